@@ -119,6 +119,63 @@ __device__ __forceinline__ float weight_rel(float lw, fpair R) {
     return x > 0.f ? __fmaf_rn(x, __fmaf_rn(d_lo, 0.5f * d_lo, d_lo), x) : 0.f;
 }
 
+// The same for two log-weights at once, in packed single precision (each half
+// rounds as the scalar operation does, so the bits are weight_rel's), without
+// the selection of zero for a zero weight: where expf gives 0 the result is 0,
+// or NaN for lw = -inf (whose error term is inf - inf).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+
+__device__ __forceinline__ float2 weight_rel2(float2 lw, float2 neg_hi, float2 neg_lo) {
+    const float2 s = __fadd2_rn(lw, neg_hi);
+    const float2 bb = sub2(s, lw);
+    const float2 e = __fadd2_rn(sub2(lw, sub2(s, bb)), sub2(neg_hi, bb));
+    const float2 d = __fadd2_rn(e, neg_lo);
+    const float2 x = make_float2(expf(s.x), expf(s.y));
+    const float2 half = make_float2(0.5f, 0.5f);
+    return __ffma2_rn(x, __ffma2_rn(d, __fmul2_rn(half, d), d), x);
+}
+
+// Minimum of three that propagates NaN (one instruction on this part).
+__device__ __forceinline__ float fmin3_nan(float a, float b, float c) {
+    float d;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// Maximum of three that propagates NaN.
+__device__ __forceinline__ float fmax3_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// ---------------------------------------------------------------------------
+// 64-bit fixed point (2^-48) <-> float without the 64-bit conversion
+// instructions, which run on the FP64 pipe: 16 cycles a warp each on this part.
+// Bit for bit the values of __float2ll_rn and of (float)(long long).
+// ---------------------------------------------------------------------------
+// __float2ll_rn(s 2^48) + __float2ll_rn(-c 2^48) for a compensated sum (s, c), s >= 0.
+__device__ __forceinline__ long long fixed48_of(float s, float c) {
+    const float sc = __fmul_rn(s, 0x1p48f), cc = __fmul_rn(-c, 0x1p48f);
+    if (!(s < 64.f)) return __float2ll_rn(sc) + __float2ll_rn(cc);  // weights far above 1, or NaN: c may be large too
+    // s < 64 has an error term below 2^-16, so cc fits 32 bits; sc is an integer from 2^24 on
+    const uint32_t b = __float_as_uint(sc);
+    const int sh = (int)(b >> 23) - 150;
+    const long long whole = (long long)((b & 0x7fffffu) | 0x800000u) << (sh > 0 ? sh : 0);
+    return (sh > 0 ? whole : (long long)__float2int_rn(sc)) + (long long)__float2int_rn(cc);
+}
+
+// (float)v 2^-48 for v >= 0: the top 32 bits of v normalised, the rest kept as a
+// sticky bit, so that one 32-bit conversion rounds to nearest as the 64-bit one.
+__device__ __forceinline__ float fixed48_to_float(long long v) {
+    const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
+    const int sh = __clz((int)hi);  // 32 when hi = 0
+    uint32_t top = __funnelshift_lc(lo, hi, sh);
+    const uint32_t rest = sh < 32 ? lo << sh : 0u;
+    top |= rest != 0u ? 1u : 0u;
+    return __fmul_rn(__uint2float_rn(top), __uint_as_float((uint32_t)(127 - 16 - sh) << 23));
+}
+
 // ---------------------------------------------------------------------------
 // Status word and bounded waits.
 // ---------------------------------------------------------------------------

@@ -23,12 +23,12 @@ constexpr int kWarps = kThreads / 32;
 struct TileShared {
     long long wtot[kWarps];  // per-warp sums of the thread totals (fixed point)
     float redf[kWarps];
-    int i_last;
+    int wlast[kWarps];  // per-warp last positive element
 };
 
 struct TileSummary {
     int k;        // tile exponent
-    fpair S;      // tile sum relative to 2^k (compensated pair)
+    fpair S;      // tile sum relative to 2^k (compensated pair); thread 0 only
     int i_last;   // tile-local index of the last positive weight, -1 if none
     int bad;      // a NaN or +inf log-weight was seen
 };
@@ -74,7 +74,7 @@ __device__ __forceinline__ void tile_load_k(const float* __restrict__ base, int 
 
 // Block-wide; every thread of the CTA must call it.  Scans base[0..n) with the
 // first `lo` slots taken as zero weights; fills th (this thread's elements) and
-// returns the tile summary (identical in every thread).
+// returns the tile summary (identical in every thread, but S in thread 0 alone).
 // KK elements per thread (n <= KK * kThreads); tile_scan picks KK from n.
 template <int KK, bool SMEM = false>  // SMEM: base is a copy of the tile in shared memory
 __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ base, int lo, int n, TileShared& sm,
@@ -84,47 +84,66 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
     th.K = KK;
     th.e0 = e0;
 
-    if (tid == 0) sm.i_last = -1;
-
     float* x = th.v;
     tile_load_k<KK, SMEM>(base, lo, n, e0, th.v);
 
-    // 1. tile maximum and domain check: the thread's maximum propagates NaN, so
-    // one test of it finds a NaN or +inf element
-    float m = -INFINITY;
+    // 1. tile maximum and domain check: the maxima propagate NaN (which the
+    // integer reduction places above +inf), so the tile's maximum alone tells
+    // whether the tile holds a NaN or +inf
+    float m = fmax_nan(x[0], x[1]);
 #pragma unroll
-    for (int i = 0; i < KK; ++i) m = fmax_nan(m, x[i]);
-    int bad = !(m <= 3.402823466e38f);
+    for (int i = 2; i < KK; i += 2) m = fmax3_nan(m, x[i], x[i + 1]);
     m = warp_max_redux(m);
     if (lane == 0) sm.redf[warp] = m;
-    bad = __syncthreads_or(bad);
+    __syncthreads();
     const float mt = warp_max_redux(lane < kWarps ? sm.redf[lane] : -INFINITY);
+    const int bad = !(mt <= 3.402823466e38f);
     const int k = tile_exponent(mt);
     const fpair R = tile_reference(k);
 
-    // 2-3. weights and the compensated per-thread scan (x[] becomes the running sum)
+    // 2. weights, two at a time; a thread all of whose weights are positive (the
+    // minimum propagates the NaN of a zero weight) skips the zero handling
+    const float2 nhi = make_float2(-R.hi, -R.hi), nlo = make_float2(-R.lo, -R.lo);
+    float mn;
+#pragma unroll
+    for (int i = 0; i < KK; i += 2) {
+        const float2 w = weight_rel2(make_float2(x[i], x[i + 1]), nhi, nlo);
+        x[i] = w.x;
+        x[i + 1] = w.y;
+        mn = i ? fmin3_nan(mn, w.x, w.y) : fmin3_nan(w.x, w.x, w.y);
+    }
+    int p = KK - 1;
+    uint32_t posbits = (1u << KK) - 1u;
+    if (!(mn > 0.f)) {
+        p = -1;
+        posbits = 0;
+#pragma unroll
+        for (int i = 0; i < KK; ++i) {
+            if (x[i] > 0.f) {
+                p = i;
+                posbits |= 1u << i;
+            } else {
+                x[i] = 0.f;
+            }
+        }
+    }
+    th.pos = posbits;
+
+    // 3. the compensated per-thread scan (x[] becomes the running sum)
     float s = 0.f, c = 0.f;
-    int p = -1;
-    uint32_t posbits = 0;
 #pragma unroll
     for (int i = 0; i < KK; ++i) {
-        const float w = weight_rel(x[i], R);
-        if (w > 0.f) {
-            p = i;
-            posbits |= 1u << i;
-        }
-        const float y = __fsub_rn(w, c);
+        const float y = __fsub_rn(x[i], c);
         const float t = __fadd_rn(s, y);
         c = __fsub_rn(__fsub_rn(t, s), y);
         s = t;
         x[i] = s;
     }
-    th.pos = posbits;
 
     // block exclusive scan of the per-thread totals in exact 64-bit fixed point
     // (resolution 2^-48 relative to 2^k; a tile sum is below 2^14): exact
     // sums are monotone, and every thread knows its own next base
-    const long long tot = __float2ll_rn(s * 0x1p48f) + __float2ll_rn(-c * 0x1p48f);
+    const long long tot = fixed48_of(s, c);
     long long inc = tot;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -133,10 +152,11 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
     }
     if (lane == 31) sm.wtot[warp] = inc;
     const int il = __reduce_max_sync(0xffffffffu, p >= 0 ? e0 + p : -1);
-    if (lane == 0 && il >= 0) atomicMax(&sm.i_last, il);
+    if (lane == 0) sm.wlast[warp] = il;
     __syncthreads();
     // every warp scans the kWarps warp totals (lane w holds warp w's)
     long long ws = lane < kWarps ? sm.wtot[lane] : 0;
+    const int i_last = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.wlast[lane] : -1);
 #pragma unroll
     for (int o = 1; o < kWarps; o <<= 1) {
         const long long h = __shfl_up_sync(0xffffffffu, ws, o);
@@ -145,19 +165,31 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
     const long long total = __shfl_sync(0xffffffffu, ws, kWarps - 1);
     const long long wbase = warp > 0 ? __shfl_sync(0xffffffffu, ws, warp - 1) : 0;
     const long long excl = wbase + inc - tot;
-    const float Vk = (float)excl * 0x1p-48f, Vn = (float)(excl + tot) * 0x1p-48f;
-    const float S_hi = (float)total;
-    const fpair S = {S_hi * 0x1p-48f, (float)(total - (long long)S_hi) * 0x1p-48f};
+    const float Vk = fixed48_to_float(excl), Vn = fixed48_to_float(excl + tot);
 
     // 4. tile-local cumulative weights; elements from the last positive one on
     // take the next base so that no gap is left between threads
+    if (p == KK - 1) {
+        const float2 Vk2 = make_float2(Vk, Vk);
 #pragma unroll
-    for (int i = 0; i < KK; ++i) x[i] = (i >= p) ? Vn : fminf(__fadd_rn(Vk, x[i]), Vn);
+        for (int i = 0; i < KK; i += 2) {
+            const float2 v = __fadd2_rn(Vk2, make_float2(x[i], x[i + 1]));
+            x[i] = fminf(v.x, Vn);
+            x[i + 1] = i + 1 < KK - 1 ? fminf(v.y, Vn) : Vn;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < KK; ++i) x[i] = (i >= p) ? Vn : fminf(__fadd_rn(Vk, x[i]), Vn);
+    }
 
     TileSummary ts;
     ts.k = k;
-    ts.S = S;
-    ts.i_last = sm.i_last;
+    ts.S = {0.f, 0.f};
+    if (tid == 0) {  // the tile sum, a pair: thread 0 records it
+        const float S_hi = (float)total;
+        ts.S = {S_hi * 0x1p-48f, (float)(total - (long long)S_hi) * 0x1p-48f};
+    }
+    ts.i_last = i_last;
     ts.bad = bad;
     return ts;
 }
