@@ -368,6 +368,237 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same assignment warp by warp, for tiles of at most kWarpOffsets offsets
+// (nearly all: a tile's count varies around its length).  No barrier of the CTA:
+// a warp's elements own one contiguous range of the tile's offsets, and where
+// that range begins follows from the thread's base (the cumulative weight of the
+// element before its first), because the element before it has exactly that
+// cumulative weight and so the same count N.  Each warp marks its runs in its
+// own 32 S staging entries (all -1 between chunks), a warp max-scan fills them,
+// and the entries are set back to -1 as they are read for the last time.
+//
+// The CTA-wide decode below this bound waited at three barriers a tile with 40% of
+// the issue slots used.  Systematic launch at P = 2^25 + 4096 94 us (41 instructions
+// per particle), stratified 156 us (88); whole calls now: stratified at 10^8
+// particles 691 -> 527 us, 4096 filters systematic 293 -> 264 us, the 2^24 heavy-tail
+// step 252 -> 230 us.
+//
+// N by a rounded addition: y + 1.5 2^23 rounded up (down) has ceil(y)
+// (floor(y)) in its low bits, exact for |y| < 2^22; it replaces the conversion,
+// which issues at a quarter of the rate.  y is monotone along the thread, so only
+// a thread whose first or last count falls outside the tile's range clamps.
+// ---------------------------------------------------------------------------
+// A tile with more offsets than this goes to the CTA-wide decode: its excess sits in
+// few warps (the mean is 512 offsets a warp), and one warp decoding 16384 offsets alone
+// takes about 26 chunks, the time the CTA needs for two of its own and the two clears.
+constexpr int kWarpOffsets = 2 * kTileMax;
+constexpr float kRoundMagic = 12582912.f;      // 1.5 2^23
+constexpr int kRoundMagicBits = 0x4b400000;
+
+// Staging entries per lane: 32 S covers a warp's usual range (its 32 KK elements'
+// worth of offsets and four standard deviations of N(0,1) weights) in one chunk, and an
+// odd multiple of four words between lanes keeps the 16-byte reads free of bank conflicts.
+constexpr int warp_stage_per_lane(int KK) { return KK == 16 ? 20 : (KK == 8 ? 12 : 8); }
+
+// marks: this warp's 32 S entries, 16-byte aligned, all -1 on entry and on return.
+// ubuf (stratified): this warp's 32 S floats for the strata's uniforms.
+template <int KIND, int KK, int S>
+__device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap map, int32_t* marks, float* ubuf,
+                                            TileThread& th, int i_last, int64_t index0) {
+    const int lane = threadIdx.x & 31;
+    const int noff = map.noff;
+    if (noff <= 0) return;
+    const float x0 = map.x0, ir = map.ir;
+    constexpr uint32_t kFull = (1u << KK) - 1u;
+    const uint32_t pos = th.pos;
+    if (!__any_sync(0xffffffffu, pos != 0u)) return;  // no positive weight in the warp
+    const int il = i_last - th.e0;  // this thread's index of the tile's last positive element, if any
+    const float yb = __fmaf_rn(th.base, ir, x0), yl = __fmaf_rn(th.v[KK - 1], ir, x0);
+    int start0;  // offsets below the element before this thread's first
+    if (KIND == KIND_SYS) {
+        const int nb = __float_as_int(__fadd_ru(yb, kRoundMagic)) - kRoundMagicBits;
+        const int nl = __float_as_int(__fadd_ru(yl, kRoundMagic)) - kRoundMagicBits;
+        start0 = min(max(nb, 0), noff);
+        const bool clamp = nb < 0 || nl > noff;
+#pragma unroll
+        for (int i = 0; i < KK; ++i)
+            th.v[i] = __int_as_float(__float_as_int(__fadd_ru(__fmaf_rn(th.v[i], ir, x0), kRoundMagic)) - kRoundMagicBits);
+        if (clamp) {
+#pragma unroll
+            for (int i = 0; i < KK; ++i)
+                th.v[i] = __int_as_float(min(max(__float_as_int(th.v[i]), 0), noff));
+        }
+    } else {
+        const int kmax = noff - 1;
+        // stratum of a coordinate and the coordinate's place in it
+        auto stratum = [&](float y, float& frac) -> int {
+            const float t = __fadd_rd(y, kRoundMagic);
+            int k = __float_as_int(t) - kRoundMagicBits;
+            frac = __fsub_rn(y, __fsub_rn(t, kRoundMagic));
+            return k;
+        };
+        float fb, fl;
+        const int kb0 = stratum(yb, fb), kl0 = stratum(yl, fl);
+        const bool clamp = kb0 < 0 || kl0 > kmax;
+        const int kb = min(max(kb0, 0), kmax), kl = min(max(kl0, 0), kmax);
+        if (clamp) fb = __fsub_rn(yb, (float)kb);
+        // the uniforms of the warp's strata, four per Philox block, drawn once into ubuf
+        const int k_first = __shfl_sync(0xffffffffu, kb, 0);
+        const int k_last = __reduce_max_sync(0xffffffffu, max(kb, kl));
+        const long long g0 = (map.jlo + k_first) >> 2;
+        const int blocks = (int)(((map.jlo + k_last) >> 2) - g0) + 1;
+        const int at = (int)(map.jlo - 4 * g0);  // ubuf index of stratum 0 (may be negative)
+        if (blocks <= 8 * S) {
+            __syncwarp();  // the last tile's reads of ubuf
+            for (int b = lane; b < blocks; b += 32) {
+                const u32x4 r = philox((uint32_t)(g0 + b), 0u, p.filter, TAG_STRAT, p.key0, p.key1);
+                *reinterpret_cast<float4*>(ubuf + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
+            }
+            __syncwarp();
+            start0 = min(noff, kb + (ubuf[at + kb] < fb ? 1 : 0));
+            if (!clamp) {
+#pragma unroll
+                for (int i = 0; i < KK; ++i) {
+                    float frac;
+                    const int k = stratum(__fmaf_rn(th.v[i], ir, x0), frac);
+                    th.v[i] = __int_as_float(k + (ubuf[at + k] < frac ? 1 : 0));
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < KK; ++i) {
+                    const float y = __fmaf_rn(th.v[i], ir, x0);
+                    float frac;
+                    const int k = min(max(stratum(y, frac), 0), kmax);
+                    th.v[i] = __int_as_float(min(noff, k + (ubuf[at + k] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                }
+            }
+        } else {
+            // strata beyond the buffer (a dominant particle): each thread draws the blocks its elements need
+            uint32_t cq = 0xffffffffu;
+            u32x4 cw = {0, 0, 0, 0};
+            auto u_of = [&](int k) -> float {
+                const long long j = map.jlo + k;
+                const uint32_t q = (uint32_t)(j >> 2);
+                if (q != cq) {
+                    cq = q;
+                    cw = philox(q, 0u, p.filter, TAG_STRAT, p.key0, p.key1);
+                }
+                return u23f(word_of(cw, (int)(j & 3)));
+            };
+            start0 = min(noff, kb + (u_of(kb) < fb ? 1 : 0));
+#pragma unroll
+            for (int i = 0; i < KK; ++i) {
+                const float y = __fmaf_rn(th.v[i], ir, x0);
+                float frac;
+                const int k = min(max(stratum(y, frac), 0), kmax);
+                th.v[i] = __int_as_float(min(noff, k + (u_of(k) < __fsub_rn(y, (float)k) ? 1 : 0)));
+            }
+        }
+    }
+    int last_n;  // count at this thread's last positive element
+    if ((uint32_t)il < (uint32_t)KK || pos != kFull) {
+        last_n = start0;
+#pragma unroll
+        for (int i = 0; i < KK; ++i) {
+            if (i == il) th.v[i] = __int_as_float(noff);  // the tile's last positive element takes the rest
+            if ((pos >> i) & 1u) last_n = __float_as_int(th.v[i]);
+        }
+    } else {
+        last_n = __float_as_int(th.v[KK - 1]);
+    }
+    const int A = __shfl_sync(0xffffffffu, start0, 0);
+    const int B = __reduce_max_sync(0xffffffffu, pos ? last_n : 0);
+    const int32_t e_base = (int32_t)index0 + th.e0;  // ancestor of this thread's element 0
+    const int xl = lane * S;
+    for (int c0 = A; c0 < B;) {
+        const int shift = (int)(((uintptr_t)(p.anc + map.jlo + c0) >> 2) & 3u);  // to a 16-byte boundary
+        const int c1 = min(B, c0 + 32 * S - shift);
+        // marks: each run's first slot in the chunk
+        int a = start0;
+        int32_t* mk = marks + (shift - c0);
+        if (c0 == A && c1 == B && pos == kFull) {  // the usual case: one chunk, every weight positive
+#pragma unroll
+            for (int i = 0; i < KK; ++i) {
+                const int b = __float_as_int(th.v[i]);
+                if (b > a) mk[a] = e_base + i;
+                a = b;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KK; ++i) {
+                if ((pos >> i) & 1u) {
+                    const int b = __float_as_int(th.v[i]);
+                    const int m = max(a, c0);
+                    if (b > m && m < c1) mk[m] = e_base + i;
+                    a = b;
+                }
+            }
+        }
+        __syncwarp();
+        int run = -1;
+#pragma unroll
+        for (int q = 0; q < S / 4; ++q) {
+            const int4 v = *reinterpret_cast<const int4*>(&marks[xl + 4 * q]);
+            run = max(run, max(max(v.x, v.y), max(v.z, v.w)));
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int h = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run = max(run, h);
+        }
+        int rr = __shfl_up_sync(0xffffffffu, run, 1);
+        if (lane == 0) rr = -1;
+        const int end = shift + (c1 - c0);  // the chunk's entries: [shift, end)
+        int32_t* g = p.anc + (map.jlo + c0 - shift) + xl;  // 16-byte aligned
+#pragma unroll
+        for (int q = 0; q < S / 4; ++q) {
+            const int x = xl + 4 * q;
+            int4 v = *reinterpret_cast<const int4*>(&marks[x]);
+            *reinterpret_cast<int4*>(&marks[x]) = make_int4(-1, -1, -1, -1);
+            v.x = rr = max(rr, v.x);
+            v.y = rr = max(rr, v.y);
+            v.z = rr = max(rr, v.z);
+            v.w = rr = max(rr, v.w);
+            if (x >= shift && x + 4 <= end) {
+                *reinterpret_cast<int4*>(g + 4 * q) = v;
+            } else if (x + 4 > shift && x < end) {
+                if (x >= shift) g[4 * q] = v.x;
+                if (x + 1 >= shift && x + 1 < end) g[4 * q + 1] = v.y;
+                if (x + 2 >= shift && x + 2 < end) g[4 * q + 2] = v.z;
+                if (x + 3 < end) g[4 * q + 3] = v.w;
+            }
+        }
+        __syncwarp();  // the entries are clear before the next marks
+        c0 = c1;
+    }
+}
+
+// One tile's assignment: warp by warp, or, for a tile that owns so many offsets
+// that one warp's share could be most of them, chunk by chunk over the CTA (whose
+// staging starts and leaves everything at -1).  Block-uniform choice.
+template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK)>
+__device__ __forceinline__ void assign_tile(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
+                                            TileThread& th, const TileSummary& ts, int64_t index0) {
+    // a warp's entries lie at the same place whatever KK and S: the CTA's warps may be in
+    // different tiles, of different KK
+    constexpr int kStride = (KIND == KIND_STRAT || CAP >= kIoCapSmall ? CAP : 2 * CAP) / kWarps;
+    static_assert(32 * S <= kStride && kStride % 4 == 0, "a warp's entries fit its share of the staging");
+    if (map.noff <= kWarpOffsets) {
+        const int at = (threadIdx.x >> 5) * kStride;
+        assign_warp<KIND, KK, S>(p, map, stage + at, reinterpret_cast<float*>(stage + CAP) + at, th, ts.i_last, index0);
+        return;
+    }
+    __syncthreads();
+    stage_init<CAP>(stage);
+    __syncthreads();
+    uint32_t epoch = 0;
+    assign_offspring<KIND, KK, CAP>(p, sm, map, stage, epoch, th, ts, index0);
+    __syncthreads();
+    stage_init<CAP>(stage);
+    __syncthreads();
+}
+
 // Four multinomial draws (the words of one Philox block) of one filter
 // (Figure 1a).  Draw s targets u_s W (float pair); a binary search over the
 // tile table (shared memory) finds the last tile whose carry is <= the
@@ -828,47 +1059,100 @@ __device__ __forceinline__ void write_tile_samples(const TileThread& th, int n, 
     }
 }
 
+// Eight floats in one 256-bit access (32-byte aligned): a thread's share of a tile
+// is 64 bytes, so each access moves whole 32-byte sectors where two 128-bit ones
+// move each sector twice.
+__device__ __forceinline__ void ld_cg_v8(const float* p, float* o) {
+    asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]), "=f"(o[4]), "=f"(o[5]), "=f"(o[6]), "=f"(o[7])
+                 : "l"(p)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_v8(float* p, const float* o) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(o[0]), "f"(o[1]), "f"(o[2]),
+                 "f"(o[3]), "f"(o[4]), "f"(o[5]), "f"(o[6]), "f"(o[7])
+                 : "memory");
+}
+
 // Reloads a tile stored by write_tile_v into th (elements of tile-local
 // indices [0, n)): v from the magnitudes, the positive-weight mask from the
 // sign bits.  Slots at or beyond n are not read.  SMEM: vg0 is a copy of the
-// tile in shared memory.
+// tile in shared memory.  Every lane of the warp must call it (the bases come
+// from the lane below).
 template <int KK = 0, bool SMEM = false>  // KK: elements per thread when fixed (the tile was scanned with KK), 0 = from n
 __device__ __forceinline__ void read_tile_v(const float* vg0, int n, TileThread& th) {
     const int K = KK ? KK : per_thread_count(n);
     th.K = K;
     th.e0 = threadIdx.x * K;
     const float* vg = vg0 + th.e0;
-    uint32_t pos = 0;
+    const bool whole = th.e0 + K <= n;
+    if (!SMEM && KK >= 8 && whole && (((uintptr_t)vg) & 31u) == 0) {
 #pragma unroll
-    for (int q = 0; q < kMaxPerThread / 4; ++q) {
-        if (4 * q < K) {
-            float o[4];
-            if (th.e0 + 4 * q + 3 < n) {
-                const float4 t = SMEM ? *reinterpret_cast<const float4*>(vg + 4 * q)
-                                      : __ldcg(reinterpret_cast<const float4*>(vg + 4 * q));
-                o[0] = t.x;
-                o[1] = t.y;
-                o[2] = t.z;
-                o[3] = t.w;
-            } else {
+        for (int q = 0; q < KK / 8; ++q) ld_cg_v8(vg + 8 * q, th.v + 8 * q);
+    } else {
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    o[r] = th.e0 + 4 * q + r < n ? (SMEM ? vg[4 * q + r] : __ldcg(vg + 4 * q + r)) : -0.0f;
-            }
+        for (int q = 0; q < kMaxPerThread / 4; ++q) {
+            if (4 * q < K) {
+                if (th.e0 + 4 * q + 3 < n) {
+                    const float4 t = SMEM ? *reinterpret_cast<const float4*>(vg + 4 * q)
+                                          : __ldcg(reinterpret_cast<const float4*>(vg + 4 * q));
+                    th.v[4 * q] = t.x;
+                    th.v[4 * q + 1] = t.y;
+                    th.v[4 * q + 2] = t.z;
+                    th.v[4 * q + 3] = t.w;
+                } else {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                th.v[4 * q + r] = fabsf(o[r]);
-                if (!zero_flag(o[r])) pos |= 1u << (4 * q + r);
+                    for (int r = 0; r < 4; ++r)
+                        th.v[4 * q + r] = th.e0 + 4 * q + r < n ? (SMEM ? vg[4 * q + r] : __ldcg(vg + 4 * q + r)) : -0.0f;
+                }
             }
         }
     }
+    // the sign bits: none set in the usual thread
+    uint32_t any = 0, pos = K >= 32 ? 0xffffffffu : (1u << K) - 1u;
+#pragma unroll
+    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
+        if (KK || i < K) any |= __float_as_uint(th.v[i]);
+    if (any >> 31) {
+        pos = 0;
+        float run = 0.f;
+#pragma unroll
+        for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
+            if (KK || i < K) {
+                if (!zero_flag(th.v[i])) pos |= 1u << i;
+                // monotone also past the tile's end, where -0 stands for no element
+                th.v[i] = run = fmaxf(run, fabsf(th.v[i]));
+            }
+    }
     th.pos = pos;
+    // the element before this thread's first: the lane below's last, or a load by lane 0
+    float last = th.v[0];
+#pragma unroll
+    for (int i = 1; i < (KK ? KK : kMaxPerThread); ++i)
+        if (KK || i < K) last = th.v[i];
+    th.base = __shfl_up_sync(0xffffffffu, last, 1);
+    if ((threadIdx.x & 31) == 0)
+        th.base = th.e0 > 0 && th.e0 <= n ? fabsf(SMEM ? vg[-1] : __ldcg(vg - 1)) : 0.f;
 }
 
 // The tile's cumulative weights to global memory (sign bit: zero weight), for the searches.
 template <int KK = 0>
 __device__ __forceinline__ void write_tile_v(const SortedParams& p, const TileThread& th, int64_t t0, int n) {
     float* vg = p.v_out + t0 + th.e0;
+    const int K = KK ? KK : th.K;
+    if (KK && th.pos == (1u << KK) - 1u && th.e0 + K <= n) {  // the usual thread: whole, every weight positive
+        if (KK >= 8 && (((uintptr_t)vg) & 31u) == 0) {
+#pragma unroll
+            for (int q = 0; q < KK / 8; ++q) st_v8(vg + 8 * q, th.v + 8 * q);
+        } else {
+#pragma unroll
+            for (int q = 0; q < KK / 4; ++q)
+                *reinterpret_cast<float4*>(vg + 4 * q) =
+                    make_float4(th.v[4 * q], th.v[4 * q + 1], th.v[4 * q + 2], th.v[4 * q + 3]);
+        }
+        return;
+    }
 #pragma unroll
     for (int q = 0; q < (KK ? KK : kMaxPerThread) / 4; ++q) {
         if (KK || 4 * q < th.K) {

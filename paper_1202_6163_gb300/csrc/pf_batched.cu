@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
     const int tid = threadIdx.x, lane = tid & 31;
     const int n_items = (int)ld_relaxed_u32(bp.ctl + CTL_ITEMS);
     TileThread th;
-    uint32_t chunks = 0;  // staging chunks decoded by this CTA
     if (KIND != KIND_MULTI) stage_init<kIoCap>(reinterpret_cast<int32_t*>(region));  // before the first ticket's barriers
     for (;;) {
         if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
@@ -206,11 +205,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                     ts.i_last = sm.ril[c];
                     const TileMap map = sm.maps[c];
                     if (th.K == 16)
-                        assign_offspring<KIND, 16>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 16, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else if (th.K == 8)
-                        assign_offspring<KIND, 8>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 8, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else
-                        assign_offspring<KIND, 4>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 4, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                 }
                 if (bp.trace) {
                     __syncthreads();
@@ -276,11 +275,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                     const TileMap map = {sm.as.jlo, sm.as.noff, sm.as.tau0, sm.as.inv_rho};
                     // elements per thread as a constant: 16 for full tiles, fewer for small filters
                     if (th.K == 16)
-                        assign_offspring<KIND, 16>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 16, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else if (th.K == 8)
-                        assign_offspring<KIND, 8>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 8, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else
-                        assign_offspring<KIND, 4>(p, sm.as, map, stage, chunks, th, ts, t0 - lead);
+                        assign_tile<KIND, 4, kIoCap>(p, sm.as, map, stage, th, ts, t0 - lead);
                     if (bp.trace) {
                         __syncthreads();
                         trace_stamp(bp.trace, bp.trace_cap, ticket, 4);

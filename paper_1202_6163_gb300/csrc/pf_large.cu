@@ -230,7 +230,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, co
     // tile r + 1's copy is issued once every thread has taken tile r out of the
     // buffer, and lands while tile r is assigned
     if (tid == 0) issue_tile_copy(p.v_out, PA, 0, vbuf, &sm.bar);
-    uint32_t chunks = 0;  // staging chunks decoded by this CTA
     TileThread th;
     for (int r = 0; r < n_mine; ++r) {
         const int t = (int)blockIdx.x + r * (int)gridDim.x;
@@ -255,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, co
         fence_proxy_async_smem();  // this thread's reads of the buffer before its next copy
         __syncthreads();
         if (tid == 0 && r + 1 < n_mine) issue_tile_copy(p.v_out, PA, r + 1, vbuf, &sm.bar);
-        assign_offspring<KIND, 16, kIoCap>(p, sm.as, sm.map, stage, chunks, th, ts, t0 - p.lead);
+        assign_tile<KIND, 16, kIoCap>(p, sm.as, sm.map, stage, th, ts, t0 - p.lead);
         __syncthreads();  // the map is reused by the next tile
     }
 }
@@ -282,7 +281,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_guide(SortedParams pg, in
     }
     stage_init<kIoCap>(stage);
     __syncthreads();
-    uint32_t chunks = 0;
     TileThread th;
     for (int t = blockIdx.x; t < pg.n_tiles; t += gridDim.x) {
         const int64_t t0 = (int64_t)t * kLargeTile;
@@ -299,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_guide(SortedParams pg, in
             if (tid == 0) sm.map = m;
         }
         __syncthreads();
-        assign_offspring<KIND_SYS, 16, kIoCap>(pg, sm.as, sm.map, stage, chunks, th, ts, t0 - pg.lead);
+        assign_tile<KIND_SYS, 16, kIoCap, 8>(pg, sm.as, sm.map, stage, th, ts, t0 - pg.lead);
         __syncthreads();
     }
 }

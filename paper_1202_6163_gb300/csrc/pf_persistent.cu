@@ -372,6 +372,7 @@ __device__ void multinomial_draws(const SortedParams& p, PersistShared& sm, cons
 // before any draw reads one.  Returns false when that wait ran out.
 // ---------------------------------------------------------------------------
 constexpr int kGuideCap = 2048;  // staging entries per buffer: offsets per chunk + room for the shift
+constexpr int kGuidePerLane = 8; // the warp decode's entries per lane: a warp's 512 elements hold ~128 bucket edges
 static_assert(2 * kGuideCap <= kLut + 1, "the guide's staging fits the tile lookup's area");
 
 template <int KK>
@@ -392,14 +393,13 @@ __device__ bool build_guide(const SortedParams& p, PersistShared& sm, int32_t* s
     }
     __syncthreads();
     const int64_t PA = p.P + p.lead;
-    uint32_t chunks = 0;
     for (int r = t_count - 1; r >= 0; --r) {  // the last tile's scan is still in registers
         const int64_t t0 = (int64_t)(t_first + r) * p.tile;
         if (r != t_count - 1) {
             read_tile_v<KK>(p.v_out + t0, (int)min((int64_t)p.tile, PA - t0), th);
             ts.i_last = sm.own_il[r];
         }
-        assign_offspring<KIND_SYS, KK, kGuideCap>(pg, sm.as, sm.own_map[r], stage, chunks, th, ts, t0 - p.lead);
+        assign_tile<KIND_SYS, KK, kGuideCap, kGuidePerLane>(pg, sm.as, sm.own_map[r], stage, th, ts, t0 - p.lead);
     }
     __threadfence();
     __syncthreads();
@@ -560,7 +560,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
     // pass 2: offsets of every owned tile (the last tile's scan is still in
     // registers; the others reload their cumulative weights)
     int32_t* stage = reinterpret_cast<int32_t*>(region);
-    uint32_t chunks = 0;  // staging chunks decoded by this CTA
     for (int r = t_count - 1; r >= 0; --r) {
         const int t = t_first + r;
         const int64_t t0 = (int64_t)t * p.tile;
@@ -568,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
             read_tile_v<KK>(p.v_out + t0, (int)min((int64_t)p.tile, PA - t0), th);
             ts.i_last = sm.own_il[r];
         }
-        assign_offspring<KIND, KK, stage_cap(KK)>(p, sm.as, sm.own_map[r], stage, chunks, th, ts, t0 - p.lead);
+        assign_tile<KIND, KK, stage_cap(KK)>(p, sm.as, sm.own_map[r], stage, th, ts, t0 - p.lead);
     }
     if (p.trace) {
         __syncthreads();
