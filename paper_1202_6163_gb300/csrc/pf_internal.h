@@ -33,6 +33,7 @@ enum : int {
     CTL_HEAVY = 11,       // batched Metropolis: filters on the list of shared (heavy) filters
     CTL_ARRIVE2 = 12,     // second arrival counters of the single-launch multinomial kernel
     CTL_ARRIVE3 = 13,     //   (after its guide table), alternating like CTL_ARRIVE0 / 1
+    CTL_PERM_COUNT = 14,  // CTAs done in the permutation's tile sums (zero between calls)
     CTL_WORDS = 16
 };
 

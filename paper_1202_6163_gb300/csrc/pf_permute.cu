@@ -10,16 +10,26 @@
 // moved in place: row j is overwritten only if particle j has no offspring,
 // and every row read belongs to a particle that keeps its slot.
 //
-// Passes (all bandwidth-light): offspring counts (atomics); per-tile sums of
-// the extra copies max(o_i - 1, 0) and of the empty slots [o_i == 0]; their
-// exclusive scan; placement (survivors to their own slot, each survivor's run
-// start marked in the extras list E, each empty slot listed in DS); a
-// max-scan over E that fills the runs (survivor indices increase along E);
-// and the fill out[DS[r]] = E[r].
+// Passes, each over tiles of 4096 slots: offspring counts o (one atomic per run of
+// equal neighbours in a row of 32: sorted ancestors, as the offset schemes give
+// them, need one per survivor); per-tile sums of the extra copies max(o_i - 1, 0)
+// and of the empty slots [o_i == 0], whose last CTA to finish forms their
+// exclusive scans; the list E of the extra copies, each tile's run starts marked
+// in shared memory and filled by a block max-scan (tiles with more than kPermPart
+// extras are split over several CTAs); and the result, every slot written once in
+// order: i where o_i > 0, else E at the rank of the empty slot.
+//
+// Bound by its launches and by L2 latency (five passes of 4 bytes a slot, of which
+// only the first and the last touch the caller's arrays): one memset and four
+// launches where there were three memsets and seven.  Stratified resampling,
+// permutation and in-place move of 3 M rows of 64 bytes: 212 -> 150 us, and 136 us
+// with the rows in 256-bit chunks.
 #include <climits>
+#include <type_traits>
 
 #include "pf_device.cuh"
 #include "pf_internal.h"
+#include "pf_rows.cuh"
 
 namespace pf {
 namespace {
@@ -28,14 +38,35 @@ constexpr int kPermThreads = 512;
 constexpr int kPermPer = 8;
 constexpr int kPermTile = kPermThreads * kPermPer;
 constexpr int kPermWarps = kPermThreads / 32;
-constexpr int kScanThreads = 1024;
+constexpr int kPermPart = 8192;  // extras one CTA lists: twice a tile's mean share
 
+// One count per ancestor.  A warp takes four rows of 32 consecutive entries; the
+// first lane of each run of equal entries in a row adds the run's length.
 __global__ void __launch_bounds__(256) k_perm_count(const int32_t* __restrict__ anc, int64_t P,
                                                     int32_t* __restrict__ o, uint32_t* ctl) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < P; j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t a = anc[j];
-        if (a < 0 || a >= P) set_status(ctl + CTL_STATUS, ST_INVALID);
-        else atomicAdd(o + a, 1);
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 128; j0 < P; j0 += warps * 128) {
+        int32_t a[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int64_t j = j0 + 32 * r + lane;
+            a[r] = j < P ? __ldg(anc + j) : INT_MIN;  // INT_MIN: past the end, counted nowhere
+            if (j < P && (a[r] < 0 || a[r] >= P)) {
+                set_status(ctl + CTL_STATUS, ST_INVALID);
+                a[r] = INT_MIN;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int32_t below = __shfl_up_sync(0xffffffffu, a[r], 1);
+            const bool head = lane == 0 || below != a[r];
+            const uint32_t heads = __ballot_sync(0xffffffffu, head);
+            if (head && a[r] >= 0) {
+                const uint32_t later = heads & ~(0xffffffffu >> (31 - lane));  // heads above this lane
+                atomicAdd(o + a[r], (later ? __ffs((int)later) - 1 : 32) - lane);
+            }
+        }
     }
 }
 
@@ -50,246 +81,274 @@ __device__ __forceinline__ int block_excl_scan(int x, int* red, int& total) {
     }
     if (lane == 31) red[warp] = inc;
     __syncthreads();
-    int base = 0;
-    total = 0;
+    int w = lane < kPermWarps ? red[lane] : 0;
 #pragma unroll
-    for (int w = 0; w < kPermWarps; ++w) {
-        const int v = red[w];
-        base += w < warp ? v : 0;
-        total += v;
+    for (int off = 1; off < kPermWarps; off <<= 1) {
+        const int h = __shfl_up_sync(0xffffffffu, w, off);
+        if (lane >= off) w += h;
     }
+    total = __shfl_sync(0xffffffffu, w, kPermWarps - 1);
+    const int base = warp > 0 ? __shfl_sync(0xffffffffu, w, warp - 1) : 0;
     __syncthreads();
     return base + inc - x;
 }
 
+// This thread's kPermPer counts of its tile (1 past the end: neither extra nor empty).
+__device__ __forceinline__ void load_counts(const int32_t* __restrict__ o, int64_t i0, int64_t P, int (&c)[kPermPer]) {
+    if (i0 + kPermPer <= P) {  // the counts start on a 256-byte boundary
+#pragma unroll
+        for (int q = 0; q < kPermPer / 4; ++q) {
+            const int4 v = __ldg(reinterpret_cast<const int4*>(o + i0) + q);
+            c[4 * q] = v.x;
+            c[4 * q + 1] = v.y;
+            c[4 * q + 2] = v.z;
+            c[4 * q + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) c[k] = i0 + k < P ? __ldg(o + i0 + k) : 1;
+    }
+}
+
+// Per-tile prefixes: extra copies, empty slots, and parts (CTAs of the listing pass).
+struct TilePrefix {
+    int32_t extra, dead, part;
+};
+
+// Tile sums; the last CTA to finish turns them into exclusive prefixes, pre[T] holding the totals.
 __global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* __restrict__ o, int64_t P,
-                                                             int32_t* __restrict__ t_extra, int32_t* __restrict__ t_dead) {
+                                                             TilePrefix* __restrict__ pre, int T, uint32_t* ctl) {
     __shared__ int red[kPermWarps];
-    const int64_t i0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
+    __shared__ int last;
+    int c[kPermPer];
+    load_counts(o, (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer, P, c);
     int e = 0, d = 0;
 #pragma unroll
     for (int k = 0; k < kPermPer; ++k) {
-        if (i0 + k < P) {
-            const int c = o[i0 + k];
-            e += c > 1 ? c - 1 : 0;
-            d += c == 0;
-        }
+        e += c[k] > 1 ? c[k] - 1 : 0;
+        d += c[k] == 0;
     }
     int te, td;
     block_excl_scan(e, red, te);
     block_excl_scan(d, red, td);
     if (threadIdx.x == 0) {
-        t_extra[blockIdx.x] = te;
-        t_dead[blockIdx.x] = td;
+        pre[blockIdx.x] = {te, td, 0};
+        __threadfence();
+        last = atomicAdd(ctl + CTL_PERM_COUNT, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    int ce = 0, cd = 0, cp = 0;  // carries over rounds of kPermThreads tiles
+    for (int base = 0; base < T; base += kPermThreads) {
+        const int t = base + threadIdx.x;
+        const int xe = t < T ? __ldcg(&pre[t].extra) : 0, xd = t < T ? __ldcg(&pre[t].dead) : 0;
+        const int xp = (xe + kPermPart - 1) / kPermPart;
+        int se, sd, sp;
+        const int pe = block_excl_scan(xe, red, se), pd = block_excl_scan(xd, red, sd), pp = block_excl_scan(xp, red, sp);
+        if (t < T) pre[t] = {ce + pe, cd + pd, cp + pp};
+        ce += se;
+        cd += sd;
+        cp += sp;
+    }
+    if (threadIdx.x == 0) {
+        pre[T] = {ce, cd, cp};
+        ctl[CTL_PERM_COUNT] = 0u;  // ready for the next call on this stream
     }
 }
 
-// One CTA: exclusive scans (sum) of two arrays of T ints, in place; or, with
-// max_mode, an exclusive running maximum of one array (starting at -1).
-__global__ void __launch_bounds__(kScanThreads) k_perm_scan(int32_t* a, int32_t* b, int T, int max_mode) {
-    __shared__ int red[kScanThreads / 32];
-    __shared__ int carry_a, carry_b;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        carry_a = max_mode ? -1 : 0;
-        carry_b = 0;
-    }
-    __syncthreads();
-    for (int base = 0; base < T; base += kScanThreads) {
-        const int t = base + threadIdx.x;
-        for (int which = 0; which < (max_mode ? 1 : 2); ++which) {
-            int32_t* arr = which ? b : a;
-            const int x = t < T ? arr[t] : (max_mode ? -1 : 0);
-            int inc = x;
+// Lists the extra copies: E[r], r < extras, in increasing particle order.  CTA b is
+// part b of the listing: part pt of tile t, ranks [pt kPermPart, ...) of the tile's.
+__global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __restrict__ o, int64_t P,
+                                                            const TilePrefix* __restrict__ pre, int T,
+                                                            int32_t* __restrict__ E) {
+    __shared__ int red[kPermWarps];
+    __shared__ __align__(16) int32_t mark[kPermPart + 4];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int b = blockIdx.x; b < pre[T].part; b += gridDim.x) {
+        int lo = 0, hi = T - 1;  // the last tile with pre.part <= b
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(&pre[mid].part) <= b) lo = mid;
+            else hi = mid - 1;
+        }
+        const int t = lo;
+        const int s0 = (b - __ldg(&pre[t].part)) * kPermPart;                          // this part's ranks within the tile:
+        const int s1 = min(s0 + kPermPart, __ldg(&pre[t + 1].extra) - __ldg(&pre[t].extra));  // [s0, s1)
+        int32_t* out = E + __ldg(&pre[t].extra) + s0;
+        const int shift = (int)(((uintptr_t)out >> 2) & 3u);  // to a 16-byte boundary
+        const int end = s1 - s0 + shift;
+        for (int i = 4 * tid; i < end; i += 4 * kPermThreads)
+            *reinterpret_cast<int4*>(mark + i) = make_int4(-1, -1, -1, -1);
+        const int64_t i0 = (int64_t)t * kPermTile + (int64_t)tid * kPermPer;
+        int c[kPermPer];
+        load_counts(o, i0, P, c);
+        int e = 0, te;
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) e += c[k] > 1 ? c[k] - 1 : 0;
+        int r = block_excl_scan(e, red, te);  // also orders the clears before the marks
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) {
+            if (c[k] > 1) {
+                const int r1 = r + c[k] - 1;
+                if (r1 > s0 && r < s1) mark[max(r, s0) - s0 + shift] = (int32_t)(i0 + k);
+                r = r1;
+            }
+        }
+        __syncthreads();
+        // running maximum over the marks, four entries a thread and round
+        int carry = -1;
+        for (int x0 = 0; x0 < end; x0 += 4 * kPermThreads) {
+            const int x = x0 + 4 * tid;
+            int4 v = make_int4(-1, -1, -1, -1);
+            if (x < end) v = *reinterpret_cast<const int4*>(mark + x);
+            v.y = max(v.x, v.y);
+            v.z = max(v.y, v.z);
+            v.w = max(v.z, v.w);
+            int m = v.w;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
-                const int h = __shfl_up_sync(0xffffffffu, inc, off);
-                if (lane >= off) inc = max_mode ? max(inc, h) : inc + h;
+                const int h = __shfl_up_sync(0xffffffffu, m, off);
+                if (lane >= off) m = max(m, h);
             }
-            if (lane == 31) red[warp] = inc;
+            int below = __shfl_up_sync(0xffffffffu, m, 1);
+            if (lane == 0) below = -1;
+            if (lane == 31) red[warp] = m;
             __syncthreads();
-            int wb = max_mode ? -1 : 0, tot = max_mode ? -1 : 0;
-            for (int w = 0; w < kScanThreads / 32; ++w) {
-                const int v = red[w];
-                if (w < warp) wb = max_mode ? max(wb, v) : wb + v;
-                tot = max_mode ? max(tot, v) : tot + v;
+            below = max(max(below, carry), __reduce_max_sync(0xffffffffu, lane < warp ? red[lane] : -1));
+            carry = max(carry, __reduce_max_sync(0xffffffffu, lane < kPermWarps ? red[lane] : -1));
+            v.x = max(v.x, below);
+            v.y = max(v.y, below);
+            v.z = max(v.z, below);
+            v.w = max(v.w, below);
+            int32_t* g = out - shift + x;  // 16-byte aligned
+            if (x >= shift && x + 4 <= end) {
+                *reinterpret_cast<int4*>(g) = v;
+            } else if (x < end) {
+                if (x >= shift) g[0] = v.x;
+                if (x + 1 >= shift && x + 1 < end) g[1] = v.y;
+                if (x + 2 >= shift && x + 2 < end) g[2] = v.z;
+                if (x + 3 < end) g[3] = v.w;
             }
-            const int c = which ? carry_b : carry_a;
-            // exclusive value: carry (+) the block prefix before this thread
-            int excl;
-            if (max_mode) {
-                const int prev = __shfl_up_sync(0xffffffffu, inc, 1);
-                excl = max(c, max(wb, lane > 0 ? prev : -1));
-            } else {
-                excl = c + wb + inc - x;
-            }
-            __syncthreads();
-            if (t < T) arr[t] = excl;
-            if (threadIdx.x == 0) {
-                if (which) carry_b = c + tot;
-                else carry_a = max_mode ? max(c, tot) : c + tot;
-            }
-            __syncthreads();
+            __syncthreads();  // red and (next part) mark are reused
         }
     }
 }
 
-__global__ void __launch_bounds__(kPermThreads) k_perm_place(const int32_t* __restrict__ o, int64_t P,
-                                                             const int32_t* __restrict__ t_extra,
-                                                             const int32_t* __restrict__ t_dead,
-                                                             int32_t* __restrict__ out, int32_t* __restrict__ E,
-                                                             int32_t* __restrict__ DS) {
+// The result: a particle with offspring keeps its slot, the empty slots take E in order.
+__global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __restrict__ o, int64_t P,
+                                                            const TilePrefix* __restrict__ pre,
+                                                            const int32_t* __restrict__ E, int32_t* __restrict__ out) {
     __shared__ int red[kPermWarps];
     const int64_t i0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
     int c[kPermPer];
-    int e = 0, d = 0;
+    load_counts(o, i0, P, c);
+    int d = 0, td;
 #pragma unroll
-    for (int k = 0; k < kPermPer; ++k) {
-        c[k] = i0 + k < P ? o[i0 + k] : 1;  // past the end: neither extra nor empty
-        e += c[k] > 1 ? c[k] - 1 : 0;
-        d += c[k] == 0;
-    }
-    int te, td;
-    int pe = t_extra[blockIdx.x] + block_excl_scan(e, red, te);
-    int pd = t_dead[blockIdx.x] + block_excl_scan(d, red, td);
-#pragma unroll
-    for (int k = 0; k < kPermPer; ++k) {
-        const int64_t i = i0 + k;
-        if (i >= P) break;
-        if (c[k] > 0) {
-            out[i] = (int32_t)i;
-            if (c[k] > 1) {
-                E[pe] = (int32_t)i;  // start of i's run of extra copies
-                pe += c[k] - 1;
-            }
-        } else {
-            DS[pd++] = (int32_t)i;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kPermThreads) k_perm_tile_max(const int32_t* __restrict__ E, int64_t D,
-                                                                int32_t* __restrict__ t_max) {
-    __shared__ int red[kPermWarps];
-    const int64_t r0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
-    int m = -1;
-#pragma unroll
-    for (int k = 0; k < kPermPer; ++k)
-        if (r0 + k < D) m = max(m, E[r0 + k]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int mm = -1;
-        for (int w = 0; w < kPermWarps; ++w) mm = max(mm, red[w]);
-        t_max[blockIdx.x] = mm;
-    }
-}
-
-__global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __restrict__ E, int64_t D,
-                                                            const int32_t* __restrict__ t_carry,
-                                                            const int32_t* __restrict__ DS,
-                                                            int32_t* __restrict__ out) {
-    __shared__ int red[kPermWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
+    for (int k = 0; k < kPermPer; ++k) d += c[k] == 0;
+    const int32_t* src = E + __ldg(&pre[blockIdx.x].dead) + block_excl_scan(d, red, td);  // ranks below P: inside E
     int v[kPermPer];
-    int run = -1;
 #pragma unroll
-    for (int k = 0; k < kPermPer; ++k) {
-        v[k] = r0 + k < D ? E[r0 + k] : -1;
-        run = max(run, v[k]);
-        v[k] = run;
-    }
-    // exclusive running maximum of the threads' maxima, then the tile's carry
-    int inc = run;
+    for (int k = 0; k < kPermPer; ++k) v[k] = c[k] == 0 ? __ldg(src++) : (int)(i0 + k);
+    if (i0 + kPermPer <= P && (((uintptr_t)out) & 15u) == 0) {
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int h = __shfl_up_sync(0xffffffffu, inc, off);
-        if (lane >= off) inc = max(inc, h);
-    }
-    int prev = __shfl_up_sync(0xffffffffu, inc, 1);
-    if (lane == 0) prev = -1;
-    if (lane == 31) red[warp] = inc;
-    __syncthreads();
-    for (int w = 0; w < warp; ++w) prev = max(prev, red[w]);
-    prev = max(prev, t_carry[blockIdx.x]);
+        for (int q = 0; q < kPermPer / 4; ++q)
+            reinterpret_cast<int4*>(out + i0)[q] = make_int4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    } else {
 #pragma unroll
-    for (int k = 0; k < kPermPer; ++k) {
-        if (r0 + k >= D) break;
-        const int32_t slot = DS[r0 + k];  // -1 past the last empty slot
-        if (slot >= 0 && slot < D) out[slot] = max(prev, v[k]);
+        for (int k = 0; k < kPermPer; ++k)
+            if (i0 + k < P) out[i0 + k] = v[k];
     }
 }
 
 // In-place gather: row j <- row perm[j] where they differ; a source must keep
 // its own slot (perm[perm[j]] = perm[j]), else the row is left and
-// PF_ERR_INVALID recorded.
-template <typename VT>
-__global__ void __launch_bounds__(256) k_gather_inplace(VT* __restrict__ x, int64_t P, int64_t vecs,
+// PF_ERR_INVALID recorded.  Chunks as in the gather; a source row is read beside
+// its own perm entry, before that is known to be itself (a row being overwritten
+// meanwhile is read to no effect).
+template <typename VT, int U, bool POW2>
+__global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSplit split,
                                                         const int32_t* __restrict__ perm, uint32_t* ctl) {
-    const int64_t total = P * vecs;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = idx / vecs, c = idx - j * vecs;
-        const int32_t a = perm[j];
-        if (a == j) continue;
-        if (a < 0 || a >= P || perm[a] != a) {
-            if (c == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
-            continue;
+    const int64_t total = P * split.vecs;
+    const int64_t stride = (int64_t)gridDim.x * (256 * U);
+    for (int64_t base = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; base < total; base += stride) {
+        int32_t a[U], own[U];
+        uint32_t c[U];
+        VT v[U];
+        bool move[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = base + u * 256;
+            move[u] = false;
+            a[u] = 0;
+            if (i < total) {
+                const int64_t j = split.row<POW2>(i, c[u]);
+                a[u] = __ldg(perm + j);
+                move[u] = a[u] != j;
+            }
         }
-        x[idx] = x[(int64_t)a * vecs + c];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            own[u] = -1;
+            if (move[u] && a[u] >= 0 && a[u] < P) {
+                own[u] = __ldg(perm + a[u]);
+                v[u] = load_chunk(x + (int64_t)a[u] * split.vecs + c[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (!move[u]) continue;
+            if (own[u] >= 0 && own[u] == a[u]) store_chunk_cs(x + base + u * 256, v[u]);
+            else if (c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
+        }
     }
 }
 
 }  // namespace
 
+// Scratch: the tile prefixes, then the counts o and the list E (16-byte loads of o: 256-byte aligned).
+static size_t perm_counts_at(int64_t T) { return (((size_t)T + 1) * sizeof(TilePrefix) + 255) & ~(size_t)255; }
+
 size_t permute_scratch_bytes(int64_t P) {
     const int64_t T = (P + kPermTile - 1) / kPermTile;
-    return ((size_t)3 * P + 4 * (size_t)T + 64) * sizeof(int32_t);
+    return perm_counts_at(T) + (((size_t)P * sizeof(int32_t) + 255) & ~(size_t)255) + (size_t)P * sizeof(int32_t);
 }
 
 cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* scratch, uint32_t* ctl, int num_sms,
                            cudaStream_t s) {
-    const int64_t T = (P + kPermTile - 1) / kPermTile;
-    int32_t* o = static_cast<int32_t*>(scratch);
-    int32_t* E = o + P;
-    int32_t* DS = E + P;
-    int32_t* t_extra = DS + P;
-    int32_t* t_dead = t_extra + T;
-    int32_t* t_max = t_dead + T;
+    const int T = (int)((P + kPermTile - 1) / kPermTile);
+    TilePrefix* pre = static_cast<TilePrefix*>(scratch);
+    int32_t* o = reinterpret_cast<int32_t*>((char*)scratch + perm_counts_at(T));
+    int32_t* E = reinterpret_cast<int32_t*>((char*)o + (((size_t)P * sizeof(int32_t) + 255) & ~(size_t)255));
     cudaError_t e = cudaMemsetAsync(o, 0, (size_t)P * sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(E, 0xff, (size_t)P * sizeof(int32_t), s);  // -1: no mark
-    if (e == cudaSuccess) e = cudaMemsetAsync(DS, 0xff, (size_t)P * sizeof(int32_t), s);  // -1: no slot
     if (e != cudaSuccess) return e;
-    int64_t blocks = (P + 255) / 256;
+    int64_t blocks = (P + 1023) / 1024;  // 8 warps of 128 entries
     if (blocks > (int64_t)num_sms * 8) blocks = (int64_t)num_sms * 8;
     k_perm_count<<<(unsigned)blocks, 256, 0, s>>>(anc, P, o, ctl);
-    k_perm_tiles<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, t_extra, t_dead);
-    k_perm_scan<<<1, kScanThreads, 0, s>>>(t_extra, t_dead, (int)T, 0);
-    k_perm_place<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, t_extra, t_dead, out, E, DS);
-    // the extras list has as many entries as there are empty slots, at most P;
-    // entries past that count stay -1 and their DS entries -1, so nothing is written for them
-    k_perm_tile_max<<<(unsigned)T, kPermThreads, 0, s>>>(E, P, t_max);
-    k_perm_scan<<<1, kScanThreads, 0, s>>>(t_max, nullptr, (int)T, 1);
-    k_perm_fill<<<(unsigned)T, kPermThreads, 0, s>>>(E, P, t_max, DS, out);
+    k_perm_tiles<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, pre, T, ctl);
+    // at most T + P / kPermPart parts; a resident wave takes them in turn
+    const int64_t parts = T + P / kPermPart, wave = (int64_t)num_sms * 4;
+    k_perm_list<<<(unsigned)(parts < wave ? parts : wave), kPermThreads, 0, s>>>(o, P, pre, T, E);
+    k_perm_fill<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, pre, E, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const int32_t* perm, uint32_t* ctl,
                                   int num_sms, cudaStream_t s) {
-    const int64_t blocks_cap = (int64_t)num_sms * 8;
-    auto go = [&](auto* p, int64_t vecs) {
-        int64_t blocks = (P * vecs + 255) / 256;
-        if (blocks > blocks_cap) blocks = blocks_cap;
-        if (blocks < 1) blocks = 1;
-        k_gather_inplace<<<(unsigned)blocks, 256, 0, s>>>(p, P, vecs, perm, ctl);
+    auto go = [&](auto* p, auto unroll) {
+        using VT = std::remove_pointer_t<decltype(p)>;
+        constexpr int U = decltype(unroll)::value;
+        const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
+        const RowSplit split = row_split(vecs, P * vecs);
+        const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, 8, 40);
+        if (split.pow2) k_gather_inplace<VT, U, true><<<blocks, 256, 0, s>>>(p, P, split, perm, ctl);
+        else k_gather_inplace<VT, U, false><<<blocks, 256, 0, s>>>(p, P, split, perm, ctl);
     };
     const uintptr_t a = (uintptr_t)x | (uintptr_t)row_bytes;
-    if ((a & 15) == 0) go(static_cast<uint4*>(x), row_bytes / 16);
-    else if ((a & 7) == 0) go(static_cast<uint2*>(x), row_bytes / 8);
-    else go(static_cast<uint32_t*>(x), row_bytes / 4);
+    if ((a & 31) == 0) go(static_cast<u32x8*>(x), std::integral_constant<int, 2>());
+    else if ((a & 15) == 0) go(static_cast<uint4*>(x), std::integral_constant<int, 4>());
+    else if ((a & 7) == 0) go(static_cast<uint2*>(x), std::integral_constant<int, 4>());
+    else go(static_cast<uint32_t*>(x), std::integral_constant<int, 4>());
     return cudaGetLastError();
 }
 
