@@ -4,76 +4,79 @@
 #include <climits>
 
 #include "pf_fixed.cuh"
+#include "pf_rows.cuh"
 
 namespace pf {
 
 // ---------------------------------------------------------------------------
-// Gather: dst row j <- src row anc[j].  One thread moves one VT-sized chunk;
-// each thread handles kUnroll chunks spread a grid apart, issuing all loads
-// before the stores so that several random row reads are in flight.
+// Gather: dst row j <- src row anc[j].  One thread moves U chunks of VT, adjacent
+// blocks of a CTA's threads, issuing all loads before the stores so that several
+// random row reads are in flight.  Bound by DRAM writes and the latency of the
+// row reads.  Rows of a multiple of 32 bytes move in 256-bit accesses, two a thread:
+// 2^24 rows of 32 bytes 133 -> 100 us (576 MB of rows and ancestors: 5.7 TB/s),
+// 2^22 rows of 64 bytes 94 -> 78 us, of 128 bytes 154 -> 124 us against four 128-bit
+// chunks a thread spaced a grid apart (four 256-bit ones: 116 us at 2^24).
 // ---------------------------------------------------------------------------
 constexpr int kGatherThreads = 256;
-constexpr int kUnroll = 4;
+constexpr int kGatherWave = 8;        // resident CTAs per SM of one wave
+constexpr int kGatherFullGrid = 40;   // CTAs per SM from which the grid is not cut to a wave
 
-template <typename VT, bool POW2>
-__global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict__ src, int64_t P_src, int64_t vecs,
-                                                           int vshift, const int32_t* __restrict__ anc,
-                                                           int64_t P_dst, VT* __restrict__ dst, uint32_t* ctl) {
-    const int64_t total = P_dst * vecs;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; base < total; base += stride * kUnroll) {
-        VT v[kUnroll];
-        int64_t idx[kUnroll];
-        bool ok[kUnroll];
+template <typename VT, int U, bool POW2>
+__global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict__ src, int64_t P_src, RowSplit split,
+                                                           const int32_t* __restrict__ anc, int64_t total,
+                                                           VT* __restrict__ dst, uint32_t* ctl) {
+    const int64_t stride = (int64_t)gridDim.x * (kGatherThreads * U);
+    for (int64_t base = (int64_t)blockIdx.x * (kGatherThreads * U) + threadIdx.x; base < total; base += stride) {
+        VT v[U];
+        int32_t a[U];
+        uint32_t c[U];
+        bool ok[U];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            idx[u] = base + u * stride;
-            ok[u] = false;
-            if (idx[u] < total) {
-                const int64_t j = POW2 ? (idx[u] >> vshift) : idx[u] / vecs;
-                const int64_t c = POW2 ? (idx[u] & (vecs - 1)) : idx[u] - j * vecs;
-                const int32_t a = __ldg(anc + j);
-                if (a >= 0 && a < P_src) {
-                    v[u] = __ldg(src + (int64_t)a * vecs + c);
-                    ok[u] = true;
-                } else if (c == 0) {
-                    set_status(ctl + CTL_STATUS, ST_INVALID);
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = base + u * kGatherThreads;
+            ok[u] = i < total;
+            a[u] = 0;
+            c[u] = 0;
+            if (ok[u]) a[u] = __ldg(anc + split.row<POW2>(i, c[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (ok[u]) {
+                if (a[u] >= 0 && a[u] < P_src) {
+                    v[u] = load_chunk_nc(src + (int64_t)a[u] * split.vecs + c[u]);
+                } else {
+                    ok[u] = false;
+                    if (c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
                 }
             }
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
-            if (ok[u]) __stcs(dst + idx[u], v[u]);
+        for (int u = 0; u < U; ++u)
+            if (ok[u]) store_chunk_cs(dst + base + u * kGatherThreads, v[u]);
     }
 }
 
-template <typename VT>
+template <typename VT, int U>
 static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
                              void* dst, uint32_t* ctl, int num_sms, cudaStream_t s) {
     const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
     const int64_t total = P_dst * vecs;
-    int64_t blocks = (total + (int64_t)kGatherThreads * kUnroll - 1) / ((int64_t)kGatherThreads * kUnroll);
-    const int64_t cap = (int64_t)num_sms * 8;  // one resident wave (8 CTAs of 256 threads per SM)
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    const bool pow2 = (vecs & (vecs - 1)) == 0;
-    int vshift = 0;
-    while (pow2 && (1LL << vshift) < vecs) ++vshift;
-    if (pow2)
-        k_gather<VT, true><<<(unsigned)blocks, kGatherThreads, 0, s>>>(
-            (const VT*)src, P_src, vecs, vshift, anc, P_dst, (VT*)dst, ctl);
+    const RowSplit split = row_split(vecs, total);
+    const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, kGatherWave, kGatherFullGrid);
+    if (split.pow2)
+        k_gather<VT, U, true><<<blocks, kGatherThreads, 0, s>>>((const VT*)src, P_src, split, anc, total, (VT*)dst, ctl);
     else
-        k_gather<VT, false><<<(unsigned)blocks, kGatherThreads, 0, s>>>(
-            (const VT*)src, P_src, vecs, vshift, anc, P_dst, (VT*)dst, ctl);
+        k_gather<VT, U, false><<<blocks, kGatherThreads, 0, s>>>((const VT*)src, P_src, split, anc, total, (VT*)dst, ctl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gather(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
                           void* dst, uint32_t* ctl, int num_sms, cudaStream_t s) {
     const uintptr_t a = (uintptr_t)src | (uintptr_t)dst | (uintptr_t)row_bytes;
-    if ((a & 15) == 0) return gather_vt<uint4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
-    if ((a & 7) == 0) return gather_vt<uint2>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
-    return gather_vt<uint32_t>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
+    if ((a & 31) == 0) return gather_vt<u32x8, 2>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
+    if ((a & 15) == 0) return gather_vt<uint4, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
+    if ((a & 7) == 0) return gather_vt<uint2, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
+    return gather_vt<uint32_t, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
 }
 
 // ---------------------------------------------------------------------------
