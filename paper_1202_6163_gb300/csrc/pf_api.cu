@@ -705,15 +705,15 @@ pf_status pf_lg_init(int F, int64_t P, int D, float m0, float p0, uint64_t seed,
     p.sigma = (float)std::sqrt((double)p0);
     p.m0 = m0;
     p.log_P = std::log((double)P);
-    p.key0 = (uint32_t)(seed & 0xffffffffu);
-    p.key1 = (uint32_t)(seed >> 32);
+    p.n_tiles = (int)((P + lg_tile() - 1) / lg_tile());
+    p.keys = philox_round_keys((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
     p.x_next = x;
     p.lw = logw;
     p.loglik = loglik;
     p.log_sum = log_sum;
     p.ess = ess;
     p.resample = resample;
-    return cuda_fail(launch_lg_init(p, info->num_sms, s), "lg init launch");
+    return cuda_fail(launch_lg_init(p, s), "lg init launch");
 }
 
 pf_status pf_lg_step(int F, int64_t P, int D, const float* a, double q, double r, double threshold,
@@ -759,8 +759,7 @@ pf_status pf_lg_step(int F, int64_t P, int D, const float* a, double q, double r
     p.log_P = std::log((double)P);
     p.y = y;
     p.t = (uint32_t)t;
-    p.key0 = (uint32_t)(seed & 0xffffffffu);
-    p.key1 = (uint32_t)(seed >> 32);
+    p.keys = philox_round_keys((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
     p.anc = ancestors;
     p.x_prev = x_prev;
     p.x_next = x_next;

@@ -41,13 +41,30 @@ __device__ __forceinline__ u32x4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
     return {c0, c1, c2, c3};
 }
 
+// The ten-round function with the round keys given (kernel parameters: the keys are
+// then operands of the xors, where advancing them costs two additions a round).
+__device__ __forceinline__ u32x4 philox_keys(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const PhiloxKeys& k) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t a = (uint64_t)0xD2511F53u * c0;
+        const uint64_t b = (uint64_t)0xCD9E8D57u * c2;
+        c0 = (uint32_t)(b >> 32) ^ c1 ^ k.k0[r];
+        c1 = (uint32_t)b;
+        c2 = (uint32_t)(a >> 32) ^ c3 ^ k.k1[r];
+        c3 = (uint32_t)a;
+    }
+    return {c0, c1, c2, c3};
+}
+
 __device__ __forceinline__ uint32_t word_of(const u32x4& r, int s) {
     return s == 0 ? r.x : (s == 1 ? r.y : (s == 2 ? r.z : r.w));
 }
 
-// u23: odd multiples of 2^-24 in (0,1); exact in float.
+// u23: odd multiples of 2^-24 in (0,1); exact in float.  The word's top 23 bits
+// make 1 + m 2^-23, and taking 1 - 2^-24 off leaves (2m + 1) 2^-24 exactly: no
+// integer conversion, which issues at a quarter of the rate.
 __device__ __forceinline__ float u23f(uint32_t x) {
-    return __uint2float_rn(((x >> 9) << 1) | 1u) * 0x1p-24f;
+    return __fsub_rn(__uint_as_float((x >> 9) | 0x3f800000u), 0x1.fffffep-1f);
 }
 
 // u32 = (2x+1) 2^-33 as an exact float pair (hi carries the top 24 bits).

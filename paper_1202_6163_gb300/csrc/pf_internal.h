@@ -120,6 +120,19 @@ __device__ __forceinline__ void trace_stamp(uint64_t* trace, int64_t cap, int64_
     }
 }
 
+// The round keys of a Philox-4x32-10 key.
+struct PhiloxKeys {
+    uint32_t k0[10], k1[10];
+};
+inline PhiloxKeys philox_round_keys(uint32_t k0, uint32_t k1) {
+    PhiloxKeys k;
+    for (int r = 0; r < 10; ++r) {
+        k.k0[r] = k0 + (uint32_t)r * 0x9E3779B9u;
+        k.k1[r] = k1 + (uint32_t)r * 0xBB67AE85u;
+    }
+    return k;
+}
+
 // One step of F bootstrap filters on the linear-Gaussian test model.
 struct LgParams {
     int F;
@@ -135,7 +148,7 @@ struct LgParams {
     double log_P;
     const float* y;  // [F][D] observation of this step
     uint32_t t;
-    uint32_t key0, key1;
+    PhiloxKeys keys;
     const int32_t* anc;
     const float* x_prev;
     float* x_next;
@@ -155,7 +168,7 @@ uint64_t current_wait_ns();
 // Kernel launchers (defined in the .cu files; return the launch error).
 cudaError_t launch_sorted_persistent(int kind, const SortedParams& p, int grid, cudaStream_t s);
 int lg_tile();
-cudaError_t launch_lg_init(const LgParams& p, int num_sms, cudaStream_t s);
+cudaError_t launch_lg_init(const LgParams& p, cudaStream_t s);
 cudaError_t launch_lg_step(const LgParams& p, cudaStream_t s);
 size_t permute_scratch_bytes(int64_t P);
 cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* scratch, uint32_t* ctl, int num_sms,
