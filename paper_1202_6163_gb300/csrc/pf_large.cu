@@ -6,20 +6,19 @@
 //      into shared memory while the CTA's previous tile is scanned: the tile
 //      scan (pf_tile.cuh), a 16-byte record (k_t, S_t, i_last) and the tile's
 //      cumulative weights v_i (sign bit: zero weight);
-//   2. k_large_carries: one CTA: the largest tile exponent K and the exact
-//      exclusive prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} of every tile
-//      (128-bit fixed point; each thread a contiguous run of records, then one
-//      block scan of the run totals), W = B_T, and the multinomial's tile table;
-//   3. k_large_assign (systematic, stratified): grid-stride over tiles: the
-//      tile's v_i read back (not rescanned: 6-7% faster at 2^25 - 2^27 for the
-//      extra 4 B written and read per particle; bulk-copied into shared memory
-//      while the previous tile is assigned), the tile's offset map from B_t and
-//      B_{t+1}, the offsets and their run-length decode (pf_assign.cuh).
-//      Multinomial: k_large_guide decodes the guide table (the first particle
-//      above each of P/4 evenly spaced targets) from the stored v_i, then
-//      k_large_draws runs the draws, each through its guide entry and one
-//      window of v_i, or, where that does not settle it, by binary searches over
-//      the tile table and the tile's v_i.
+//   2. k_large_carries: a thread per tile: the largest tile exponent K, the exact
+//      prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} (128-bit fixed point; each CTA sums the
+//      tiles before its own), W = B_T, every tile's offset map from B_t and B_{t+1}
+//      (the same function of a boundary for both ends, so neighbouring tiles share their
+//      end exactly), and the multinomial's tile table;
+//   3. k_large_assign (systematic, stratified): the tiles' offsets and their run-length
+//      decode (pf_assign.cuh), warp by warp: a warp reads its share of a tile's v_i back
+//      (not rescanned: 6-7% faster at 2^25 - 2^27 for the extra 4 B written and read per
+//      particle) and meets no barrier; tiles that own too many offsets for that are left
+//      to the whole CTA at the end.  Multinomial: the same pass decodes the guide table
+//      (the first particle above each of P/4 evenly spaced targets), then k_large_draws
+//      runs the draws, each through its guide entry and one window of v_i, or, where
+//      that does not settle it, by binary searches over the tile table and the tile's v_i.
 // The tiles, the exact boundaries and the per-tile arithmetic are those of the
 // single-launch kernels, so the results follow the same rules.  A NaN/+inf or
 // all-zero weight set records PF_ERR_DOMAIN in launch 1 or 2, and launch 3
@@ -35,18 +34,18 @@ namespace {
 
 // What launch 2 hands to launch 3 (global memory).
 struct LargeScalars {
-    i128 Wt;  // W in fixed point (units of 2^K)
-    int K;    // largest tile exponent with weight
-    int ok;   // 0: a domain error was recorded, launch 3 writes nothing
+    int ok;  // 0: a domain error was recorded, launch 3 writes nothing
     float W_hi, W_lo;
 };
 
-struct LargeShared {
-    AssignShared as;
-    TileMap map;
-    uint64_t bar;  // the assignment's tile copies
+// A tile for launch 3: its offset map and its last positive element.
+struct __align__(32) LargeMap {
+    long long jlo;
+    int noff;
+    float x0, ir;
+    int il;
 };
-static_assert(sizeof(LargeShared) % 16 == 0, "the staging buffers are 16-byte aligned");
+static_assert(sizeof(LargeMap) == 32, "one sector a tile");
 
 constexpr int kLargeTile = kTileMax;  // full tiles, 16 log-weights per thread
 
@@ -118,187 +117,141 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_scan(SortedParams p, uint
 }
 
 // ---------------------------------------------------------------------------
-// Launch 2: one CTA forms K, every tile's exact lower boundary B_t (bnd[0..T],
-// bnd[T] = W) and, for the multinomial, the tile table the draws search.
+// Launch 2: kThreads tiles per CTA.  Every CTA reads all records for K and the mass
+// below its own tiles (a few microseconds from L2, where one CTA doing all tiles took
+// 13 us at 4097 of them); integer sums, so the order does not matter.
+// pm: the parameters of the offsets (multinomial: the guide's M bucket edges).
 // ---------------------------------------------------------------------------
 template <int KIND>
-__global__ void __launch_bounds__(kThreads) k_large_carries(SortedParams p, const uint4* rec, i128* bnd,
+__global__ void __launch_bounds__(kThreads) k_large_carries(SortedParams pm, const uint4* rec, LargeMap* maps,
                                                             TableEntry* table, LargeScalars* out) {
     __shared__ int red[kWarps];
-    __shared__ i128 wsum[kWarps];
-    __shared__ i128 total;
+    __shared__ i128 wsum[kWarps], wall[kWarps];
+    __shared__ long long jnext[kThreads + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int T = p.n_tiles;
+    const int T = pm.n_tiles;
+    const int t_first = (int)blockIdx.x * kThreads, t = t_first + tid;
     // the largest exponent among tiles with weight, and the domain check
     int kmax = INT_MIN, bad = 0;
-    for (int t = tid; t < T; t += kThreads) {
-        const uint4 r = rec[t];
+    for (int i = tid; i < T; i += kThreads) {
+        const uint4 r = __ldg(rec + i);
         const float sh = __uint_as_float(r.y);
         bad |= !(sh <= FLT_MAX);
         if (sh > 0.f) kmax = max(kmax, (int)r.x);
     }
-    kmax = warp_max_i(kmax);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) red[warp] = kmax;
     bad = __syncthreads_or(bad);
-    int K = INT_MIN;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) K = max(K, red[w]);
+    const int K = __reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : INT_MIN);
     if (K == INT_MIN || bad) {
-        if (tid == 0) {
-            set_status(p.ctl + CTL_STATUS, ST_DOMAIN);
+        if (tid == 0 && blockIdx.x == 0) {
+            set_status(pm.ctl + CTL_STATUS, ST_DOMAIN);
             out->ok = 0;
         }
         return;
     }
-    // each thread a contiguous run [t_lo, t_hi) of records, read eight at a time
-    const int per = (T + kThreads - 1) / kThreads;
-    const int t_lo = min(T, tid * per), t_hi = min(T, t_lo + per);
-    i128 run = 0;
-    for (int t0 = t_lo; t0 < t_hi; t0 += 8) {
-        uint4 r[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) r[u] = t0 + u < t_hi ? rec[t0 + u] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) run += record_mass(r[u], K);
+    // the mass of every tile, split into what lies below this CTA's tiles and the rest
+    i128 below = 0, all = 0;
+    for (int i = tid; i < T; i += kThreads) {
+        const i128 m = record_mass(__ldg(rec + i), K);
+        all += m;
+        if (i < t_first) below += m;
     }
-    // exclusive block scan of the run totals (integer sums: exact in any order)
-    const i128 inc = warp_scan_i128(run, lane);
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        const i128 v = lane < kWarps ? wsum[lane] : (i128)0;
-        const i128 vi = warp_scan_i128(v, lane);
-        if (lane < kWarps) wsum[lane] = vi - v;
-        if (lane == kWarps - 1) total = vi;
+    const uint4 r = t < T ? __ldg(rec + t) : make_uint4(0u, 0u, 0u, 0xffffffffu);
+    const i128 mine = record_mass(r, K);
+    const i128 inc = warp_scan_i128(mine, lane);
+    // one block scan: the CTA's own masses, its base added to the first warp's
+    const i128 bw = warp_scan_i128(below, lane), aw = warp_scan_i128(all, lane);
+    if (lane == 31) {
+        wsum[warp] = inc;
+        wall[warp] = aw;
     }
+    __shared__ i128 wbelow[kWarps];
+    if (lane == 31) wbelow[warp] = bw;
     __syncthreads();
-    i128 B = wsum[warp] + inc - run;  // the boundary of tile t_lo
-    for (int t0 = t_lo; t0 < t_hi; t0 += 8) {
-        uint4 r[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) r[u] = t0 + u < t_hi ? rec[t0 + u] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (t0 + u < t_hi) {
-                bnd[t0 + u] = B;
-                if (KIND == KIND_MULTI) {
-                    const fpair b = fixed_to_pair(B);
-                    table[t0 + u] = {b.hi, b.lo, pow2f(K - (int)r[u].x), (int)r[u].w};
-                }
-                B += record_mass(r[u], K);
-            }
+    i128 B = inc - mine, Wt = 0;
+    for (int w = 0; w < kWarps; ++w) {
+        B += wbelow[w];
+        if (w < warp) B += wsum[w];
+        Wt += wall[w];
+    }
+    AssignShared as;
+    as.Wt = Wt;
+    as.K = K;
+    const fpair W = fixed_to_pair(Wt);
+    as.W_hi = W.hi;
+    as.W_lo = W.lo;
+    // this tile's lower end; the upper one is the next tile's lower
+    const fpair Pp = fast_two_sum((float)pm.P, (float)(pm.P - (int64_t)(float)pm.P));  // P exactly
+    const fpair PW = pair_div(Pp, W);
+    constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;
+    float x0 = 0.f, x0_end;
+    const long long jlo = t <= T ? offsets_below<kMapKind>(pm, as, PW, B, x0) : 0;
+    jnext[tid] = jlo;
+    if (tid == kThreads - 1 && t < T) jnext[kThreads] = offsets_below<kMapKind>(pm, as, PW, B + mine, x0_end);
+    __syncthreads();
+    if (t < T) {
+        LargeMap m;
+        m.jlo = jlo;
+        m.noff = (int)max(0LL, jnext[tid + 1] - jlo);
+        m.x0 = x0;
+        m.ir = PW.hi * pow2f((int)r.x - K);
+        m.il = (int)r.w;
+        maps[t] = m;
+        if (KIND == KIND_MULTI) {
+            const fpair b = fixed_to_pair(B);
+            table[t] = {b.hi, b.lo, pow2f(K - (int)r.x), (int)r.w};
         }
     }
-    if (tid == 0) {
-        bnd[T] = total;
-        const fpair Wp = fixed_to_pair(total);
-        out->Wt = total;
-        out->K = K;
-        out->W_hi = Wp.hi;
-        out->W_lo = Wp.lo;
-        out->ok = 1;
-    }
+    if (tid == 0 && blockIdx.x == 0) *out = {1, W.hi, W.lo};
 }
 
 // ---------------------------------------------------------------------------
-// Launch 3, systematic / stratified: each tile's stored cumulative weights and
-// record read back, its offset map from its two boundaries (the same function
-// of a boundary for both ends, so neighbouring tiles share their end exactly),
-// then its offsets decoded.
+// Launch 3, systematic / stratified, and the multinomial's guide table g[b], b < M =
+// P / 4, the first particle whose cumulative weight exceeds the bucket edge (b / M) W:
+// the systematic assignment of M offsets with no uniform shift (p: the call's
+// parameters, or those with anc = g, P = M, guide = 1; PA the call's P + lead).
 // ---------------------------------------------------------------------------
-template <int KIND>
-__global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, const uint4* rec, const i128* bnd,
+constexpr int kMapBatch = 64;  // tiles whose maps a CTA holds at once
+
+struct LargeShared {
+    AssignShared as;
+    LargeMap maps[kMapBatch];
+};
+static_assert(sizeof(LargeShared) % 16 == 0, "the staging buffers are 16-byte aligned");
+
+template <int KIND, int S>
+__global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, int64_t PA, const LargeMap* maps,
                                                               const LargeScalars* sc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LargeShared& sm = *reinterpret_cast<LargeShared*>(smem_raw);
     int32_t* stage = reinterpret_cast<int32_t*>(smem_raw + sizeof(LargeShared));
-    float* vbuf = reinterpret_cast<float*>(stage + 2 * kIoCap);  // one tile's stored cumulative weights
     const int tid = threadIdx.x;
     if (!sc->ok) return;  // launch 2 recorded a domain error
-    const int64_t PA = p.P + p.lead;
     const int n_mine = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // grid <= tiles
-    if (tid == 0) {
-        sm.as.Wt = sc->Wt;
-        sm.as.K = sc->K;
-        sm.as.W_hi = sc->W_hi;
-        sm.as.W_lo = sc->W_lo;
-        mbar_init(&sm.bar, 1);
-        fence_mbar_init();
-    }
     stage_init<kIoCap>(stage);
-    __syncthreads();
-    // tile r + 1's copy is issued once every thread has taken tile r out of the
-    // buffer, and lands while tile r is assigned
-    if (tid == 0) issue_tile_copy(p.v_out, PA, 0, vbuf, &sm.bar);
     TileThread th;
-    for (int r = 0; r < n_mine; ++r) {
-        const int t = (int)blockIdx.x + r * (int)gridDim.x;
-        const int64_t t0 = (int64_t)t * kLargeTile;
-        const int n = (int)min((int64_t)kLargeTile, PA - t0);
-        // bounded from this wait's start; the results are then unspecified
-        if (!mbar_wait(&sm.bar, (uint32_t)r & 1u, global_ns(), p.wait_ns) && tid == 0)
-            set_status(p.ctl + CTL_STATUS, ST_TIMEOUT);
-        // a ragged last tile: its tail is not in the copy; read it from global memory
-        if ((n & 3) == 0) read_tile_v<16, true>(vbuf, n, th);
-        else read_tile_v<16>(p.v_out + t0, n, th);
-        const uint4 rc = rec[t];
-        TileSummary ts;
-        ts.k = (int)rc.x;
-        ts.i_last = (int)rc.w;
-        ts.bad = 0;
-        ts.S = {__uint_as_float(rc.y), __uint_as_float(rc.z)};
-        if (tid < 32) {  // lanes 0 and 1 form the map (the other pairs of warp 0 the same one)
-            const TileMap m = tile_map_pair<KIND>(p, sm.as, bnd[t], bnd[t + 1], ts.k, 0xffffffffu);
-            if (tid == 0) sm.map = m;
+    TileSummary ts;
+    for (int r0 = 0; r0 < n_mine; r0 += kMapBatch) {
+        const int n = min(kMapBatch, n_mine - r0);
+        if (tid < n) sm.maps[tid] = maps[(int)blockIdx.x + (r0 + tid) * (int)gridDim.x];
+        __syncthreads();
+        auto tile = [&](int r, bool heavy) {
+            const LargeMap m = sm.maps[r];
+            if ((m.noff > kWarpOffsets) != heavy) return;
+            const int64_t t0 = (int64_t)((int)blockIdx.x + (r0 + r) * (int)gridDim.x) * kLargeTile;
+            read_tile_v<16>(p.v_out + t0, (int)min((int64_t)kLargeTile, PA - t0), th);
+            ts.i_last = m.il;
+            assign_tile<KIND, 16, kIoCap, S>(p, sm.as, {m.jlo, m.noff, m.x0, m.ir}, stage, th, ts, t0 - p.lead);
+        };
+        bool any = false;
+        for (int r = 0; r < n; ++r) {
+            any |= sm.maps[r].noff > kWarpOffsets;
+            tile(r, false);
         }
-        fence_proxy_async_smem();  // this thread's reads of the buffer before its next copy
-        __syncthreads();
-        if (tid == 0 && r + 1 < n_mine) issue_tile_copy(p.v_out, PA, r + 1, vbuf, &sm.bar);
-        assign_tile<KIND, 16, kIoCap>(p, sm.as, sm.map, stage, th, ts, t0 - p.lead);
-        __syncthreads();  // the map is reused by the next tile
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Multinomial, between launches 2 and 3: the guide table g[b], b < M = P / 4,
-// the first particle whose cumulative weight exceeds the bucket edge
-// (b / M) W -- the systematic assignment of M offsets with no uniform shift,
-// from each tile's stored cumulative weights (pg: the call's parameters with
-// anc = g, P = M, guide = 1; PA the call's P + lead).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 2) k_large_guide(SortedParams pg, int64_t PA, const uint4* rec,
-                                                             const i128* bnd, const LargeScalars* sc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    LargeShared& sm = *reinterpret_cast<LargeShared*>(smem_raw);
-    int32_t* stage = reinterpret_cast<int32_t*>(smem_raw + sizeof(LargeShared));
-    const int tid = threadIdx.x;
-    if (!sc->ok) return;
-    if (tid == 0) {
-        sm.as.Wt = sc->Wt;
-        sm.as.K = sc->K;
-        sm.as.W_hi = sc->W_hi;
-        sm.as.W_lo = sc->W_lo;
-    }
-    stage_init<kIoCap>(stage);
-    __syncthreads();
-    TileThread th;
-    for (int t = blockIdx.x; t < pg.n_tiles; t += gridDim.x) {
-        const int64_t t0 = (int64_t)t * kLargeTile;
-        const int n = (int)min((int64_t)kLargeTile, PA - t0);
-        read_tile_v<16>(pg.v_out + t0, n, th);
-        const uint4 r = rec[t];
-        TileSummary ts;
-        ts.k = (int)r.x;
-        ts.i_last = (int)r.w;
-        ts.bad = 0;
-        ts.S = {__uint_as_float(r.y), __uint_as_float(r.z)};
-        if (tid < 32) {
-            const TileMap m = tile_map_pair<KIND_SYS>(pg, sm.as, bnd[t], bnd[t + 1], ts.k, 0xffffffffu);
-            if (tid == 0) sm.map = m;
-        }
-        __syncthreads();
-        assign_tile<KIND_SYS, 16, kIoCap, 8>(pg, sm.as, sm.map, stage, th, ts, t0 - pg.lead);
-        __syncthreads();
+        if (any)  // block-uniform: the same maps in every thread
+            for (int r = 0; r < n; ++r) tile(r, true);
+        __syncthreads();  // the maps are replaced
     }
 }
 
@@ -355,7 +308,7 @@ namespace {
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct LargeLayout {
-    size_t rec, bnd, table, scalars, v, g, total;
+    size_t rec, maps, table, scalars, v, g, total;
 };
 
 // Multinomial guide buckets: a quarter of the particles.
@@ -366,8 +319,8 @@ LargeLayout large_layout(int kind, int64_t PA) {
     const bool multi = kind == KIND_MULTI;
     LargeLayout l;
     l.rec = 0;
-    l.bnd = align256(T * sizeof(uint4));
-    l.table = align256(l.bnd + (T + 1) * sizeof(i128));
+    l.maps = align256(T * sizeof(uint4));
+    l.table = align256(l.maps + T * sizeof(LargeMap));
     l.scalars = align256(l.table + (multi ? T * sizeof(TableEntry) : 0));
     l.v = align256(l.scalars + sizeof(LargeScalars));
     l.g = align256(l.v + (size_t)PA * sizeof(float));
@@ -375,8 +328,8 @@ LargeLayout large_layout(int kind, int64_t PA) {
     return l;
 }
 
-constexpr size_t kGuideSmem = sizeof(LargeShared) + 2 * (size_t)kIoCap * sizeof(int32_t);
-constexpr size_t kAssignSmem = kGuideSmem + (size_t)kLargeTile * sizeof(float);  // and one tile's copy
+constexpr size_t kAssignSmem = sizeof(LargeShared) + 2 * (size_t)kIoCap * sizeof(int32_t);
+constexpr int kGuideS = 8;  // guide: a warp's 512 elements hold ~128 bucket edges
 
 template <int KIND>
 cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sms, cudaStream_t s) {
@@ -384,7 +337,7 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
     const LargeLayout l = large_layout(KIND, PA);
     const int T = p.n_tiles;
     uint4* rec = reinterpret_cast<uint4*>(scratch + l.rec);
-    i128* bnd = reinterpret_cast<i128*>(scratch + l.bnd);
+    LargeMap* maps = reinterpret_cast<LargeMap*>(scratch + l.maps);
     TableEntry* table = reinterpret_cast<TableEntry*>(scratch + l.table);
     LargeScalars* sc = reinterpret_cast<LargeScalars*>(scratch + l.scalars);
     p.v_out = reinterpret_cast<float*>(scratch + l.v);
@@ -392,27 +345,28 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
     k_large_scan<KIND><<<grid, kThreads, kScanSmem, s>>>(p, rec);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_large_carries<KIND><<<1, kThreads, 0, s>>>(p, rec, bnd, table, sc);
+    SortedParams pm = p;  // of the offsets: the call's, or the guide's
+    const int64_t M = guide_buckets(p.P);
+    int32_t* g = reinterpret_cast<int32_t*>(scratch + l.g);
+    if (KIND == KIND_MULTI) {
+        pm.anc = g;
+        pm.P = M;
+        pm.Pd = (double)M;
+        pm.guide = 1;
+    }
+    k_large_carries<KIND><<<(T + kThreads - 1) / kThreads, kThreads, 0, s>>>(pm, rec, maps, table, sc);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;
+    constexpr int S = KIND == KIND_MULTI ? kGuideS : warp_stage_per_lane(16);
+    k_large_assign<kMapKind, S><<<grid, kThreads, kAssignSmem, s>>>(pm, PA, maps, sc);
     if constexpr (KIND == KIND_MULTI) {
-        // the guide table, then the draws through it
-        int32_t* g = reinterpret_cast<int32_t*>(scratch + l.g);
-        const int64_t M = guide_buckets(p.P);
-        SortedParams pg = p;
-        pg.anc = g;
-        pg.P = M;
-        pg.Pd = (double)M;
-        pg.guide = 1;
-        k_large_guide<<<grid, kThreads, kGuideSmem, s>>>(pg, PA, rec, bnd, sc);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t nq = (p.P + 3) >> 2;
         int64_t gd = (nq + kThreads - 1) / kThreads;
         if (gd > (int64_t)num_sms * 16) gd = (int64_t)num_sms * 16;
         k_large_draws<true><<<(unsigned)gd, kThreads, 0, s>>>(p, table, sc, g, M);
-    } else {
-        k_large_assign<KIND><<<grid, kThreads, kAssignSmem, s>>>(p, rec, bnd, sc);
     }
     return cudaGetLastError();
 }
@@ -421,13 +375,15 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
 // Once per device: the scans' tile buffers and the assignment kernels' staging
 // buffers exceed the default dynamic shared-memory limit.
 cudaError_t prepare_large() {
-    cudaError_t e = cudaFuncSetAttribute(k_large_assign<KIND_SYS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    constexpr int S = warp_stage_per_lane(16);
+    cudaError_t e = cudaFuncSetAttribute(k_large_assign<KIND_SYS, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAssignSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_large_assign<KIND_STRAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_large_assign<KIND_STRAT, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kAssignSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_large_guide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGuideSmem);
+        e = cudaFuncSetAttribute(k_large_assign<KIND_SYS, kGuideS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kAssignSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_large_scan<KIND_MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScanSmem);
     if (e == cudaSuccess)
