@@ -381,7 +381,7 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
 // The CTA-wide decode below this bound waited at three barriers a tile with 40% of
 // the issue slots used.  Systematic launch at P = 2^25 + 4096 94 us (41 instructions
 // per particle), stratified 156 us (88); whole calls now: stratified at 10^8
-// particles 691 -> 527 us, 4096 filters systematic 293 -> 264 us, the 2^24 heavy-tail
+// particles 691 -> 417 us, 4096 filters systematic 293 -> 264 us, the 2^24 heavy-tail
 // step 252 -> 230 us.
 //
 // N by a rounded addition: y + 1.5 2^23 rounded up (down) has ceil(y)
@@ -1121,8 +1121,8 @@ __device__ __forceinline__ void read_tile_v(const float* vg0, int n, TileThread&
         for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
             if (KK || i < K) {
                 if (!zero_flag(th.v[i])) pos |= 1u << i;
-                // monotone also past the tile's end, where -0 stands for no element
-                th.v[i] = run = fmaxf(run, fabsf(th.v[i]));
+                if (th.e0 + i < n) run = fabsf(th.v[i]);
+                th.v[i] = run;  // past the tile's end: the last element's
             }
     }
     th.pos = pos;

@@ -35,6 +35,12 @@ __device__ __forceinline__ i128 shfl_up_i128(i128 v, int o) {
     return (i128)(((unsigned __int128)h2 << 64) | l2);
 }
 
+__device__ __forceinline__ i128 shfl_i128(i128 v, int src) {
+    const unsigned long long lo = __shfl_sync(0xffffffffu, (unsigned long long)v, src);
+    const unsigned long long hi = __shfl_sync(0xffffffffu, (unsigned long long)(v >> 64), src);
+    return (i128)(((unsigned __int128)hi << 64) | lo);
+}
+
 __device__ __forceinline__ i128 warp_scan_i128(i128 v, int lane) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

@@ -6,9 +6,8 @@
 //      into shared memory while the CTA's previous tile is scanned: the tile
 //      scan (pf_tile.cuh), a 16-byte record (k_t, S_t, i_last) and the tile's
 //      cumulative weights v_i (sign bit: zero weight);
-//   2. k_large_carries: a thread per tile: the largest tile exponent K, the exact
-//      prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} (128-bit fixed point; each CTA sums the
-//      tiles before its own), W = B_T, every tile's offset map from B_t and B_{t+1}
+//   2. k_large_carries: one cluster of CTAs: the largest tile exponent K, the exact
+//      prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} (128-bit fixed point), W = B_T, every tile's offset map from B_t and B_{t+1}
 //      (the same function of a boundary for both ends, so neighbouring tiles share their
 //      end exactly), and the multinomial's tile table;
 //   3. k_large_assign (systematic, stratified): the tiles' offsets and their run-length
@@ -25,6 +24,8 @@
 // then writes nothing.
 #include <cfloat>
 #include <climits>
+
+#include <cooperative_groups.h>
 
 #include "pf_assign.cuh"
 
@@ -117,63 +118,91 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_scan(SortedParams p, uint
 }
 
 // ---------------------------------------------------------------------------
-// Launch 2: kThreads tiles per CTA.  Every CTA reads all records for K and the mass
-// below its own tiles (a few microseconds from L2, where one CTA doing all tiles took
-// 13 us at 4097 of them); integer sums, so the order does not matter.
+// Launch 2: one cluster of kCarryCtas CTAs, each a contiguous range of tiles; the
+// ranges' largest exponents and exact masses are exchanged through distributed
+// shared memory.  Bound by the latency of its chain (128-bit shifts, two divisions, the
+// strata's draws): at 4097 tiles 13 us for one CTA, for nine CTAs each summing all
+// records, and for the cluster, whose share of records per thread stays an eighth.
 // pm: the parameters of the offsets (multinomial: the guide's M bucket edges).
 // ---------------------------------------------------------------------------
+constexpr int kCarryCtas = 8;
+
 template <int KIND>
-__global__ void __launch_bounds__(kThreads) k_large_carries(SortedParams pm, const uint4* rec, LargeMap* maps,
-                                                            TableEntry* table, LargeScalars* out) {
+__global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
+    k_large_carries(SortedParams pm, const uint4* rec, LargeMap* maps, TableEntry* table, LargeScalars* out) {
+    namespace cg = cooperative_groups;
     __shared__ int red[kWarps];
-    __shared__ i128 wsum[kWarps], wall[kWarps];
+    __shared__ i128 wsum[kWarps];
+    __shared__ int cta_k;     // this CTA's largest exponent with weight (kBadRange: a NaN or +inf tile)
+    __shared__ i128 cta_sum;  // this CTA's mass
     __shared__ long long jnext[kThreads + 1];
+    constexpr int kBadRange = INT_MAX;
+    cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int T = pm.n_tiles;
-    const int t_first = (int)blockIdx.x * kThreads, t = t_first + tid;
+    const int per = ((T + kCarryCtas - 1) / kCarryCtas + 1) & ~1;
+    const int t_lo = min(T, (int)blockIdx.x * per), t_hi = min(T, t_lo + per);
     // the largest exponent among tiles with weight, and the domain check
-    int kmax = INT_MIN, bad = 0;
-    for (int i = tid; i < T; i += kThreads) {
-        const uint4 r = __ldg(rec + i);
-        const float sh = __uint_as_float(r.y);
-        bad |= !(sh <= FLT_MAX);
-        if (sh > 0.f) kmax = max(kmax, (int)r.x);
+    constexpr int kBatch = 4;  // records in flight per thread
+    int kmax = INT_MIN;
+    for (int t0 = t_lo + tid; t0 < t_hi; t0 += kBatch * kThreads) {
+        uint2 r[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+            r[u] = t0 + u * kThreads < t_hi ? __ldg(reinterpret_cast<const uint2*>(rec + t0 + u * kThreads))
+                                            : make_uint2(0u, 0u);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const float sh = __uint_as_float(r[u].y);
+            if (!(sh <= FLT_MAX)) kmax = kBadRange;
+            else if (sh > 0.f) kmax = max(kmax, (int)r[u].x);
+        }
     }
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) red[warp] = kmax;
-    bad = __syncthreads_or(bad);
-    const int K = __reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : INT_MIN);
-    if (K == INT_MIN || bad) {
+    __syncthreads();
+    kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : INT_MIN);
+    if (tid == 0) cta_k = kmax;
+    cluster.sync();
+    int K = INT_MIN;
+    for (int c = 0; c < kCarryCtas; ++c) K = max(K, *cluster.map_shared_rank(&cta_k, c));
+    const bool ok = K != INT_MIN && K != kBadRange;  // the same in every CTA
+    // this CTA's mass, then those before it and the total (integer sums: any order)
+    if (ok) {
+        i128 run = 0;
+        for (int t0 = t_lo + tid; t0 < t_hi; t0 += kBatch * kThreads) {
+            uint4 r[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                r[u] = t0 + u * kThreads < t_hi ? __ldg(rec + t0 + u * kThreads) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                if (t0 + u * kThreads < t_hi) run += record_mass(r[u], K);
+        }
+        run = warp_scan_i128(run, lane);
+        if (lane == 31) wsum[warp] = run;
+        __syncthreads();
+        if (warp == 0) {
+            const i128 v = warp_scan_i128(lane < kWarps ? wsum[lane] : (i128)0, lane);
+            if (lane == 31) cta_sum = v;
+        }
+    }
+    cluster.sync();
+    i128 base = 0, Wt = 0;
+    if (ok) {
+        for (int c = 0; c < kCarryCtas; ++c) {
+            const i128 v = *cluster.map_shared_rank(&cta_sum, c);
+            if (c < (int)blockIdx.x) base += v;
+            Wt += v;
+        }
+    }
+    cluster.sync();  // no CTA leaves while another may still read its shared memory
+    if (!ok) {
         if (tid == 0 && blockIdx.x == 0) {
             set_status(pm.ctl + CTL_STATUS, ST_DOMAIN);
             out->ok = 0;
         }
         return;
-    }
-    // the mass of every tile, split into what lies below this CTA's tiles and the rest
-    i128 below = 0, all = 0;
-    for (int i = tid; i < T; i += kThreads) {
-        const i128 m = record_mass(__ldg(rec + i), K);
-        all += m;
-        if (i < t_first) below += m;
-    }
-    const uint4 r = t < T ? __ldg(rec + t) : make_uint4(0u, 0u, 0u, 0xffffffffu);
-    const i128 mine = record_mass(r, K);
-    const i128 inc = warp_scan_i128(mine, lane);
-    // one block scan: the CTA's own masses, its base added to the first warp's
-    const i128 bw = warp_scan_i128(below, lane), aw = warp_scan_i128(all, lane);
-    if (lane == 31) {
-        wsum[warp] = inc;
-        wall[warp] = aw;
-    }
-    __shared__ i128 wbelow[kWarps];
-    if (lane == 31) wbelow[warp] = bw;
-    __syncthreads();
-    i128 B = inc - mine, Wt = 0;
-    for (int w = 0; w < kWarps; ++w) {
-        B += wbelow[w];
-        if (w < warp) B += wsum[w];
-        Wt += wall[w];
     }
     AssignShared as;
     as.Wt = Wt;
@@ -181,27 +210,41 @@ __global__ void __launch_bounds__(kThreads) k_large_carries(SortedParams pm, con
     const fpair W = fixed_to_pair(Wt);
     as.W_hi = W.hi;
     as.W_lo = W.lo;
-    // this tile's lower end; the upper one is the next tile's lower
     const fpair Pp = fast_two_sum((float)pm.P, (float)(pm.P - (int64_t)(float)pm.P));  // P exactly
     const fpair PW = pair_div(Pp, W);
     constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;
-    float x0 = 0.f, x0_end;
-    const long long jlo = t <= T ? offsets_below<kMapKind>(pm, as, PW, B, x0) : 0;
-    jnext[tid] = jlo;
-    if (tid == kThreads - 1 && t < T) jnext[kThreads] = offsets_below<kMapKind>(pm, as, PW, B + mine, x0_end);
-    __syncthreads();
-    if (t < T) {
-        LargeMap m;
-        m.jlo = jlo;
-        m.noff = (int)max(0LL, jnext[tid + 1] - jlo);
-        m.x0 = x0;
-        m.ir = PW.hi * pow2f((int)r.x - K);
-        m.il = (int)r.w;
-        maps[t] = m;
-        if (KIND == KIND_MULTI) {
-            const fpair b = fixed_to_pair(B);
-            table[t] = {b.hi, b.lo, pow2f(K - (int)r.x), (int)r.w};
+    for (int t0 = t_lo; t0 < t_hi; t0 += kThreads) {
+        const int t = t0 + tid;
+        const uint4 r = t < t_hi ? __ldg(rec + t) : make_uint4(0u, 0u, 0u, 0xffffffffu);
+        const i128 mine = t < t_hi ? record_mass(r, K) : (i128)0;
+        const i128 inc = warp_scan_i128(mine, lane);
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        const i128 ws = warp_scan_i128(lane < kWarps ? wsum[lane] : (i128)0, lane);  // every warp: the warps' totals
+        const i128 before = shfl_i128(ws, max(warp, 1) - 1), round = shfl_i128(ws, kWarps - 1);
+        const i128 B = base + (warp > 0 ? before : (i128)0) + inc - mine;
+        base += round;
+        // this tile's lower end; its upper one is the next tile's lower
+        float x0 = 0.f, x0_end;
+        const long long jlo = offsets_below<kMapKind>(pm, as, PW, B, x0);
+        jnext[tid] = jlo;
+        if (tid == kThreads - 1) jnext[kThreads] = offsets_below<kMapKind>(pm, as, PW, B + mine, x0_end);
+        __syncthreads();
+        if (t < t_hi) {
+            LargeMap m;
+            m.jlo = jlo;
+            m.noff = (int)max(0LL, jnext[tid + 1] - jlo);
+            m.x0 = x0;
+            m.ir = PW.hi * pow2f((int)r.x - K);
+            m.il = (int)r.w;
+            maps[t] = m;
+            if (KIND == KIND_MULTI) {
+                const fpair b = fixed_to_pair(B);
+                table[t] = {b.hi, b.lo, pow2f(K - (int)r.x), (int)r.w};
+            }
         }
+        // the next round writes wsum only after every thread has read it (the barrier
+        // above), and jnext only after its own first barrier
     }
     if (tid == 0 && blockIdx.x == 0) *out = {1, W.hi, W.lo};
 }
@@ -220,6 +263,11 @@ struct LargeShared {
 };
 static_assert(sizeof(LargeShared) % 16 == 0, "the staging buffers are 16-byte aligned");
 
+// Bound by DRAM and its latency (systematic: 5 TB/s of reads and writes) and, with the
+// strata's draws, by instruction issue (65% of the slots).  Maps formed by warp 0 behind
+// a barrier per tile, and tiles staged by bulk copies behind another, had taken 77 us
+// (systematic) and 112 us (stratified) at P = 2^25 + 4096; without any barrier between
+// the maps' batches 53 and 79 us.  Asking L2 for the next share while decoding one: 56 and 77 us.
 template <int KIND, int S>
 __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, int64_t PA, const LargeMap* maps,
                                                               const LargeScalars* sc) {
@@ -354,7 +402,7 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
         pm.Pd = (double)M;
         pm.guide = 1;
     }
-    k_large_carries<KIND><<<(T + kThreads - 1) / kThreads, kThreads, 0, s>>>(pm, rec, maps, table, sc);
+    k_large_carries<KIND><<<kCarryCtas, kThreads, 0, s>>>(pm, rec, maps, table, sc);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;

@@ -198,12 +198,6 @@ __device__ __forceinline__ i128 warp_sum_i128(i128 v) {
     return v;
 }
 
-__device__ __forceinline__ i128 shfl_i128(i128 v, int src) {
-    const unsigned long long lo = __shfl_sync(0xffffffffu, (unsigned long long)v, src);
-    const unsigned long long hi = __shfl_sync(0xffffffffu, (unsigned long long)(v >> 64), src);
-    return (i128)(((unsigned __int128)hi << 64) | lo);
-}
-
 // v 2^{-sh} for v >= 0, truncated; sh >= 0.
 __device__ __forceinline__ i128 shr_i128(i128 v, int sh) { return sh >= 127 ? (i128)0 : (v >> sh); }
 
