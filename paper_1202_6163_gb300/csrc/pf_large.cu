@@ -2,7 +2,7 @@
 // schemes (Section 2, Figure 1a-c) for P + lead > PF_MAX_CUMULATIVE, up to
 // 2^31 - 1 particles.  Three ordinary launches in stream order, with no wait of
 // one CTA on another:
-//   1. k_large_scan: tiles of 8192 log-weights, grid-stride, each bulk-copied
+//   1. k_large_scan: tiles of 8192 log-weights, grid-stride, each copied
 //      into shared memory while the CTA's previous tile is scanned: the tile
 //      scan (pf_tile.cuh), a 16-byte record (k_t, S_t, i_last) and the tile's
 //      cumulative weights v_i (sign bit: zero weight);
@@ -59,61 +59,48 @@ __device__ __forceinline__ i128 record_mass(uint4 r, int K) {
 
 // ---------------------------------------------------------------------------
 // Launch 1: the tile scans.  A CTA's tiles are t = blockIdx.x + r gridDim.x;
-// tile r + 1 is bulk-copied into one of two shared-memory buffers while tile r
-// is scanned from the other.
+// tile r + 1 is copied into one of two shared-memory buffers while tile r is
+// scanned from the other.  P = 2^25 + 4096: 66 us with bulk copies (cp.async.bulk,
+// whose plain order makes the scan's 16-byte reads conflict four ways), 61 us with
+// per-thread copies into the conflict-free order.
 // ---------------------------------------------------------------------------
-struct ScanShared {
-    TileShared tile;
-    uint64_t bar[2];
-};
-constexpr size_t kScanSmem = ((sizeof(ScanShared) + 15) & ~(size_t)15) + 2 * (size_t)kLargeTile * sizeof(float);
-
-// Thread 0: the copy of this CTA's tile r (its whole 16-byte pieces) into buf,
-// completing on bar.
-__device__ __forceinline__ void issue_tile_copy(const float* src, int64_t PA, int r, float* buf, uint64_t* bar) {
-    const int64_t t0 = (int64_t)(blockIdx.x + (int64_t)r * gridDim.x) * kLargeTile;
-    const uint32_t bytes = (uint32_t)((int)min((int64_t)kLargeTile, PA - t0) & ~3) * 4u;
-    if (bytes) bulk_load(buf, src + t0, bytes, bar);
-    else mbar_arrive(bar);
-}
+constexpr size_t kScanSmem = ((sizeof(TileShared) + 15) & ~(size_t)15) + 2 * (size_t)kLargeTile * sizeof(float);
 
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2) k_large_scan(SortedParams p, uint4* rec) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ScanShared& sm = *reinterpret_cast<ScanShared*>(smem_raw);
-    float* slot = reinterpret_cast<float*>(smem_raw + ((sizeof(ScanShared) + 15) & ~(size_t)15));
+    TileShared& sm = *reinterpret_cast<TileShared*>(smem_raw);
+    float* slot = reinterpret_cast<float*>(smem_raw + ((sizeof(TileShared) + 15) & ~(size_t)15));
     const int tid = threadIdx.x;
     const int64_t PA = p.P + p.lead;
     const int n_mine = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // grid <= tiles
-    if (tid == 0) {
-        mbar_init(&sm.bar[0], 1);
-        mbar_init(&sm.bar[1], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (tid == 0) issue_tile_copy(p.lw, PA, 0, slot, &sm.bar[0]);
+    auto start = [&](int r) {
+        const int64_t t0 = (int64_t)(blockIdx.x + (int64_t)r * gridDim.x) * kLargeTile;
+        stage_tile(p.lw + t0, (int)min((int64_t)kLargeTile, PA - t0), slot + (r & 1) * kLargeTile);
+    };
+    start(0);
     TileThread th;
     for (int r = 0; r < n_mine; ++r) {
         const int t = (int)blockIdx.x + r * (int)gridDim.x;
         const int64_t t0 = (int64_t)t * kLargeTile;
         const int n = (int)min((int64_t)kLargeTile, PA - t0);
-        if (tid == 0 && r + 1 < n_mine)
-            issue_tile_copy(p.lw, PA, r + 1, slot + ((r + 1) & 1) * kLargeTile, &sm.bar[(r + 1) & 1]);
-        // a copy not complete within the wait limit (from this wait's start) is
-        // reported; the results are then unspecified
-        if (!mbar_wait(&sm.bar[r & 1], (uint32_t)(r >> 1) & 1u, global_ns(), p.wait_ns) && tid == 0)
-            set_status(p.ctl + CTL_STATUS, ST_TIMEOUT);
+        if (r + 1 < n_mine) {
+            start(r + 1);
+            async_wait<1>();
+        } else {
+            async_wait<0>();
+        }
+        __syncthreads();
         // a ragged last tile: its tail is not in the copy; read it from global memory
         const int lo = t == 0 ? p.lead : 0;
-        const TileSummary ts = (n & 3) == 0 ? tile_scan_k<16, true>(slot + (r & 1) * kLargeTile, lo, n, sm.tile, th)
-                                            : tile_scan_k<16>(p.lw + t0, lo, n, sm.tile, th);
+        const TileSummary ts = (n & 3) == 0 ? tile_scan_k<16, true>(slot + (r & 1) * kLargeTile, lo, n, sm, th)
+                                            : tile_scan_k<16>(p.lw + t0, lo, n, sm, th);
         if (ts.bad && tid == 0) set_status(p.ctl + CTL_STATUS, ST_DOMAIN);
         write_tile_v<16>(p, th, t0, n);  // read back by launch 3
         if (tid == 0)
             rec[t] = make_uint4((uint32_t)ts.k, __float_as_uint(ts.bad ? NAN : ts.S.hi), __float_as_uint(ts.S.lo),
                                 (uint32_t)ts.i_last);
-        fence_proxy_async_smem();  // this tile's reads of its buffer before the buffer's next copy
-        __syncthreads();           // and the tile scan's shared fields are reused by the next tile
+        __syncthreads();  // the buffer and the tile scan's shared fields are reused
     }
 }
 

@@ -56,27 +56,49 @@ __device__ __forceinline__ int per_thread_count(int n) {
 
 __device__ __forceinline__ bool zero_flag(float v) { return __float_as_uint(v) >> 31; }
 
+// A tile staged in shared memory (16 elements per thread): 16-byte chunk (t, q), the
+// q-th of thread t's four, lies at place (q + t / 2) mod 4 of the thread's 64 bytes, so
+// that eight neighbouring threads' reads of their q-th chunks meet no bank conflict
+// (in plain order they meet four-way ones).
+__device__ __forceinline__ int stage_place(int t, int q) { return 16 * t + 4 * ((q + (t >> 1)) & 3); }
+
+// Block-wide: this CTA's asynchronous copies of the whole 16-byte chunks of src[0..n) (src 16-byte
+// aligned) into buf, as one group per thread; the caller waits for the group and meets a barrier.
+__device__ __forceinline__ void stage_tile(const float* src, int n, float* buf) {
+    const int c0 = threadIdx.x;  // chunk q kThreads + c0: coalesced
+    float* to = buf + stage_place(c0 >> 2, c0 & 3);
+    const float* from = src + 4 * c0;
+#pragma unroll
+    for (int q = 0; q < kMaxPerThread / 4; ++q)
+        if (n == kTileMax || 4 * (q * kThreads + c0) + 3 < n)
+            async_copy16(to + q * kThreads * 4, from + q * kThreads * 4);
+    async_commit();
+}
+static_assert((kThreads / 4) % 8 == 0, "chunks a CTA apart have the same place");
+
 // Loads this thread's KK elements (tile-local e0 .. e0+KK) of base[lo..n);
-// base is 16-byte aligned, in global memory or (SMEM) in shared memory.
+// base is 16-byte aligned in global memory, or (SMEM) a tile staged by stage_tile.
 // Slots outside [lo, n) read as -inf (zero weight).
 template <int KK, bool SMEM = false>
 __device__ __forceinline__ void tile_load_k(const float* __restrict__ base, int lo, int n, int e0,
                                             float (&x)[kMaxPerThread]) {
+    static_assert(!SMEM || KK == kMaxPerThread, "tiles are staged in full");
+    if (e0 >= lo && e0 + KK <= n) {  // nearly every thread
 #pragma unroll
-    for (int q = 0; q < KK / 4; ++q) {
-        const int idx = e0 + 4 * q;
-        if (idx >= lo && idx + 3 < n) {
-            const float4 v = SMEM ? *reinterpret_cast<const float4*>(base + idx)
-                                  : __ldg(reinterpret_cast<const float4*>(base + idx));
+        for (int q = 0; q < KK / 4; ++q) {
+            const float4 v = SMEM ? *reinterpret_cast<const float4*>(base + stage_place(threadIdx.x, q))
+                                  : __ldg(reinterpret_cast<const float4*>(base + e0 + 4 * q));
             x[4 * q + 0] = v.x;
             x[4 * q + 1] = v.y;
             x[4 * q + 2] = v.z;
             x[4 * q + 3] = v.w;
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-                x[4 * q + r] = (idx + r >= lo && idx + r < n) ? (SMEM ? base[idx + r] : __ldg(base + idx + r)) : -INFINITY;
         }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < KK; ++i) {
+        const float* src = SMEM ? base + stage_place(threadIdx.x, i >> 2) + (i & 3) : base + e0 + i;
+        x[i] = (e0 + i >= lo && e0 + i < n) ? (SMEM ? *src : __ldg(src)) : -INFINITY;
     }
 }
 
