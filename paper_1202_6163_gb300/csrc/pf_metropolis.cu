@@ -21,6 +21,7 @@ namespace pf {
 
 constexpr int kMetroThreads = 256;
 constexpr int kMetroSmemFloats = 48 * 1024;  // 192 KiB staging limit
+constexpr float kWeightFloor = 0x1p-100f;    // staged weights below it decide in log space
 
 // Accept a move from k to j (log-weights lk, lj) with uniform u.
 __device__ __forceinline__ bool metropolis_accept(float lj, float lk, float u) {
@@ -32,25 +33,82 @@ __device__ __forceinline__ bool metropolis_accept(float lj, float lk, float u) {
     return u < r;
 }
 
-// B steps of chain i from state (k, lk).  The proposals do not depend on the
-// chain's state, so each group of kAhead steps draws its proposals first and
-// issues all their log-weight loads before resolving the steps in order.
+// The chain's Philox stream with everything taken out of the steps that does not
+// depend on the step.  Of the counter (i, step / 2, filter, tag) only one word varies, so
+// the first three rounds come down to two products: round 0 multiplies i and filter,
+// round 1 multiplies the step's word (xored with a constant) and a constant, round 2 a
+// constant and what round 1 made of the step.  The later rounds' keys are kept in
+// registers (opaque to the compiler, which otherwise forms them anew in every call: two
+// additions a round).  34 instructions a call instead of about 60; a call serves two steps.
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+template <int ROUNDS>
+struct ChainStream {
+    uint32_t f0, e2, h0, j2, g3;
+    uint32_t k0[ROUNDS - 3], k1[ROUNDS - 3];
+
+    __device__ __forceinline__ void set_key(uint32_t key0, uint32_t key1) {
+#pragma unroll
+        for (int r = 3; r < ROUNDS; ++r) {
+            k0[r - 3] = key0 + (uint32_t)r * 0x9E3779B9u;
+            k1[r - 3] = key1 + (uint32_t)r * 0xBB67AE85u;
+            asm volatile("" : "+r"(k0[r - 3]), "+r"(k1[r - 3]));
+        }
+    }
+    __device__ __forceinline__ void set_chain(uint32_t i, uint32_t filter, uint32_t key0, uint32_t key1) {
+        const uint64_t b0 = (uint64_t)kPhiloxM1 * filter, a0 = (uint64_t)kPhiloxM0 * i;
+        f0 = (uint32_t)(b0 >> 32) ^ key0;
+        const uint32_t c2 = (uint32_t)(a0 >> 32) ^ (uint32_t)TAG_METRO ^ key1;
+        const uint64_t b1 = (uint64_t)kPhiloxM1 * c2;
+        const uint32_t d0 = (uint32_t)(b1 >> 32) ^ (uint32_t)b0 ^ (key0 + 0x9E3779B9u);
+        e2 = (uint32_t)a0 ^ (key1 + 0xBB67AE85u);
+        h0 = (uint32_t)b1 ^ (key0 + 2u * 0x9E3779B9u);
+        const uint64_t a2 = (uint64_t)kPhiloxM0 * d0;
+        j2 = (uint32_t)(a2 >> 32) ^ (key1 + 2u * 0xBB67AE85u);
+        g3 = (uint32_t)a2;
+    }
+    __device__ __forceinline__ u32x4 words(uint32_t half_step) const {
+        const uint64_t a1 = (uint64_t)kPhiloxM0 * (f0 ^ half_step);
+        const uint64_t b2 = (uint64_t)kPhiloxM1 * ((uint32_t)(a1 >> 32) ^ e2);
+        uint32_t c0 = (uint32_t)(b2 >> 32) ^ h0, c1 = (uint32_t)b2, c2 = (uint32_t)a1 ^ j2, c3 = g3;
+#pragma unroll
+        for (int r = 0; r < ROUNDS - 3; ++r) {
+            const uint64_t a = (uint64_t)kPhiloxM0 * c0, b = (uint64_t)kPhiloxM1 * c2;
+            c0 = (uint32_t)(b >> 32) ^ c1 ^ k0[r];
+            c1 = (uint32_t)b;
+            c2 = (uint32_t)(a >> 32) ^ c3 ^ k1[r];
+            c3 = (uint32_t)a;
+        }
+        return {c0, c1, c2, c3};
+    }
+};
+
+// Proposals and uniforms of steps b0 .. b0 + kAhead - 1 (b0 even).
 constexpr int kAhead = 4;
 
 template <int ROUNDS>
-__device__ __forceinline__ void run_chain(const float* __restrict__ lw, uint32_t Pu, uint32_t i, int steps,
-                                          uint32_t filter, uint32_t key0, uint32_t key1, uint32_t& k, float& lk) {
+__device__ __forceinline__ void draw_steps(const ChainStream<ROUNDS>& rng, int b0, uint32_t Pu, uint32_t (&jj)[kAhead],
+                                           float (&uu)[kAhead]) {
+#pragma unroll
+    for (int q = 0; q < kAhead / 2; ++q) {
+        const u32x4 r = rng.words((uint32_t)((b0 >> 1) + q));
+        jj[2 * q] = draw_index(r.x, Pu);
+        uu[2 * q] = u23f(r.y);
+        jj[2 * q + 1] = draw_index(r.z, Pu);
+        uu[2 * q + 1] = u23f(r.w);
+    }
+}
+
+// B steps of a chain from state (k, lk).  The proposals do not depend on the
+// chain's state, so each group of kAhead steps draws its proposals first and
+// issues all their log-weight loads before resolving the steps in order.
+template <int ROUNDS>
+__device__ __forceinline__ void run_chain(const float* __restrict__ lw, uint32_t Pu, const ChainStream<ROUNDS>& rng,
+                                          int steps, uint32_t& k, float& lk) {
     for (int b0 = 0; b0 < steps; b0 += kAhead) {
         uint32_t jj[kAhead];
         float uu[kAhead], ll[kAhead];
-#pragma unroll
-        for (int q = 0; q < kAhead / 2; ++q) {
-            const u32x4 r = philox<ROUNDS>(i, (uint32_t)((b0 >> 1) + q), filter, TAG_METRO, key0, key1);
-            jj[2 * q] = draw_index(r.x, Pu);
-            uu[2 * q] = u23f(r.y);
-            jj[2 * q + 1] = draw_index(r.z, Pu);
-            uu[2 * q + 1] = u23f(r.w);
-        }
+        draw_steps(rng, b0, Pu, jj, uu);
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) ll[s] = __ldg(lw + jj[s]);
 #pragma unroll
@@ -63,44 +121,67 @@ __device__ __forceinline__ void run_chain(const float* __restrict__ lw, uint32_t
     }
 }
 
-// B steps of chain i from state k over staged weights w (shared memory).
-constexpr float kWeightFloor = 0x1p-100f;
-
-template <int ROUNDS>
-__device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const float* w, uint32_t Pu, uint32_t i,
-                                            int steps, uint32_t filter, uint32_t key0, uint32_t key1, uint32_t& k) {
+// B steps of a chain from state k over staged weights w (shared memory).  CLEAN:
+// every staged weight is at least kWeightFloor, so no step looks at the log-weights.
+template <int ROUNDS, bool CLEAN>
+__device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const float* w, uint32_t Pu,
+                                            const ChainStream<ROUNDS>& rng, int steps, uint32_t& k) {
     float wk = w[k];
-    for (int b0 = 0; b0 < steps; b0 += kAhead) {
-        uint32_t jj[kAhead];
-        float uu[kAhead], ww[kAhead];
-#pragma unroll
-        for (int q = 0; q < kAhead / 2; ++q) {
-            const u32x4 r = philox<ROUNDS>(i, (uint32_t)((b0 >> 1) + q), filter, TAG_METRO, key0, key1);
-            jj[2 * q] = draw_index(r.x, Pu);
-            uu[2 * q] = u23f(r.y);
-            jj[2 * q + 1] = draw_index(r.z, Pu);
-            uu[2 * q + 1] = u23f(r.w);
+    auto step = [&](uint32_t j, float u, float wj) {
+        const bool acc = CLEAN || wk >= kWeightFloor ? __fmul_rn(u, wk) < wj
+                                                     : metropolis_accept(__ldg(lw + j), __ldg(lw + k), u);
+        if (acc) {
+            k = j;
+            wk = wj;
         }
+    };
+    uint32_t jj[kAhead];
+    float uu[kAhead], ww[kAhead];
+    int b0 = 0;
+    for (; b0 + kAhead <= steps; b0 += kAhead) {
+        draw_steps(rng, b0, Pu, jj, uu);
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) ww[s] = w[jj[s]];
 #pragma unroll
-        for (int s = 0; s < kAhead; ++s) {
-            if (b0 + s < steps) {
-                const bool acc = wk >= kWeightFloor ? __fmul_rn(uu[s], wk) < ww[s]
-                                                    : metropolis_accept(__ldg(lw + jj[s]), __ldg(lw + k), uu[s]);
-                if (acc) {
-                    k = jj[s];
-                    wk = ww[s];
-                }
-            }
-        }
+        for (int s = 0; s < kAhead; ++s) step(jj[s], uu[s], ww[s]);
     }
+    if (b0 < steps) {
+        draw_steps(rng, b0, Pu, jj, uu);
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s)
+            if (b0 + s < steps) step(jj[s], uu[s], w[jj[s]]);
+    }
+}
+
+// Chain i of a filter with staged or unstaged weights, written to anc[i].
+template <int ROUNDS>
+__device__ __forceinline__ void run_staged(const float* lw, const float* w, bool clean, uint32_t Pu, uint32_t i, int steps,
+                                           uint32_t filter, uint32_t key0, uint32_t key1, ChainStream<ROUNDS>& rng,
+                                           int32_t* anc) {
+    uint32_t k = i;
+    rng.set_chain(i, filter, key0, key1);
+    if (clean) run_chain_w<ROUNDS, true>(lw, w, Pu, rng, steps, k);
+    else run_chain_w<ROUNDS, false>(lw, w, Pu, rng, steps, k);
+    anc[i] = (int32_t)k;
+}
+
+template <int ROUNDS>
+__device__ __forceinline__ void run_unstaged(const float* __restrict__ lw, uint32_t Pu, uint32_t i, int steps,
+                                             uint32_t filter, uint32_t key0, uint32_t key1, ChainStream<ROUNDS>& rng,
+                                             int32_t* anc, uint32_t* ctl) {
+    uint32_t k = i;
+    float lk = __ldg(lw + i);
+    if (!(lk <= 3.402823466e38f)) set_status(ctl + CTL_STATUS, ST_DOMAIN);  // NaN or +inf
+    rng.set_chain(i, filter, key0, key1);
+    run_chain<ROUNDS>(lw, Pu, rng, steps, k, lk);
+    anc[i] = (int32_t)k;
 }
 
 // Block-wide: copy lw[0..n) to w[] as weights exp(lw - m), m = max lw (0 when
 // every weight is zero); records PF_ERR_DOMAIN for a NaN or +inf log-weight.
+// Returns whether every weight is at least kWeightFloor.
 template <int THREADS>
-__device__ void stage_weights(const float* __restrict__ lw, int64_t n, float* w, float* red, uint32_t* ctl) {
+__device__ bool stage_weights(const float* __restrict__ lw, int64_t n, float* w, float* red, uint32_t* ctl) {
     const int tid = threadIdx.x;
     float m = -INFINITY;
     int bad = 0;
@@ -135,8 +216,13 @@ __device__ void stage_weights(const float* __restrict__ lw, int64_t n, float* w,
 #pragma unroll
     for (int q = 1; q < THREADS / 32; ++q) mt = fmaxf(mt, red[q]);
     const fpair R = {mt > -INFINITY ? mt : 0.f, 0.f};
-    for (int64_t q = tid; q < n; q += THREADS) w[q] = weight_rel(w[q], R);
-    __syncthreads();
+    bool clean = true;
+    for (int64_t q = tid; q < n; q += THREADS) {
+        const float x = weight_rel(w[q], R);
+        w[q] = x;
+        clean = clean && x >= kWeightFloor;
+    }
+    return __syncthreads_and(clean) != 0;
 }
 
 // Block-wide: the largest normalised weight w_max = max_i w_i / sum_i w_i of
@@ -217,19 +303,15 @@ __global__ void __launch_bounds__(kMetroThreads) k_metropolis(const float* __res
                                                               int32_t* __restrict__ anc, uint32_t* ctl) {
     extern __shared__ float wsm[];
     __shared__ float red[kMetroThreads / 32];
-    if (STAGED) stage_weights<kMetroThreads>(lw, P, wsm, red, ctl);  // every CTA: the whole vector
+    bool clean = false;
+    if (STAGED) clean = stage_weights<kMetroThreads>(lw, P, wsm, red, ctl);  // every CTA: the whole vector
     const int steps = B_dev ? (int)__ldg(B_dev) : B;
     const uint32_t Pu = (uint32_t)P;
+    ChainStream<ROUNDS> rng;
+    rng.set_key(key0, key1);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t k = (uint32_t)i;
-        if (STAGED) {
-            run_chain_w<ROUNDS>(lw, wsm, Pu, (uint32_t)i, steps, filter, key0, key1, k);
-        } else {
-            float lk = __ldg(lw + i);
-            if (!(lk <= 3.402823466e38f)) set_status(ctl + CTL_STATUS, ST_DOMAIN);  // NaN or +inf
-            run_chain<ROUNDS>(lw, Pu, (uint32_t)i, steps, filter, key0, key1, k, lk);
-        }
-        anc[i] = (int32_t)k;
+        if (STAGED) run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc);
+        else run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc, ctl);
     }
 }
 
@@ -311,8 +393,9 @@ __device__ __forceinline__ uint32_t claim_block(unsigned long long* w, uint32_t 
 // The chains of blocks claimed from filter f (block-wide; the weights are staged).
 template <int ROUNDS>
 __device__ __forceinline__ void run_claimed_blocks(const BatchParams& bp, const float* lw, const float* wsm, bool staged,
-                                                   int64_t Pf, int64_t off0, int steps, int f, uint32_t epoch,
-                                                   uint32_t key0, uint32_t key1, int* blk_sm) {
+                                                   bool clean, int64_t Pf, int64_t off0, int steps, int f,
+                                                   uint32_t epoch, uint32_t key0, uint32_t key1,
+                                                   ChainStream<ROUNDS>& rng, int* blk_sm) {
     const int tid = threadIdx.x;
     const uint32_t Pu = (uint32_t)Pf;
     const int64_t nblk = (Pf + kMetroBThreads - 1) / kMetroBThreads;
@@ -324,15 +407,10 @@ __device__ __forceinline__ void run_claimed_blocks(const BatchParams& bp, const 
         if (blk >= nblk) break;
         const int64_t i = blk * kMetroBThreads + tid;
         if (i < Pf) {
-            uint32_t k = (uint32_t)i;
-            if (staged) {
-                run_chain_w<ROUNDS>(lw, wsm, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, k);
-            } else {
-                float lk = __ldg(lw + i);
-                if (!(lk <= 3.402823466e38f)) set_status(bp.ctl + CTL_STATUS, ST_DOMAIN);
-                run_chain<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, k, lk);
-            }
-            bp.anc[off0 + i] = (int32_t)k;
+            if (staged)
+                run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0);
+            else
+                run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0, bp.ctl);
         }
     }
 }
@@ -345,6 +423,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
     const int tid = threadIdx.x;
     const int n_items = (int)ld_relaxed_u32(bp.ctl + CTL_ITEMS);
     const uint32_t epoch = ld_relaxed_u32(bp.ctl + CTL_METRO_EPOCH);
+    ChainStream<ROUNDS> rng;
     for (;;) {
         if (tid == 0) f_sm = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
         __syncthreads();
@@ -366,7 +445,8 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             trace_put(bp.trace, bp.trace_cap, ticket, 6, (uint64_t)f);
             trace_put(bp.trace, bp.trace_cap, ticket, 7, (uint64_t)(bp.items[ticket] & 31));
         }
-        if (staged) stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
+        bool clean = false;
+        if (staged) clean = stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
         for (int w = 1; w <= 2; ++w) trace_stamp(bp.trace, bp.trace_cap, ticket, w);
         // B < 0: this filter's own step count from Eq. 5 and its largest normalised weight
         int steps = bp.B;
@@ -384,6 +464,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
         const uint64_t seed = bp.seeds[f];
         const uint32_t key0 = (uint32_t)(seed & 0xffffffffu), key1 = (uint32_t)(seed >> 32);
         const uint32_t Pu = (uint32_t)Pf;
+        rng.set_key(key0, key1);
         const bool heavy = bp.metro != nullptr && Pf > kMetroBThreads && Pf * (long long)max(steps, 1) >= kHeavyWork;
         if (heavy) {
             // publish the step count, then list the filter for CTAs with nothing left to take
@@ -396,18 +477,15 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
                     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(list + h), "r"(f + 1) : "memory");
                 }
             }
-            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, Pf, off0, steps, f, epoch, key0, key1, &blk_sm);
+            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
         } else {
             for (int64_t i = tid; i < Pf; i += kMetroBThreads) {
-                uint32_t k = (uint32_t)i;
-                if (staged) {
-                    run_chain_w<ROUNDS>(lw, wsm, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, k);
-                } else {
-                    float lk = __ldg(lw + i);
-                    if (!(lk <= 3.402823466e38f)) set_status(bp.ctl + CTL_STATUS, ST_DOMAIN);
-                    run_chain<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, k, lk);
-                }
-                bp.anc[off0 + i] = (int32_t)k;
+                if (staged)
+                    run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng,
+                                       bp.anc + off0);
+                else
+                    run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0,
+                                         bp.ctl);
             }
         }
         __syncthreads();  // the staging buffer is reused by the next filter
@@ -451,10 +529,12 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             const int64_t Pf = bp.offsets[f + 1] - off0;
             const float* lw = bp.lw + off0;
             const bool staged = Pf <= kMetroBStage;
-            if (staged) stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
+            bool clean = false;
+            if (staged) clean = stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
             const uint64_t seed = bp.seeds[f];
-            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, Pf, off0, steps, f, epoch, (uint32_t)(seed & 0xffffffffu),
-                               (uint32_t)(seed >> 32), &blk_sm);
+            const uint32_t key0 = (uint32_t)(seed & 0xffffffffu), key1 = (uint32_t)(seed >> 32);
+            rng.set_key(key0, key1);
+            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
             __syncthreads();  // the staging buffer is reused by the next listed filter
         }
     }
