@@ -199,6 +199,11 @@ pf_status ensure_metro(Workspace& w, size_t n, cudaStream_t s) {
     return PF_OK;
 }
 
+// Floats of scratch per CTA of a batched call.
+int64_t batched_scratch_of(int kind) {
+    return kind == PF_METROPOLIS ? (int64_t)kMetroScratchFloats : (int64_t)batched_scratch_floats_per_cta();
+}
+
 size_t lg_record_bytes(int F, int64_t P) {
     const int64_t tiles = (P + lg_tile() - 1) / lg_tile();
     return (size_t)F * (size_t)tiles * sizeof(float4);
@@ -465,8 +470,8 @@ pf_status resample_batched(int kind, const float* logw, const int64_t* offsets, 
     // scratch: per-CTA cumulative weights (multinomial), the plan's items, the
     // split filters' tile records; two counters per filter
     // per-CTA scratch: the cumulative weights of a whole filter's tiles (multinomial, and
-    // systematic / stratified filters kept whole in one CTA)
-    const int64_t per_cta = kind != PF_METROPOLIS ? (int64_t)batched_scratch_floats_per_cta() : 0;
+    // systematic / stratified filters kept whole in one CTA), the Metropolis weights beyond the staging
+    const int64_t per_cta = batched_scratch_of(kind);
     const size_t items_at = ((size_t)grid * per_cta * sizeof(float) + 255) & ~(size_t)255;
     const size_t n_items = (size_t)F * kMaxItemsPerFilter;
     const size_t records_at = (items_at + n_items * sizeof(int32_t) + 255) & ~(size_t)255;
@@ -549,7 +554,7 @@ pf_status pf_reserve(int64_t P_max, int64_t total_max, int F_max, void* stream) 
     }
     if (F_max > 0) {
         for (int k = PF_MULTINOMIAL; k <= PF_METROPOLIS; ++k) {
-            const size_t per_cta = k != PF_METROPOLIS ? batched_scratch_floats_per_cta() : 0;
+            const size_t per_cta = (size_t)batched_scratch_of(k);
             const size_t items_at =
                 ((size_t)info->num_sms * info->batched_per_sm[k] * per_cta * sizeof(float) + 255) & ~(size_t)255;
             const size_t n_items = (size_t)F_max * kMaxItemsPerFilter;

@@ -87,7 +87,7 @@ struct BatchParams {
     const uint64_t* seeds;
     int32_t* anc;
     uint32_t* ctl;
-    float* scratch;           // multinomial: per-CTA cumulative weights of multi-tile filters
+    float* scratch;           // per CTA: cumulative weights of multi-tile filters; Metropolis: weights beyond the staging
     int64_t scratch_per_cta;  // floats per CTA
     const int32_t* items;     // work items from the plan pass: f * 32 + tile, or f * 32 + 31 (whole filter)
     uint4* records;           // one 16-byte tile record per item (split filters)
@@ -183,6 +183,7 @@ constexpr int kMaxHeavy = 4096;  // batched Metropolis: length of the list of sh
 constexpr int kMaxItemsPerFilter = 16;  // tiles of a batched filter (kMaxOwnB)
 int batched_blocks_per_sm(int kind);
 size_t batched_scratch_floats_per_cta();
+constexpr int kMetroScratchFloats = 56 * 1024;  // batched Metropolis: a CTA's scratch for the weights it cannot stage
 cudaError_t launch_batched_metropolis(const BatchParams& bp, int grid, cudaStream_t s);
 int batched_metropolis_blocks_per_sm();
 

@@ -121,15 +121,35 @@ __device__ __forceinline__ void run_chain(const float* __restrict__ lw, uint32_t
     }
 }
 
-// B steps of a chain from state k over staged weights w (shared memory).  CLEAN:
-// every staged weight is at least kWeightFloor, so no step looks at the log-weights.
-template <int ROUNDS, bool CLEAN>
-__device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const float* w, uint32_t Pu,
+// A filter's staged weights: those below `held` in shared memory, the rest (SPLIT) in
+// global memory.
+struct StagedWeights {
+    float* w;
+    float* rest;    // weight of particle held + i at rest[i]
+    uint32_t held;
+    template <bool SPLIT>
+    __device__ __forceinline__ float at(uint32_t j) const {
+        if (!SPLIT || j < held) return w[j];
+        return rest[j - held];
+    }
+};
+
+// B steps of a chain from state k over staged weights.  CLEAN: every staged weight is
+// at least kWeightFloor, so no step looks at the log-weights.  SPLIT: a filter
+// beyond shared memory, whose steps decide by the rule on log-weights: the product
+// decides where it is further from a tie than the weights' errors reach (7e-7
+// relative, five times over), and the log-weights where it is not.
+constexpr float kTieBand = 4e-6f;
+
+template <int ROUNDS, bool CLEAN, bool SPLIT>
+__device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const StagedWeights& sw, uint32_t Pu,
                                             const ChainStream<ROUNDS>& rng, int steps, uint32_t& k) {
-    float wk = w[k];
+    float wk = sw.at<SPLIT>(k);
     auto step = [&](uint32_t j, float u, float wj) {
-        const bool acc = CLEAN || wk >= kWeightFloor ? __fmul_rn(u, wk) < wj
-                                                     : metropolis_accept(__ldg(lw + j), __ldg(lw + k), u);
+        const float t = __fmul_rn(u, wk);
+        bool acc = t < wj;
+        if ((!CLEAN && !(wk >= kWeightFloor)) || (SPLIT && fabsf(__fsub_rn(t, wj)) <= kTieBand * wj))
+            acc = metropolis_accept(__ldg(lw + j), __ldg(lw + k), u);
         if (acc) {
             k = j;
             wk = wj;
@@ -141,7 +161,7 @@ __device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const 
     for (; b0 + kAhead <= steps; b0 += kAhead) {
         draw_steps(rng, b0, Pu, jj, uu);
 #pragma unroll
-        for (int s = 0; s < kAhead; ++s) ww[s] = w[jj[s]];
+        for (int s = 0; s < kAhead; ++s) ww[s] = sw.at<SPLIT>(jj[s]);
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) step(jj[s], uu[s], ww[s]);
     }
@@ -149,19 +169,19 @@ __device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const 
         draw_steps(rng, b0, Pu, jj, uu);
 #pragma unroll
         for (int s = 0; s < kAhead; ++s)
-            if (b0 + s < steps) step(jj[s], uu[s], w[jj[s]]);
+            if (b0 + s < steps) step(jj[s], uu[s], sw.at<SPLIT>(jj[s]));
     }
 }
 
-// Chain i of a filter with staged or unstaged weights, written to anc[i].
-template <int ROUNDS>
-__device__ __forceinline__ void run_staged(const float* lw, const float* w, bool clean, uint32_t Pu, uint32_t i, int steps,
-                                           uint32_t filter, uint32_t key0, uint32_t key1, ChainStream<ROUNDS>& rng,
-                                           int32_t* anc) {
+// Chain i of a filter with staged weights, written to anc[i].
+template <int ROUNDS, bool SPLIT>
+__device__ __forceinline__ void run_staged(const float* lw, const StagedWeights& sw, bool clean, uint32_t Pu, uint32_t i,
+                                           int steps, uint32_t filter, uint32_t key0, uint32_t key1,
+                                           ChainStream<ROUNDS>& rng, int32_t* anc) {
     uint32_t k = i;
     rng.set_chain(i, filter, key0, key1);
-    if (clean) run_chain_w<ROUNDS, true>(lw, w, Pu, rng, steps, k);
-    else run_chain_w<ROUNDS, false>(lw, w, Pu, rng, steps, k);
+    if (clean) run_chain_w<ROUNDS, true, SPLIT>(lw, sw, Pu, rng, steps, k);
+    else run_chain_w<ROUNDS, false, SPLIT>(lw, sw, Pu, rng, steps, k);
     anc[i] = (int32_t)k;
 }
 
@@ -177,37 +197,35 @@ __device__ __forceinline__ void run_unstaged(const float* __restrict__ lw, uint3
     anc[i] = (int32_t)k;
 }
 
-// Block-wide: copy lw[0..n) to w[] as weights exp(lw - m), m = max lw (0 when
-// every weight is zero); records PF_ERR_DOMAIN for a NaN or +inf log-weight.
-// Returns whether every weight is at least kWeightFloor.
+// Block-wide: copy lw[0..n) as weights exp(lw - m), m = max lw (0 when every weight is
+// zero), to shared memory and, from sw.held on, to sw.rest; records PF_ERR_DOMAIN
+// for a NaN or +inf log-weight.  Returns whether every weight is at least kWeightFloor.
 template <int THREADS>
-__device__ bool stage_weights(const float* __restrict__ lw, int64_t n, float* w, float* red, uint32_t* ctl) {
+__device__ bool stage_weights(const float* __restrict__ lw, int64_t n, const StagedWeights& sw, float* red,
+                              uint32_t* ctl) {
     const int tid = threadIdx.x;
+    const int64_t ns = n < (int64_t)sw.held ? n : (int64_t)sw.held;  // those held in shared memory
     float m = -INFINITY;
     int bad = 0;
-    if ((((uintptr_t)lw) & 15u) == 0) {
-        const int64_t n4 = n >> 2;
-        for (int64_t q = tid; q < n4; q += THREADS) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(lw) + q);
-            reinterpret_cast<float4*>(w)[q] = v;
-            m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-            bad |= !(v.x <= 3.402823466e38f) | !(v.y <= 3.402823466e38f) | !(v.z <= 3.402823466e38f) |
-                   !(v.w <= 3.402823466e38f);
-        }
-        for (int64_t q = 4 * n4 + tid; q < n; q += THREADS) {
-            const float x = __ldg(lw + q);
-            w[q] = x;
-            m = fmaxf(m, x);
-            bad |= !(x <= 3.402823466e38f);
-        }
-    } else {
-        for (int64_t q = tid; q < n; q += THREADS) {
-            const float x = __ldg(lw + q);
-            w[q] = x;
-            m = fmaxf(m, x);
-            bad |= !(x <= 3.402823466e38f);
-        }
+    auto see = [&](float x) {
+        m = fmaxf(m, x);
+        bad |= !(x <= 3.402823466e38f);
+    };
+    const int64_t n4 = (((uintptr_t)lw) & 15u) == 0 ? ns >> 2 : 0;
+    for (int64_t q = tid; q < n4; q += THREADS) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(lw) + q);
+        reinterpret_cast<float4*>(sw.w)[q] = v;
+        see(v.x);
+        see(v.y);
+        see(v.z);
+        see(v.w);
     }
+    for (int64_t q = 4 * n4 + tid; q < ns; q += THREADS) {
+        const float x = __ldg(lw + q);
+        sw.w[q] = x;
+        see(x);
+    }
+    for (int64_t q = ns + tid; q < n; q += THREADS) see(__ldg(lw + q));
     m = warp_max(m);
     if ((tid & 31) == 0) red[tid >> 5] = m;
     bad = __syncthreads_or(bad);
@@ -217,9 +235,14 @@ __device__ bool stage_weights(const float* __restrict__ lw, int64_t n, float* w,
     for (int q = 1; q < THREADS / 32; ++q) mt = fmaxf(mt, red[q]);
     const fpair R = {mt > -INFINITY ? mt : 0.f, 0.f};
     bool clean = true;
-    for (int64_t q = tid; q < n; q += THREADS) {
-        const float x = weight_rel(w[q], R);
-        w[q] = x;
+    for (int64_t q = tid; q < ns; q += THREADS) {
+        const float x = weight_rel(sw.w[q], R);
+        sw.w[q] = x;
+        clean = clean && x >= kWeightFloor;
+    }
+    for (int64_t q = ns + tid; q < n; q += THREADS) {
+        const float x = weight_rel(__ldg(lw + q), R);
+        sw.rest[q - ns] = x;
         clean = clean && x >= kWeightFloor;
     }
     return __syncthreads_and(clean) != 0;
@@ -304,13 +327,14 @@ __global__ void __launch_bounds__(kMetroThreads) k_metropolis(const float* __res
     extern __shared__ float wsm[];
     __shared__ float red[kMetroThreads / 32];
     bool clean = false;
-    if (STAGED) clean = stage_weights<kMetroThreads>(lw, P, wsm, red, ctl);  // every CTA: the whole vector
+    const StagedWeights sw = {wsm, nullptr, 0xffffffffu};
+    if (STAGED) clean = stage_weights<kMetroThreads>(lw, P, sw, red, ctl);  // every CTA: the whole vector
     const int steps = B_dev ? (int)__ldg(B_dev) : B;
     const uint32_t Pu = (uint32_t)P;
     ChainStream<ROUNDS> rng;
     rng.set_key(key0, key1);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        if (STAGED) run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc);
+        if (STAGED) run_staged<ROUNDS, false>(lw, sw, clean, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc);
         else run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc, ctl);
     }
 }
@@ -366,6 +390,19 @@ cudaError_t launch_metropolis(const float* lw, int64_t P, int B, const uint32_t*
 constexpr int kMetroBThreads = 1024;
 constexpr int kMetroBStage = 56 * 1024;  // floats staged per CTA (224 KiB)
 constexpr uint32_t kBatchedBCap = 1u << 24;  // largest step count chosen for B < 0
+// A filter of up to twice the staging holds the rest of its weights in the CTA's
+// scratch: its steps then cost L2 only for the proposals that fall there.  Without, the
+// CTA's 32 random L2 reads a warp step bound it: 65 cycles a warp step at 65536
+// particles against 13 staged and 18 split; beyond, half or more of the reads go
+// to L2 either way.
+constexpr int64_t kMetroBSplit = 2 * (int64_t)kMetroBStage;
+static_assert(kMetroBSplit - kMetroBStage <= kMetroScratchFloats, "the CTA's scratch holds the rest");
+
+// How a filter's weights are reached.
+enum WeightsAt { kAllStaged, kSplit, kUnstaged };
+__device__ __forceinline__ WeightsAt weights_at(int64_t Pf) {
+    return Pf <= kMetroBStage ? kAllStaged : (Pf <= kMetroBSplit ? kSplit : kUnstaged);
+}
 
 // Chain blocks of a filter shared by several CTAs: a filter whose chains
 // number more than one block and whose work P_f B_f reaches kHeavyWork steps
@@ -390,10 +427,22 @@ __device__ __forceinline__ uint32_t claim_block(unsigned long long* w, uint32_t 
     }
 }
 
+// Chain i of a batched filter.
+template <int ROUNDS>
+__device__ __forceinline__ void run_batched_chain(const BatchParams& bp, const float* lw, const StagedWeights& sw,
+                                                  WeightsAt where, bool clean, uint32_t Pu, int64_t off0, uint32_t i,
+                                                  int steps, int f, uint32_t key0, uint32_t key1,
+                                                  ChainStream<ROUNDS>& rng) {
+    int32_t* anc = bp.anc + off0;
+    if (where == kAllStaged) run_staged<ROUNDS, false>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
+    else if (where == kSplit) run_staged<ROUNDS, true>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
+    else run_unstaged<ROUNDS>(lw, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc, bp.ctl);
+}
+
 // The chains of blocks claimed from filter f (block-wide; the weights are staged).
 template <int ROUNDS>
-__device__ __forceinline__ void run_claimed_blocks(const BatchParams& bp, const float* lw, const float* wsm, bool staged,
-                                                   bool clean, int64_t Pf, int64_t off0, int steps, int f,
+__device__ __forceinline__ void run_claimed_blocks(const BatchParams& bp, const float* lw,
+                                                   const StagedWeights& sw, WeightsAt where, bool clean, int64_t Pf, int64_t off0, int steps, int f,
                                                    uint32_t epoch, uint32_t key0, uint32_t key1,
                                                    ChainStream<ROUNDS>& rng, int* blk_sm) {
     const int tid = threadIdx.x;
@@ -406,12 +455,8 @@ __device__ __forceinline__ void run_claimed_blocks(const BatchParams& bp, const 
         __syncthreads();
         if (blk >= nblk) break;
         const int64_t i = blk * kMetroBThreads + tid;
-        if (i < Pf) {
-            if (staged)
-                run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0);
-            else
-                run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0, bp.ctl);
-        }
+        if (i < Pf)
+            run_batched_chain<ROUNDS>(bp, lw, sw, where, clean, Pu, off0, (uint32_t)i, steps, f, key0, key1, rng);
     }
 }
 
@@ -424,6 +469,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
     const int n_items = (int)ld_relaxed_u32(bp.ctl + CTL_ITEMS);
     const uint32_t epoch = ld_relaxed_u32(bp.ctl + CTL_METRO_EPOCH);
     ChainStream<ROUNDS> rng;
+    const StagedWeights sw = {wsm, bp.scratch + (int64_t)blockIdx.x * bp.scratch_per_cta, (uint32_t)kMetroBStage};
     for (;;) {
         if (tid == 0) f_sm = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
         __syncthreads();
@@ -438,7 +484,8 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             continue;
         }
         const float* lw = bp.lw + off0;
-        const bool staged = Pf <= kMetroBStage;
+        const WeightsAt where = weights_at(Pf);
+        const bool staged = where == kAllStaged;
         if (bp.trace) {
             trace_stamp(bp.trace, bp.trace_cap, ticket, 0);
             trace_put(bp.trace, bp.trace_cap, ticket, 5, blockIdx.x);
@@ -446,7 +493,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             trace_put(bp.trace, bp.trace_cap, ticket, 7, (uint64_t)(bp.items[ticket] & 31));
         }
         bool clean = false;
-        if (staged) clean = stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
+        if (where != kUnstaged) clean = stage_weights<kMetroBThreads>(lw, Pf, sw, red, bp.ctl);
         for (int w = 1; w <= 2; ++w) trace_stamp(bp.trace, bp.trace_cap, ticket, w);
         // B < 0: this filter's own step count from Eq. 5 and its largest normalised weight
         int steps = bp.B;
@@ -477,16 +524,10 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
                     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(list + h), "r"(f + 1) : "memory");
                 }
             }
-            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
+            run_claimed_blocks<ROUNDS>(bp, lw, sw, where, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
         } else {
-            for (int64_t i = tid; i < Pf; i += kMetroBThreads) {
-                if (staged)
-                    run_staged<ROUNDS>(lw, wsm, clean, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng,
-                                       bp.anc + off0);
-                else
-                    run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, (uint32_t)f, key0, key1, rng, bp.anc + off0,
-                                         bp.ctl);
-            }
+            for (int64_t i = tid; i < Pf; i += kMetroBThreads)
+                run_batched_chain<ROUNDS>(bp, lw, sw, where, clean, Pu, off0, (uint32_t)i, steps, f, key0, key1, rng);
         }
         __syncthreads();  // the staging buffer is reused by the next filter
         trace_stamp(bp.trace, bp.trace_cap, ticket, 4);
@@ -528,13 +569,13 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             const int64_t off0 = bp.offsets[f];
             const int64_t Pf = bp.offsets[f + 1] - off0;
             const float* lw = bp.lw + off0;
-            const bool staged = Pf <= kMetroBStage;
+            const WeightsAt where = weights_at(Pf);
             bool clean = false;
-            if (staged) clean = stage_weights<kMetroBThreads>(lw, Pf, wsm, red, bp.ctl);
+            if (where != kUnstaged) clean = stage_weights<kMetroBThreads>(lw, Pf, sw, red, bp.ctl);
             const uint64_t seed = bp.seeds[f];
             const uint32_t key0 = (uint32_t)(seed & 0xffffffffu), key1 = (uint32_t)(seed >> 32);
             rng.set_key(key0, key1);
-            run_claimed_blocks<ROUNDS>(bp, lw, wsm, staged, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
+            run_claimed_blocks<ROUNDS>(bp, lw, sw, where, clean, Pf, off0, steps, f, epoch, key0, key1, rng, &blk_sm);
             __syncthreads();  // the staging buffer is reused by the next listed filter
         }
     }
