@@ -117,8 +117,10 @@ enum {
  *   B         ignored
  *   seed      Philox key
  *   ancestors [P] int32, 4-byte aligned       (out)
- * One cooperative launch while P + ((logw mod 16) / 4) <= PF_MAX_CUMULATIVE:
- * every CTA scans its tiles, publishes one record for them, waits (bounded)
+ * One launch of a thread-block cluster up to 16 tiles (P = 32768 at the default
+ * minimum tile), else one cooperative launch while
+ * P + ((logw mod 16) / 4) <= PF_MAX_CUMULATIVE: every CTA scans its tiles,
+ * publishes one record for them, waits (bounded)
  * for all records, forms its carries and assigns its ancestors; larger P as
  * PF_MAX_CUMULATIVE describes.  Errors: PF_ERR_INVALID for null or misaligned
  * pointers or P out of range; device status PF_ERR_DOMAIN for NaN/+inf or all

@@ -22,6 +22,9 @@ cudaError_t prepare_metropolis();
 cudaError_t prepare_large();
 cudaError_t launch_large(int kind, SortedParams p, void* scratch, int num_sms, cudaStream_t s);
 size_t large_scratch_bytes(int kind, int64_t PA);
+cudaError_t prepare_small(int (&tiles)[3]);
+bool small_fits(int kind, const SortedParams& p, int tiles);
+cudaError_t launch_small(int kind, const SortedParams& p, cudaStream_t s);
 cudaError_t launch_gather(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
                           void* dst, uint32_t* ctl, int num_sms, cudaStream_t s);
 cudaError_t launch_reduce(const float* lw, int64_t P, void* rec, uint32_t* ctl, float* ess_out, double* log_sum_out,
@@ -47,6 +50,7 @@ struct DeviceInfo {
     int num_sms = 0;
     int persist_per_sm[3] = {0, 0, 0};
     int batched_per_sm[4] = {0, 0, 0, 0};
+    int small_tiles[3] = {0, 0, 0};  // tiles of a single filter served by one cluster (pf_small.cu)
 };
 
 struct Workspace {
@@ -101,6 +105,8 @@ pf_status device_info(int& dev, DeviceInfo*& info) {
     if (e != cudaSuccess) return cuda_fail(e, "prepare_metropolis");
     e = prepare_large();
     if (e != cudaSuccess) return cuda_fail(e, "prepare_large");
+    e = prepare_small(info->small_tiles);
+    if (e != cudaSuccess) return cuda_fail(e, "prepare_small");
     info->ready = true;
     return PF_OK;
 }
@@ -300,6 +306,28 @@ pf_status resample_cumulative(int kind, const float* logw, int64_t P, uint64_t s
         return PF_ERR_INVALID;  // P beyond kMaxTilesTotal full tiles
     }
     Workspace* w;
+    // few tiles: one cluster (the test hook's withheld record needs the single launch's bounded wait)
+    if (R == 1 && g_skip_tile < 0) {
+        SortedParams p;
+        std::memset(&p, 0, sizeof(p));
+        p.lw = logw - lead;
+        p.anc = anc;
+        p.lead = lead;
+        p.P = P;
+        p.Pd = (double)P;
+        p.tile = tile;
+        p.n_tiles = T;
+        p.key0 = (uint32_t)(seed & 0xffffffffu);
+        p.key1 = (uint32_t)(seed >> 32);
+        p.trace = g_trace;
+        p.trace_cap = g_trace_cap;
+        if (small_fits(kind, p, info->small_tiles[kind])) {
+            st = workspace(s, 0, w);
+            if (st) return st;
+            p.ctl = w->ctl;
+            return cuda_fail(launch_small(kind, p, s), "small launch");
+        }
+    }
     // multinomial: the tiles' cumulative weights (PA floats), then samples of
     // every 16th (c2) and 256th (c1) for the three-level draws, when the c1
     // samples fit in shared memory beside the tile table

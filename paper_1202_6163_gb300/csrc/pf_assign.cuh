@@ -574,15 +574,31 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
     }
 }
 
+// Where a warp's entries lie in the staging: at the same place whatever KK and S, as the
+// CTA's warps may be in different tiles, of different KK.
+template <int KIND, int CAP>
+__host__ __device__ constexpr int warp_stage_stride() {
+    return (KIND == KIND_STRAT || CAP >= kIoCapSmall ? CAP : 2 * CAP) / kWarps;
+}
+
+// Sets this warp's entries to -1 (once, before its first tile).
+template <int KIND, int CAP>
+__device__ __forceinline__ void warp_stage_init(int32_t* stage) {
+    constexpr int kStride = warp_stage_stride<KIND, CAP>();
+    int4* mine = reinterpret_cast<int4*>(stage + (threadIdx.x >> 5) * kStride);
+#pragma unroll
+    for (int i = threadIdx.x & 31; i < kStride / 4; i += 32) mine[i] = make_int4(-1, -1, -1, -1);
+    __syncwarp();
+}
+
 // One tile's assignment: warp by warp, or, for a tile that owns so many offsets
-// that one warp's share could be most of them, chunk by chunk over the CTA (whose
-// staging starts and leaves everything at -1).  Block-uniform choice.
+// that one warp's share could be most of them, chunk by chunk over the CTA (which sets
+// the staging before, and back to -1 after).  Block-uniform choice.  The warp's
+// entries are -1 on entry (warp_stage_init) and on return.
 template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK)>
 __device__ __forceinline__ void assign_tile(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
                                             TileThread& th, const TileSummary& ts, int64_t index0) {
-    // a warp's entries lie at the same place whatever KK and S: the CTA's warps may be in
-    // different tiles, of different KK
-    constexpr int kStride = (KIND == KIND_STRAT || CAP >= kIoCapSmall ? CAP : 2 * CAP) / kWarps;
+    constexpr int kStride = warp_stage_stride<KIND, CAP>();
     static_assert(32 * S <= kStride && kStride % 4 == 0, "a warp's entries fit its share of the staging");
     if (map.noff <= kWarpOffsets) {
         const int at = (threadIdx.x >> 5) * kStride;
@@ -605,15 +621,14 @@ __device__ __forceinline__ void assign_tile(const SortedParams& p, AssignShared&
 // target, then a lower-bound search in that tile's cumulative weights finds
 // the first element whose weight exceeds the tile-local target.  The four
 // in-tile searches advance in lockstep, so their loads overlap.
-//   table[T]  tile entries;  v  the filter's cumulative weights by tile
-//   (sign bit: zero weight; shared memory if SMEM_V, else global/L2);
-//   tile  tile length;  PA = P + lead.  Writes filter-local ancestors to a[].
-template <bool SMEM_V>
-__device__ __forceinline__ void multinomial_draws4(const u32x4& r, const TableEntry* table, int T,
-                                                   const float* v, int tile, int64_t PA, int lead, float Wh,
-                                                   float Wl, int32_t (&a)[4]) {
+//   table[T]  tile entries;  v(t, i)  reads element i of tile t's cumulative weights
+//   (sign bit: zero weight);  tile  tile length;  PA = P + lead.
+//   Writes filter-local ancestors to a[].
+template <class V>
+__device__ __forceinline__ void multinomial_draws4(const u32x4& r, const TableEntry* table, int T, V v, int tile,
+                                                   int64_t PA, int lead, float Wh, float Wl, int32_t (&a)[4]) {
     float xh[4], xl[4];
-    int lo[4], n[4], il[4];
+    int lo[4], n[4], il[4], at[4];
     int64_t b0[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -638,6 +653,7 @@ __device__ __forceinline__ void multinomial_draws4(const u32x4& r, const TableEn
         }
         xh[s] = h;
         xl[s] = l;
+        at[s] = tlo;
         b0[s] = (int64_t)tlo * tile;
         n[s] = (int)min((int64_t)tile, PA - b0[s]);
         lo[s] = 0;
@@ -649,8 +665,7 @@ __device__ __forceinline__ void multinomial_draws4(const u32x4& r, const TableEn
         float val[4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            const float* q = v + b0[s] + lo[s] + (n[s] >> 1);
-            val[s] = n[s] > 0 ? (SMEM_V ? *q : __ldcg(q)) : 0.f;
+            val[s] = n[s] > 0 ? v(at[s], lo[s] + (n[s] >> 1)) : 0.f;
         }
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
@@ -667,8 +682,7 @@ __device__ __forceinline__ void multinomial_draws4(const u32x4& r, const TableEn
     }
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-        const float* vt = v + b0[s];
-        auto ld = [&](int i) -> float { return SMEM_V ? vt[i] : __ldcg(vt + i); };
+        auto ld = [&](int i) -> float { return v(at[s], i); };
         int idx = il[s];
         if (lo[s] < nt[s]) {
             idx = lo[s];

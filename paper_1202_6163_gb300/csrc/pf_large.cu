@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
     const int tid = threadIdx.x;
     if (!sc->ok) return;  // launch 2 recorded a domain error
     const int n_mine = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // grid <= tiles
-    stage_init<kIoCap>(stage);
+    warp_stage_init<KIND, kIoCap>(stage);
     TileThread th;
     TileSummary ts;
     for (int r0 = 0; r0 < n_mine; r0 += kMapBatch) {
@@ -325,7 +325,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, con
                 settled = settled && ok;
             }
         }
-        if (!settled) multinomial_draws4<false>(r, table, p.n_tiles, p.v_out, kLargeTile, PA, p.lead, Wh, Wl, a);
+        if (!settled)
+            multinomial_draws4(r, table, p.n_tiles,
+                               [&](int t, int i) { return __ldcg(p.v_out + (int64_t)t * kLargeTile + i); }, kLargeTile, PA,
+                               p.lead, Wh, Wl, a);
         if (!mine) continue;
         const int64_t j = 4 * q;
         if (j + 3 < p.P && (((uintptr_t)(p.anc + j)) & 15u) == 0) {

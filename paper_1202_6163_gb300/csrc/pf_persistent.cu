@@ -341,7 +341,8 @@ __device__ void multinomial_draws(const SortedParams& p, PersistShared& sm, cons
                 }
             }
         } else {
-            multinomial_draws4<false>(r, table, T, p.v_out, p.tile, p.P + p.lead, p.lead, Wh, Wl, a);
+            multinomial_draws4(r, table, T, [&](int t, int i) { return __ldcg(p.v_out + (int64_t)t * p.tile + i); },
+                               p.tile, p.P + p.lead, p.lead, Wh, Wl, a);
         }
         const int64_t j = 4 * q;
         if (!mine) continue;
@@ -377,7 +378,7 @@ __device__ bool build_guide(const SortedParams& p, PersistShared& sm, int32_t* s
     pg.P = p.M;
     pg.Pd = (double)p.M;
     pg.guide = 1;
-    stage_init<kGuideCap>(stage);
+    warp_stage_init<KIND_SYS, kGuideCap>(stage);
     // the guide's offset map of every owned tile, two lanes per tile
     if (tid < 2 * ((t_count + 15) & ~15)) {
         const int r = min(tid >> 1, t_count - 1);
@@ -422,10 +423,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
     }
 
     static_assert(sizeof(PersistShared) % 16 == 0, "the staging buffers are 16-byte aligned");
-    // the staging buffers start pass 2 at -1 (below every decode tag); with tile
-    // copies in pass 1 they are set after it
+    // pass 2's staging: before pass 1, or after it where pass 1 copies tiles there
     if (KIND != KIND_MULTI && (KK != kMaxPerThread || t_count <= 1))
-        stage_init<stage_cap(KK)>(reinterpret_cast<int32_t*>(region));
+        warp_stage_init<KIND, stage_cap(KK)>(reinterpret_cast<int32_t*>(region));
 
     // pass 1: scan and record every owned tile.  Systematic / stratified with
     // several tiles per CTA: tile r + 1 is copied into one of the two staging
@@ -490,7 +490,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
         }
         __syncthreads();
     }
-    if (kCopies && copies) stage_init<stage_cap(KK)>(reinterpret_cast<int32_t*>(region));  // ordered by the arrival
+    if (kCopies && copies)  // the loop ended with a barrier
+        warp_stage_init<KIND, stage_cap(KK)>(reinterpret_cast<int32_t*>(region));
     int kc = 0;
     if (KIND != KIND_MULTI && warp == 0) kc = publish_cta_record(p, sm, t_count);
 

@@ -38,6 +38,7 @@ struct TileSummary {
     fpair S;      // tile sum relative to 2^k (compensated pair); thread 0 only
     int i_last;   // tile-local index of the last positive weight, -1 if none
     int bad;      // a NaN or +inf log-weight was seen
+    long long total;  // tile sum in fixed point (2^-48 relative to 2^k)
 };
 
 // This thread's share of the tile.
@@ -100,6 +101,12 @@ __device__ __forceinline__ void tile_load_k(const float* __restrict__ base, int 
         const float* src = SMEM ? base + stage_place(threadIdx.x, i >> 2) + (i & 3) : base + e0 + i;
         x[i] = (e0 + i >= lo && e0 + i < n) ? (SMEM ? *src : __ldg(src)) : -INFINITY;
     }
+}
+
+// A tile's sum as a pair, from its fixed-point total.
+__device__ __forceinline__ fpair tile_sum_pair(long long total) {
+    const float hi = (float)total;
+    return {hi * 0x1p-48f, (float)(total - (long long)hi) * 0x1p-48f};
 }
 
 // Block-wide; every thread of the CTA must call it.  Scans base[0..n) with the
@@ -216,10 +223,8 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
     TileSummary ts;
     ts.k = k;
     ts.S = {0.f, 0.f};
-    if (tid == 0) {  // the tile sum, a pair: thread 0 records it
-        const float S_hi = (float)total;
-        ts.S = {S_hi * 0x1p-48f, (float)(total - (long long)S_hi) * 0x1p-48f};
-    }
+    if (tid == 0) ts.S = tile_sum_pair(total);  // thread 0 records it
+    ts.total = total;
     ts.i_last = i_last;
     ts.bad = bad;
     return ts;
