@@ -409,6 +409,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __re
                                                                int32_t* __restrict__ items, uint32_t* ctl, int metro,
                                                                int split_min) {
     __shared__ int count[kMaxOwnB + 1], start[kMaxOwnB + 1], split_sm;
+    grid_begin();
     const int tid = threadIdx.x;
     if (tid <= kMaxOwnB) count[tid] = 0;
     if (metro) {
@@ -470,8 +471,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __re
 
 cudaError_t launch_batched_plan(const float* lw, const int64_t* offsets, int F, const int32_t* mask, int split,
                                 int32_t* items, uint32_t* ctl, cudaStream_t s, int metro, int split_min) {
-    k_batched_plan<<<1, kPlanThreads, 0, s>>>(lw, offsets, F, mask, split, items, ctl, metro, split_min);
-    return cudaGetLastError();
+    return launch_overlapped(k_batched_plan, 1, kPlanThreads, 0, s, lw, offsets, F, mask, split, items, ctl, metro,
+                             split_min);
 }
 
 template <int KIND>

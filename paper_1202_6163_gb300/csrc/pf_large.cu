@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_scan(SortedParams p, uint
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileShared& sm = *reinterpret_cast<TileShared*>(smem_raw);
     float* slot = reinterpret_cast<float*>(smem_raw + ((sizeof(TileShared) + 15) & ~(size_t)15));
+    grid_begin();
     const int tid = threadIdx.x;
     const int64_t PA = p.P + p.lead;
     const int n_mine = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // grid <= tiles
@@ -124,6 +125,7 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
     __shared__ i128 cta_sum;  // this CTA's mass
     __shared__ long long jnext[kThreads + 1];
     constexpr int kBadRange = INT_MAX;
+    grid_begin();
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int T = pm.n_tiles;
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LargeShared& sm = *reinterpret_cast<LargeShared*>(smem_raw);
     int32_t* stage = reinterpret_cast<int32_t*>(smem_raw + sizeof(LargeShared));
+    grid_begin();
     const int tid = threadIdx.x;
     if (!sc->ok) return;  // launch 2 recorded a domain error
     const int n_mine = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // grid <= tiles
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
 template <bool GUIDE>
 __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, const TableEntry* table,
                                                              const LargeScalars* sc, const int32_t* g, int64_t M) {
+    grid_begin();
     if (!sc->ok) return;
     const float Wh = sc->W_hi, Wl = sc->W_lo;
     const int64_t PA = p.P + p.lead;
@@ -380,8 +384,7 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
     LargeScalars* sc = reinterpret_cast<LargeScalars*>(scratch + l.scalars);
     p.v_out = reinterpret_cast<float*>(scratch + l.v);
     const int grid = T < 2 * num_sms ? T : 2 * num_sms;  // two resident CTAs per SM, grid-stride over tiles
-    k_large_scan<KIND><<<grid, kThreads, kScanSmem, s>>>(p, rec);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_overlapped(k_large_scan<KIND>, grid, kThreads, kScanSmem, s, p, rec);
     if (e != cudaSuccess) return e;
     SortedParams pm = p;  // of the offsets: the call's, or the guide's
     const int64_t M = guide_buckets(p.P);
@@ -392,21 +395,19 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
         pm.Pd = (double)M;
         pm.guide = 1;
     }
-    k_large_carries<KIND><<<kCarryCtas, kThreads, 0, s>>>(pm, rec, maps, table, sc);
-    e = cudaGetLastError();
+    e = launch_overlapped(k_large_carries<KIND>, kCarryCtas, kThreads, 0, s, pm, rec, maps, table, sc);
     if (e != cudaSuccess) return e;
     constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;
     constexpr int S = KIND == KIND_MULTI ? kGuideS : warp_stage_per_lane(16);
-    k_large_assign<kMapKind, S><<<grid, kThreads, kAssignSmem, s>>>(pm, PA, maps, sc);
+    e = launch_overlapped(k_large_assign<kMapKind, S>, grid, kThreads, kAssignSmem, s, pm, PA, maps, sc);
     if constexpr (KIND == KIND_MULTI) {
-        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t nq = (p.P + 3) >> 2;
         int64_t gd = (nq + kThreads - 1) / kThreads;
         if (gd > (int64_t)num_sms * 16) gd = (int64_t)num_sms * 16;
-        k_large_draws<true><<<(unsigned)gd, kThreads, 0, s>>>(p, table, sc, g, M);
+        e = launch_overlapped(k_large_draws<true>, (unsigned)gd, kThreads, 0, s, p, table, sc, g, M);
     }
-    return cudaGetLastError();
+    return e;
 }
 }  // namespace
 

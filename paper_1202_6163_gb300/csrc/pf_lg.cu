@@ -100,6 +100,7 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* ra, float*
 // (as a grid-stride loop over all particles, 37% of the warps resident); its 335 MB take 49 us.
 template <int GS>
 __global__ void __launch_bounds__(kLgThreads) k_lg_init(LgParams p) {
+    grid_begin();
     const int f = (int)(blockIdx.x / (unsigned)p.n_tiles);
     const int tile = (int)(blockIdx.x - (unsigned)f * (unsigned)p.n_tiles);
     const int G = GS > 0 ? GS : (p.D >> 2);
@@ -138,6 +139,7 @@ template <int GS>
 __global__ void __launch_bounds__(kLgThreads) k_lg_step(LgParams p) {
     __shared__ float ra[kLgWarps], rb[kLgWarps];
     __shared__ int last;
+    grid_begin();
     const int f = (int)(blockIdx.x / (unsigned)p.n_tiles);
     const int tile = (int)(blockIdx.x - (unsigned)f * (unsigned)p.n_tiles);
     const int tid = threadIdx.x;
@@ -268,23 +270,21 @@ int lg_tile() { return kLgThreads * kLgPerThread; }
 cudaError_t launch_lg_init(const LgParams& p, cudaStream_t s) {
     const unsigned blocks = (unsigned)((int64_t)p.F * p.n_tiles);
     switch (p.D) {
-    case 4: k_lg_init<1><<<blocks, kLgThreads, 0, s>>>(p); break;
-    case 8: k_lg_init<2><<<blocks, kLgThreads, 0, s>>>(p); break;
-    case 16: k_lg_init<4><<<blocks, kLgThreads, 0, s>>>(p); break;
-    default: k_lg_init<0><<<blocks, kLgThreads, 0, s>>>(p); break;
+    case 4: return launch_overlapped(k_lg_init<1>, blocks, kLgThreads, 0, s, p);
+    case 8: return launch_overlapped(k_lg_init<2>, blocks, kLgThreads, 0, s, p);
+    case 16: return launch_overlapped(k_lg_init<4>, blocks, kLgThreads, 0, s, p);
+    default: return launch_overlapped(k_lg_init<0>, blocks, kLgThreads, 0, s, p);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_lg_step(const LgParams& p, cudaStream_t s) {
     const unsigned blocks = (unsigned)((int64_t)p.F * p.n_tiles);
     switch (p.D) {
-    case 4: k_lg_step<1><<<blocks, kLgThreads, 0, s>>>(p); break;
-    case 8: k_lg_step<2><<<blocks, kLgThreads, 0, s>>>(p); break;
-    case 16: k_lg_step<4><<<blocks, kLgThreads, 0, s>>>(p); break;
-    default: k_lg_step<0><<<blocks, kLgThreads, 0, s>>>(p); break;
+    case 4: return launch_overlapped(k_lg_step<1>, blocks, kLgThreads, 0, s, p);
+    case 8: return launch_overlapped(k_lg_step<2>, blocks, kLgThreads, 0, s, p);
+    case 16: return launch_overlapped(k_lg_step<4>, blocks, kLgThreads, 0, s, p);
+    default: return launch_overlapped(k_lg_step<0>, blocks, kLgThreads, 0, s, p);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace pf

@@ -326,6 +326,7 @@ __global__ void __launch_bounds__(kMetroThreads) k_metropolis(const float* __res
                                                               int32_t* __restrict__ anc, uint32_t* ctl) {
     extern __shared__ float wsm[];
     __shared__ float red[kMetroThreads / 32];
+    grid_begin();
     bool clean = false;
     const StagedWeights sw = {wsm, nullptr, 0xffffffffu};
     if (STAGED) clean = stage_weights<kMetroThreads>(lw, P, sw, red, ctl);  // every CTA: the whole vector
@@ -362,15 +363,14 @@ static cudaError_t launch_metropolis_r(const float* lw, int64_t P, int B, const 
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_metropolis<true, ROUNDS>, kMetroThreads, smem);
         if (per_sm < 1) per_sm = 1;
         const int64_t grid = blocks_needed < (int64_t)num_sms * per_sm ? blocks_needed : (int64_t)num_sms * per_sm;
-        k_metropolis<true, ROUNDS><<<(unsigned)grid, kMetroThreads, smem, s>>>(lw, P, B, B_dev, key0, key1, filter,
-                                                                               anc, ctl);
+        return launch_overlapped(k_metropolis<true, ROUNDS>, (unsigned)grid, kMetroThreads, smem, s, lw, P, B, B_dev, key0,
+                                 key1, filter, anc, ctl);
     } else {
         const int64_t cap = (int64_t)num_sms * 64;
         const int64_t grid = blocks_needed < cap ? blocks_needed : cap;
-        k_metropolis<false, ROUNDS><<<(unsigned)grid, kMetroThreads, 0, s>>>(lw, P, B, B_dev, key0, key1, filter,
-                                                                             anc, ctl);
+        return launch_overlapped(k_metropolis<false, ROUNDS>, (unsigned)grid, kMetroThreads, 0, s, lw, P, B, B_dev, key0,
+                                 key1, filter, anc, ctl);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_metropolis(const float* lw, int64_t P, int B, const uint32_t* B_dev, uint32_t key0, uint32_t key1,

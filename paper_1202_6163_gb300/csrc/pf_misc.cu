@@ -25,6 +25,7 @@ template <typename VT, int U, bool POW2>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict__ src, int64_t P_src, RowSplit split,
                                                            const int32_t* __restrict__ anc, int64_t total,
                                                            VT* __restrict__ dst, uint32_t* ctl) {
+    grid_begin();
     const int64_t stride = (int64_t)gridDim.x * (kGatherThreads * U);
     for (int64_t base = (int64_t)blockIdx.x * (kGatherThreads * U) + threadIdx.x; base < total; base += stride) {
         VT v[U];
@@ -64,10 +65,10 @@ static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, 
     const RowSplit split = row_split(vecs, total);
     const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, kGatherWave, kGatherFullGrid);
     if (split.pow2)
-        k_gather<VT, U, true><<<blocks, kGatherThreads, 0, s>>>((const VT*)src, P_src, split, anc, total, (VT*)dst, ctl);
-    else
-        k_gather<VT, U, false><<<blocks, kGatherThreads, 0, s>>>((const VT*)src, P_src, split, anc, total, (VT*)dst, ctl);
-    return cudaGetLastError();
+        return launch_overlapped(k_gather<VT, U, true>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc,
+                                 total, (VT*)dst, ctl);
+    return launch_overlapped(k_gather<VT, U, false>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc, total,
+                             (VT*)dst, ctl);
 }
 
 cudaError_t launch_gather(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const float* __restrict_
     __shared__ int rk[kRedThreads / 32];
     __shared__ i128 rS[kRedThreads / 32], rQ[kRedThreads / 32];
     __shared__ int last;
+    grid_begin();
     const float eps_f = (float)eps;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t t0 = (int64_t)blockIdx.x * kRedTile;
@@ -364,9 +366,8 @@ size_t reduce_record_bytes() { return sizeof(RedRecord); }
 
 cudaError_t launch_reduce(const float* lw, int64_t P, void* rec, uint32_t* ctl, float* ess_out, double* log_sum_out,
                           uint32_t* B_out, double eps, uint32_t B_cap, cudaStream_t s) {
-    k_reduce<<<reduce_tiles(P), kRedThreads, 0, s>>>(lw, P, (RedRecord*)rec, ctl, ess_out, log_sum_out, B_out, eps,
-                                                     B_cap);
-    return cudaGetLastError();
+    return launch_overlapped(k_reduce, reduce_tiles(P), kRedThreads, 0, s, lw, P, (RedRecord*)rec, ctl, ess_out,
+                             log_sum_out, B_out, eps, B_cap);
 }
 
 }  // namespace pf

@@ -44,6 +44,7 @@ constexpr int kPermPart = 8192;  // extras one CTA lists: twice a tile's mean sh
 // first lane of each run of equal entries in a row adds the run's length.
 __global__ void __launch_bounds__(256) k_perm_count(const int32_t* __restrict__ anc, int64_t P,
                                                     int32_t* __restrict__ o, uint32_t* ctl) {
+    grid_begin();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 128; j0 < P; j0 += warps * 128) {
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* __re
                                                              TilePrefix* __restrict__ pre, int T, uint32_t* ctl) {
     __shared__ int red[kPermWarps];
     __shared__ int last;
+    grid_begin();
     int c[kPermPer];
     load_counts(o, (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer, P, c);
     int e = 0, d = 0;
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __res
                                                             int32_t* __restrict__ E) {
     __shared__ int red[kPermWarps];
     __shared__ __align__(16) int32_t mark[kPermPart + 4];
+    grid_begin();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int b = blockIdx.x; b < pre[T].part; b += gridDim.x) {
         int lo = 0, hi = T - 1;  // the last tile with pre.part <= b
@@ -240,6 +243,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __res
                                                             const TilePrefix* __restrict__ pre,
                                                             const int32_t* __restrict__ E, int32_t* __restrict__ out) {
     __shared__ int red[kPermWarps];
+    grid_begin();
     const int64_t i0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
     int c[kPermPer];
     load_counts(o, i0, P, c);
@@ -269,6 +273,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __res
 template <typename VT, int U, bool POW2>
 __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSplit split,
                                                         const int32_t* __restrict__ perm, uint32_t* ctl) {
+    grid_begin();
     const int64_t total = P * split.vecs;
     const int64_t stride = (int64_t)gridDim.x * (256 * U);
     for (int64_t base = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; base < total; base += stride) {
@@ -324,13 +329,14 @@ cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* sc
     if (e != cudaSuccess) return e;
     int64_t blocks = (P + 1023) / 1024;  // 8 warps of 128 entries
     if (blocks > (int64_t)num_sms * 8) blocks = (int64_t)num_sms * 8;
-    k_perm_count<<<(unsigned)blocks, 256, 0, s>>>(anc, P, o, ctl);
-    k_perm_tiles<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, pre, T, ctl);
+    e = launch_overlapped(k_perm_count, (unsigned)blocks, 256, 0, s, anc, P, o, ctl);
+    if (e == cudaSuccess) e = launch_overlapped(k_perm_tiles, (unsigned)T, kPermThreads, 0, s, o, P, pre, T, ctl);
     // at most T + P / kPermPart parts; a resident wave takes them in turn
     const int64_t parts = T + P / kPermPart, wave = (int64_t)num_sms * 4;
-    k_perm_list<<<(unsigned)(parts < wave ? parts : wave), kPermThreads, 0, s>>>(o, P, pre, T, E);
-    k_perm_fill<<<(unsigned)T, kPermThreads, 0, s>>>(o, P, pre, E, out);
-    return cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_overlapped(k_perm_list, (unsigned)(parts < wave ? parts : wave), kPermThreads, 0, s, o, P, pre, T, E);
+    if (e == cudaSuccess) e = launch_overlapped(k_perm_fill, (unsigned)T, kPermThreads, 0, s, o, P, pre, E, out);
+    return e;
 }
 
 cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const int32_t* perm, uint32_t* ctl,
@@ -341,15 +347,14 @@ cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const i
         const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
         const RowSplit split = row_split(vecs, P * vecs);
         const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, 8, 40);
-        if (split.pow2) k_gather_inplace<VT, U, true><<<blocks, 256, 0, s>>>(p, P, split, perm, ctl);
-        else k_gather_inplace<VT, U, false><<<blocks, 256, 0, s>>>(p, P, split, perm, ctl);
+        return launch_overlapped(split.pow2 ? k_gather_inplace<VT, U, true> : k_gather_inplace<VT, U, false>, blocks, 256, 0, s,
+                                 p, P, split, perm, ctl);
     };
     const uintptr_t a = (uintptr_t)x | (uintptr_t)row_bytes;
-    if ((a & 31) == 0) go(static_cast<u32x8*>(x), std::integral_constant<int, 2>());
-    else if ((a & 15) == 0) go(static_cast<uint4*>(x), std::integral_constant<int, 4>());
-    else if ((a & 7) == 0) go(static_cast<uint2*>(x), std::integral_constant<int, 4>());
-    else go(static_cast<uint32_t*>(x), std::integral_constant<int, 4>());
-    return cudaGetLastError();
+    if ((a & 31) == 0) return go(static_cast<u32x8*>(x), std::integral_constant<int, 2>());
+    if ((a & 15) == 0) return go(static_cast<uint4*>(x), std::integral_constant<int, 4>());
+    if ((a & 7) == 0) return go(static_cast<uint2*>(x), std::integral_constant<int, 4>());
+    return go(static_cast<uint32_t*>(x), std::integral_constant<int, 4>());
 }
 
 }  // namespace pf

@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(kThreads) k_small(SortedParams p) {
     const int slot = weight_slot(p.tile);
     constexpr int CAP = small_stage_cap(KK);
     const int tid = threadIdx.x, lane = tid & 31, t = blockIdx.x, T = p.n_tiles;
+    grid_begin();
     uint64_t* const trace = t < T ? p.trace : nullptr;  // CTAs beyond the tiles write no record
     if (trace) {
         trace_stamp(trace, p.trace_cap, t, 0);
@@ -277,6 +278,11 @@ cudaError_t launch_kk(const SortedParams& p, cudaStream_t s) {
     cfg.dynamicSmemBytes = small_smem(KIND, KK);
     if (KIND == KIND_MULTI) cfg.dynamicSmemBytes += (size_t)p.n_tiles * weight_slot(p.tile) * sizeof(float);
     cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     if (p.n_tiles == 1) {
         cfg.gridDim = dim3(1);
         return cudaLaunchKernelEx(&cfg, k_small<KIND, KK, true>, p);
@@ -284,13 +290,11 @@ cudaError_t launch_kk(const SortedParams& p, cudaStream_t s) {
     int c = 2;
     while (c < p.n_tiles) c *= 2;
     cfg.gridDim = dim3(c);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = c;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = c;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_small<KIND, KK, false>, p);
 }
 
