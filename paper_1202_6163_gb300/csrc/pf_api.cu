@@ -55,7 +55,7 @@ struct DeviceInfo {
 
 struct Workspace {
     uint32_t* ctl = nullptr;     // CTL_WORDS control words
-    uint64_t* slots = nullptr;   // one 16-byte record per tile of the single-launch kernels
+    uint64_t* slots = nullptr;   // one 16-byte record per tile of the single-launch kernels, then the tagged records
     void* scratch = nullptr;     // per-call scratch (multinomial cumulative weights, reduction records)
     size_t scratch_bytes = 0;
     uint32_t* counters = nullptr;  // per-filter arrival counters, zero between launches
@@ -130,12 +130,13 @@ pf_status workspace(cudaStream_t s, size_t scratch, Workspace*& out) {
         uint32_t* ctl = nullptr;
         uint64_t* slots = nullptr;
         if (cudaMalloc(&ctl, CTL_WORDS * sizeof(uint32_t)) != cudaSuccess) return PF_ERR_NOMEM;
-        if (cudaMalloc(&slots, 2 * kMaxRecords * sizeof(uint64_t)) != cudaSuccess) {
+        const size_t slot_bytes = (2 * (size_t)kMaxRecords + kTaggedWords * (size_t)kThreads) * sizeof(uint64_t);
+        if (cudaMalloc(&slots, slot_bytes) != cudaSuccess) {
             cudaFree(ctl);
             return PF_ERR_NOMEM;
         }
         e = cudaMemsetAsync(ctl, 0, CTL_WORDS * sizeof(uint32_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(slots, 0, 2 * kMaxRecords * sizeof(uint64_t), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(slots, 0, slot_bytes, s);
         if (e != cudaSuccess) {
             cudaFree(slots);
             cudaFree(ctl);
@@ -369,6 +370,7 @@ pf_status resample_cumulative(int kind, const float* logw, int64_t P, uint64_t s
     p.filter = 0;
     p.ctl = w->ctl;
     p.slots = w->slots;
+    p.tagged = w->slots + 2 * (size_t)kMaxRecords;
     p.wait_ns = g_wait_ns;
     p.skip_tile = (int)g_skip_tile;
     g_skip_tile = -1;

@@ -51,14 +51,17 @@ __device__ __forceinline__ float pair_minus_int(fpair a, long long j) {
     return __fadd_rn(__fadd_rn((float)((long long)fh - j), __fsub_rn(a.hi, fh)), a.lo);
 }
 
+// The uniform of the systematic scheme; the multinomial guide places its offsets at (j / P) W: none.
+__device__ __forceinline__ float offset_uniform(const SortedParams& p) {
+    return p.guide ? 0.f : u23f(philox(0u, 0u, p.filter, TAG_SYS, p.key0, p.key1).x);
+}
+
 template <int KIND>
 __device__ __forceinline__ long long offsets_below(const SortedParams& p, const AssignShared& sm, fpair PW, i128 B_i,
-                                                   float& x0) {
+                                                   float u, float& x0) {
     const fpair y = pair_mul(fixed_to_pair(B_i), PW);  // B P / W
     long long j;
     if (KIND == KIND_SYS) {
-        // the multinomial guide places its offsets at (j / P) W: no uniform shift
-        const float u = p.guide ? 0.f : u23f(philox(0u, 0u, p.filter, TAG_SYS, p.key0, p.key1).x);
         const fpair d = pair_sub_f(y, u);
         j = B_i <= 0 ? 0 : (B_i >= sm.Wt ? p.P : max(0LL, min((long long)p.P, pair_ceil(d))));
         x0 = pair_minus_int(d, j);  // N(v) = ceil(v * inv_rho + x0)
@@ -94,20 +97,27 @@ struct TileMap {
 // warp together: the even lane forms the lower end, the odd lane the upper;
 // `mask` names the participating lanes (both lanes of every pair).  Both lanes
 // return the map.
+// u: offset_uniform (systematic).
 template <int KIND>
 __device__ __forceinline__ TileMap tile_map_pair(const SortedParams& p, const AssignShared& sm, i128 Bl_i, i128 Bh_i,
-                                                 int k_tile, unsigned mask) {
+                                                 int k_tile, unsigned mask, float u) {
     const int lane = threadIdx.x & 31;
     const bool upper = lane & 1;
     const fpair W = {sm.W_hi, sm.W_lo};
     const fpair Pp = fast_two_sum((float)p.P, (float)(p.P - (int64_t)(float)p.P));  // P exactly
     const fpair PW = pair_div(Pp, W);
     float x0;
-    const long long j = offsets_below<KIND>(p, sm, PW, upper ? Bh_i : Bl_i, x0);
+    const long long j = offsets_below<KIND>(p, sm, PW, upper ? Bh_i : Bl_i, u, x0);
     const long long jl = __shfl_sync(mask, j, lane & ~1);
     const long long jh = __shfl_sync(mask, j, lane | 1);
     const float x0l = __shfl_sync(mask, x0, lane & ~1);
     return {jl, (int)max(0LL, jh - jl), x0l, PW.hi * pow2f(k_tile - sm.K)};
+}
+
+template <int KIND>
+__device__ __forceinline__ TileMap tile_map_pair(const SortedParams& p, const AssignShared& sm, i128 Bl_i, i128 Bh_i,
+                                                 int k_tile, unsigned mask) {
+    return tile_map_pair<KIND>(p, sm, Bl_i, Bh_i, k_tile, mask, KIND == KIND_SYS ? offset_uniform(p) : 0.f);
 }
 
 // The same for one tile into sm (lanes 0 and 1 of warp 0 together).

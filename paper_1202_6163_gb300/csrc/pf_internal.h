@@ -40,6 +40,7 @@ enum : int {
 constexpr int kThreads = 512;     // threads per CTA of the tile kernels
 constexpr int kMaxPerThread = 16; // elements per thread (multiple of 4)
 constexpr int kTileMax = kThreads * kMaxPerThread;
+constexpr int kTaggedWords = 4;   // 64-bit words of an epoch-tagged record
 constexpr int kMaxTilesTotal = 4096;  // tiles of one single-launch call (P <= 2^25)
 
 // Per-tile record of the multi-pass scan (decoupled lookback).
@@ -62,7 +63,8 @@ struct SortedParams {
     int tiles_per_cta;  // consecutive tiles owned by each CTA (R >= 1; 0 means 1)
     uint32_t key0, key1, filter;
     uint32_t* ctl;
-    uint64_t* slots;  // one 16-byte record per tile
+    uint64_t* slots;   // one 16-byte record per tile
+    uint64_t* tagged;  // kTaggedWords per CTA: epoch-tagged records of the one-tile-per-CTA launches, which alone write them
     uint64_t wait_ns;
     int skip_tile;
     float* v_out;     // tile-local cumulative weights (P + lead floats): multinomial, and the tiles

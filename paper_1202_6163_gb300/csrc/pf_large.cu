@@ -202,6 +202,7 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
     const fpair Pp = fast_two_sum((float)pm.P, (float)(pm.P - (int64_t)(float)pm.P));  // P exactly
     const fpair PW = pair_div(Pp, W);
     constexpr int kMapKind = KIND == KIND_MULTI ? KIND_SYS : KIND;
+    const float u = kMapKind == KIND_SYS ? offset_uniform(pm) : 0.f;
     for (int t0 = t_lo; t0 < t_hi; t0 += kThreads) {
         const int t = t0 + tid;
         const uint4 r = t < t_hi ? __ldg(rec + t) : make_uint4(0u, 0u, 0u, 0xffffffffu);
@@ -215,9 +216,9 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
         base += round;
         // this tile's lower end; its upper one is the next tile's lower
         float x0 = 0.f, x0_end;
-        const long long jlo = offsets_below<kMapKind>(pm, as, PW, B, x0);
+        const long long jlo = offsets_below<kMapKind>(pm, as, PW, B, u, x0);
         jnext[tid] = jlo;
-        if (tid == kThreads - 1) jnext[kThreads] = offsets_below<kMapKind>(pm, as, PW, B + mine, x0_end);
+        if (tid == kThreads - 1) jnext[kThreads] = offsets_below<kMapKind>(pm, as, PW, B + mine, u, x0_end);
         __syncthreads();
         if (t < t_hi) {
             LargeMap m;

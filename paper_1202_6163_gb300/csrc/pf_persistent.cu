@@ -559,6 +559,171 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// Systematic / stratified with one tile per CTA (P up to one tile per resident CTA,
+// 2.49 M on this part): the same cooperative launch with a shorter chain between
+// the scan and the decode.  A CTA's record carries the launch's epoch in every
+// 64-bit word, so that with few CTAs a thread per CTA polls that CTA's record itself (no
+// counter, no second round trip for the data; with 304 CTAs 92000 polling threads
+// took 5.6 us where the counter takes 1.4); the masses are summed as 27-bit limbs (one
+// warp reduction instruction and one shared-memory atomic each) instead of 128-bit
+// shuffles.  Bound by latency.  Back to back in a graph, before and here: systematic P =
+// 65536 9.0 and 6.0 us, 2^18 9.2 and 7.3, 2^20 13.1 and 10.7, 2^21 17.6 and 13.9; stratified
+// 10.1 and 6.6, 10.3 and 8.0, 15.2 and 12.0, 21.4 and 15.0.
+// ---------------------------------------------------------------------------
+constexpr int kLimbBits = 27, kLimbs = 4;  // 108 bits: a mass is below 2^104 (2^14 with 90 fraction bits)
+
+struct OneTileShared {
+    TileShared tile;
+    AssignShared as;
+    unsigned long long below[kLimbs], all[kLimbs];  // limb sums
+    i128 mine;
+    TileMap map;
+    int red_k[kWarps];
+    int ok;
+};
+constexpr int kPollCtas = 40;  // CTAs up to which each polls all records (59: stratified 9.2 us, by the counter 7.7)
+constexpr size_t one_tile_header() { return (sizeof(OneTileShared) + 15) & ~(size_t)15; }
+constexpr size_t one_tile_smem(int KK) { return one_tile_header() + 2 * (size_t)stage_cap(KK) * sizeof(int32_t); }
+
+__device__ __forceinline__ i128 of_limbs(const unsigned long long (&limb)[kLimbs]) {
+    i128 v = 0;
+#pragma unroll
+    for (int i = kLimbs - 1; i >= 0; --i) v = (v << kLimbBits) + (i128)limb[i];
+    return v;
+}
+
+template <int KIND, int KK>
+__global__ void __launch_bounds__(kThreads, 2) k_one_tile(SortedParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OneTileShared& sm = *reinterpret_cast<OneTileShared*>(smem_raw);
+    int32_t* stage = reinterpret_cast<int32_t*>(smem_raw + ((sizeof(OneTileShared) + 15) & ~(size_t)15));
+    constexpr int CAP = stage_cap(KK);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x, t = blockIdx.x;
+    const uint64_t t_start = global_ns();
+    const uint32_t epoch = ld_relaxed_u32(p.ctl + CTL_EPOCH) + 1u;
+    if (p.trace) {
+        trace_put(p.trace, p.trace_cap, t, 0, t_start);
+        for (int w = 1; w <= 4; ++w) trace_put(p.trace, p.trace_cap, t, w, 0);
+        trace_put(p.trace, p.trace_cap, t, 5, t);
+        trace_put(p.trace, p.trace_cap, t, 6, 0);
+        trace_put(p.trace, p.trace_cap, t, 7, 1);
+    }
+    warp_stage_init<KIND, CAP>(stage);
+    if (tid < kLimbs) sm.below[tid] = sm.all[tid] = 0ull;  // ordered by the scan's barriers
+    const int64_t PA = p.P + p.lead, t0 = (int64_t)t * p.tile;
+    TileThread th;
+    const TileSummary ts =
+        tile_scan_k<KK>(p.lw + t0, t == 0 ? p.lead : 0, (int)min((int64_t)p.tile, PA - t0), sm.tile, th);
+    const uint64_t tag = (uint64_t)epoch << 32;
+    if (tid == 0 && t != p.skip_tile) {
+        uint64_t* rec = p.tagged + kTaggedWords * t;
+        st_relaxed_v2(rec, tag | (uint32_t)ts.k, tag | __float_as_uint(ts.bad ? NAN : ts.S.hi));
+        st_relaxed_v2(rec + 2, tag | __float_as_uint(ts.S.lo), tag);
+        if (G > kPollCtas) red_release_add_u32(p.ctl + CTL_ARRIVE0 + (epoch & 1u), 1u);
+    }
+    trace_stamp(p.trace, p.trace_cap, t, 1);
+    const float u = KIND == KIND_SYS ? offset_uniform(p) : 0.f;  // while the records travel
+
+    int k = 0, late = 0;
+    float hi = 0.f, lo = 0.f;
+    if (G > kPollCtas) {  // one thread waits for the counter
+        if (tid == 0) {
+            const uint32_t* arrive = p.ctl + CTL_ARRIVE0 + (epoch & 1u);
+            for (uint32_t it = 1; ld_acquire_u32(arrive) < (uint32_t)G; ++it)
+                if ((it & 7u) == 0u && global_ns() - t_start > p.wait_ns) {
+                    late = 1;
+                    break;
+                }
+            sm.ok = !late;
+        }
+        __syncthreads();
+        late = !sm.ok;
+    }
+    if (tid < G && !late) {  // thread c: CTA c's record
+        const uint64_t* rec = p.tagged + kTaggedWords * tid;
+        uint64_t a, b, c, d;
+        for (uint32_t it = 1;; ++it) {
+            ld_relaxed_v2(rec, a, b);
+            ld_relaxed_v2(rec + 2, c, d);
+            if ((a >> 32) == epoch && (b >> 32) == epoch && (c >> 32) == epoch) break;
+            if ((it & 7u) == 0u && global_ns() - t_start > p.wait_ns) {
+                late = 1;
+                break;
+            }
+        }
+        k = (int)(uint32_t)a;
+        hi = __uint_as_float((uint32_t)b);
+        lo = __uint_as_float((uint32_t)c);
+    }
+    const bool bad = !(hi <= 3.402823466e38f);
+    const int kw = __reduce_max_sync(0xffffffffu, bad ? INT_MAX : (hi > 0.f ? k : INT_MIN));
+    if (lane == 0) sm.red_k[warp] = kw;
+    late = __syncthreads_or(late);
+    trace_stamp(p.trace, p.trace_cap, t, 2);
+    // every CTA read the epoch before it published, and CTA 0 has seen all records (or
+    // waited out its limit): ready for the next launch, of whatever kind
+    if (t == 0 && tid == 0) {
+        atomicExch(p.ctl + CTL_ARRIVE0 + ((epoch + 1u) & 1u), 0u);
+        atomicExch(p.ctl + CTL_ARRIVE2 + ((epoch + 1u) & 1u), 0u);
+        atomicExch(p.ctl + CTL_EPOCH, epoch);
+    }
+    const int K = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.red_k[lane] : INT_MIN);
+    if (late || K == INT_MIN || K == INT_MAX) {  // a record that never came; all weights zero; NaN/+inf
+        if (tid == 0) set_status(p.ctl + CTL_STATUS, late ? ST_TIMEOUT : ST_DOMAIN);
+        return;
+    }
+    if (warp * 32 < G) {
+        const i128 v = hi > 0.f ? shr_i128(fixed_of(hi, 0) + fixed_of(lo, 0), K - k) : (i128)0;
+        if (tid == t) sm.mine = v;
+#pragma unroll
+        for (int i = 0; i < kLimbs; ++i) {
+            const uint32_t limb = (uint32_t)(v >> (kLimbBits * i)) & ((1u << kLimbBits) - 1u);
+            const uint32_t all = __reduce_add_sync(0xffffffffu, limb);
+            const uint32_t below = __reduce_add_sync(0xffffffffu, tid < t ? limb : 0u);
+            if (lane == 0) {
+                atomicAdd(&sm.all[i], (unsigned long long)all);
+                atomicAdd(&sm.below[i], (unsigned long long)below);
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        AssignShared as;
+        as.Wt = of_limbs(sm.all);
+        as.K = K;
+        const fpair W = fixed_to_pair(as.Wt);
+        as.W_hi = W.hi;
+        as.W_lo = W.lo;
+        const i128 B = of_limbs(sm.below);
+        const TileMap m = tile_map_pair<KIND>(p, as, B, B + sm.mine, ts.k, 0xffffffffu, u);
+        if (lane == 0) sm.map = m;
+    }
+    __syncthreads();
+    const TileMap map = sm.map;
+    trace_stamp(p.trace, p.trace_cap, t, 3);
+    assign_tile<KIND, KK, CAP>(p, sm.as, map, stage, th, ts, t0 - p.lead);
+    if (p.trace) {
+        __syncthreads();
+        trace_stamp(p.trace, p.trace_cap, t, 4);
+    }
+}
+
+template <int KIND, int KK>
+static cudaError_t launch_one_tile(const SortedParams& p, int grid, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = one_tile_smem(KK);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_one_tile<KIND, KK>, p);
+}
+
 template <int KIND, int KK, bool GUIDE = false>
 static cudaError_t set_smem_attr() {
     return cudaFuncSetAttribute(k_persistent<KIND, KK, GUIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -589,6 +754,13 @@ static cudaError_t launch_k(const SortedParams& p, int grid, cudaStream_t s) {
         if (q <= 8) return launch_kind<KIND, 8, true>(p, grid, s);
         return launch_kind<KIND, 16, true>(p, grid, s);
     }
+    if constexpr (KIND != KIND_MULTI) {
+        if (p.tiles_per_cta <= 1 && p.tagged != nullptr && grid == p.n_tiles && grid <= kThreads) {
+            if (q <= 4) return launch_one_tile<KIND, 4>(p, grid, s);
+            if (q <= 8) return launch_one_tile<KIND, 8>(p, grid, s);
+            return launch_one_tile<KIND, 16>(p, grid, s);
+        }
+    }
     if (q <= 4) return launch_kind<KIND, 4>(p, grid, s);
     if (q <= 8) return launch_kind<KIND, 8>(p, grid, s);
     return launch_kind<KIND, 16>(p, grid, s);
@@ -617,7 +789,7 @@ static int blocks_per_sm_kk() {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_persistent<KIND, KK>, kThreads,
                                                       persistent_smem_bytes(KIND, kMaxTilesTotal, KK)) != cudaSuccess)
         return 0;
-    if (KIND == KIND_MULTI) {  // the guide variant: the same launch shape, so the smaller of the two
+    if constexpr (KIND == KIND_MULTI) {  // the guide variant: the same launch shape, so the smaller of the two
         int ng = 0;
         if (set_smem_attr<KIND, KK, true>() != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ng, k_persistent<KIND, KK, true>, kThreads,
@@ -625,6 +797,14 @@ static int blocks_per_sm_kk() {
                 cudaSuccess)
             return 0;
         nb = min(nb, ng);
+    } else {  // the one-tile-per-CTA variant: as many CTAs too
+        int n1 = 0;
+        if (cudaFuncSetAttribute(k_one_tile<KIND, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)one_tile_smem(KK)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_one_tile<KIND, KK>, kThreads, one_tile_smem(KK)) !=
+                cudaSuccess)
+            return 0;
+        nb = min(nb, n1);
     }
     return nb;
 }
