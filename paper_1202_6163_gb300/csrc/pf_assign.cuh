@@ -601,6 +601,26 @@ __device__ __forceinline__ void warp_stage_init(int32_t* stage) {
     __syncwarp();
 }
 
+// W of a one-tile filter as a pair, as fixed_to_pair gives it for the tile sum's 128-bit
+// value: the top 24 bits and the next 24 of the pair's exact sum.
+__device__ __forceinline__ fpair total_pair(long long total) {
+    const float hi = (float)total;
+    const long long sum = (long long)hi + (long long)(float)(total - (long long)hi);
+    const int n = 64 - __clzll(sum), s = max(n - 24, 0);
+    const uint32_t top = (uint32_t)(sum >> s);
+    const long long rem = sum - ((long long)top << s);
+    const int s2 = max(s - 24, 0);
+    return {(float)top * pow2f(s - 48), (float)(uint32_t)(rem >> s2) * pow2f(s2 - 48)};
+}
+
+// The map of a tile that owns every offset (tile_map_pair with the boundaries 0 and W).
+template <int KIND>
+__device__ __forceinline__ TileMap only_tile_map(const SortedParams& p, fpair W) {
+    const fpair Pp = fast_two_sum((float)p.P, (float)(p.P - (int64_t)(float)p.P));
+    const float u = KIND == KIND_SYS ? u23f(philox(0u, 0u, p.filter, TAG_SYS, p.key0, p.key1).x) : 0.f;
+    return {0, (int)p.P, -u, pair_div(Pp, W).hi};
+}
+
 // One tile's assignment: warp by warp, or, for a tile that owns so many offsets
 // that one warp's share could be most of them, chunk by chunk over the CTA (which sets
 // the staging before, and back to -1 after).  Block-uniform choice.  The warp's

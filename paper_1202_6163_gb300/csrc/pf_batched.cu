@@ -4,11 +4,13 @@
 // A one-CTA plan pass turns the filters into a list of work items, largest
 // filters first (a counting sort by tile count), skipping masked and empty
 // filters.  A persistent grid then takes items from a ticket counter:
-//   - a filter of one tile (or any multinomial filter) is one item, done by
-//     one CTA with no wait on any other: scan and record each tile
-//     (pf_tile.cuh), warp 0 forms the tiles' exact fixed-point carries, then
-//     offsets are assigned (systematic, stratified) or the filter's uniforms
-//     drawn and searched (multinomial);
+//   - a systematic or stratified filter of one tile is one item, done by one
+//     CTA with no barrier but the scan's own: every thread has the tile's
+//     total and forms the offset map from it;
+//   - any multinomial filter is one item, done by one CTA with no wait on any
+//     other: scan and record each tile (pf_tile.cuh), warp 0 forms the tiles'
+//     exact fixed-point carries, then the filter's uniforms are drawn and
+//     searched;
 //   - a systematic or stratified filter of Tf > 1 tiles is Tf items with
 //     consecutive tickets, one tile each: every CTA scans its tile in
 //     registers, publishes a 16-byte record, waits (bounded) until all Tf
@@ -17,10 +19,16 @@
 //     tickets and a filter has at most kMaxOwnB < grid tiles, so every tile a
 //     CTA waits for has been or will be taken by a running CTA (the launch is
 //     cooperative, so all CTAs are resident);
-//   - unless such filters are at least as many as the resident CTAs: then the
-//     plan keeps each one whole, a single item whose CTA scans all its tiles
+//   - unless such filters load the resident CTAs well enough by themselves
+//     (k_batched_plan has the rule): then the plan keeps each one whole, a single item whose CTA scans all its tiles
 //     (cumulative weights to the CTA's scratch), forms the carries and every
 //     tile's offset map, and assigns the tiles, with no wait on another CTA.
+// What bounds it: the scan's and the decode's instructions and barriers at two
+// CTAs an SM (registers), about 45% of the issue slots.  4096 filters of 256 to
+// 65536 particles, systematic: 254 us with a one-tile filter's records and
+// carries through shared memory and its tile widths found at run time, 229 us
+// now; the next ticket drawn ahead of its item 232, without the prefetch of a
+// filter's next tile into L2 230.
 // A filter's data may start at any 4-byte boundary: tiles are laid out on the
 // aligned window, with the leading slots taken as zero weights.  The last CTA
 // to finish resets the ticket; the last CTA of a split filter resets its
@@ -127,6 +135,34 @@ __device__ __forceinline__ void filter_carries(BatchShared& sm, const BatchParam
     }
 }
 
+// A systematic or stratified filter of one tile: scan, map and assignment with no barrier
+// but the scan's own, every thread forming the map from the tile's total.
+template <int KIND, int KK>
+__device__ __forceinline__ void one_tile_filter(const BatchParams& bp, const SortedParams& p, BatchShared& sm, int lead,
+                                                int n, int32_t* stage, int ticket) {
+    TileThread th;
+    const TileSummary ts = tile_scan_k<KK>(p.lw, lead, n, sm.tile, th);
+    trace_stamp(bp.trace, bp.trace_cap, ticket, 1);
+    trace_stamp(bp.trace, bp.trace_cap, ticket, 2);
+    if (ts.bad || ts.total <= 0) {
+        if (threadIdx.x == 0) set_status(bp.ctl + CTL_STATUS, ST_DOMAIN);
+        return;
+    }
+    const TileMap map = only_tile_map<KIND>(p, total_pair(ts.total));
+    trace_stamp(bp.trace, bp.trace_cap, ticket, 3);
+    assign_tile<KIND, KK, kIoCap>(p, sm.as, map, stage, th, ts, -lead);
+    if (bp.trace) {
+        __syncthreads();
+        trace_stamp(bp.trace, bp.trace_cap, ticket, 4);
+    }
+}
+
+// Asks L2 for a tile that is scanned soon (its whole 128-byte lines).
+__device__ __forceinline__ void prefetch_tile(const float* src, int n) {
+    const int at = threadIdx.x * 32;
+    if (at < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + at));
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -136,11 +172,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
     const int n_items = (int)ld_relaxed_u32(bp.ctl + CTL_ITEMS);
     TileThread th;
     if (KIND != KIND_MULTI) warp_stage_init<KIND, kIoCap>(reinterpret_cast<int32_t*>(region));
+    if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
     for (;;) {
-        if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
-        __syncthreads();
+        __syncthreads();  // the ticket, and the last item's shared memory is free
         const int ticket = sm.f;
-        __syncthreads();
         if (ticket >= n_items) break;
         const int item = bp.items[ticket];
         const int f = item >> 5, c_item = item & 31;
@@ -160,7 +195,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             trace_put(bp.trace, bp.trace_cap, ticket, 7, (uint64_t)c_item);
         }
 
-        if (KIND != KIND_MULTI && c_item == kWhole && Tf > 1) {
+        if (KIND != KIND_MULTI && c_item == kWhole && Tf == 1) {
+            const int n = (int)PA, K = per_thread_count(n);
+            if (K == 16)
+                one_tile_filter<KIND, 16>(bp, p, sm, lead, n, stage, ticket);
+            else if (K == 8)
+                one_tile_filter<KIND, 8>(bp, p, sm, lead, n, stage, ticket);
+            else
+                one_tile_filter<KIND, 4>(bp, p, sm, lead, n, stage, ticket);
+            __syncthreads();
+            if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
+            continue;
+        }
+        if (KIND != KIND_MULTI && c_item == kWhole) {
             // ---- systematic / stratified: a whole filter of several tiles in this CTA (the plan
             // gives whole filters when there are enough of them to occupy the grid): every tile is
             // scanned (the cumulative weights of all but the last kept in this CTA's scratch), warp 0
@@ -172,6 +219,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             for (int c = 0; c < Tf; ++c) {
                 const int64_t t0 = (int64_t)c * kTileMax;
                 const int n = (int)min((int64_t)kTileMax, PA - t0);
+                if (c + 1 < Tf) prefetch_tile(p.lw + t0 + kTileMax, (int)min((int64_t)kTileMax, PA - t0 - kTileMax));
                 ts = tile_scan(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
                 bad |= ts.bad;
                 if (tid == 0) {
@@ -180,7 +228,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                     sm.rsl[c] = ts.S.lo;
                     sm.ril[c] = ts.i_last;
                 }
-                if (c + 1 < Tf) write_tile_v(p, th, t0, n);  // reloaded for its assignment
+                if (c + 1 < Tf) write_tile_v<16>(p, th, t0, kTileMax);  // reloaded for its assignment
                 __syncthreads();
             }
             trace_stamp(bp.trace, bp.trace_cap, ticket, 1);
@@ -201,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 __syncthreads();
                 for (int c = Tf - 1; c >= 0; --c) {
                     const int64_t t0 = (int64_t)c * kTileMax;
-                    if (c != Tf - 1) read_tile_v(p.v_out + t0, (int)min((int64_t)kTileMax, PA - t0), th);
+                    if (c != Tf - 1) read_tile_v<16>(p.v_out + t0, kTileMax, th);
                     ts.i_last = sm.ril[c];
                     const TileMap map = sm.maps[c];
                     if (th.K == 16)
@@ -217,6 +265,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 }
             }
             __syncthreads();
+            if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
             continue;
         }
         if (KIND != KIND_MULTI) {
@@ -292,6 +341,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 atomicExch(bp.counters + 2 * f + 1, 0u);
             }
             __syncthreads();
+            if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
             continue;
         }
 
@@ -328,10 +378,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                                  in ? sm.rsl[lane] : 0.f, in ? sm.ril[lane] : -1, bad, true);
         }
         __syncthreads();
-        if (sm.skip) continue;
-        trace_stamp(bp.trace, bp.trace_cap, ticket, 3);
+        const bool go = !sm.skip;
+        if (go) trace_stamp(bp.trace, bp.trace_cap, ticket, 3);
 
-        if (KIND == KIND_MULTI) {
+        if (KIND == KIND_MULTI && go) {
             const int64_t nq = (Pf + 3) >> 2;  // four draws per Philox block
             // the same number of passes in every thread (the windowed draws read
             // quad-cooperatively); a lane past the end redraws block 0
@@ -357,8 +407,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             }
             __syncthreads();
             trace_stamp(bp.trace, bp.trace_cap, ticket, 4);
-            continue;
         }
+        if (tid == 0) sm.f = (int)atomicAdd(bp.ctl + CTL_QUEUE, 1u);
     }
     // every CTA has drawn a ticket past the end: the last one to leave resets the queue
     if (tid == 0) {
@@ -442,10 +492,19 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __re
     }
     __syncthreads();
     if (tid == 0) {
-        // several-tile filters are split over CTAs only while they are too few to occupy the grid
-        int multi = 0;
-        for (int T = 2; T <= kMaxOwnB; ++T) multi += count[T];
-        const int sp = split && multi < split_min;
+        // Split tiles pay for their records' round trip (10-12 us a tile and CTA against
+        // 8.6-9.8 of a whole filter's), whole filters for the largest one's serial tiles.  The
+        // line where the two meet: the tiles as many as 3/4 of what the resident CTAs do while
+        // one does the largest filter's.  Systematic, split / whole, us, 304 CTAs: 65536
+        // particles 204 filters 70 / 78, 228: 78 / 78, 256: 87 / 79, 290: 98 / 81; 131072
+        // particles 200: 134 / 139, 228: 149 / 139; 20000 particles 152: 29 / 33, 228: 37 / 34;
+        // 256 to 131072 particles, 800 filters 111 / 134, 1500: 186 / 140.
+        int tiles_multi = 0, largest = 0;
+        for (int T = 2; T <= kMaxOwnB; ++T) {
+            tiles_multi += count[T] * T;
+            if (count[T]) largest = T;
+        }
+        const int sp = split && 4 * tiles_multi < 3 * split_min * largest;
         split_sm = sp;
         int run = 0;
         for (int T = kMaxOwnB; T >= 1; --T) {

@@ -52,18 +52,6 @@ __host__ __device__ constexpr int weight_slot(int tile) { return (tile + 31) & ~
 // otherwise all fall in one bank (P = 2048: 8.2 us, 2000: 5.9).
 __device__ __forceinline__ int weight_place(int i) { return i ^ ((i >> 3) & 0x1c); }
 
-// W of a one-tile filter as a pair, as fixed_to_pair gives it for the tile sum's 128-bit
-// value: the top 24 bits and the next 24 of the pair's exact sum.
-__device__ __forceinline__ fpair total_pair(long long total) {
-    const float hi = (float)total;
-    const long long sum = (long long)hi + (long long)(float)(total - (long long)hi);
-    const int n = 64 - __clzll(sum), s = max(n - 24, 0);
-    const uint32_t top = (uint32_t)(sum >> s);
-    const long long rem = sum - ((long long)top << s);
-    const int s2 = max(s - 24, 0);
-    return {(float)top * pow2f(s - 48), (float)(uint32_t)(rem >> s2) * pow2f(s2 - 48)};
-}
-
 // Two multinomial draws, their searches in lockstep and without branches: the last tile
 // whose boundary is at or below the target, then the number of the tile's elements at or
 // below it.
@@ -165,10 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_small(SortedParams p) {
         ok = !ts.bad && ts.total > 0;
         W = total_pair(ts.total);
         if (KIND != KIND_MULTI) {
-            // the map of a tile that owns every offset (tile_map_pair with boundaries 0 and W)
-            const fpair Pp = fast_two_sum((float)p.P, (float)(p.P - (int64_t)(float)p.P));
-            const float u = KIND == KIND_SYS ? u23f(philox(0u, 0u, p.filter, TAG_SYS, p.key0, p.key1).x) : 0.f;
-            map = {0, (int)p.P, -u, pair_div(Pp, W).hi};
+            map = only_tile_map<KIND>(p, W);
         } else {
             if (tid == 0) sm.table[0] = {0.f, 0.f, 1.f, ts.i_last};
             __syncthreads();
