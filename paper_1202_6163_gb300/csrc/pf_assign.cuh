@@ -30,7 +30,7 @@ struct AssignShared {
     int noff;      // offsets of the tile being assigned
     long long jlo; // first offset of that tile
     float tau0, inv_rho, W_hi, W_lo;
-    int red_n[kWarps];
+    int red_n[kWarps], red_next[kWarps];
 };
 
 // ---------------------------------------------------------------------------
@@ -149,6 +149,51 @@ __device__ __forceinline__ void stage_init(int32_t* stage) {  // stage: 16-byte 
         reinterpret_cast<int4*>(stage)[i] = make_int4(-1, -1, -1, -1);
 }
 
+// The run that covers offset c0 and where the next one begins, over this thread's elements
+// (counts N in v, starting from start0): cur the last element whose run covers c0 (-1:
+// none), next the first start beyond c0 (INT_MAX: none).
+template <int KK>  // 0: th.K elements
+__device__ __forceinline__ void run_at(const TileThread& th, int start0, int c0, int& cur, int& next) {
+    cur = -1;
+    next = INT_MAX;
+    int a = start0;
+#pragma unroll
+    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
+        if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+            const int b = __float_as_int(th.v[i]);
+            if (b > a) {
+                if (a > c0) next = min(next, a);
+                else if (b > c0) cur = i;
+            }
+            a = b;
+        }
+    }
+}
+
+// The longest run of this thread's elements (as run_at).
+template <int KK>
+__device__ __forceinline__ int longest_run(const TileThread& th, int start0) {
+    int a = start0, longest = 0;
+#pragma unroll
+    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
+        if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+            const int b = __float_as_int(th.v[i]);
+            longest = max(longest, b - a);
+            a = b;
+        }
+    }
+    return longest;
+}
+
+// dst[0, n) = v by `threads` threads, this one the t-th; 16-byte stores between the ends.
+__device__ __forceinline__ void fill_run(int32_t* dst, int n, int32_t v, int t, int threads) {
+    const int head = min((int)((4u - (uint32_t)((uintptr_t)dst >> 2)) & 3u), n), body = (n - head) & ~3;
+    if (t < head) dst[t] = v;
+    for (int x = head + 4 * t; x < head + body; x += 4 * threads)
+        *reinterpret_cast<int4*>(dst + x) = make_int4(v, v, v, v);
+    if (t < n - head - body) dst[head + body + t] = v;
+}
+
 // One chunk [c0, c1) of the tile's offsets: each positive element marks the
 // first slot of its run [N_{i-1}, N_i) with its tagged tile-local index (runs
 // of later elements start later, so tags increase along the chunk), the
@@ -234,7 +279,8 @@ __device__ __forceinline__ void decode_chunk(const SortedParams& p, AssignShared
 
 // stage: the two staging buffers (2 * CAP entries, stage_init<CAP>'ed once per
 // launch); epoch: the chunk counter of the launch, identical in every thread.
-template <int KIND, int KK = 0, int CAP = kIoCap>  // KK: elements per thread when fixed, 0 = th.K
+template <int KIND, int KK = 0, int CAP = kIoCap, bool LONG = true>  // KK: elements per thread when fixed, 0 = th.K;
+                                                                     // LONG: look for long runs
 __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
                                  uint32_t& epoch, TileThread& th, const TileSummary& ts, int64_t index0) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -333,13 +379,36 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
     __syncthreads();
     prev = max(prev, __reduce_max_sync(0xffffffffu, lane < warp ? sm.red_n[lane] : -1));
     const int start0 = max(prev, 0);
+    constexpr int kLongRun = 2 * CAP;
+    const bool long_runs = LONG && noff >= kLongRun && __syncthreads_or(longest_run<KK>(th, start0) >= kLongRun);
     const int32_t tile_base = (int32_t)index0;  // particle index of the tile's element 0
 
     // Run-length decode, one staging chunk at a time (decode_chunk); chunks
     // of at most 2044 / 4092 / 8188 offsets use 4 / 8 / 16 staging entries per
     // thread, larger ones 20.
     constexpr int kChunk = CAP - 4;  // offsets per chunk (room for the shift)
-    for (int c0 = 0; c0 < noff; c0 += kChunk) {
+    for (int c0 = 0; c0 < noff;) {
+        if (long_runs && noff - c0 >= kLongRun) {  // block-uniform
+            // a run that goes on for two chunks or more is stored as it is
+            int cur, next;
+            run_at<KK>(th, start0, c0, cur, next);
+            cur = __reduce_max_sync(0xffffffffu, cur < 0 ? -1 : th.e0 + cur);
+            next = __reduce_min_sync(0xffffffffu, next);
+            __syncthreads();  // the last reads of red_n
+            if (lane == 0) {
+                sm.red_n[warp] = cur;
+                sm.red_next[warp] = next;
+            }
+            __syncthreads();
+            cur = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.red_n[lane] : -1);
+            next = min(__reduce_min_sync(0xffffffffu, lane < kWarps ? sm.red_next[lane] : INT_MAX), noff);
+            __syncthreads();  // red_n is written again
+            if (cur >= 0 && next - c0 >= kLongRun) {
+                fill_run(p.anc + jlo + c0, next - c0, tile_base + cur, tid, kThreads);
+                c0 = next;
+                continue;
+            }
+        }
         if (++epoch > kEpochMax) {  // tags exhausted (uniform): clear both buffers and restart
             __syncthreads();
             stage_init<CAP>(stage);
@@ -375,6 +444,7 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
         else
             decode_chunk<(CAP > 16 * kThreads ? CAP : 16 * kThreads + 4) / kThreads, KK>(
                 p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
+        c0 = c1;
     }
 }
 
@@ -398,22 +468,36 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
 // (floor(y)) in its low bits, exact for |y| < 2^22; it replaces the conversion,
 // which issues at a quarter of the rate.  y is monotone along the thread, so only
 // a thread whose first or last count falls outside the tile's range clamps.
+//
+// Skewed weights: a warp whose offsets are several chunks looks for a run that goes on
+// for two chunks or more and stores it as it is, and a warp with more strata than its
+// buffer holds draws them one buffer at a time, passing over those inside a run.  With
+// every chunk decoded and each thread drawing its own strata, systematic, exp(4 N(0,1))
+// weights: 2^20 particles 66 us, now 27; 3 M 127, now 52; 2^24 394, now 150; stratified
+// 2^20 41, now 25; 4096 filters, exp(2 N), which look for no runs: 387, now 339.
 // ---------------------------------------------------------------------------
-// A tile with more offsets than this goes to the CTA-wide decode: its excess sits in
-// few warps (the mean is 512 offsets a warp), and one warp decoding 16384 offsets alone
-// takes about 26 chunks, the time the CTA needs for two of its own and the two clears.
-constexpr int kWarpOffsets = 2 * kTileMax;
+// A tile with more offsets than this goes to the CTA-wide decode.  One warp may own nearly
+// all of a tile's offsets (one heavy particle, or many): long runs it stores as they are,
+// and where it must decode chunk by chunk, 640 offsets at a time, the CTA's 10236 at a
+// time behind three barriers and two clears of the staging are quicker only for a great
+// many.  One weight in about 1e4 heavy, 2^24 particles, systematic, weights exp(3 N(0,1)): 98 us with the line
+// at 16384, 80 at 65536, 79 at 262144; exp(4 N) at 6e4 particles, stratified: 14.7, 12.4, 11.7;
+// 300 equally heavy particles side by side among 2^20: 56, 50, 89.
+// Without the look for long runs (LONG false) the line is at 16384.
+constexpr int kWarpOffsets = 8 * kTileMax, kWarpOffsetsShort = 2 * kTileMax;
+// A run of so many offsets of one particle, two of the warp's chunks, is stored as it is.
+constexpr int kRunFill = 1280;
 constexpr float kRoundMagic = 12582912.f;      // 1.5 2^23
 constexpr int kRoundMagicBits = 0x4b400000;
 
 // Staging entries per lane: 32 S covers a warp's usual range (its 32 KK elements'
 // worth of offsets and four standard deviations of N(0,1) weights) in one chunk, and an
 // odd multiple of four words between lanes keeps the 16-byte reads free of bank conflicts.
-constexpr int warp_stage_per_lane(int KK) { return KK == 16 ? 20 : (KK == 8 ? 12 : 8); }
+__host__ __device__ constexpr int warp_stage_per_lane(int KK) { return KK == 16 ? 20 : (KK == 8 ? 12 : 8); }
 
 // marks: this warp's 32 S entries, 16-byte aligned, all -1 on entry and on return.
 // ubuf (stratified): this warp's 32 S floats for the strata's uniforms.
-template <int KIND, int KK, int S>
+template <int KIND, int KK, int S, bool LONG>
 __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap map, int32_t* marks, float* ubuf,
                                             TileThread& th, int i_last, int64_t index0) {
     const int lane = threadIdx.x & 31;
@@ -455,7 +539,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
         if (clamp) fb = __fsub_rn(yb, (float)kb);
         // the uniforms of the warp's strata, four per Philox block, drawn once into ubuf
         const int k_first = __shfl_sync(0xffffffffu, kb, 0);
-        const int k_last = __reduce_max_sync(0xffffffffu, max(kb, kl));
+        // one more than the last count's: a compensated sum may step back by an ulp at the end
+        const int k_last = min(__reduce_max_sync(0xffffffffu, max(kb, kl)) + 1, kmax);
         const long long g0 = (map.jlo + k_first) >> 2;
         const int blocks = (int)(((map.jlo + k_last) >> 2) - g0) + 1;
         const int at = (int)(map.jlo - 4 * g0);  // ubuf index of stratum 0 (may be negative)
@@ -484,25 +569,45 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                 }
             }
         } else {
-            // strata beyond the buffer (a dominant particle): each thread draws the blocks its elements need
-            uint32_t cq = 0xffffffffu;
-            u32x4 cw = {0, 0, 0, 0};
-            auto u_of = [&](int k) -> float {
-                const long long j = map.jlo + k;
-                const uint32_t q = (uint32_t)(j >> 2);
-                if (q != cq) {
-                    cq = q;
-                    cw = philox(q, 0u, p.filter, TAG_STRAT, p.key0, p.key1);
+            // strata beyond the buffer: one buffer of them at a time, those without a
+            // coordinate (inside a dominant particle's run) passed over.  The whole buffer each
+            // time: draws cut off at the last stratum measured slower (no longer unrolled)
+            uint32_t open = kFull;  // elements whose stratum is still to come
+            bool open0 = true;
+            for (int w = k_first; w < INT_MAX;) {
+                const long long g = (map.jlo + w) >> 2;
+                const int w_at = (int)(map.jlo - 4 * g), w_end = 32 * S - w_at;  // strata [w, w_end) are in ubuf
+                __syncwarp();
+                for (int b = lane; b < 8 * S; b += 32) {
+                    const u32x4 r = philox((uint32_t)(g + b), 0u, p.filter, TAG_STRAT, p.key0, p.key1);
+                    *reinterpret_cast<float4*>(ubuf + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
                 }
-                return u23f(word_of(cw, (int)(j & 3)));
-            };
-            start0 = min(noff, kb + (u_of(kb) < fb ? 1 : 0));
+                __syncwarp();
+                int next = INT_MAX;
+                if (open0) {
+                    if (kb < w_end) {
+                        start0 = min(noff, kb + (ubuf[w_at + kb] < fb ? 1 : 0));
+                        open0 = false;
+                    } else {
+                        next = kb;
+                    }
+                }
 #pragma unroll
-            for (int i = 0; i < KK; ++i) {
-                const float y = __fmaf_rn(th.v[i], ir, x0);
-                float frac;
-                const int k = min(max(stratum(y, frac), 0), kmax);
-                th.v[i] = __int_as_float(min(noff, k + (u_of(k) < __fsub_rn(y, (float)k) ? 1 : 0)));
+                for (int i = 0; i < KK; ++i) {
+                    if ((open >> i) & 1u) {
+                        const float y = __fmaf_rn(th.v[i], ir, x0);
+                        float frac;
+                        const int k = min(max(stratum(y, frac), 0), kmax);
+                        if (k < w_end) {
+                            th.v[i] =
+                                __int_as_float(min(noff, k + (ubuf[w_at + k] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                            open &= ~(1u << i);
+                        } else {
+                            next = min(next, k);
+                        }
+                    }
+                }
+                w = __reduce_min_sync(0xffffffffu, next);
             }
         }
     }
@@ -521,9 +626,22 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
     const int B = __reduce_max_sync(0xffffffffu, pos ? last_n : 0);
     const int32_t e_base = (int32_t)index0 + th.e0;  // ancestor of this thread's element 0
     const int xl = lane * S;
+    const bool long_runs = LONG && B - A > 32 * S && __any_sync(0xffffffffu, longest_run<KK>(th, start0) >= kRunFill);
     for (int c0 = A; c0 < B;) {
         const int shift = (int)(((uintptr_t)(p.anc + map.jlo + c0) >> 2) & 3u);  // to a 16-byte boundary
         const int c1 = min(B, c0 + 32 * S - shift);
+        if (long_runs && B - c0 >= kRunFill) {
+            // a run that goes on for kRunFill offsets or more is stored as it is
+            int cur, next;
+            run_at<KK>(th, start0, c0, cur, next);
+            cur = __reduce_max_sync(0xffffffffu, cur < 0 ? -1 : e_base + cur);
+            next = min(__reduce_min_sync(0xffffffffu, next), B);
+            if (cur >= 0 && next - c0 >= kRunFill) {
+                fill_run(p.anc + map.jlo + c0, next - c0, cur, lane, 32);
+                c0 = next;
+                continue;
+            }
+        }
         // marks: each run's first slot in the chunk
         int a = start0;
         int32_t* mk = marks + (shift - c0);
@@ -625,21 +743,21 @@ __device__ __forceinline__ TileMap only_tile_map(const SortedParams& p, fpair W)
 // that one warp's share could be most of them, chunk by chunk over the CTA (which sets
 // the staging before, and back to -1 after).  Block-uniform choice.  The warp's
 // entries are -1 on entry (warp_stage_init) and on return.
-template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK)>
+template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK), bool LONG = true>  // LONG: as assign_offspring
 __device__ __forceinline__ void assign_tile(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
                                             TileThread& th, const TileSummary& ts, int64_t index0) {
     constexpr int kStride = warp_stage_stride<KIND, CAP>();
     static_assert(32 * S <= kStride && kStride % 4 == 0, "a warp's entries fit its share of the staging");
-    if (map.noff <= kWarpOffsets) {
+    if (map.noff <= (LONG ? kWarpOffsets : kWarpOffsetsShort)) {
         const int at = (threadIdx.x >> 5) * kStride;
-        assign_warp<KIND, KK, S>(p, map, stage + at, reinterpret_cast<float*>(stage + CAP) + at, th, ts.i_last, index0);
+        assign_warp<KIND, KK, S, LONG>(p, map, stage + at, reinterpret_cast<float*>(stage + CAP) + at, th, ts.i_last, index0);
         return;
     }
     __syncthreads();
     stage_init<CAP>(stage);
     __syncthreads();
     uint32_t epoch = 0;
-    assign_offspring<KIND, KK, CAP>(p, sm, map, stage, epoch, th, ts, index0);
+    assign_offspring<KIND, KK, CAP, LONG>(p, sm, map, stage, epoch, th, ts, index0);
     __syncthreads();
     stage_init<CAP>(stage);
     __syncthreads();

@@ -21,8 +21,7 @@ KINDS = {"systematic": (pf.PF_SYSTEMATIC, pf.pf_resample_systematic, oracle.syst
 @pytest.mark.parametrize("name", list(KINDS))
 @pytest.mark.parametrize("share", [0.002, 0.02, 0.3, 0.409, 0.41, 0.9])
 def test_dominant_particle(name, share):
-    """One particle with `share` of the weight: 80 to 36000 of 40000 offsets in one warp
-    (16384 = 0.4096 of them is the most a tile keeps in the warp-by-warp form)."""
+    """One particle with `share` of the weight: 80 to 36000 of 40000 offsets in one warp."""
     _, fn, orc = KINDS[name]
     P = 40000
     lw = np.random.default_rng(3).standard_normal(P).astype(np.float32)
@@ -62,3 +61,33 @@ def test_whole_filters_of_mixed_widths(name):
         rep = check_cumulative(name, part, got[off[f]:off[f + 1]], orc(part, int(seeds[f]), f), int(seeds[f]),
                                filter_id=f)
         assert rep.ok, (f, rep.summary())
+
+
+@pytest.mark.parametrize("name", list(KINDS))
+@pytest.mark.parametrize("runs", [(1279,), (1280, 1281), (640, 5000, 3), (65000,), (30000, 36000), (20479, 20480, 41000),
+                                  (150000, 9000)])
+def test_long_runs(name, runs):
+    """Neighbouring particles with long runs (some in one thread, some across threads), in
+    tiles on either side of the 65536 offsets that send a tile to the CTA-wide decode, with
+    particles of a few offsets around them and zero weights between: the runs stored as they
+    are, and the chunks between them, at every alignment."""
+    _, fn, orc = KINDS[name]
+    P = 300000
+    lw = np.random.default_rng(len(runs)).standard_normal(P).astype(np.float32)
+    lw[70001:70010:3] = -np.inf
+    places = [70002, 70003, 70035][:len(runs)]
+    lw[places] = -np.inf
+    rest = np.exp(lw.astype(np.float64)).sum()
+    total = rest * P / (P - sum(runs))
+    lw[places] = np.log(np.array(runs) / P * total)
+    lw[70300:70400] = np.log(30.0 * total / P)  # a warp of many middling runs
+    d = torch.from_numpy(lw).cuda()
+    ref = orc(lw, 11)
+    for shift in range(4):
+        buf = torch.full((P + 8,), -3, dtype=torch.int32, device="cuda")
+        fn(d, P, 0, 11, buf[shift:])
+        assert pf.pf_get_device_status() == pf.PF_OK
+        got = buf.cpu().numpy()
+        assert (got[:shift] == -3).all() and (got[shift + P:] == -3).all()
+        rep = check_cumulative(name, lw, got[shift:shift + P], ref, 11)
+        assert rep.ok, rep.summary()
