@@ -22,8 +22,8 @@
 // Bound by its launches and by L2 latency (five passes of 4 bytes a slot, of which
 // only the first and the last touch the caller's arrays): one memset and four
 // launches where there were three memsets and seven.  Stratified resampling,
-// permutation and in-place move of 3 M rows of 64 bytes: 212 -> 150 us, and 136 us
-// with the rows in 256-bit chunks.
+// permutation and in-place move of 3 M rows of 64 bytes: 212 -> 150 us, 136 us
+// with the rows in 256-bit chunks, and 116 us with more of their reads in flight.
 #include <climits>
 #include <type_traits>
 
@@ -269,42 +269,59 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __res
 // its own slot (perm[perm[j]] = perm[j]), else the row is left and
 // PF_ERR_INVALID recorded.  Chunks as in the gather; a source row is read beside
 // its own perm entry, before that is known to be itself (a row being overwritten
-// meanwhile is read to no effect).
+// meanwhile is read to no effect).  The next piece's entries of perm are asked for while
+// this piece's rows are on their way.
+//
+// Bound by the reads in flight: a chunk waits for its entry of perm, then its row.
+// us, row i of 3000017 moved where stratified resampling of exp(2 N(0,1)) weights moves it, rows
+// of 32, 64, 96, 128 bytes, two chunks a thread without the early entries: 32, 51, 77, 80;
+// four chunks a thread, a CTA for each piece: 25, 44, 80, 67; three a thread in one
+// resident wave with the early entries: 27, 47, 67, 53.
 template <typename VT, int U, bool POW2>
 __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSplit split,
                                                         const int32_t* __restrict__ perm, uint32_t* ctl) {
     grid_begin();
     const int64_t total = P * split.vecs;
     const int64_t stride = (int64_t)gridDim.x * (256 * U);
-    for (int64_t base = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; base < total; base += stride) {
-        int32_t a[U], own[U];
-        uint32_t c[U];
+    int64_t base = (int64_t)blockIdx.x * (256 * U) + threadIdx.x;
+    int32_t a[U];  // this piece's entries of perm, and the chunks' places in their rows
+    uint32_t c[U];
+    auto entries = [&](int64_t b, int32_t (&e)[U], uint32_t (&at)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = b + u * 256;
+            e[u] = -1;
+            at[u] = 0;
+            if (i < total) e[u] = __ldg(perm + split.row<POW2>(i, at[u]));
+        }
+    };
+    entries(base, a, c);
+    for (; base < total; base += stride) {
+        int32_t own[U];
         VT v[U];
         bool move[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t i = base + u * 256;
-            move[u] = false;
-            a[u] = 0;
-            if (i < total) {
-                const int64_t j = split.row<POW2>(i, c[u]);
-                a[u] = __ldg(perm + j);
-                move[u] = a[u] != j;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
+            uint32_t cc;
+            move[u] = i < total && a[u] != (int32_t)split.row<POW2>(i, cc);
             own[u] = -1;
             if (move[u] && a[u] >= 0 && a[u] < P) {
                 own[u] = __ldg(perm + a[u]);
                 v[u] = load_chunk(x + (int64_t)a[u] * split.vecs + c[u]);
             }
         }
+        int32_t an[U];
+        uint32_t cn[U];
+        entries(base + stride, an, cn);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (!move[u]) continue;
-            if (own[u] >= 0 && own[u] == a[u]) store_chunk_cs(x + base + u * 256, v[u]);
-            else if (c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
+            if (move[u]) {
+                if (own[u] >= 0 && own[u] == a[u]) store_chunk_cs(x + base + u * 256, v[u]);
+                else if (c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
+            }
+            a[u] = an[u];
+            c[u] = cn[u];
         }
     }
 }
@@ -341,20 +358,29 @@ cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* sc
 
 cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const int32_t* perm, uint32_t* ctl,
                                   int num_sms, cudaStream_t s) {
-    auto go = [&](auto* p, auto unroll) {
+    auto go = [&](auto* p, auto unroll, int wave, int full) {
         using VT = std::remove_pointer_t<decltype(p)>;
         constexpr int U = decltype(unroll)::value;
         const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
         const RowSplit split = row_split(vecs, P * vecs);
-        const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, 8, 40);
+        const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, wave, full);
         return launch_overlapped(split.pow2 ? k_gather_inplace<VT, U, true> : k_gather_inplace<VT, U, false>, blocks, 256, 0, s,
                                  p, P, split, perm, ctl);
     };
     const uintptr_t a = (uintptr_t)x | (uintptr_t)row_bytes;
-    if ((a & 31) == 0) return go(static_cast<u32x8*>(x), std::integral_constant<int, 2>());
-    if ((a & 15) == 0) return go(static_cast<uint4*>(x), std::integral_constant<int, 4>());
-    if ((a & 7) == 0) return go(static_cast<uint2*>(x), std::integral_constant<int, 4>());
-    return go(static_cast<uint32_t*>(x), std::integral_constant<int, 4>());
+    constexpr int kNever = 1 << 22;  // one resident wave however many pieces there are
+    const std::integral_constant<int, 3> three;
+    const std::integral_constant<int, 4> four;
+    // 256-bit chunks: rows of one or two are read one row's length apart and do best with the
+    // most reads in flight; longer rows with the wave (both sides measured above)
+    if ((a & 31) == 0) {
+        u32x8* q = static_cast<u32x8*>(x);
+        return row_bytes <= 64 ? go(q, four, 4, 12) : go(q, three, 4, kNever);
+    }
+    if ((a & 15) == 0) return go(static_cast<uint4*>(x), four, 8, 40);
+    // 4-byte chunks (1.2e7 rows of 4 and 12 bytes: 27 and 93 us as a wave, 33 and 110 in full)
+    if ((a & 7) == 0) return go(static_cast<uint2*>(x), four, 5, kNever);
+    return go(static_cast<uint32_t*>(x), four, 5, kNever);
 }
 
 }  // namespace pf

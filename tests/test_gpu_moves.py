@@ -72,3 +72,22 @@ def test_bad_rows_are_left_and_reported():
     want = before.clone()
     want[101] = before[102]
     assert torch.equal(x, want)
+
+
+@pytest.mark.parametrize("dim", [1, 3, 24, 32])
+def test_in_place_waves_of_several_pieces(dim):
+    """More chunks than one resident wave takes at once, so that every CTA goes on to further
+    pieces with their entries asked for early; odd sizes leave a ragged last piece."""
+    P = 1000003
+    g = torch.Generator(device="cuda")
+    g.manual_seed(dim)
+    lw = 2.0 * torch.randn(P, device="cuda", generator=g)
+    a = torch.empty(P, dtype=torch.int32, device="cuda")
+    perm = torch.empty_like(a)
+    pf.pf_resample_systematic(lw, P, 0, 3, a)
+    pf.pf_permute(a, P, perm)
+    x = torch.randn(P, dim, device="cuda", generator=g)
+    ref = x[perm.long()]
+    pf.pf_gather_inplace(x, P, 4 * dim, perm)
+    assert pf.pf_get_device_status() == pf.PF_OK
+    assert torch.equal(x, ref)
