@@ -75,7 +75,7 @@ def test_bad_rows_are_left_and_reported():
 
 
 @pytest.mark.parametrize("dim", [1, 3, 24, 32])
-def test_in_place_waves_of_several_pieces(dim):
+def test_waves_of_several_pieces(dim):
     """More chunks than one resident wave takes at once, so that every CTA goes on to further
     pieces with their entries asked for early; odd sizes leave a ragged last piece."""
     P = 1000003
@@ -88,6 +88,9 @@ def test_in_place_waves_of_several_pieces(dim):
     pf.pf_permute(a, P, perm)
     x = torch.randn(P, dim, device="cuda", generator=g)
     ref = x[perm.long()]
+    out = torch.empty_like(x)
+    pf.pf_gather(x, P, 4 * dim, a, P, out)
+    assert torch.equal(out, x[a.long()])
     pf.pf_gather_inplace(x, P, 4 * dim, perm)
     assert pf.pf_get_device_status() == pf.PF_OK
     assert torch.equal(x, ref)
