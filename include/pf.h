@@ -91,7 +91,7 @@ enum {
 /* Largest P (plus the alignment lead of logw) that a single-filter
  * systematic, stratified or multinomial call resamples in one cooperative
  * launch (4096 tiles of 8192 log-weights).  Beyond it the call runs three
- * ordinary launches on the stream -- the tile scans, one CTA forming every
+ * ordinary launches on the stream -- the tile scans, one cluster forming every
  * tile's exact carry, then the assignment (systematic, stratified: from the
  * tiles' stored cumulative weights) or, for the multinomial, a guide table
  * and the draws (each through its guide entry and one window of the stored

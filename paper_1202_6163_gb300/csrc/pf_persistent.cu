@@ -27,8 +27,8 @@
 //      tile owns the offsets j whose position (j + u_j) W / P lies in
 //      [B_t, B_{t+1}); each element counts the offsets below its cumulative
 //      weight, N_i, and its index fills [N_{i-1}, N_i) by a run-length decode
-//      in shared memory (mark run starts, block max-scan), stored with 128-bit
-//      writes;
+//      in shared memory (mark run starts, max-scan; a warp at a time, pf_assign.cuh),
+//      stored with 128-bit writes;
 //      multinomial: the CTA draws a balanced slice of the P uniforms; a draw
 //      finds its tile from a lookup of the tile boundaries and its element in
 //      three levels (every 2^c1shift-th v_i in shared memory, then one
@@ -725,12 +725,6 @@ static cudaError_t launch_one_tile(const SortedParams& p, int grid, cudaStream_t
 }
 
 template <int KIND, int KK, bool GUIDE = false>
-static cudaError_t set_smem_attr() {
-    return cudaFuncSetAttribute(k_persistent<KIND, KK, GUIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)persistent_smem_bytes(KIND, kMaxTilesTotal, KK));
-}
-
-template <int KIND, int KK, bool GUIDE = false>
 static cudaError_t launch_kind(const SortedParams& p, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -749,20 +743,17 @@ static cudaError_t launch_kind(const SortedParams& p, int grid, cudaStream_t s) 
 template <int KIND>
 static cudaError_t launch_k(const SortedParams& p, int grid, cudaStream_t s) {
     const int q = (p.tile + kThreads - 1) / kThreads;  // elements per thread of a full tile
-    if (KIND == KIND_MULTI && p.g_out) {
-        if (q <= 4) return launch_kind<KIND, 4, true>(p, grid, s);
-        if (q <= 8) return launch_kind<KIND, 8, true>(p, grid, s);
-        return launch_kind<KIND, 16, true>(p, grid, s);
-    }
-    if constexpr (KIND != KIND_MULTI) {
+    if constexpr (KIND == KIND_MULTI) {
+        if (p.g_out) return launch_kind<KIND, 16, true>(p, grid, s);  // several tiles per CTA: full ones
+        if (q <= 4) return launch_kind<KIND, 4>(p, grid, s);
+        if (q <= 8) return launch_kind<KIND, 8>(p, grid, s);
+    } else {
         if (p.tiles_per_cta <= 1 && p.tagged != nullptr && grid == p.n_tiles && grid <= kThreads) {
             if (q <= 4) return launch_one_tile<KIND, 4>(p, grid, s);
             if (q <= 8) return launch_one_tile<KIND, 8>(p, grid, s);
             return launch_one_tile<KIND, 16>(p, grid, s);
         }
     }
-    if (q <= 4) return launch_kind<KIND, 4>(p, grid, s);
-    if (q <= 8) return launch_kind<KIND, 8>(p, grid, s);
     return launch_kind<KIND, 16>(p, grid, s);
 }
 
@@ -784,28 +775,17 @@ cudaError_t launch_sorted_persistent(int kind, const SortedParams& p, int grid, 
 // their dynamic shared memory limits on the way).  Called once per device.
 template <int KIND, int KK>
 static int blocks_per_sm_kk() {
-    int nb = 0;
-    if (set_smem_attr<KIND, KK>() != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_persistent<KIND, KK>, kThreads,
-                                                      persistent_smem_bytes(KIND, kMaxTilesTotal, KK)) != cudaSuccess)
-        return 0;
-    if constexpr (KIND == KIND_MULTI) {  // the guide variant: the same launch shape, so the smaller of the two
-        int ng = 0;
-        if (set_smem_attr<KIND, KK, true>() != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ng, k_persistent<KIND, KK, true>, kThreads,
-                                                          persistent_smem_bytes(KIND, kMaxTilesTotal, KK)) !=
-                cudaSuccess)
-            return 0;
-        nb = min(nb, ng);
-    } else {  // the one-tile-per-CTA variant: as many CTAs too
-        int n1 = 0;
-        if (cudaFuncSetAttribute(k_one_tile<KIND, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)one_tile_smem(KK)) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_one_tile<KIND, KK>, kThreads, one_tile_smem(KK)) !=
-                cudaSuccess)
-            return 0;
-        nb = min(nb, n1);
-    }
+    int nb = INT_MAX;
+    auto take = [&](auto kernel, size_t smem) {
+        int n = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, smem) != cudaSuccess)
+            n = 0;
+        nb = min(nb, n);
+    };
+    if constexpr (KIND == KIND_MULTI || KK == 16) take(k_persistent<KIND, KK, false>, persistent_smem_bytes(KIND, kMaxTilesTotal, KK));
+    if constexpr (KIND == KIND_MULTI && KK == 16) take(k_persistent<KIND, KK, true>, persistent_smem_bytes(KIND, kMaxTilesTotal, KK));
+    if constexpr (KIND != KIND_MULTI) take(k_one_tile<KIND, KK>, one_tile_smem(KK));
     return nb;
 }
 
