@@ -20,6 +20,7 @@ cudaError_t launch_metropolis(const float* lw, int64_t P, int B, const uint32_t*
                               uint32_t filter, int32_t* anc, uint32_t* ctl, int num_sms, cudaStream_t s, int rounds);
 cudaError_t prepare_metropolis();
 cudaError_t prepare_large();
+cudaError_t prepare_permute();
 cudaError_t launch_large(int kind, SortedParams p, void* scratch, int num_sms, cudaStream_t s);
 size_t large_scratch_bytes(int kind, int64_t PA);
 cudaError_t prepare_small(int (&tiles)[3]);
@@ -105,6 +106,8 @@ pf_status device_info(int& dev, DeviceInfo*& info) {
     if (e != cudaSuccess) return cuda_fail(e, "prepare_metropolis");
     e = prepare_large();
     if (e != cudaSuccess) return cuda_fail(e, "prepare_large");
+    e = prepare_permute();
+    if (e != cudaSuccess) return cuda_fail(e, "prepare_permute");
     e = prepare_small(info->small_tiles);
     if (e != cudaSuccess) return cuda_fail(e, "prepare_small");
     info->ready = true;

@@ -265,6 +265,97 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __res
     }
 }
 
+// Few particles: the whole permutation in one CTA and shared memory, where the passes above
+// are five launches of two to three microseconds each whatever they move.  Counts and
+// list lie at i + i / 32, so that threads reading their own consecutive entries meet no
+// bank conflict.
+// Bound by its serial phases, which grow with the particles a thread holds: 100, 4096, 8192,
+// 16384 particles 3.6, 4.8, 7.1, 12.1 us against 13.5, 13.3, 13.7, 14.5 by the passes; the
+// line is where shared memory ends, a little before the two meet.
+constexpr int kPermSmall = 16384;  // both arrays in 132 KiB
+constexpr int kPermSmallThreads = 1024;
+constexpr int kPermSmallPer = kPermSmall / kPermSmallThreads;
+constexpr int perm_small_at(int i) { return i + (i >> 5); }
+constexpr size_t kPermSmallSmem = 2 * (size_t)(perm_small_at(kPermSmall)) * sizeof(int32_t);
+
+__global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t* __restrict__ anc, int P,
+                                                                  int32_t* __restrict__ out, uint32_t* ctl) {
+    extern __shared__ int32_t perm_smem[];
+    __shared__ int red[32];
+    int32_t* o = perm_smem;
+    int32_t* E = perm_smem + (kPermSmall + (kPermSmall >> 5));
+    auto at = [](int i) { return i + (i >> 5); };
+    grid_begin();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < P; i += kPermSmallThreads) {
+        o[at(i)] = 0;
+        E[at(i)] = -1;
+    }
+    __syncthreads();
+    // counts: one addition per run of equal neighbours in a row of 32 (as k_perm_count)
+    for (int j0 = 32 * warp; j0 < P; j0 += kPermSmallThreads) {
+        const int j = j0 + lane;
+        int32_t a = j < P ? __ldg(anc + j) : INT_MIN;
+        if (j < P && (a < 0 || a >= P)) {
+            set_status(ctl + CTL_STATUS, ST_INVALID);
+            a = INT_MIN;
+        }
+        const int32_t below = __shfl_up_sync(0xffffffffu, a, 1);
+        const bool head = lane == 0 || below != a;
+        const uint32_t heads = __ballot_sync(0xffffffffu, head);
+        if (head && a >= 0) {
+            const uint32_t later = heads & ~(0xffffffffu >> (31 - lane));
+            atomicAdd(o + at(a), (later ? __ffs((int)later) - 1 : 32) - lane);
+        }
+    }
+    __syncthreads();
+    // extra copies and empty slots before this thread's entries: both below 2^15, one scan
+    const int per = (P + kPermSmallThreads - 1) / kPermSmallThreads, i0 = tid * per, i1 = min(P, i0 + per);
+    int x = 0;
+    for (int i = i0; i < i1; ++i) {
+        const int c = o[at(i)];
+        x += c == 0 ? 1 : (c - 1) << 16;
+    }
+    int inc = x;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int h = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += h;
+    }
+    if (lane == 31) red[warp] = inc;
+    __syncthreads();
+    const int before = inc - x + __reduce_add_sync(0xffffffffu, lane < warp ? red[lane] : 0);
+    int r = before >> 16;
+    for (int i = i0; i < i1; ++i) {
+        const int c = o[at(i)];
+        if (c > 1) {
+            E[at(r)] = i;
+            r += c - 1;
+        }
+    }
+    __syncthreads();
+    // running maximum over the marks
+    int m = -1;
+    for (int i = i0; i < i1; ++i) m = max(m, E[at(i)]);
+    int mm = m;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int h = __shfl_up_sync(0xffffffffu, mm, off);
+        if (lane >= off) mm = max(mm, h);
+    }
+    int carry = __shfl_up_sync(0xffffffffu, mm, 1);
+    if (lane == 0) carry = -1;
+    if (lane == 31) red[warp] = mm;  // every read of the sums is behind the barrier above
+    __syncthreads();
+    carry = max(carry, __reduce_max_sync(0xffffffffu, lane < warp ? red[lane] : -1));
+    for (int i = i0; i < i1; ++i) E[at(i)] = carry = max(carry, E[at(i)]);
+    __syncthreads();
+    int d = before & 0xffff;
+    for (int i = i0; i < i1; ++i) o[at(i)] = o[at(i)] == 0 ? E[at(d++)] : i;  // ranks below P: inside E
+    __syncthreads();
+    for (int i = tid; i < P; i += kPermSmallThreads) out[i] = o[at(i)];
+}
+
 // In-place gather: row j <- row perm[j] where they differ; a source must keep
 // its own slot (perm[perm[j]] = perm[j]), else the row is left and
 // PF_ERR_INVALID recorded.  Chunks as in the gather; a source row is read beside
@@ -336,8 +427,16 @@ size_t permute_scratch_bytes(int64_t P) {
     return perm_counts_at(T) + (((size_t)P * sizeof(int32_t) + 255) & ~(size_t)255) + (size_t)P * sizeof(int32_t);
 }
 
+// Once per device.
+cudaError_t prepare_permute() {
+    return cudaFuncSetAttribute(k_perm_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPermSmallSmem);
+}
+
 cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* scratch, uint32_t* ctl, int num_sms,
                            cudaStream_t s) {
+    if (P <= kPermSmall) {
+        return launch_overlapped(k_perm_small, 1, kPermSmallThreads, kPermSmallSmem, s, anc, (int)P, out, ctl);
+    }
     const int T = (int)((P + kPermTile - 1) / kPermTile);
     TilePrefix* pre = static_cast<TilePrefix*>(scratch);
     int32_t* o = reinterpret_cast<int32_t*>((char*)scratch + perm_counts_at(T));

@@ -94,3 +94,16 @@ def test_waves_of_several_pieces(dim):
     pf.pf_gather_inplace(x, P, 4 * dim, perm)
     assert pf.pf_get_device_status() == pf.PF_OK
     assert torch.equal(x, ref)
+
+
+@pytest.mark.parametrize("law", ["sorted", "random", "one", "runs"])
+@pytest.mark.parametrize("P", [2, 32, 1023, 1024, 1025, 12321, 16383, 16384, 16385])
+def test_permute_in_one_cta(P, law):
+    """Either side of the count up to which one CTA forms the permutation, and where its
+    threads' shares of the particles end unevenly."""
+    a = ancestors(P, law, seed=P)
+    out = torch.full((P + 2,), -3, dtype=torch.int32, device="cuda")
+    pf.pf_permute(torch.from_numpy(a).cuda(), P, out[1:])
+    assert pf.pf_get_device_status() == pf.PF_OK
+    got = out.cpu().numpy()
+    assert np.array_equal(got[1:P + 1], oracle.permute(a)) and got[0] == -3 and got[-1] == -3
