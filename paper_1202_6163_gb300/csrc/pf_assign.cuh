@@ -4,6 +4,7 @@
 #pragma once
 
 #include "pf_fixed.cuh"
+#include "pf_index.h"
 #include "pf_tile.cuh"
 
 namespace pf {
@@ -574,16 +575,16 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
         };
         float fb, fl;
         const int kb0 = stratum(yb, fb), kl0 = stratum(yl, fl);
-        const bool clamp = kb0 < 0 || kl0 > kmax;
+        const bool clamp = strata_clamped(kb0, kl0, kmax, pos);
         const int kb = min(max(kb0, 0), kmax), kl = min(max(kl0, 0), kmax);
         if (clamp) fb = __fsub_rn(yb, (float)kb);
         // the uniforms of the warp's strata, four per Philox block, drawn once into ubuf
         const int k_first = __shfl_sync(0xffffffffu, kb, 0);
         // one more than the last count's: a compensated sum may step back by an ulp at the end
         const int k_last = min(__reduce_max_sync(0xffffffffu, max(kb, kl)) + 1, kmax);
-        const long long g0 = (map.jlo + k_first) >> 2;
-        const int blocks = (int)(((map.jlo + k_last) >> 2) - g0) + 1;
-        const int at = (int)(map.jlo - 4 * g0);  // ubuf index of stratum 0 (may be negative)
+        const long long g0 = strata_block(map.jlo, k_first);
+        const int blocks = (int)(strata_block(map.jlo, k_last) - g0) + 1;
+        const int at = strata_at(map.jlo, g0);  // ubuf index of stratum 0 (may be negative)
         if (blocks <= 8 * S) {
             __syncwarp();  // the last tile's reads of ubuf
             for (int b = lane; b < blocks; b += 32) {
@@ -591,7 +592,7 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                 *reinterpret_cast<float4*>(ubuf + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
             }
             __syncwarp();
-            start0 = min(noff, kb + (ubuf[at + kb] < fb ? 1 : 0));
+            start0 = min(noff, kb + (ubuf[strata_index(at, kb)] < fb ? 1 : 0));
             if (!clamp) {
 #pragma unroll
                 for (int i = 0; i < KK; ++i) {
@@ -605,7 +606,7 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                     const float y = __fmaf_rn(th.v[i], ir, x0);
                     float frac;
                     const int k = min(max(stratum(y, frac), 0), kmax);
-                    th.v[i] = __int_as_float(min(noff, k + (ubuf[at + k] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                    th.v[i] = __int_as_float(min(noff, k + (ubuf[strata_index(at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
                 }
             }
         } else {
@@ -615,8 +616,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
             uint32_t open = kFull;  // elements whose stratum is still to come
             bool open0 = true;
             for (int w = k_first; w < INT_MAX;) {
-                const long long g = (map.jlo + w) >> 2;
-                const int w_at = (int)(map.jlo - 4 * g), w_end = 32 * S - w_at;  // strata [w, w_end) are in ubuf
+                const long long g = strata_block(map.jlo, w);
+                const int w_at = strata_at(map.jlo, g), w_end = 32 * S - w_at;  // strata [w, w_end) are in ubuf
                 __syncwarp();
                 for (int b = lane; b < 8 * S; b += 32) {
                     const u32x4 r = philox((uint32_t)(g + b), 0u, p.filter, TAG_STRAT, p.key0, p.key1);
@@ -626,7 +627,7 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                 int next = INT_MAX;
                 if (open0) {
                     if (kb < w_end) {
-                        start0 = min(noff, kb + (ubuf[w_at + kb] < fb ? 1 : 0));
+                        start0 = min(noff, kb + (ubuf[strata_index(w_at, kb)] < fb ? 1 : 0));
                         open0 = false;
                     } else {
                         next = kb;
@@ -639,8 +640,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                         float frac;
                         const int k = min(max(stratum(y, frac), 0), kmax);
                         if (k < w_end) {
-                            th.v[i] =
-                                __int_as_float(min(noff, k + (ubuf[w_at + k] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                            th.v[i] = __int_as_float(
+                                min(noff, k + (ubuf[strata_index(w_at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
                             open &= ~(1u << i);
                         } else {
                             next = min(next, k);
@@ -1279,7 +1280,8 @@ __device__ __forceinline__ void st_v8(float* p, const float* o) {
 
 // Reloads a tile stored by write_tile_v into th (elements of tile-local
 // indices [0, n)): v from the magnitudes, the positive-weight mask from the
-// sign bits.  Slots at or beyond n are not read.  SMEM: vg0 is a copy of the
+// sign bits.  Slots at or beyond n are not read: they and, in threads wholly past n, the base
+// hold the last element's v, as after a scan.  SMEM: vg0 is a copy of the
 // tile in shared memory.  Every lane of the warp must call it (the bases come
 // from the lane below).
 template <int KK = 0, bool SMEM = false>  // KK: elements per thread when fixed (the tile was scanned with KK), 0 = from n
@@ -1318,7 +1320,7 @@ __device__ __forceinline__ void read_tile_v(const float* vg0, int n, TileThread&
         if (KK || i < K) any |= __float_as_uint(th.v[i]);
     if (any >> 31) {
         pos = 0;
-        float run = 0.f;
+        float run = th.e0 >= n ? fabsf(SMEM ? vg0[n - 1] : __ldcg(vg0 + n - 1)) : 0.f;
 #pragma unroll
         for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
             if (KK || i < K) {
@@ -1335,7 +1337,7 @@ __device__ __forceinline__ void read_tile_v(const float* vg0, int n, TileThread&
         if (KK || i < K) last = th.v[i];
     th.base = __shfl_up_sync(0xffffffffu, last, 1);
     if ((threadIdx.x & 31) == 0)
-        th.base = th.e0 > 0 && th.e0 <= n ? fabsf(SMEM ? vg[-1] : __ldcg(vg - 1)) : 0.f;
+        th.base = th.e0 == 0 ? 0.f : (th.e0 <= n ? fabsf(SMEM ? vg[-1] : __ldcg(vg - 1)) : th.v[0]);
 }
 
 // The tile's cumulative weights to global memory (sign bit: zero weight), for the searches.

@@ -1,0 +1,32 @@
+// Index arithmetic of the kernels, written so that host code can run it too: where a
+// mistake would read or write out of range, it is checked on the CPU over more shapes than
+// a GPU test can reach.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define PF_HD __host__ __device__ __forceinline__
+#else
+#define PF_HD inline
+#endif
+
+namespace pf {
+
+// ---------------------------------------------------------------------------
+// The strata of one warp of the stratified assignment, counted from its tile's first offset
+// jlo.  Their uniforms lie in the warp's buffer by whole Philox blocks of four, from that of
+// lane 0's lowest stratum on.
+// ---------------------------------------------------------------------------
+PF_HD long long strata_block(long long jlo, int k) { return (jlo + k) >> 2; }
+// The place of stratum 0 (negative in all warps but the first) for a buffer from block g0 on.
+PF_HD int strata_at(long long jlo, long long g0) { return (int)(jlo - 4 * g0); }
+// The place of stratum k.  A lane without weight may ask for one below the buffer's (past the
+// tile's end it may hold any coordinate); what it gets is not used.
+PF_HD int strata_index(int at, int k) { return at + k < 0 ? 0 : at + k; }
+// Whether a lane bounds each of its look-ups: its lowest stratum kb0 or its highest kl0 lies
+// outside the tile (at the tile's ends, by rounding), or no element of it has weight (pos = 0).
+// The strata of any other lane are lane 0's or later, and rise along the lane.
+PF_HD bool strata_clamped(int kb0, int kl0, int kmax, uint32_t pos) { return kb0 < 0 || kl0 > kmax || pos == 0u; }
+
+}  // namespace pf
