@@ -29,4 +29,13 @@ PF_HD int strata_index(int at, int k) { return at + k < 0 ? 0 : at + k; }
 // The strata of any other lane are lane 0's or later, and rise along the lane.
 PF_HD bool strata_clamped(int kb0, int kl0, int kmax, uint32_t pos) { return kb0 < 0 || kl0 > kmax || pos == 0u; }
 
+// ---------------------------------------------------------------------------
+// Parts of the permutation's listing (pf_permute.cu): a tile's extra copies, up to P - 1 =
+// 2^31 - 2 of them, kPermPart to a part.  Sums with kPermPart would pass 2^31.
+// ---------------------------------------------------------------------------
+constexpr int kPermPart = 8192;  // extras one CTA lists: twice a tile's mean share
+PF_HD int perm_parts(int extras) { return extras / kPermPart + (extras % kPermPart != 0 ? 1 : 0); }
+// The end of the part that starts at rank s0 < extras.
+PF_HD int perm_part_end(int s0, int extras) { return s0 + (extras - s0 < kPermPart ? extras - s0 : kPermPart); }
+
 }  // namespace pf

@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "pf_device.cuh"
+#include "pf_index.h"
 #include "pf_internal.h"
 #include "pf_rows.cuh"
 
@@ -38,7 +39,6 @@ constexpr int kPermThreads = 512;
 constexpr int kPermPer = 8;
 constexpr int kPermTile = kPermThreads * kPermPer;
 constexpr int kPermWarps = kPermThreads / 32;
-constexpr int kPermPart = 8192;  // extras one CTA lists: twice a tile's mean share
 
 // One count per ancestor.  A warp takes four rows of 32 consecutive entries; the
 // first lane of each run of equal entries in a row adds the run's length.
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* __re
     for (int base = 0; base < T; base += kPermThreads) {
         const int t = base + threadIdx.x;
         const int xe = t < T ? __ldcg(&pre[t].extra) : 0, xd = t < T ? __ldcg(&pre[t].dead) : 0;
-        const int xp = (xe + kPermPart - 1) / kPermPart;
+        const int xp = perm_parts(xe);
         int se, sd, sp;
         const int pe = block_excl_scan(xe, red, se), pd = block_excl_scan(xd, red, sd), pp = block_excl_scan(xp, red, sp);
         if (t < T) pre[t] = {ce + pe, cd + pd, cp + pp};
@@ -176,8 +176,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __res
             else hi = mid - 1;
         }
         const int t = lo;
-        const int s0 = (b - __ldg(&pre[t].part)) * kPermPart;                          // this part's ranks within the tile:
-        const int s1 = min(s0 + kPermPart, __ldg(&pre[t + 1].extra) - __ldg(&pre[t].extra));  // [s0, s1)
+        const int s0 = (b - __ldg(&pre[t].part)) * kPermPart;  // this part's ranks within the tile:
+        const int s1 = perm_part_end(s0, __ldg(&pre[t + 1].extra) - __ldg(&pre[t].extra));  // [s0, s1)
         int32_t* out = E + __ldg(&pre[t].extra) + s0;
         const int shift = (int)(((uintptr_t)out >> 2) & 3u);  // to a 16-byte boundary
         const int end = s1 - s0 + shift;

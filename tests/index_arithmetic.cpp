@@ -115,9 +115,27 @@ static void strata() {
     for (int empty = 0; empty < 3; ++empty) strata_of_tile(rng, 16, 20, 4153, v, 34152, 0.25f, 1.f, 33550000, empty);
 }
 
+// ---------------------------------------------------------------------------
+// The permutation's parts: they cover a tile's extra copies once, in order, up to the largest count.
+// ---------------------------------------------------------------------------
+static void permute_parts() {
+    for (long long extras : {0LL, 1LL, 8191LL, 8192LL, 8193LL, 1000003LL, (1LL << 31) - 8194, (1LL << 31) - 8193,
+                             (1LL << 31) - 8192, (1LL << 31) - 8191, (1LL << 31) - 2}) {
+        const int x = (int)extras, parts = pf::perm_parts(x);
+        long long at = 0;
+        for (int b = 0; b < parts; ++b) {
+            const int s0 = b * pf::kPermPart, s1 = pf::perm_part_end(s0, x);
+            REQUIRE(s0 == at && s1 > s0 && s1 - s0 <= pf::kPermPart, "parts: [%d, %d) at %lld of %lld extras", s0, s1, at, extras);
+            at = s1;
+        }
+        REQUIRE(at == extras, "parts: %d parts list %lld of %lld extras", parts, at, extras);
+    }
+}
+
 int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!std::strcmp(what, "strata")) strata();
+    else if (!std::strcmp(what, "permute_parts")) permute_parts();
     else return 2;
     return 0;
 }

@@ -1,0 +1,21 @@
+"""The largest particle counts the entry points accept, where 32-bit index arithmetic has no
+room left: the calls run to the end and every entry is right."""
+import pytest
+
+from paper_1202_6163_gb300 import pf
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+P_MAX = 2147483647  # PF_MAX_PARTICLES
+
+
+@pytest.mark.parametrize("P", [P_MAX, P_MAX - 8192])
+def test_permute_all_offspring_of_one_particle(P):
+    """Every tile but one is empty slots; one tile lists P - 1 extra copies."""
+    kept = 1234567890
+    a = torch.full((P,), kept, dtype=torch.int32, device="cuda")
+    out = torch.full((P + 1,), -3, dtype=torch.int32, device="cuda")
+    pf.pf_permute(a, P, out)
+    assert pf.pf_get_device_status() == pf.PF_OK
+    assert bool(torch.equal(out[:P], a)) and int(out[P]) == -3
