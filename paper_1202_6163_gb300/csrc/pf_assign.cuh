@@ -195,8 +195,8 @@ __device__ __forceinline__ int longest_run(const TileThread& th, int start0) {
 __device__ __forceinline__ void fill_run(int32_t* dst, int n, int32_t v, int t, int threads) {
     const int head = min((int)((4u - (uint32_t)((uintptr_t)dst >> 2)) & 3u), n), body = (n - head) & ~3;
     if (t < head) dst[t] = v;
-    for (int x = head + 4 * t; x < head + body; x += 4 * threads)
-        *reinterpret_cast<int4*>(dst + x) = make_int4(v, v, v, v);
+    for (FillPieces f(head, body, t, threads); f.x < f.end; f.x += f.step)
+        *reinterpret_cast<int4*>(dst + f.x) = make_int4(v, v, v, v);
     if (t < n - head - body) dst[head + body + t] = v;
 }
 
@@ -436,7 +436,7 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
     // thread, larger ones 20.
     constexpr int kChunk = CAP - 4;  // offsets per chunk (room for the shift)
     for (int c0 = 0; c0 < noff;) {
-        int c1 = min(noff, c0 + kChunk);
+        int c1 = chunk_end(c0, noff, kChunk);
         if (n_runs > 0) {  // block-uniform
             int beyond = 0, next = INT_MAX;
             for (int r = lane; r < n_runs; r += 32) {

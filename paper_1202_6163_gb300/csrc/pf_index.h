@@ -38,4 +38,19 @@ PF_HD int perm_parts(int extras) { return extras / kPermPart + (extras % kPermPa
 // The end of the part that starts at rank s0 < extras.
 PF_HD int perm_part_end(int s0, int extras) { return s0 + (extras - s0 < kPermPart ? extras - s0 : kPermPart); }
 
+// ---------------------------------------------------------------------------
+// Runs and chunks of a tile's offsets (pf_assign.cuh), up to 2^31 - 1 of them in one tile.
+// ---------------------------------------------------------------------------
+// The end of the chunk of at most `chunk` offsets that starts at c0 < noff.
+PF_HD int chunk_end(int c0, int noff, int chunk) { return c0 + (noff - c0 < chunk ? noff - c0 : chunk); }
+
+// The pieces of four entries that thread t of `threads` stores of the `body` entries (a
+// multiple of four) behind the first `head` of a run.  Unsigned: the step past the end of a
+// run of 2^31 - 1 entries stays above every entry.
+struct FillPieces {
+    uint32_t x, end, step;
+    PF_HD FillPieces(int head, int body, int t, int threads)
+        : x((uint32_t)(head + 4 * t)), end((uint32_t)(head + body)), step(4u * (uint32_t)threads) {}
+};
+
 }  // namespace pf

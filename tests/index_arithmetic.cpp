@@ -132,10 +132,43 @@ static void permute_parts() {
     }
 }
 
+// ---------------------------------------------------------------------------
+// A tile's chunks and a run's pieces cover them once, up to the largest counts.
+// ---------------------------------------------------------------------------
+static void runs_and_chunks() {
+    for (int noff : {1, 10236, 10237, 70001, INT_MAX - 10237, INT_MAX - 10236, INT_MAX - 10235, INT_MAX}) {
+        for (int chunk : {10236, 8188, 2044}) {
+            int c0 = 0;
+            while (c0 < noff) {
+                const int c1 = pf::chunk_end(c0, noff, chunk);
+                REQUIRE(c1 > c0 && c1 - c0 <= chunk && c1 <= noff, "chunk [%d, %d) of %d", c0, c1, noff);
+                c0 = c1;
+            }
+        }
+    }
+    for (int threads : {32, 512})
+        for (int n : {0, 3, 4, 1283, 70001, INT_MAX - 2051, INT_MAX - 2047, INT_MAX - 1, INT_MAX})
+            for (int head = 0; head < 4 && head <= n; ++head) {
+                const int body = (n - head) & ~3;
+                long long pieces = 0;
+                for (int t = 0; t < threads; t += n > 1000000 && t + 3 < threads ? threads / 2 - 1 : 1) {
+                    uint32_t at = (uint32_t)head + 4u * (uint32_t)t;
+                    for (pf::FillPieces f(head, body, t, threads); f.x < f.end; f.x += f.step) {
+                        REQUIRE(f.x == at && f.x + 4 <= (uint32_t)(head + body), "run of %d: piece at %u", n, f.x);
+                        at += 4u * (uint32_t)threads;
+                        ++pieces;
+                    }
+                    REQUIRE(at >= (uint32_t)(head + body), "run of %d: thread %d ends at %u", n, t, at);
+                }
+                REQUIRE(n > 1000000 || 4 * pieces == body, "run of %d: %lld pieces", n, pieces);
+            }
+}
+
 int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!std::strcmp(what, "strata")) strata();
     else if (!std::strcmp(what, "permute_parts")) permute_parts();
+    else if (!std::strcmp(what, "runs_and_chunks")) runs_and_chunks();
     else return 2;
     return 0;
 }

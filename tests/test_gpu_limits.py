@@ -19,3 +19,15 @@ def test_permute_all_offspring_of_one_particle(P):
     pf.pf_permute(a, P, out)
     assert pf.pf_get_device_status() == pf.PF_OK
     assert bool(torch.equal(out[:P], a)) and int(out[P]) == -3
+
+
+@pytest.mark.parametrize("name", ["systematic", "stratified"])
+def test_one_particle_takes_every_offset(name):
+    """All other weights are zero: one run of P offspring from one tile."""
+    kept = 1234567890
+    lw = torch.full((P_MAX,), float("-inf"), device="cuda")
+    lw[kept] = 0.5
+    out = torch.full((P_MAX + 2,), -3, dtype=torch.int32, device="cuda")
+    getattr(pf, "pf_resample_" + name)(lw, P_MAX, 0, 3, out[1:])
+    assert pf.pf_get_device_status() == pf.PF_OK
+    assert bool((out[1:-1] == kept).all()) and int(out[0]) == -3 and int(out[-1]) == -3
