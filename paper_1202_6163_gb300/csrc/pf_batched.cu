@@ -151,7 +151,7 @@ template <int KIND, int KK>
 __device__ __forceinline__ void one_tile_filter(const BatchParams& bp, const SortedParams& p, BatchShared& sm, int lead,
                                                 int n, int32_t* stage, int ticket) {
     TileThread th;
-    const TileSummary ts = tile_scan_k<KK>(p.lw, lead, n, sm.tile, th);
+    const TileSummary ts = tile_scan_k<KK, false, kReadOnly>(p.lw, lead, n, sm.tile, th);
     trace_stamp(bp.trace, bp.trace_cap, ticket, 1);
     trace_stamp(bp.trace, bp.trace_cap, ticket, 2);
     if (ts.bad || ts.total <= 0) {
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 const int64_t t0 = (int64_t)c * kTileMax;
                 const int n = (int)min((int64_t)kTileMax, PA - t0);
                 if (c + 1 < Tf) prefetch_tile(p.lw + t0 + kTileMax, (int)min((int64_t)kTileMax, PA - t0 - kTileMax));
-                ts = tile_scan(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
+                ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
                 bad |= ts.bad;
                 if (tid == 0) {
                     sm.rk[c] = ts.k;
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             // ---- systematic / stratified: one tile (a one-tile filter is its own item) ----
             const int c = c_item == kWhole ? 0 : c_item;
             const int64_t t0 = (int64_t)c * kTileMax;
-            TileSummary ts = tile_scan(p.lw + t0, c == 0 ? lead : 0, (int)min((int64_t)kTileMax, PA - t0), sm.tile, th);
+            TileSummary ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, (int)min((int64_t)kTileMax, PA - t0), sm.tile, th);
             uint32_t* rec = reinterpret_cast<uint32_t*>(bp.records + (ticket - c));  // the filter's Tf records
             uint32_t* arrive = bp.counters + 2 * f;
             if (tid == 0) {
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
         for (int c = 0; c < Tf; ++c) {
             const int64_t t0 = (int64_t)c * kTileMax;
             const int n = (int)min((int64_t)kTileMax, PA - t0);
-            ts = tile_scan(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
+            ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
             bad |= ts.bad;
             if (tid == 0) {
                 sm.rk[c] = ts.k;
@@ -463,27 +463,16 @@ size_t batched_scratch_floats_per_cta() { return (size_t)kMaxOwnB * kTileMax; }
 // filters get no item; a negative size or a filter beyond kMaxOwnB tiles sets
 // PF_ERR_INVALID and gets none.  The item count goes to ctl[CTL_ITEMS].
 constexpr int kPlanThreads = 1024;
-__global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __restrict__ lw,
-                                                               const int64_t* __restrict__ offsets, int F,
-                                                               const int32_t* __restrict__ mask, int split,
-                                                               int32_t* __restrict__ items, uint32_t* ctl, int metro,
-                                                               int split_min) {
+__global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* lw, const int64_t* offsets, int F,
+                                                               const int32_t* mask, int split, int32_t* items,
+                                                               uint32_t* ctl, int metro, int split_min) {
     __shared__ int count[kMaxOwnB + 1], start[kMaxOwnB + 1], split_sm;
     grid_begin();
     const int tid = threadIdx.x;
-    if (tid <= kMaxOwnB) count[tid] = 0;
-    if (metro) {
-        // Metropolis: a new launch epoch, and an empty list of shared filters after the items
-        if (tid == 0) {
-            ctl[CTL_METRO_EPOCH] += 1u;
-            ctl[CTL_HEAVY] = 0u;
-        }
-        for (int i = tid; i < min(F, kMaxHeavy); i += kPlanThreads) items[F + i] = 0;
-    }
-    __syncthreads();
     auto tiles = [&](int f) -> int {  // 0: no item
-        if (mask && mask[f] == 0) return 0;
+        const int32_t chosen = mask ? mask[f] : 1;
         const int64_t off0 = offsets[f], n = offsets[f + 1] - off0;
+        if (chosen == 0) return 0;
         if (n <= 0) {
             if (n < 0) set_status(ctl + CTL_STATUS, ST_INVALID);
             return 0;
@@ -496,8 +485,19 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __re
         }
         return (int)T;
     };
+    const int first = tid < F ? tiles(tid) : 0;  // on its way before the barrier, and used twice
+    if (tid <= kMaxOwnB) count[tid] = 0;
+    if (metro) {
+        // Metropolis: a new launch epoch, and an empty list of shared filters after the items
+        if (tid == 0) {
+            ctl[CTL_METRO_EPOCH] += 1u;
+            ctl[CTL_HEAVY] = 0u;
+        }
+        for (int i = tid; i < min(F, kMaxHeavy); i += kPlanThreads) items[F + i] = 0;
+    }
+    __syncthreads();
     for (int f = tid; f < F; f += kPlanThreads) {
-        const int T = tiles(f);
+        const int T = f == tid ? first : tiles(f);
         if (T) atomicAdd(&count[T], 1);
     }
     __syncthreads();
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* __re
     __syncthreads();
     const int sp = split_sm;
     for (int f = tid; f < F; f += kPlanThreads) {
-        const int T = tiles(f);
+        const int T = f == tid ? first : tiles(f);
         if (!T) continue;
         const int per = sp && T > 1 ? T : 1;
         const int at = atomicAdd(&start[T], per);

@@ -194,7 +194,10 @@ __device__ __forceinline__ float fixed48_to_float(long long v) {
 }
 
 // First statement of a kernel launched by launch_overlapped, in every thread and before any
-// access to global memory: waits for the work before this grid.  A grid of few CTAs
+// access to global memory: waits for the work before this grid.  The kernel may be resident
+// while that work still writes, so nothing it reads counts as read-only for its lifetime: no
+// load through the read-only path (__ldg, ld.global.nc), and no const __restrict__ pointer, which
+// lets the compiler choose that path (ld_input).  A grid of few CTAs
 // first lets the next such launch take its place on the GPU; a larger one leaves that
 // to its CTAs' exits, as a grid placed beside another that fills the SMs is spread
 // unevenly over them (Metropolis at P = 65536: 17 us, 36 with the early start).
@@ -262,6 +265,16 @@ __device__ __forceinline__ void ld_cg_v2(const uint64_t* p, uint64_t& a, uint64_
 
 __device__ __forceinline__ void st_v2(uint64_t* p, uint64_t a, uint64_t b) {
     asm volatile("st.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+
+// Reads of what earlier work on the stream may have written: log-weights, ancestors.
+// kReadOnly, by the read-only path, which the compiler may move past stores and barriers: only
+// in kernels launched the ordinary way, which start after that work.
+constexpr bool kReadOnly = true;
+template <bool RO = false, typename T>
+__device__ __forceinline__ T ld_input(const T* p) {
+    if constexpr (RO) return __ldg(p);
+    return *p;
 }
 
 // The same as relaxed accesses at GPU scope (records another CTA polls).

@@ -138,7 +138,7 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
         uint2 r[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u)
-            r[u] = t0 + u * kThreads < t_hi ? __ldg(reinterpret_cast<const uint2*>(rec + t0 + u * kThreads))
+            r[u] = t0 + u * kThreads < t_hi ? *reinterpret_cast<const uint2*>(rec + t0 + u * kThreads)
                                             : make_uint2(0u, 0u);
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
@@ -163,7 +163,7 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
             uint4 r[kBatch];
 #pragma unroll
             for (int u = 0; u < kBatch; ++u)
-                r[u] = t0 + u * kThreads < t_hi ? __ldg(rec + t0 + u * kThreads) : make_uint4(0u, 0u, 0u, 0u);
+                r[u] = t0 + u * kThreads < t_hi ? rec[t0 + u * kThreads] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int u = 0; u < kBatch; ++u)
                 if (t0 + u * kThreads < t_hi) run += record_mass(r[u], K);
@@ -205,7 +205,7 @@ __global__ void __cluster_dims__(kCarryCtas) __launch_bounds__(kThreads)
     const float u = kMapKind == KIND_SYS ? offset_uniform(pm) : 0.f;
     for (int t0 = t_lo; t0 < t_hi; t0 += kThreads) {
         const int t = t0 + tid;
-        const uint4 r = t < t_hi ? __ldg(rec + t) : make_uint4(0u, 0u, 0u, 0xffffffffu);
+        const uint4 r = t < t_hi ? rec[t] : make_uint4(0u, 0u, 0u, 0xffffffffu);
         const i128 mine = t < t_hi ? record_mass(r, K) : (i128)0;
         const i128 inc = warp_scan_i128(mine, lane);
         if (lane == 31) wsum[warp] = inc;

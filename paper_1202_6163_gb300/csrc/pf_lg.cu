@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kLgThreads) k_lg_step(LgParams p) {
     const int D = 4 * G;
     const int64_t base = (int64_t)f * p.P;
     const int rf = __ldcg(p.resample + f);
-    const float a = __ldg(p.a + f);
+    const float a = p.a[f];
     const float* yf = p.y + (int64_t)f * D;
     const uint32_t c1 = p.t * (uint32_t)G;
 

@@ -99,18 +99,29 @@ __device__ __forceinline__ void draw_steps(const ChainStream<ROUNDS>& rng, int b
     }
 }
 
+// A log-weight read at random.  Where the read-only path is closed (ld_input) the load stays
+// where it is written: moved about by the compiler, the chain's loads took seven registers
+// more, and with them a quarter of the resident warps.
+template <bool RO>
+__device__ __forceinline__ float read_logw(const float* p) {
+    if constexpr (RO) return ld_input<true>(p);
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 // B steps of a chain from state (k, lk).  The proposals do not depend on the
 // chain's state, so each group of kAhead steps draws its proposals first and
 // issues all their log-weight loads before resolving the steps in order.
-template <int ROUNDS>
-__device__ __forceinline__ void run_chain(const float* __restrict__ lw, uint32_t Pu, const ChainStream<ROUNDS>& rng,
+template <int ROUNDS, bool RO>
+__device__ __forceinline__ void run_chain(const float* lw, uint32_t Pu, const ChainStream<ROUNDS>& rng,
                                           int steps, uint32_t& k, float& lk) {
     for (int b0 = 0; b0 < steps; b0 += kAhead) {
         uint32_t jj[kAhead];
         float uu[kAhead], ll[kAhead];
         draw_steps(rng, b0, Pu, jj, uu);
 #pragma unroll
-        for (int s = 0; s < kAhead; ++s) ll[s] = __ldg(lw + jj[s]);
+        for (int s = 0; s < kAhead; ++s) ll[s] = read_logw<RO>(lw + jj[s]);
 #pragma unroll
         for (int s = 0; s < kAhead; ++s) {
             if (b0 + s < steps && metropolis_accept(ll[s], lk, uu[s])) {
@@ -141,15 +152,15 @@ struct StagedWeights {
 // relative, five times over), and the log-weights where it is not.
 constexpr float kTieBand = 4e-6f;
 
-template <int ROUNDS, bool CLEAN, bool SPLIT>
-__device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const StagedWeights& sw, uint32_t Pu,
+template <int ROUNDS, bool CLEAN, bool SPLIT, bool RO>
+__device__ __forceinline__ void run_chain_w(const float* lw, const StagedWeights& sw, uint32_t Pu,
                                             const ChainStream<ROUNDS>& rng, int steps, uint32_t& k) {
     float wk = sw.at<SPLIT>(k);
     auto step = [&](uint32_t j, float u, float wj) {
         const float t = __fmul_rn(u, wk);
         bool acc = t < wj;
         if ((!CLEAN && !(wk >= kWeightFloor)) || (SPLIT && fabsf(__fsub_rn(t, wj)) <= kTieBand * wj))
-            acc = metropolis_accept(__ldg(lw + j), __ldg(lw + k), u);
+            acc = metropolis_accept(ld_input<RO>(lw + j), ld_input<RO>(lw + k), u);
         if (acc) {
             k = j;
             wk = wj;
@@ -174,34 +185,34 @@ __device__ __forceinline__ void run_chain_w(const float* __restrict__ lw, const 
 }
 
 // Chain i of a filter with staged weights, written to anc[i].
-template <int ROUNDS, bool SPLIT>
+template <int ROUNDS, bool SPLIT, bool RO>
 __device__ __forceinline__ void run_staged(const float* lw, const StagedWeights& sw, bool clean, uint32_t Pu, uint32_t i,
                                            int steps, uint32_t filter, uint32_t key0, uint32_t key1,
                                            ChainStream<ROUNDS>& rng, int32_t* anc) {
     uint32_t k = i;
     rng.set_chain(i, filter, key0, key1);
-    if (clean) run_chain_w<ROUNDS, true, SPLIT>(lw, sw, Pu, rng, steps, k);
-    else run_chain_w<ROUNDS, false, SPLIT>(lw, sw, Pu, rng, steps, k);
+    if (clean) run_chain_w<ROUNDS, true, SPLIT, RO>(lw, sw, Pu, rng, steps, k);
+    else run_chain_w<ROUNDS, false, SPLIT, RO>(lw, sw, Pu, rng, steps, k);
     anc[i] = (int32_t)k;
 }
 
-template <int ROUNDS>
-__device__ __forceinline__ void run_unstaged(const float* __restrict__ lw, uint32_t Pu, uint32_t i, int steps,
+template <int ROUNDS, bool RO>
+__device__ __forceinline__ void run_unstaged(const float* lw, uint32_t Pu, uint32_t i, int steps,
                                              uint32_t filter, uint32_t key0, uint32_t key1, ChainStream<ROUNDS>& rng,
                                              int32_t* anc, uint32_t* ctl) {
     uint32_t k = i;
-    float lk = __ldg(lw + i);
+    float lk = read_logw<RO>(lw + i);
     if (!(lk <= 3.402823466e38f)) set_status(ctl + CTL_STATUS, ST_DOMAIN);  // NaN or +inf
     rng.set_chain(i, filter, key0, key1);
-    run_chain<ROUNDS>(lw, Pu, rng, steps, k, lk);
+    run_chain<ROUNDS, RO>(lw, Pu, rng, steps, k, lk);
     anc[i] = (int32_t)k;
 }
 
 // Block-wide: copy lw[0..n) as weights exp(lw - m), m = max lw (0 when every weight is
 // zero), to shared memory and, from sw.held on, to sw.rest; records PF_ERR_DOMAIN
 // for a NaN or +inf log-weight.  Returns whether every weight is at least kWeightFloor.
-template <int THREADS>
-__device__ bool stage_weights(const float* __restrict__ lw, int64_t n, const StagedWeights& sw, float* red,
+template <int THREADS, bool RO>
+__device__ bool stage_weights(const float* lw, int64_t n, const StagedWeights& sw, float* red,
                               uint32_t* ctl) {
     const int tid = threadIdx.x;
     const int64_t ns = n < (int64_t)sw.held ? n : (int64_t)sw.held;  // those held in shared memory
@@ -212,20 +223,37 @@ __device__ bool stage_weights(const float* __restrict__ lw, int64_t n, const Sta
         bad |= !(x <= 3.402823466e38f);
     };
     const int64_t n4 = (((uintptr_t)lw) & 15u) == 0 ? ns >> 2 : 0;
-    for (int64_t q = tid; q < n4; q += THREADS) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(lw) + q);
-        reinterpret_cast<float4*>(sw.w)[q] = v;
-        see(v.x);
-        see(v.y);
-        see(v.z);
-        see(v.w);
+    constexpr int kBatch = RO ? 1 : 4;  // reads in flight per thread (RO: as many as the compiler sees fit)
+    for (int64_t q0 = tid; q0 < n4; q0 += kBatch * THREADS) {
+        float4 v[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+            if (q0 + u * THREADS < n4) v[u] = ld_input<RO>(reinterpret_cast<const float4*>(lw) + q0 + u * THREADS);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (q0 + u * THREADS < n4) {
+                reinterpret_cast<float4*>(sw.w)[q0 + u * THREADS] = v[u];
+                see(v[u].x);
+                see(v[u].y);
+                see(v[u].z);
+                see(v[u].w);
+            }
+        }
     }
-    for (int64_t q = 4 * n4 + tid; q < ns; q += THREADS) {
-        const float x = __ldg(lw + q);
-        sw.w[q] = x;
-        see(x);
+    for (int64_t q0 = 4 * n4 + tid; q0 < ns; q0 += kBatch * THREADS) {
+        float x[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+            if (q0 + u * THREADS < ns) x[u] = ld_input<RO>(lw + q0 + u * THREADS);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (q0 + u * THREADS < ns) {
+                sw.w[q0 + u * THREADS] = x[u];
+                see(x[u]);
+            }
+        }
     }
-    for (int64_t q = ns + tid; q < n; q += THREADS) see(__ldg(lw + q));
+    for (int64_t q = ns + tid; q < n; q += THREADS) see(ld_input<RO>(lw + q));
     m = warp_max(m);
     if ((tid & 31) == 0) red[tid >> 5] = m;
     bad = __syncthreads_or(bad);
@@ -234,18 +262,17 @@ __device__ bool stage_weights(const float* __restrict__ lw, int64_t n, const Sta
 #pragma unroll
     for (int q = 1; q < THREADS / 32; ++q) mt = fmaxf(mt, red[q]);
     const fpair R = {mt > -INFINITY ? mt : 0.f, 0.f};
-    bool clean = true;
-    for (int64_t q = tid; q < ns; q += THREADS) {
-        const float x = weight_rel(sw.w[q], R);
-        sw.w[q] = x;
-        clean = clean && x >= kWeightFloor;
+    float least = INFINITY;
+    for (int q = tid; q < (int)(ns >> 2); q += THREADS) {
+        float4 x = reinterpret_cast<const float4*>(sw.w)[q];
+        x = make_float4(weight_rel(x.x, R), weight_rel(x.y, R), weight_rel(x.z, R), weight_rel(x.w, R));
+        reinterpret_cast<float4*>(sw.w)[q] = x;
+        least = fminf(least, fminf(fminf(x.x, x.y), fminf(x.z, x.w)));
     }
-    for (int64_t q = ns + tid; q < n; q += THREADS) {
-        const float x = weight_rel(__ldg(lw + q), R);
-        sw.rest[q - ns] = x;
-        clean = clean && x >= kWeightFloor;
-    }
-    return __syncthreads_and(clean) != 0;
+    for (int q = (int)(ns & ~(int64_t)3) + tid; q < (int)ns; q += THREADS)
+        least = fminf(least, sw.w[q] = weight_rel(sw.w[q], R));
+    for (int64_t q = ns + tid; q < n; q += THREADS) least = fminf(least, sw.rest[q - ns] = weight_rel(ld_input<RO>(lw + q), R));
+    return __syncthreads_and(least >= kWeightFloor) != 0;
 }
 
 // Block-wide: the largest normalised weight w_max = max_i w_i / sum_i w_i of
@@ -254,7 +281,7 @@ __device__ bool stage_weights(const float* __restrict__ lw, int64_t n, const Sta
 // pass of running (max, sum) pairs, rescaled as the maximum grows).  Returns
 // 0 when every weight is zero.  red: THREADS/32 floats of shared memory.
 template <int THREADS, bool STAGED>
-__device__ float largest_weight(const float* __restrict__ lw, const float* w, int64_t n, float* red) {
+__device__ float largest_weight(const float* lw, const float* w, int64_t n, float* red) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float m = -INFINITY, sum = 0.f, c = 0.f;
     for (int64_t q = tid; q < n; q += THREADS) {
@@ -264,7 +291,7 @@ __device__ float largest_weight(const float* __restrict__ lw, const float* w, in
             c = __fsub_rn(__fsub_rn(t, sum), y);
             sum = t;
         } else {
-            const float x = __ldg(lw + q);
+            const float x = ld_input<kReadOnly>(lw + q);
             if (x > m) {
                 sum = (m > -INFINITY ? sum * expf(m - x) : 0.f) + 1.f;
                 m = x;
@@ -320,23 +347,22 @@ __device__ uint32_t bound_B(int64_t P, double w_max, double eps, uint32_t cap) {
 }
 
 template <bool STAGED, int ROUNDS>
-__global__ void __launch_bounds__(kMetroThreads) k_metropolis(const float* __restrict__ lw, int64_t P, int B,
-                                                              const uint32_t* __restrict__ B_dev, uint32_t key0,
-                                                              uint32_t key1, uint32_t filter,
-                                                              int32_t* __restrict__ anc, uint32_t* ctl) {
+__global__ void __launch_bounds__(kMetroThreads) k_metropolis(const float* lw, int64_t P, int B,
+                                                              const uint32_t* B_dev, uint32_t key0, uint32_t key1,
+                                                              uint32_t filter, int32_t* anc, uint32_t* ctl) {
     extern __shared__ float wsm[];
     __shared__ float red[kMetroThreads / 32];
     grid_begin();
     bool clean = false;
     const StagedWeights sw = {wsm, nullptr, 0xffffffffu};
-    if (STAGED) clean = stage_weights<kMetroThreads>(lw, P, sw, red, ctl);  // every CTA: the whole vector
-    const int steps = B_dev ? (int)__ldg(B_dev) : B;
+    if (STAGED) clean = stage_weights<kMetroThreads, false>(lw, P, sw, red, ctl);  // every CTA: the whole vector
+    const int steps = B_dev ? (int)*B_dev : B;
     const uint32_t Pu = (uint32_t)P;
     ChainStream<ROUNDS> rng;
     rng.set_key(key0, key1);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (int64_t)gridDim.x * blockDim.x) {
-        if (STAGED) run_staged<ROUNDS, false>(lw, sw, clean, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc);
-        else run_unstaged<ROUNDS>(lw, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc, ctl);
+        if (STAGED) run_staged<ROUNDS, false, false>(lw, sw, clean, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc);
+        else run_unstaged<ROUNDS, false>(lw, Pu, (uint32_t)i, steps, filter, key0, key1, rng, anc, ctl);
     }
 }
 
@@ -434,9 +460,9 @@ __device__ __forceinline__ void run_batched_chain(const BatchParams& bp, const f
                                                   int steps, int f, uint32_t key0, uint32_t key1,
                                                   ChainStream<ROUNDS>& rng) {
     int32_t* anc = bp.anc + off0;
-    if (where == kAllStaged) run_staged<ROUNDS, false>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
-    else if (where == kSplit) run_staged<ROUNDS, true>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
-    else run_unstaged<ROUNDS>(lw, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc, bp.ctl);
+    if (where == kAllStaged) run_staged<ROUNDS, false, kReadOnly>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
+    else if (where == kSplit) run_staged<ROUNDS, true, kReadOnly>(lw, sw, clean, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc);
+    else run_unstaged<ROUNDS, kReadOnly>(lw, Pu, i, steps, (uint32_t)f, key0, key1, rng, anc, bp.ctl);
 }
 
 // The chains of blocks claimed from filter f (block-wide; the weights are staged).
@@ -493,7 +519,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             trace_put(bp.trace, bp.trace_cap, ticket, 7, (uint64_t)(bp.items[ticket] & 31));
         }
         bool clean = false;
-        if (where != kUnstaged) clean = stage_weights<kMetroBThreads>(lw, Pf, sw, red, bp.ctl);
+        if (where != kUnstaged) clean = stage_weights<kMetroBThreads, kReadOnly>(lw, Pf, sw, red, bp.ctl);
         for (int w = 1; w <= 2; ++w) trace_stamp(bp.trace, bp.trace_cap, ticket, w);
         // B < 0: this filter's own step count from Eq. 5 and its largest normalised weight
         int steps = bp.B;
@@ -571,7 +597,7 @@ __global__ void __launch_bounds__(kMetroBThreads) k_batched_metropolis(BatchPara
             const float* lw = bp.lw + off0;
             const WeightsAt where = weights_at(Pf);
             bool clean = false;
-            if (where != kUnstaged) clean = stage_weights<kMetroBThreads>(lw, Pf, sw, red, bp.ctl);
+            if (where != kUnstaged) clean = stage_weights<kMetroBThreads, kReadOnly>(lw, Pf, sw, red, bp.ctl);
             const uint64_t seed = bp.seeds[f];
             const uint32_t key0 = (uint32_t)(seed & 0xffffffffu), key1 = (uint32_t)(seed >> 32);
             rng.set_key(key0, key1);

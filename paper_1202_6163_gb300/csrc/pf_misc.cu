@@ -25,9 +25,8 @@ constexpr int kGatherWave = 8;        // resident CTAs per SM of one wave
 constexpr int kGatherFullGrid = 40;   // CTAs per SM from which the grid is not cut to a wave
 
 template <typename VT, int U, bool POW2>
-__global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict__ src, int64_t P_src, RowSplit split,
-                                                           const int32_t* __restrict__ anc, int64_t total,
-                                                           VT* __restrict__ dst, uint32_t* ctl) {
+__global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_t P_src, RowSplit split,
+                                                           const int32_t* anc, int64_t total, VT* dst, uint32_t* ctl) {
     grid_begin();
     const int64_t stride = (int64_t)gridDim.x * (kGatherThreads * U);
     int64_t base = (int64_t)blockIdx.x * (kGatherThreads * U) + threadIdx.x;
@@ -39,7 +38,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict_
             const int64_t i = b + u * kGatherThreads;
             e[u] = 0;
             at[u] = 0;
-            if (i < total) e[u] = __ldg(anc + split.row<POW2>(i, at[u]));
+            if (i < total) e[u] = anc[split.row<POW2>(i, at[u])];
         }
     };
     ancestors(base, a, c);
@@ -48,15 +47,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict_
         bool ok[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            ok[u] = base + u * kGatherThreads < total;
-            if (ok[u]) {
-                if (a[u] >= 0 && a[u] < P_src) {
-                    v[u] = load_chunk_nc(src + (int64_t)a[u] * split.vecs + c[u]);
-                } else {
-                    ok[u] = false;
-                    if (c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
-                }
-            }
+            ok[u] = base + u * kGatherThreads < total && a[u] >= 0 && a[u] < P_src;
+            if (ok[u]) v[u] = load_chunk(src + (int64_t)a[u] * split.vecs + c[u]);
         }
         int32_t an[U];
         uint32_t cn[U];
@@ -64,6 +56,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* __restrict_
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (ok[u]) store_chunk_cs(dst + base + u * kGatherThreads, v[u]);
+            else if (base + u * kGatherThreads < total && c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
             a[u] = an[u];
             c[u] = cn[u];
         }
@@ -125,7 +118,7 @@ __device__ __forceinline__ i128 shfl_xor_i128(i128 v, int o) {
     return (i128)(((unsigned __int128)h2 << 64) | l2);
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_reduce(const float* __restrict__ lw, int64_t P, RedRecord* rec,
+__global__ void __launch_bounds__(kRedThreads) k_reduce(const float* lw, int64_t P, RedRecord* rec,
                                                         uint32_t* ctl, float* ess_out, double* log_sum_out,
                                                         uint32_t* B_out, double eps, uint32_t B_cap) {
     __shared__ float rm[kRedThreads / 32];
@@ -146,14 +139,14 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const float* __restrict_
         // coalesced: thread tid reads vector q*kRedThreads + tid
         const int e = 4 * (q * kRedThreads + tid);
         if (e + 3 < n) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(base + e));
+            const float4 v = *reinterpret_cast<const float4*>(base + e);
             x[4 * q] = v.x;
             x[4 * q + 1] = v.y;
             x[4 * q + 2] = v.z;
             x[4 * q + 3] = v.w;
         } else {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) x[4 * q + r] = (e + r < n) ? __ldg(base + e + r) : -INFINITY;
+            for (int r = 0; r < 4; ++r) x[4 * q + r] = (e + r < n) ? base[e + r] : -INFINITY;
         }
     }
     float m = -INFINITY;

@@ -42,8 +42,7 @@ constexpr int kPermWarps = kPermThreads / 32;
 
 // One count per ancestor.  A warp takes four rows of 32 consecutive entries; the
 // first lane of each run of equal entries in a row adds the run's length.
-__global__ void __launch_bounds__(256) k_perm_count(const int32_t* __restrict__ anc, int64_t P,
-                                                    int32_t* __restrict__ o, uint32_t* ctl) {
+__global__ void __launch_bounds__(256) k_perm_count(const int32_t* anc, int64_t P, int32_t* o, uint32_t* ctl) {
     grid_begin();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -52,8 +51,11 @@ __global__ void __launch_bounds__(256) k_perm_count(const int32_t* __restrict__ 
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int64_t j = j0 + 32 * r + lane;
-            a[r] = j < P ? __ldg(anc + j) : INT_MIN;  // INT_MIN: past the end, counted nowhere
-            if (j < P && (a[r] < 0 || a[r] >= P)) {
+            a[r] = j < P ? anc[j] : INT_MIN;  // INT_MIN: past the end, counted nowhere
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (j0 + 32 * r + lane < P && (a[r] < 0 || a[r] >= P)) {
                 set_status(ctl + CTL_STATUS, ST_INVALID);
                 a[r] = INT_MIN;
             }
@@ -95,11 +97,11 @@ __device__ __forceinline__ int block_excl_scan(int x, int* red, int& total) {
 }
 
 // This thread's kPermPer counts of its tile (1 past the end: neither extra nor empty).
-__device__ __forceinline__ void load_counts(const int32_t* __restrict__ o, int64_t i0, int64_t P, int (&c)[kPermPer]) {
+__device__ __forceinline__ void load_counts(const int32_t* o, int64_t i0, int64_t P, int (&c)[kPermPer]) {
     if (i0 + kPermPer <= P) {  // the counts start on a 256-byte boundary
 #pragma unroll
         for (int q = 0; q < kPermPer / 4; ++q) {
-            const int4 v = __ldg(reinterpret_cast<const int4*>(o + i0) + q);
+            const int4 v = reinterpret_cast<const int4*>(o + i0)[q];
             c[4 * q] = v.x;
             c[4 * q + 1] = v.y;
             c[4 * q + 2] = v.z;
@@ -107,7 +109,7 @@ __device__ __forceinline__ void load_counts(const int32_t* __restrict__ o, int64
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < kPermPer; ++k) c[k] = i0 + k < P ? __ldg(o + i0 + k) : 1;
+        for (int k = 0; k < kPermPer; ++k) c[k] = i0 + k < P ? o[i0 + k] : 1;
     }
 }
 
@@ -117,8 +119,8 @@ struct TilePrefix {
 };
 
 // Tile sums; the last CTA to finish turns them into exclusive prefixes, pre[T] holding the totals.
-__global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* __restrict__ o, int64_t P,
-                                                             TilePrefix* __restrict__ pre, int T, uint32_t* ctl) {
+__global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* o, int64_t P, TilePrefix* pre, int T,
+                                                             uint32_t* ctl) {
     __shared__ int red[kPermWarps];
     __shared__ int last;
     grid_begin();
@@ -161,9 +163,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* __re
 
 // Lists the extra copies: E[r], r < extras, in increasing particle order.  CTA b is
 // part b of the listing: part pt of tile t, ranks [pt kPermPart, ...) of the tile's.
-__global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __restrict__ o, int64_t P,
-                                                            const TilePrefix* __restrict__ pre, int T,
-                                                            int32_t* __restrict__ E) {
+__global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* o, int64_t P, const TilePrefix* pre, int T,
+                                                            int32_t* E) {
     __shared__ int red[kPermWarps];
     __shared__ __align__(16) int32_t mark[kPermPart + 4];
     grid_begin();
@@ -172,13 +173,13 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __res
         int lo = 0, hi = T - 1;  // the last tile with pre.part <= b
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(&pre[mid].part) <= b) lo = mid;
+            if (pre[mid].part <= b) lo = mid;
             else hi = mid - 1;
         }
         const int t = lo;
-        const int s0 = (b - __ldg(&pre[t].part)) * kPermPart;  // this part's ranks within the tile:
-        const int s1 = perm_part_end(s0, __ldg(&pre[t + 1].extra) - __ldg(&pre[t].extra));  // [s0, s1)
-        int32_t* out = E + __ldg(&pre[t].extra) + s0;
+        const int s0 = (b - pre[t].part) * kPermPart;  // this part's ranks within the tile:
+        const int s1 = perm_part_end(s0, pre[t + 1].extra - pre[t].extra);  // [s0, s1)
+        int32_t* out = E + pre[t].extra + s0;
         const int shift = (int)(((uintptr_t)out >> 2) & 3u);  // to a 16-byte boundary
         const int end = s1 - s0 + shift;
         for (int i = 4 * tid; i < end; i += 4 * kPermThreads)
@@ -239,9 +240,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_list(const int32_t* __res
 }
 
 // The result: a particle with offspring keeps its slot, the empty slots take E in order.
-__global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __restrict__ o, int64_t P,
-                                                            const TilePrefix* __restrict__ pre,
-                                                            const int32_t* __restrict__ E, int32_t* __restrict__ out) {
+__global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* o, int64_t P, const TilePrefix* pre,
+                                                            const int32_t* E, int32_t* out) {
     __shared__ int red[kPermWarps];
     grid_begin();
     const int64_t i0 = (int64_t)blockIdx.x * kPermTile + (int64_t)threadIdx.x * kPermPer;
@@ -250,10 +250,10 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_fill(const int32_t* __res
     int d = 0, td;
 #pragma unroll
     for (int k = 0; k < kPermPer; ++k) d += c[k] == 0;
-    const int32_t* src = E + __ldg(&pre[blockIdx.x].dead) + block_excl_scan(d, red, td);  // ranks below P: inside E
+    const int32_t* src = E + pre[blockIdx.x].dead + block_excl_scan(d, red, td);  // ranks below P: inside E
     int v[kPermPer];
 #pragma unroll
-    for (int k = 0; k < kPermPer; ++k) v[k] = c[k] == 0 ? __ldg(src++) : (int)(i0 + k);
+    for (int k = 0; k < kPermPer; ++k) v[k] = c[k] == 0 ? *src++ : (int)(i0 + k);
     if (i0 + kPermPer <= P && (((uintptr_t)out) & 15u) == 0) {
 #pragma unroll
         for (int q = 0; q < kPermPer / 4; ++q)
@@ -278,8 +278,8 @@ constexpr int kPermSmallPer = kPermSmall / kPermSmallThreads;
 constexpr int perm_small_at(int i) { return i + (i >> 5); }
 constexpr size_t kPermSmallSmem = 2 * (size_t)(perm_small_at(kPermSmall)) * sizeof(int32_t);
 
-__global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t* __restrict__ anc, int P,
-                                                                  int32_t* __restrict__ out, uint32_t* ctl) {
+__global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t* anc, int P, int32_t* out,
+                                                                  uint32_t* ctl) {
     extern __shared__ int32_t perm_smem[];
     __shared__ int red[32];
     int32_t* o = perm_smem;
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t*
     // counts: one addition per run of equal neighbours in a row of 32 (as k_perm_count)
     for (int j0 = 32 * warp; j0 < P; j0 += kPermSmallThreads) {
         const int j = j0 + lane;
-        int32_t a = j < P ? __ldg(anc + j) : INT_MIN;
+        int32_t a = j < P ? anc[j] : INT_MIN;
         if (j < P && (a < 0 || a >= P)) {
             set_status(ctl + CTL_STATUS, ST_INVALID);
             a = INT_MIN;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t*
 // resident wave with the early entries: 27, 47, 67, 53.
 template <typename VT, int U, bool POW2>
 __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSplit split,
-                                                        const int32_t* __restrict__ perm, uint32_t* ctl) {
+                                                        const int32_t* perm, uint32_t* ctl) {
     grid_begin();
     const int64_t total = P * split.vecs;
     const int64_t stride = (int64_t)gridDim.x * (256 * U);
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
             const int64_t i = b + u * 256;
             e[u] = -1;
             at[u] = 0;
-            if (i < total) e[u] = __ldg(perm + split.row<POW2>(i, at[u]));
+            if (i < total) e[u] = perm[split.row<POW2>(i, at[u])];
         }
     };
     entries(base, a, c);
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
             move[u] = i < total && a[u] != (int32_t)split.row<POW2>(i, cc);
             own[u] = -1;
             if (move[u] && a[u] >= 0 && a[u] < P) {
-                own[u] = __ldg(perm + a[u]);
-                v[u] = load_chunk(x + (int64_t)a[u] * split.vecs + c[u]);
+                own[u] = perm[a[u]];
+                v[u] = load_chunk_cg(x + (int64_t)a[u] * split.vecs + c[u]);
             }
         }
         int32_t an[U];

@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_persistent(SortedParams p) {
                 }
             }
         }
-        if (!staged) ts = tile_scan_k<KK>(p.lw + t0, t == 0 ? p.lead : 0, n, sm.tile, th);
+        if (!staged) ts = tile_scan_k<KK, false, kReadOnly>(p.lw + t0, t == 0 ? p.lead : 0, n, sm.tile, th);
         if (ts.bad && tid == 0) set_status(p.ctl + CTL_STATUS, ST_DOMAIN);
         skip |= (t == p.skip_tile);
         if (KIND == KIND_MULTI) {
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_one_tile(SortedParams p) {
     const int64_t PA = p.P + p.lead, t0 = (int64_t)t * p.tile;
     TileThread th;
     const TileSummary ts =
-        tile_scan_k<KK>(p.lw + t0, t == 0 ? p.lead : 0, (int)min((int64_t)p.tile, PA - t0), sm.tile, th);
+        tile_scan_k<KK, false, kReadOnly>(p.lw + t0, t == 0 ? p.lead : 0, (int)min((int64_t)p.tile, PA - t0), sm.tile, th);
     const uint64_t tag = (uint64_t)epoch << 32;
     if (tid == 0 && t != p.skip_tile) {
         uint64_t* rec = p.tagged + kTaggedWords * t;

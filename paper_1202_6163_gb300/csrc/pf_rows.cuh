@@ -14,13 +14,13 @@ struct __align__(32) u32x8 {
 };
 
 template <typename VT>
-__device__ __forceinline__ VT load_chunk_nc(const VT* p) {  // read-only data
-    return __ldg(p);
+__device__ __forceinline__ VT load_chunk(const VT* p) {
+    return *p;
 }
 template <>
-__device__ __forceinline__ u32x8 load_chunk_nc<u32x8>(const u32x8* p) {
+__device__ __forceinline__ u32x8 load_chunk<u32x8>(const u32x8* p) {
     u32x8 v;
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
                    "=r"(v.w[7])
                  : "l"(p));
@@ -28,11 +28,11 @@ __device__ __forceinline__ u32x8 load_chunk_nc<u32x8>(const u32x8* p) {
 }
 
 template <typename VT>
-__device__ __forceinline__ VT load_chunk(const VT* p) {  // data other threads may be writing
+__device__ __forceinline__ VT load_chunk_cg(const VT* p) {  // data other threads may be writing
     return __ldcg(p);
 }
 template <>
-__device__ __forceinline__ u32x8 load_chunk<u32x8>(const u32x8* p) {
+__device__ __forceinline__ u32x8 load_chunk_cg<u32x8>(const u32x8* p) {
     u32x8 v;
     asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),

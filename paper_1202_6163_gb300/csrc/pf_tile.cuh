@@ -80,15 +80,15 @@ static_assert((kThreads / 4) % 8 == 0, "chunks a CTA apart have the same place")
 // Loads this thread's KK elements (tile-local e0 .. e0+KK) of base[lo..n);
 // base is 16-byte aligned in global memory, or (SMEM) a tile staged by stage_tile.
 // Slots outside [lo, n) read as -inf (zero weight).
-template <int KK, bool SMEM = false>
-__device__ __forceinline__ void tile_load_k(const float* __restrict__ base, int lo, int n, int e0,
+template <int KK, bool SMEM = false, bool RO = false>
+__device__ __forceinline__ void tile_load_k(const float* base, int lo, int n, int e0,
                                             float (&x)[kMaxPerThread]) {
     static_assert(!SMEM || KK == kMaxPerThread, "tiles are staged in full");
     if (e0 >= lo && e0 + KK <= n) {  // nearly every thread
 #pragma unroll
         for (int q = 0; q < KK / 4; ++q) {
             const float4 v = SMEM ? *reinterpret_cast<const float4*>(base + stage_place(threadIdx.x, q))
-                                  : __ldg(reinterpret_cast<const float4*>(base + e0 + 4 * q));
+                                  : ld_input<RO>(reinterpret_cast<const float4*>(base + e0 + 4 * q));
             x[4 * q + 0] = v.x;
             x[4 * q + 1] = v.y;
             x[4 * q + 2] = v.z;
@@ -99,7 +99,7 @@ __device__ __forceinline__ void tile_load_k(const float* __restrict__ base, int 
 #pragma unroll
     for (int i = 0; i < KK; ++i) {
         const float* src = SMEM ? base + stage_place(threadIdx.x, i >> 2) + (i & 3) : base + e0 + i;
-        x[i] = (e0 + i >= lo && e0 + i < n) ? (SMEM ? *src : __ldg(src)) : -INFINITY;
+        x[i] = (e0 + i >= lo && e0 + i < n) ? (SMEM ? *src : ld_input<RO>(src)) : -INFINITY;
     }
 }
 
@@ -112,9 +112,9 @@ __device__ __forceinline__ fpair tile_sum_pair(long long total) {
 // Block-wide; every thread of the CTA must call it.  Scans base[0..n) with the
 // first `lo` slots taken as zero weights; fills th (this thread's elements) and
 // returns the tile summary (identical in every thread, but S in thread 0 alone).
-// KK elements per thread (n <= KK * kThreads); tile_scan picks KK from n.
-template <int KK, bool SMEM = false>  // SMEM: base is a copy of the tile in shared memory
-__device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ base, int lo, int n, TileShared& sm,
+// KK elements per thread (n <= KK * kThreads); tile_scan picks KK from n.  RO: as ld_input.
+template <int KK, bool SMEM = false, bool RO = false>  // SMEM: base is a copy of the tile in shared memory
+__device__ __forceinline__ TileSummary tile_scan_k(const float* base, int lo, int n, TileShared& sm,
                                                    TileThread& th) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int e0 = tid * KK;
@@ -122,7 +122,7 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
     th.e0 = e0;
 
     float* x = th.v;
-    tile_load_k<KK, SMEM>(base, lo, n, e0, th.v);
+    tile_load_k<KK, SMEM, RO>(base, lo, n, e0, th.v);
 
     // 1. tile maximum and domain check: the maxima propagate NaN (which the
     // integer reduction places above +inf), so the tile's maximum alone tells
@@ -231,12 +231,13 @@ __device__ __forceinline__ TileSummary tile_scan_k(const float* __restrict__ bas
 }
 
 // Block-wide; KK from the tile length (4, 8 or 16 elements per thread).
-__device__ __forceinline__ TileSummary tile_scan(const float* __restrict__ base, int lo, int n, TileShared& sm,
+template <bool RO = false>
+__device__ __forceinline__ TileSummary tile_scan(const float* base, int lo, int n, TileShared& sm,
                                                  TileThread& th) {
     const int K = per_thread_count(n);
-    if (K == 4) return tile_scan_k<4>(base, lo, n, sm, th);
-    if (K == 8) return tile_scan_k<8>(base, lo, n, sm, th);
-    return tile_scan_k<16>(base, lo, n, sm, th);
+    if (K == 4) return tile_scan_k<4, false, RO>(base, lo, n, sm, th);
+    if (K == 8) return tile_scan_k<8, false, RO>(base, lo, n, sm, th);
+    return tile_scan_k<16, false, RO>(base, lo, n, sm, th);
 }
 
 }  // namespace pf
