@@ -191,7 +191,7 @@ pf_status pf_gather(const void* src, int64_t P_src, int64_t row_bytes, const int
  * increasing slot order.  Then permuted[permuted[j]] = permuted[j], and
  * pf_gather_inplace moves the states without a second buffer.  Deterministic.
  *   ancestors [P] int32 (in), permuted [P] int32 (out), 4-byte aligned, not
- *   overlapping.  Uses 2P + P/1024 + 200 ints of workspace at most.
+ *   overlapping.  Uses 2P + P/1024 + 200 ints of workspace at most (none up to P = 16384).
  * Errors: PF_ERR_INVALID for bad arguments (returned) or an ancestor outside
  * [0, P) (device status; the output is then unspecified).
  */

@@ -581,6 +581,8 @@ pf_status pf_reserve(int64_t P_max, int64_t total_max, int F_max, void* stream) 
                   ((size_t)(P_max + 3) / 4 + 1) * sizeof(int32_t);
     const size_t red = reduce_scratch(P_max > 0 ? P_max : 1);
     if (red > need) need = red;
+    const size_t perm = permute_scratch_bytes(P_max);
+    if (perm > need) need = perm;
     if (P_max + 3 > ((int64_t)1 << 24)) {  // the ordinary-launch path of large single filters
         const size_t large = large_scratch_bytes(PF_MULTINOMIAL, P_max + 3);
         if (large > need) need = large;

@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
 static size_t perm_counts_at(int64_t T) { return (((size_t)T + 1) * sizeof(TilePrefix) + 255) & ~(size_t)255; }
 
 size_t permute_scratch_bytes(int64_t P) {
+    if (P <= kPermSmall) return 0;  // one CTA, in shared memory
     const int64_t T = (P + kPermTile - 1) / kPermTile;
     return perm_counts_at(T) + (((size_t)P * sizeof(int32_t) + 255) & ~(size_t)255) + (size_t)P * sizeof(int32_t);
 }
