@@ -53,4 +53,51 @@ struct FillPieces {
         : x((uint32_t)(head + 4 * t)), end((uint32_t)(head + body)), step(4u * (uint32_t)threads) {}
 };
 
+// ---------------------------------------------------------------------------
+// Chunk index -> (row, place in the row) of the row moves, for rows of `vecs` chunks: a shift
+// for a power of two; else, below 2^32 chunks, a multiplication by the rounded-up
+// reciprocal 2^(32 + shift) / vecs less its leading bit (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994, Fig. 4.1: exact
+// for every 32-bit dividend); beyond, a 64-bit division.
+// ---------------------------------------------------------------------------
+PF_HD uint32_t mulhi32(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+
+struct RowSplit {
+    int64_t vecs;
+    int pow2, shift;      // shift: ceil(log2 vecs)
+    uint32_t magic;       // 0: divide in 64 bits
+    // Place: uint32_t, or, for rows that are `wide`, uint64_t.
+    template <bool POW2, typename Place>
+    PF_HD int64_t row(int64_t i, Place& place) const {
+        if (POW2) {
+            place = (Place)(i & (vecs - 1));
+            return i >> shift;
+        }
+        int64_t j;
+        if (magic != 0u) {
+            const uint32_t n = (uint32_t)i, t = mulhi32(magic, n);
+            j = (t + ((n - t) >> 1)) >> (shift - 1);
+        } else {
+            j = i / vecs;
+        }
+        place = (Place)(i - j * vecs);
+        return j;
+    }
+    bool wide() const { return vecs > 0xffffffffLL; }  // a place takes more than 32 bits
+};
+
+inline RowSplit row_split(int64_t vecs, int64_t total) {
+    RowSplit r{vecs, (vecs & (vecs - 1)) == 0, 0, 0u};
+    while ((1LL << r.shift) < vecs) ++r.shift;
+    if (!r.pow2 && total <= 0xffffffffLL && vecs <= 0x7fffffffLL)
+        r.magic = (uint32_t)(((1ull << 32) * ((1ull << r.shift) - (uint64_t)vecs)) / (uint64_t)vecs + 1ull);
+    return r;
+}
+
 }  // namespace pf

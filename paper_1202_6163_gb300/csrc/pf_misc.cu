@@ -24,15 +24,15 @@ constexpr int kGatherThreads = 256;
 constexpr int kGatherWave = 8;        // resident CTAs per SM of one wave
 constexpr int kGatherFullGrid = 40;   // CTAs per SM from which the grid is not cut to a wave
 
-template <typename VT, int U, bool POW2>
+template <typename VT, int U, bool POW2, typename Place = uint32_t>  // Place: as RowSplit
 __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_t P_src, RowSplit split,
                                                            const int32_t* anc, int64_t total, VT* dst, uint32_t* ctl) {
     grid_begin();
     const int64_t stride = (int64_t)gridDim.x * (kGatherThreads * U);
     int64_t base = (int64_t)blockIdx.x * (kGatherThreads * U) + threadIdx.x;
     int32_t a[U];  // this piece's ancestors, and the chunks' places in their rows
-    uint32_t c[U];
-    auto ancestors = [&](int64_t b, int32_t (&e)[U], uint32_t (&at)[U]) {
+    Place c[U];
+    auto ancestors = [&](int64_t b, int32_t (&e)[U], Place (&at)[U]) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t i = b + u * kGatherThreads;
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_
             if (ok[u]) v[u] = load_chunk(src + (int64_t)a[u] * split.vecs + c[u]);
         }
         int32_t an[U];
-        uint32_t cn[U];
+        Place cn[U];
         ancestors(base + stride, an, cn);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -70,6 +70,9 @@ static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, 
     const int64_t total = P_dst * vecs;
     const RowSplit split = row_split(vecs, total);
     const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, kGatherWave, kGatherFullGrid);
+    if (split.wide())
+        return launch_overlapped(k_gather<VT, U, false, uint64_t>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split,
+                                 anc, total, (VT*)dst, ctl);
     if (split.pow2)
         return launch_overlapped(k_gather<VT, U, true>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc,
                                  total, (VT*)dst, ctl);

@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kPermSmallThreads) k_perm_small(const int32_t*
 // of 32, 64, 96, 128 bytes, two chunks a thread without the early entries: 32, 51, 77, 80;
 // four chunks a thread, a CTA for each piece: 25, 44, 80, 67; three a thread in one
 // resident wave with the early entries: 27, 47, 67, 53.
-template <typename VT, int U, bool POW2>
+template <typename VT, int U, bool POW2, typename Place = uint32_t>  // Place: as RowSplit
 __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSplit split,
                                                         const int32_t* perm, uint32_t* ctl) {
     grid_begin();
@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
     const int64_t stride = (int64_t)gridDim.x * (256 * U);
     int64_t base = (int64_t)blockIdx.x * (256 * U) + threadIdx.x;
     int32_t a[U];  // this piece's entries of perm, and the chunks' places in their rows
-    uint32_t c[U];
-    auto entries = [&](int64_t b, int32_t (&e)[U], uint32_t (&at)[U]) {
+    Place c[U];
+    auto entries = [&](int64_t b, int32_t (&e)[U], Place (&at)[U]) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t i = b + u * 256;
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t i = base + u * 256;
-            uint32_t cc;
+            Place cc;
             move[u] = i < total && a[u] != (int32_t)split.row<POW2>(i, cc);
             own[u] = -1;
             if (move[u] && a[u] >= 0 && a[u] < P) {
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(256) k_gather_inplace(VT* x, int64_t P, RowSpl
             }
         }
         int32_t an[U];
-        uint32_t cn[U];
+        Place cn[U];
         entries(base + stride, an, cn);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -464,8 +464,10 @@ cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const i
         const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
         const RowSplit split = row_split(vecs, P * vecs);
         const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, wave, full);
-        return launch_overlapped(split.pow2 ? k_gather_inplace<VT, U, true> : k_gather_inplace<VT, U, false>, blocks, 256, 0, s,
-                                 p, P, split, perm, ctl);
+        return launch_overlapped(split.wide() ? k_gather_inplace<VT, U, false, uint64_t>
+                                 : split.pow2 ? k_gather_inplace<VT, U, true>
+                                              : k_gather_inplace<VT, U, false>,
+                                 blocks, 256, 0, s, p, P, split, perm, ctl);
     };
     const uintptr_t a = (uintptr_t)x | (uintptr_t)row_bytes;
     constexpr int kNever = 1 << 22;  // one resident wave however many pieces there are

@@ -1,10 +1,12 @@
 // Row moves in vector chunks, shared by the gather and the in-place gather: the
-// chunk types (4 to 32 bytes), their loads and stores, and the split of a chunk's
-// index into row and place.
+// chunk types (4 to 32 bytes), their loads and stores, and the grid (RowSplit, the split
+// of a chunk's index into row and place, is in pf_index.h).
 #pragma once
 
 #include <cstdint>
 #include <cuda_runtime.h>
+
+#include "pf_index.h"
 
 namespace pf {
 
@@ -51,41 +53,6 @@ __device__ __forceinline__ void store_chunk_cs<u32x8>(u32x8* p, u32x8 v) {
     asm volatile("st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v.w[0]), "r"(v.w[1]),
                  "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7])
                  : "memory");
-}
-
-// Chunk index -> (row, place in the row), for rows of `vecs` chunks: a shift for a
-// power of two; else, below 2^32 chunks, a multiplication by the rounded-up
-// reciprocal 2^(32 + shift) / vecs less its leading bit (Granlund and Montgomery,
-// "Division by invariant integers using multiplication", PLDI 1994, Fig. 4.1: exact
-// for every 32-bit dividend); beyond, a 64-bit division.
-struct RowSplit {
-    int64_t vecs;
-    int pow2, shift;      // shift: ceil(log2 vecs)
-    uint32_t magic;       // 0: divide in 64 bits
-    template <bool POW2>
-    __device__ __forceinline__ int64_t row(int64_t i, uint32_t& place) const {
-        if (POW2) {
-            place = (uint32_t)(i & (vecs - 1));
-            return i >> shift;
-        }
-        int64_t j;
-        if (magic != 0u) {
-            const uint32_t n = (uint32_t)i, t = __umulhi(magic, n);
-            j = (t + ((n - t) >> 1)) >> (shift - 1);
-        } else {
-            j = i / vecs;
-        }
-        place = (uint32_t)(i - j * vecs);
-        return j;
-    }
-};
-
-inline RowSplit row_split(int64_t vecs, int64_t total) {
-    RowSplit r{vecs, (vecs & (vecs - 1)) == 0, 0, 0u};
-    while ((1LL << r.shift) < vecs) ++r.shift;
-    if (!r.pow2 && total <= 0xffffffffLL && vecs <= 0x7fffffffLL)
-        r.magic = (uint32_t)(((1ull << 32) * ((1ull << r.shift) - (uint64_t)vecs)) / (uint64_t)vecs + 1ull);
-    return r;
 }
 
 // CTAs for `total` chunks, `per_cta` each: one resident wave that strides over the

@@ -164,11 +164,46 @@ static void runs_and_chunks() {
             }
 }
 
+// ---------------------------------------------------------------------------
+// Row and place of a chunk, from one chunk a row to rows of more than 2^32 chunks, as the row
+// moves choose them (power of two or not, wide or not).
+// ---------------------------------------------------------------------------
+static void rows() {
+    std::mt19937_64 rng(2);
+    std::vector<int64_t> lengths = {0x7fffffffLL, 0x80000000LL, 0x80000001LL, 0xffffffffLL, 1LL << 32, (1LL << 32) + 1,
+                                    (1LL << 33) + 5, 1LL << 34, 16000000007LL};
+    for (int64_t v = 1; v < 300; ++v) lengths.push_back(v);
+    for (int k = 0; k < 300; ++k) lengths.push_back(1 + (int64_t)(rng() >> (33 + rng() % 29)));
+    for (int64_t vecs : lengths)
+        for (int64_t n : {1LL, 2LL, 3LL, 1000LL, 0xffffffffLL / vecs, 0xffffffffLL / vecs + 1, (1LL << 33) / vecs + 1}) {
+            if (n < 1) continue;
+            const int64_t total = n * vecs;
+            const pf::RowSplit s = pf::row_split(vecs, total);
+            auto check = [&](int64_t i) {
+                if (i < 0 || i >= total) return;
+                uint32_t narrow = 0;
+                uint64_t wide = 0;
+                const int64_t j = s.wide() ? s.row<false>(i, wide) : (s.pow2 ? s.row<true>(i, narrow) : s.row<false>(i, narrow));
+                const int64_t place = s.wide() ? (int64_t)wide : (int64_t)narrow;
+                REQUIRE(j == i / vecs && place == i % vecs, "rows of %lld: chunk %lld is (%lld, %lld)", (long long)vecs,
+                        (long long)i, (long long)j, (long long)place);
+            };
+            for (int64_t i : {int64_t(0), vecs - 1, vecs, vecs + 1, total - vecs, total - 1}) check(i);
+            for (int k = 0; k < 200; ++k) {
+                const int64_t i = (int64_t)(rng() % (uint64_t)total);
+                check(i);
+                check(i - i % vecs);
+                check(i - i % vecs - 1);
+            }
+        }
+}
+
 int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!std::strcmp(what, "strata")) strata();
     else if (!std::strcmp(what, "permute_parts")) permute_parts();
     else if (!std::strcmp(what, "runs_and_chunks")) runs_and_chunks();
+    else if (!std::strcmp(what, "rows")) rows();
     else return 2;
     return 0;
 }

@@ -21,7 +21,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("what", ["strata", "permute_parts", "runs_and_chunks"])
+@pytest.mark.parametrize("what", ["strata", "permute_parts", "runs_and_chunks", "rows"])
 def test_index_arithmetic(program, what):
     r = subprocess.run([program, what], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
