@@ -11,27 +11,33 @@ namespace pf {
 // ---------------------------------------------------------------------------
 // Gather: dst row j <- src row anc[j].  One thread moves U chunks of VT, adjacent
 // blocks of a CTA's threads, issuing all loads before the stores so that several
-// random row reads are in flight.  Bound by DRAM writes and the latency of the
-// row reads.  Rows of a multiple of 32 bytes move in 256-bit accesses, two a thread:
-// 2^24 rows of 32 bytes 133 -> 100 us (576 MB of rows and ancestors: 5.7 TB/s),
-// 2^22 rows of 64 bytes 94 -> 78 us, of 128 bytes 154 -> 124 us against four 128-bit
-// chunks a thread spaced a grid apart (four 256-bit ones: 116 us at 2^24).  A piece's
-// ancestors are asked for while the piece before is on its way: systematic ancestors of
-// N(0,1) log-weights, 2^24 rows of 4, 12, 16 bytes 48.5, 176, 99 -> 44, 145, 92 us,
-// 3000017 rows of 128 bytes 101 -> 92 us, of 4 bytes 6.1 -> 6.7 us.
+// random row reads are in flight; the next piece's ancestors are asked for while a piece
+// is on its way.  Bound by DRAM writes and the latency of the row reads.  Rows of a
+// multiple of 32 bytes move in 256-bit accesses, two a thread: systematic ancestors of
+// N(0,1) log-weights, 2^24 rows of 32 bytes 161 us, 2^22 rows of 64 bytes 76 us, of 128
+// bytes 128 us, against 170, 81 and 146 for four 128-bit chunks a thread spaced a grid apart.
+// The fewer CTAs stride over the chunks the better, down to what covers the latency (the
+// waves in launch_gather): with eight of them per SM for every type 2^24 rows of 4 and 12
+// bytes took 44 and 145 us, now 34 and 87; 3000017 random rows of 16 bytes 21.0, now 18.8, of
+// 68 bytes 155, now 95.
 // ---------------------------------------------------------------------------
 constexpr int kGatherThreads = 256;
-constexpr int kGatherWave = 8;        // resident CTAs per SM of one wave
-constexpr int kGatherFullGrid = 40;   // CTAs per SM from which the grid is not cut to a wave
+
+// CTAs per SM that the registers must leave room for (0: as they fall): 256-bit chunks come out two
+// registers above six CTAs otherwise.
+template <typename VT, typename Place>
+constexpr int gather_ctas() {
+    return sizeof(VT) == 32 && sizeof(Place) == 4 ? 6 : 0;
+}
 
 template <typename VT, int U, bool POW2, typename Place = uint32_t>  // Place: as RowSplit
-__global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_t P_src, RowSplit split,
-                                                           const int32_t* anc, int64_t total, VT* dst, uint32_t* ctl) {
+__global__ void __launch_bounds__(kGatherThreads, gather_ctas<VT, Place>())
+    k_gather(const VT* src, int64_t P_src, RowSplit split, const int32_t* anc, int64_t total, VT* dst, uint32_t* ctl) {
     grid_begin();
     const int64_t stride = (int64_t)gridDim.x * (kGatherThreads * U);
     int64_t base = (int64_t)blockIdx.x * (kGatherThreads * U) + threadIdx.x;
-    int32_t a[U];  // this piece's ancestors, and the chunks' places in their rows
-    Place c[U];
+    int32_t a[U];  // this piece's ancestors, and (POW2: formed anew) the chunks' places in their rows
+    Place c[U] = {};
     auto ancestors = [&](int64_t b, int32_t (&e)[U], Place (&at)[U]) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -41,6 +47,9 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_
             if (i < total) e[u] = anc[split.row<POW2>(i, at[u])];
         }
     };
+    auto place = [&](int u) -> Place {
+        return POW2 ? (Place)((base + u * kGatherThreads) & (split.vecs - 1)) : c[u];
+    };
     ancestors(base, a, c);
     for (; base < total; base += stride) {
         VT v[U];
@@ -48,7 +57,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             ok[u] = base + u * kGatherThreads < total && a[u] >= 0 && a[u] < P_src;
-            if (ok[u]) v[u] = load_chunk(src + (int64_t)a[u] * split.vecs + c[u]);
+            if (ok[u]) v[u] = load_chunk(src + (int64_t)a[u] * split.vecs + place(u));
         }
         int32_t an[U];
         Place cn[U];
@@ -56,7 +65,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (ok[u]) store_chunk_cs(dst + base + u * kGatherThreads, v[u]);
-            else if (base + u * kGatherThreads < total && c[u] == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
+            else if (base + u * kGatherThreads < total && place(u) == 0) set_status(ctl + CTL_STATUS, ST_INVALID);
             a[u] = an[u];
             c[u] = cn[u];
         }
@@ -65,11 +74,11 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const VT* src, int64_
 
 template <typename VT, int U>
 static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
-                             void* dst, uint32_t* ctl, int num_sms, cudaStream_t s) {
+                             void* dst, uint32_t* ctl, int num_sms, cudaStream_t s, int wave, int from = 8, int full = 40) {
     const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
     const int64_t total = P_dst * vecs;
     const RowSplit split = row_split(vecs, total);
-    const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, kGatherWave, kGatherFullGrid);
+    const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, wave, full, from);
     if (split.wide())
         return launch_overlapped(k_gather<VT, U, false, uint64_t>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split,
                                  anc, total, (VT*)dst, ctl);
@@ -83,10 +92,18 @@ static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, 
 cudaError_t launch_gather(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
                           void* dst, uint32_t* ctl, int num_sms, cudaStream_t s) {
     const uintptr_t a = (uintptr_t)src | (uintptr_t)dst | (uintptr_t)row_bytes;
-    if ((a & 31) == 0) return gather_vt<u32x8, 2>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
-    if ((a & 15) == 0) return gather_vt<uint4, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
-    if ((a & 7) == 0) return gather_vt<uint2, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
-    return gather_vt<uint32_t, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s);
+    // CTAs per SM of a wave.  us with more of them: 2^22 random rows of 16 bytes, eight 31.5 and five
+    // 27.8 (rows of 48 bytes, whose kernel leaves room for four at a time, need the eight: 2^20 of
+    // them 13.3 and 16.0); 2^20 sorted rows of 64 bytes, eight 18.8 and six 18.1; 2^22 random rows
+    // of 8 bytes 21.8 and 20.3; 2^24 sorted rows of 4 bytes 42 and 34.
+    constexpr int kNever = 1 << 22;  // one resident wave however many pieces there are
+    if ((a & 31) == 0) return gather_vt<u32x8, 2>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s, 6);
+    if ((a & 15) == 0) {
+        const int wave = (row_bytes & (row_bytes - 1)) == 0 ? 5 : 8;
+        return gather_vt<uint4, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s, wave);
+    }
+    if ((a & 7) == 0) return gather_vt<uint2, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s, 6);
+    return gather_vt<uint32_t, 4>(src, P_src, row_bytes, anc, P_dst, dst, ctl, num_sms, s, 6, 6, kNever);
 }
 
 // ---------------------------------------------------------------------------

@@ -463,7 +463,7 @@ cudaError_t launch_gather_inplace(void* x, int64_t P, int64_t row_bytes, const i
         constexpr int U = decltype(unroll)::value;
         const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
         const RowSplit split = row_split(vecs, P * vecs);
-        const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, wave, full);
+        const unsigned blocks = chunk_grid(P * vecs, 256 * U, num_sms, wave, full, wave);
         return launch_overlapped(split.wide() ? k_gather_inplace<VT, U, false, uint64_t>
                                  : split.pow2 ? k_gather_inplace<VT, U, true>
                                               : k_gather_inplace<VT, U, false>,

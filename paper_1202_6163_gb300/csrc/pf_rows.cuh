@@ -55,13 +55,13 @@ __device__ __forceinline__ void store_chunk_cs<u32x8>(u32x8* p, u32x8 v) {
                  : "memory");
 }
 
-// CTAs for `total` chunks, `per_cta` each: one resident wave that strides over the
-// chunks, or, from `full` CTAs per SM on, a CTA per piece, whose staggered starts
-// keep more reads in flight (gather of 2^22 rows of 64 bytes, 108 CTAs per SM: 88 us
-// as a wave, 78 us in full; 2^20 rows, 27 per SM: 20.7 and 22.6 us).
-inline unsigned chunk_grid(int64_t total, int per_cta, int num_sms, int wave, int full) {
+// CTAs for `total` chunks, `per_cta` each: beyond `from` CTAs per SM one resident wave of `wave`
+// per SM that strides over the chunks, or, from `full` CTAs per SM on, a CTA per piece, whose
+// staggered starts keep more reads in flight (gather of 2^22 rows of 64 bytes, 108 CTAs
+// per SM: 88 us as a wave, 78 us in full; 2^20 rows, 27 per SM: 20.7 and 22.6 us).
+inline unsigned chunk_grid(int64_t total, int per_cta, int num_sms, int wave, int full, int from) {
     int64_t blocks = (total + per_cta - 1) / per_cta;
-    if (blocks > (int64_t)num_sms * wave && blocks < (int64_t)num_sms * full) blocks = (int64_t)num_sms * wave;
+    if (blocks > (int64_t)num_sms * from && blocks < (int64_t)num_sms * full) blocks = (int64_t)num_sms * wave;
     if (blocks > 0x7fffffffLL) blocks = 0x7fffffffLL;  // the kernels stride over what is left
     return (unsigned)(blocks < 1 ? 1 : blocks);
 }
