@@ -745,7 +745,6 @@ pf_status pf_lg_init(int F, int64_t P, int D, float m0, float p0, uint64_t seed,
     p.sigma = (float)std::sqrt((double)p0);
     p.m0 = m0;
     p.log_P = std::log((double)P);
-    p.n_tiles = (int)((P + lg_tile() - 1) / lg_tile());
     p.keys = philox_round_keys((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
     p.x_next = x;
     p.lw = logw;
@@ -753,7 +752,7 @@ pf_status pf_lg_init(int F, int64_t P, int D, float m0, float p0, uint64_t seed,
     p.log_sum = log_sum;
     p.ess = ess;
     p.resample = resample;
-    return cuda_fail(launch_lg_init(p, s), "lg init launch");
+    return cuda_fail(launch_lg_init(p, info->num_sms, s), "lg init launch");
 }
 
 pf_status pf_lg_step(int F, int64_t P, int D, const float* a, double q, double r, double threshold,

@@ -190,7 +190,7 @@ uint64_t current_wait_ns();
 // Kernel launchers (defined in the .cu files; return the launch error).
 cudaError_t launch_sorted_persistent(int kind, const SortedParams& p, int grid, cudaStream_t s);
 int lg_tile();
-cudaError_t launch_lg_init(const LgParams& p, cudaStream_t s);
+cudaError_t launch_lg_init(const LgParams& p, int num_sms, cudaStream_t s);
 cudaError_t launch_lg_step(const LgParams& p, cudaStream_t s);
 size_t permute_scratch_bytes(int64_t P);
 cudaError_t launch_permute(const int32_t* anc, int64_t P, int32_t* out, void* scratch, uint32_t* ctl, int num_sms,

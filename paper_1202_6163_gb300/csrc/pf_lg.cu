@@ -95,10 +95,13 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* ra, float*
 }
 
 // The initial draw, on the step's tiles of 1024 particles (one filter per CTA, so no
-// division of a particle's index, and as many CTAs as the step).  Bound by instruction
-// issue: the noise's arithmetic.  256 filters of 2^16 particles: 141 -> 96 us
-// (as a grid-stride loop over all particles, 37% of the warps resident); its 335 MB take 49 us.
-template <int GS>
+// division of a particle's index, and as many CTAs as the step), or, where those leave SMs
+// idle, on tiles of 256.  Bound by instruction issue: the noise's arithmetic.  256 filters
+// of 2^16 particles: 141 -> 96 us (as a grid-stride loop over all particles, 37% of the warps
+// resident); its 335 MB take 49 us.  7 filters of 4097 particles of 16 dimensions: 35 CTAs of 1024
+// particles 6.0 us, 119 of 256 2.3.  Rows of many dimensions are drawn in the order of memory: 16 filters
+// of 70001 particles of 64 dimensions 258 us with a thread to a row, 112 so.
+template <int GS, int PER>
 __global__ void __launch_bounds__(kLgThreads) k_lg_init(LgParams p) {
     grid_begin();
     const int f = (int)(blockIdx.x / (unsigned)p.n_tiles);
@@ -107,18 +110,36 @@ __global__ void __launch_bounds__(kLgThreads) k_lg_init(LgParams p) {
     const uint32_t Pu = (uint32_t)p.P;
     float* lw_f = p.lw + (int64_t)f * p.P;
     float4* x_f = reinterpret_cast<float4*>(p.x_next + (int64_t)f * p.P * p.D);
-    const uint32_t j0 = (uint32_t)tile * (kLgThreads * kLgPerThread) + threadIdx.x;
+    const uint32_t j0 = (uint32_t)tile * (kLgThreads * PER) + threadIdx.x;
+    auto draw = [&](float4* xo, uint32_t j, int g) {
+        const float4 z = normals4(j, (uint32_t)g, (uint32_t)f, p.keys);
+        *xo = make_float4(p.m0 + p.sigma * z.x, p.m0 + p.sigma * z.y, p.m0 + p.sigma * z.z, p.m0 + p.sigma * z.w);
+    };
+    if constexpr (GS == 0) {  // a thread per four dimensions, in the order they lie in memory
+        const uint32_t first = (uint32_t)tile * (kLgThreads * PER), n = min(Pu - first, (uint32_t)(kLgThreads * PER));
+        uint32_t j = threadIdx.x / (uint32_t)G;
+        int g = (int)(threadIdx.x - j * (uint32_t)G);
+        const uint32_t dj = kLgThreads / (uint32_t)G;
+        const int dg = (int)(kLgThreads - dj * (uint32_t)G);
+        float4* xo = x_f + (size_t)first * G + threadIdx.x;
+        for (; j < n; xo += kLgThreads) {
+            draw(xo, first + j, g);
+            j += dj;
+            g += dg;
+            if (g >= G) {
+                g -= G;
+                ++j;
+            }
+        }
+    }
 #pragma unroll
-    for (int k = 0; k < kLgPerThread; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const uint32_t j = j0 + k * kLgThreads;
         if (j >= Pu) break;
-        float4* xo = x_f + (size_t)j * G;
+        if constexpr (GS > 0) {
+            float4* xo = x_f + (size_t)j * GS;
 #pragma unroll
-        for (int g = 0; g < (GS > 0 ? GS : 16); ++g) {
-            if (GS == 0 && g >= G) break;
-            const float4 z = normals4(j, (uint32_t)g, (uint32_t)f, p.keys);
-            xo[g] = make_float4(p.m0 + p.sigma * z.x, p.m0 + p.sigma * z.y, p.m0 + p.sigma * z.z,
-                                p.m0 + p.sigma * z.w);
+            for (int g = 0; g < GS; ++g) draw(xo + g, j, g);
         }
         lw_f[j] = 0.0f;
     }
@@ -267,14 +288,21 @@ __global__ void __launch_bounds__(kLgThreads) k_lg_step(LgParams p) {
 
 int lg_tile() { return kLgThreads * kLgPerThread; }
 
-cudaError_t launch_lg_init(const LgParams& p, cudaStream_t s) {
+template <int PER>
+static cudaError_t lg_init_tiles(LgParams p, cudaStream_t s) {
+    p.n_tiles = (int)((p.P + kLgThreads * PER - 1) / (kLgThreads * PER));
     const unsigned blocks = (unsigned)((int64_t)p.F * p.n_tiles);
     switch (p.D) {
-    case 4: return launch_overlapped(k_lg_init<1>, blocks, kLgThreads, 0, s, p);
-    case 8: return launch_overlapped(k_lg_init<2>, blocks, kLgThreads, 0, s, p);
-    case 16: return launch_overlapped(k_lg_init<4>, blocks, kLgThreads, 0, s, p);
-    default: return launch_overlapped(k_lg_init<0>, blocks, kLgThreads, 0, s, p);
+    case 4: return launch_overlapped(k_lg_init<1, PER>, blocks, kLgThreads, 0, s, p);
+    case 8: return launch_overlapped(k_lg_init<2, PER>, blocks, kLgThreads, 0, s, p);
+    case 16: return launch_overlapped(k_lg_init<4, PER>, blocks, kLgThreads, 0, s, p);
+    default: return launch_overlapped(k_lg_init<0, PER>, blocks, kLgThreads, 0, s, p);
     }
+}
+
+cudaError_t launch_lg_init(const LgParams& p, int num_sms, cudaStream_t s) {
+    const int64_t tiles = (int64_t)p.F * ((p.P + lg_tile() - 1) / lg_tile());
+    return tiles < 2 * num_sms ? lg_init_tiles<1>(p, s) : lg_init_tiles<kLgPerThread>(p, s);
 }
 
 cudaError_t launch_lg_step(const LgParams& p, cudaStream_t s) {
