@@ -536,11 +536,11 @@ constexpr int kRoundMagicBits = 0x4b400000;
 // odd multiple of four words between lanes keeps the 16-byte reads free of bank conflicts.
 __host__ __device__ constexpr int warp_stage_per_lane(int KK) { return KK == 16 ? 20 : (KK == 8 ? 12 : 8); }
 
-// marks: this warp's 32 S entries, 16-byte aligned, all -1 on entry and on return.
-// ubuf (stratified): this warp's 32 S floats for the strata's uniforms.
-template <int KIND, int KK, int S, bool LONG>
-__device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap map, int32_t* marks, float* ubuf,
-                                            TileThread& th, int i_last, int64_t index0) {
+// marks: this warp's STRIDE entries (32 S used), 16-byte aligned, all -1 on entry and on return;
+// stratified: STRIDE floats for the strata's uniforms follow.
+template <int KIND, int KK, int S, int STRIDE, bool LONG, bool SPILL>
+__device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap map, int32_t* marks, TileThread& th,
+                                            int i_last, int64_t index0) {
     const int lane = threadIdx.x & 31;
     const int noff = map.noff;
     if (noff <= 0) return;
@@ -585,20 +585,25 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
         const long long g0 = strata_block(map.jlo, k_first);
         const int blocks = (int)(strata_block(map.jlo, k_last) - g0) + 1;
         const int at = strata_at(map.jlo, g0);  // ubuf index of stratum 0 (may be negative)
-        if (blocks <= 8 * S) {
-            __syncwarp();  // the last tile's reads of ubuf
+        if (blocks <= STRIDE / (SPILL ? 2 : 4)) {
+            // SPILL: where the buffer does not hold them all, the marks' entries in front of it take their
+            // share (2^21 particles, weights u^100, u uniform: a buffer at a time 22.3 us, so 18.8)
+            const bool spill = SPILL && blocks > STRIDE / 4;
+            const int from = spill ? 0 : STRIDE;
+            float* ubuf = reinterpret_cast<float*>(marks);
+            __syncwarp();  // the last tile's reads of the buffer
             for (int b = lane; b < blocks; b += 32) {
                 const u32x4 r = philox((uint32_t)(g0 + b), 0u, p.filter, TAG_STRAT, p.key0, p.key1);
-                *reinterpret_cast<float4*>(ubuf + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
+                *reinterpret_cast<float4*>(ubuf + from + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
             }
             __syncwarp();
-            start0 = min(noff, kb + (ubuf[strata_index(at, kb)] < fb ? 1 : 0));
+            start0 = min(noff, kb + (ubuf[from + strata_index(at, kb)] < fb ? 1 : 0));
             if (!clamp) {
 #pragma unroll
                 for (int i = 0; i < KK; ++i) {
                     float frac;
                     const int k = stratum(__fmaf_rn(th.v[i], ir, x0), frac);
-                    th.v[i] = __int_as_float(k + (ubuf[at + k] < frac ? 1 : 0));
+                    th.v[i] = __int_as_float(k + (ubuf[from + at + k] < frac ? 1 : 0));
                 }
             } else {
 #pragma unroll
@@ -606,10 +611,17 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                     const float y = __fmaf_rn(th.v[i], ir, x0);
                     float frac;
                     const int k = min(max(stratum(y, frac), 0), kmax);
-                    th.v[i] = __int_as_float(min(noff, k + (ubuf[strata_index(at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                    th.v[i] = __int_as_float(min(noff, k + (ubuf[from + strata_index(at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
                 }
             }
+            if (spill) {
+                __syncwarp();
+                for (int b = lane; b < STRIDE / 4; b += 32)
+                    reinterpret_cast<int4*>(marks)[b] = make_int4(-1, -1, -1, -1);
+                __syncwarp();
+            }
         } else {
+            float* ubuf = reinterpret_cast<float*>(marks + STRIDE);
             // strata beyond the buffer: one buffer of them at a time, those without a
             // coordinate (inside a dominant particle's run) passed over.  The whole buffer each
             // time: draws cut off at the last stratum measured slower (no longer unrolled)
@@ -743,18 +755,22 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
     }
 }
 
-// Where a warp's entries lie in the staging: at the same place whatever KK and S, as the
-// CTA's warps may be in different tiles, of different KK.
+// A warp's entries in the staging, and where they begin: the same place whatever KK and S, as
+// the CTA's warps may be in different tiles, of different KK.
 template <int KIND, int CAP>
 __host__ __device__ constexpr int warp_stage_stride() {
     return (KIND == KIND_STRAT || CAP >= kIoCapSmall ? CAP : 2 * CAP) / kWarps;
+}
+template <int KIND, int CAP>
+__device__ __forceinline__ int32_t* warp_stage(int32_t* stage) {  // stratified: the uniforms' buffer behind each warp's
+    return stage + (int)(threadIdx.x >> 5) * (KIND == KIND_STRAT ? 2 : 1) * warp_stage_stride<KIND, CAP>();
 }
 
 // Sets this warp's entries to -1 (once, before its first tile).
 template <int KIND, int CAP>
 __device__ __forceinline__ void warp_stage_init(int32_t* stage) {
     constexpr int kStride = warp_stage_stride<KIND, CAP>();
-    int4* mine = reinterpret_cast<int4*>(stage + (threadIdx.x >> 5) * kStride);
+    int4* mine = reinterpret_cast<int4*>(warp_stage<KIND, CAP>(stage));
 #pragma unroll
     for (int i = threadIdx.x & 31; i < kStride / 4; i += 32) mine[i] = make_int4(-1, -1, -1, -1);
     __syncwarp();
@@ -784,14 +800,14 @@ __device__ __forceinline__ TileMap only_tile_map(const SortedParams& p, fpair W)
 // that one warp's share could be most of them, chunk by chunk over the CTA (which sets
 // the staging before, and back to -1 after).  Block-uniform choice.  The warp's
 // entries are -1 on entry (warp_stage_init) and on return.
-template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK), bool LONG = true>  // LONG: as assign_offspring
+template <int KIND, int KK, int CAP, int S = warp_stage_per_lane(KK), bool LONG = true,  // LONG: as assign_offspring
+          bool SPILL = true>                                                             // SPILL: as assign_warp
 __device__ __forceinline__ void assign_tile(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
                                             TileThread& th, const TileSummary& ts, int64_t index0) {
     constexpr int kStride = warp_stage_stride<KIND, CAP>();
     static_assert(32 * S <= kStride && kStride % 4 == 0, "a warp's entries fit its share of the staging");
     if (map.noff <= (LONG ? kWarpOffsets : kWarpOffsetsShort)) {
-        const int at = (threadIdx.x >> 5) * kStride;
-        assign_warp<KIND, KK, S, LONG>(p, map, stage + at, reinterpret_cast<float*>(stage + CAP) + at, th, ts.i_last, index0);
+        assign_warp<KIND, KK, S, kStride, LONG, SPILL>(p, map, warp_stage<KIND, CAP>(stage), th, ts.i_last, index0);
         return;
     }
     __syncthreads();

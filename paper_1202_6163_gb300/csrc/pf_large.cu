@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
             const int64_t t0 = (int64_t)((int)blockIdx.x + (r0 + r) * (int)gridDim.x) * kLargeTile;
             read_tile_v<16>(p.v_out + t0, (int)min((int64_t)kLargeTile, PA - t0), th);
             ts.i_last = m.il;
-            assign_tile<KIND, 16, kIoCap, S>(p, sm.as, {m.jlo, m.noff, m.x0, m.ir}, stage, th, ts, t0 - p.lead);
+            // without SPILL: stratified, 10^8 particles 391 us, with it 396
+            assign_tile<KIND, 16, kIoCap, S, true, false>(p, sm.as, {m.jlo, m.noff, m.x0, m.ir}, stage, th, ts, t0 - p.lead);
         };
         bool any = false;
         for (int r = 0; r < n; ++r) {

@@ -22,10 +22,11 @@
 
 // ---------------------------------------------------------------------------
 // The stratified assignment's look-ups, warp by warp, over a tile of n elements KK to a
-// thread (pf_assign.cuh, assign_warp): every index lies in the warp's buffer of 32 S.
+// thread (pf_assign.cuh, assign_warp): every index lies in the warp's buffer, UB strata at once or
+// one 32 S after another.
 // Lanes wholly past the tile's end hold: 0 the last element's weight, 1 zero, 2 anything.
 // ---------------------------------------------------------------------------
-static void strata_of_tile(std::mt19937& rng, int KK, int S, int n, const std::vector<float>& v, int noff, float x0,
+static void strata_of_tile(std::mt19937& rng, int KK, int S, int UB, int n, const std::vector<float>& v, int noff, float x0,
                            float ir, long long jlo, int empty) {
     std::uniform_real_distribution<float> any(0.f, v[n - 1]);
     const int kmax = noff - 1;
@@ -55,7 +56,7 @@ static void strata_of_tile(std::mt19937& rng, int KK, int S, int n, const std::v
             REQUIRE(index >= 0 && index < size, "strata: index %d of %d, warp %d lane %d, n %d noff %d KK %d, empty lanes %d",
                     index, size, w, l, n, noff, KK, empty);
         };
-        if (blocks <= 8 * S) {
+        if (4 * blocks <= UB) {
             for (int l = 0; l < 32; ++l) {
                 const bool clamp = pf::strata_clamped(stratum(yb[l]), stratum(y[l][KK - 1]), kmax, pos[l]);
                 inside(pf::strata_index(at, bounded(yb[l])), 4 * blocks, l);
@@ -92,6 +93,7 @@ static void strata() {
     std::uniform_real_distribution<float> unit(0.f, 1.f);
     for (int round = 0; round < 1500; ++round) {
         const int KK = 4 << (round % 3), S = KK == 16 ? 20 : (KK == 8 ? 12 : 8), tile = 512 * KK;
+        const int UB = 2 * (KK == 16 || round % 2 ? 640 : 512);
         // ragged lengths that end in every warp
         const int n = round % 5 ? 1 + (int)(rng() % tile) : 4153 % tile + 1;
         std::vector<float> v(n);
@@ -107,12 +109,12 @@ static void strata() {
         const int noff = 1 + (int)(rng() % 65536);  // up to kWarpOffsets
         const float x0 = 2.f * unit(rng) - 1.f, ir = (float)noff / s;
         const long long jlo = (long long)(rng() % 2147000000u);
-        for (int empty = 0; empty < 3; ++empty) strata_of_tile(rng, KK, S, n, v, noff, x0, ir, jlo, empty);
+        for (int empty = 0; empty < 3; ++empty) strata_of_tile(rng, KK, S, UB, n, v, noff, x0, ir, jlo, empty);
     }
     // one particle of 30000 offsets in front of a last tile of 4153 particles
     std::vector<float> v(4153);
     for (int i = 0; i < 4153; ++i) v[i] = 30000.f + (float)i;
-    for (int empty = 0; empty < 3; ++empty) strata_of_tile(rng, 16, 20, 4153, v, 34152, 0.25f, 1.f, 33550000, empty);
+    for (int empty = 0; empty < 3; ++empty) strata_of_tile(rng, 16, 20, 1280, 4153, v, 34152, 0.25f, 1.f, 33550000, empty);
 }
 
 // ---------------------------------------------------------------------------
