@@ -10,10 +10,9 @@
 namespace pf {
 
 enum { KIND_MULTI = 0, KIND_STRAT = 1, KIND_SYS = 2 };
-// Staging entries of the run-length decode (per buffer): a chunk holds up to
-// CAP - 4 offsets.  kIoCap serves tiles of up to 8192 elements, whose offset
-// count varies around the tile length, so such a tile nearly always decodes
-// in one chunk; kIoCapSmall serves tiles of up to 4096.
+// Staging entries of the run-length decode (per buffer): a chunk of the CTA-wide
+// decode holds up to CAP - 4 offsets, a warp's its share.  kIoCap serves tiles of up to
+// 8192 elements, kIoCapSmall of up to 4096.
 constexpr int kIoCap = 10240;
 constexpr int kIoCapSmall = 8192;
 static_assert(kIoCap % (4 * 512) == 0 && kIoCapSmall % (4 * 512) == 0, "decode chunks use 4-entry groups per thread");
@@ -158,14 +157,14 @@ __device__ __forceinline__ void stage_init(int32_t* stage) {  // stage: 16-byte 
 // The run that covers offset c0 and where the next one begins, over this thread's elements
 // (counts N in v, starting from start0): cur the last element whose run covers c0 (-1:
 // none), next the first start beyond c0 (INT_MAX: none).
-template <int KK>  // 0: th.K elements
+template <int KK>
 __device__ __forceinline__ void run_at(const TileThread& th, int start0, int c0, int& cur, int& next) {
     cur = -1;
     next = INT_MAX;
     int a = start0;
 #pragma unroll
-    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-        if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+    for (int i = 0; i < KK; ++i) {
+        if ((th.pos >> i) & 1u) {
             const int b = __float_as_int(th.v[i]);
             if (b > a) {
                 if (a > c0) next = min(next, a);
@@ -181,8 +180,8 @@ template <int KK>
 __device__ __forceinline__ int longest_run(const TileThread& th, int start0) {
     int a = start0, longest = 0;
 #pragma unroll
-    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-        if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+    for (int i = 0; i < KK; ++i) {
+        if ((th.pos >> i) & 1u) {
             const int b = __float_as_int(th.v[i]);
             longest = max(longest, b - a);
             a = b;
@@ -208,8 +207,7 @@ __device__ __forceinline__ void fill_run(int32_t* dst, int n, int32_t v, int t, 
 // out[s + shift] so that out[x] maps to the 16-byte aligned global position
 // gb + x; each thread scans and stores S consecutive entries
 // (S * kThreads >= c1 - c0 + shift).  Ancestor = tile_base + element.
-template <int S, int KK = 0, bool ONE = false>  // KK: elements per thread when fixed, 0 = th.K;
-                                                 // ONE: the chunk is the tile's only one (c0 = 0, c1 = noff)
+template <int S, int KK>
 __device__ __forceinline__ void decode_chunk(const SortedParams& p, AssignShared& sm, int32_t* out,
                                              const TileThread& th, long long jlo, int c0, int c1, int shift,
                                              int start0, int32_t tile_base, int32_t tag) {
@@ -218,12 +216,11 @@ __device__ __forceinline__ void decode_chunk(const SortedParams& p, AssignShared
     const int32_t mark0 = tag | th.e0;
     int a = start0;
 #pragma unroll
-    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-        if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+    for (int i = 0; i < KK; ++i) {
+        if ((th.pos >> i) & 1u) {
             const int b = __float_as_int(th.v[i]);
             if (b > a) {
-                if (ONE) out[a + shift] = mark0 + i;  // 0 <= a < b <= noff: inside the only chunk
-                else if (a >= c0 && a < c1) out[a - c0 + shift] = mark0 + i;
+                if (a >= c0 && a < c1) out[a - c0 + shift] = mark0 + i;
                 else if (a < c0 && b > c0) out[shift] = mark0 + i;
             }
             a = b;
@@ -283,93 +280,50 @@ __device__ __forceinline__ void decode_chunk(const SortedParams& p, AssignShared
     // finishing this chunk's reads of sm.red_n
 }
 
-// stage: the two staging buffers (2 * CAP entries, stage_init<CAP>'ed once per
-// launch); epoch: the chunk counter of the launch, identical in every thread.
-template <int KIND, int KK = 0, int CAP = kIoCap, bool LONG = true>  // KK: elements per thread when fixed, 0 = th.K;
-                                                                     // LONG: look for long runs
+// The assignment of a tile of many offsets (more than any chunk holds) by the whole CTA.
+// stage: the two staging buffers (2 * CAP entries, stage_init<CAP>'ed); epoch: the chunk
+// counter, identical in every thread.
+template <int KIND, int KK, int CAP, bool LONG>  // LONG: look for long runs
 __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const TileMap map, int32_t* stage,
                                  uint32_t& epoch, TileThread& th, const TileSummary& ts, int64_t index0) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int noff = map.noff;
     const long long jlo = map.jlo;
     const float x0 = map.x0, ir = map.ir;
-    // Stratified: when the tile's strata fit a staging buffer, the block draws
-    // their uniforms once, four per Philox block, into the buffer the next
-    // decode chunk will use (its last readers finished two chunks ago), stored
-    // with the sign bit set so that every entry stays below the decode's tags;
-    // otherwise each thread draws the blocks its elements need.
-    const bool coop = KIND == KIND_STRAT && noff <= CAP;
-    const int32_t* ub = stage + ((epoch + 1u) & 1u) * CAP;
-    if (KIND == KIND_STRAT && coop) {
-        int32_t* uw = stage + ((epoch + 1u) & 1u) * CAP;
-        const long long g0 = jlo >> 2, g1 = (jlo + noff - 1) >> 2;
-        for (long long g = g0 + tid; g <= g1; g += kThreads) {
-            const u32x4 r = philox((uint32_t)g, 0u, p.filter, TAG_STRAT, p.key0, p.key1);
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const long long j = 4 * g + s;
-                if (j >= jlo && j < jlo + noff)
-                    uw[j - jlo] = (int32_t)(__float_as_uint(u23f(word_of(r, s))) | 0x80000000u);
-            }
-        }
-        __syncthreads();
-    }
     // N_i: offsets of the tile below the element's cumulative weight (kept in v[] as int bits).
     // Systematic: N = min(ceil(y), noff), the conversion rounding up and saturating at 0.
-    // Stratified: with k = floor(y) (saturating at 0, at most noff - 1), N = k + [u_k < y - k],
-    // capped at noff (y - k is exact).  The tile's last positive element takes noff.
+    // Stratified: with k = floor(y), N = k + [u_k < y - k], capped at noff (y - k is exact); each
+    // thread draws the Philox blocks its elements need.  The tile's last positive element takes noff.
     int last_n = -1;
-    const int il = ts.i_last - th.e0;  // this thread's index of the tile's last positive element, if any
-    if (KIND == KIND_SYS || coop) {
-        const uint32_t kmax = (uint32_t)max(noff - 1, 0);
+    uint32_t cq = 0xffffffffu;
+    u32x4 cw = {0, 0, 0, 0};
 #pragma unroll
-        for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-            if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
-                const float y = __fmaf_rn(th.v[i], ir, x0);
-                int n;
-                if (KIND == KIND_SYS) {
-                    n = (int)min(__float2uint_ru(y), (uint32_t)noff);
-                } else {
-                    const uint32_t k = min(__float2uint_rd(y), kmax);
-                    const float u = __uint_as_float((uint32_t)ub[k] & 0x7fffffffu);
-                    n = min(noff, (int)k + (u < __fsub_rn(y, (float)k) ? 1 : 0));
-                }
-                n = i == il ? noff : n;
-                th.v[i] = __int_as_float(n);
-                last_n = n;
-            }
-        }
-    } else {
-        // stratified, strata beyond the staging buffer: each thread draws the
-        // Philox blocks its elements need
-        uint32_t cq = 0xffffffffu;
-        u32x4 cw = {0, 0, 0, 0};
-#pragma unroll
-        for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-            if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
-                int n;
-                const float y = __fmaf_rn(th.v[i], ir, x0);
-                if (th.e0 + i == ts.i_last) {
+    for (int i = 0; i < KK; ++i) {
+        if ((th.pos >> i) & 1u) {
+            const float y = __fmaf_rn(th.v[i], ir, x0);
+            int n;
+            if (th.e0 + i == ts.i_last) {
+                n = noff;
+            } else if (KIND == KIND_SYS) {
+                n = (int)min(__float2uint_ru(y), (uint32_t)noff);
+            } else if (y <= 0.f) {
+                n = 0;
+            } else {
+                const float fl = floorf(y);
+                if (fl >= (float)noff) {
                     n = noff;
-                } else if (y <= 0.f) {
-                    n = 0;
                 } else {
-                    const float fl = floorf(y);
-                    if (fl >= (float)noff) {
-                        n = noff;
-                    } else {
-                        const long long j = jlo + (long long)fl;
-                        const uint32_t q = (uint32_t)(j >> 2);
-                        if (q != cq) {
-                            cq = q;
-                            cw = philox(q, 0u, p.filter, TAG_STRAT, p.key0, p.key1);
-                        }
-                        n = min(noff, (int)fl + (u23f(word_of(cw, (int)(j & 3))) < y - fl ? 1 : 0));
+                    const long long j = jlo + (long long)fl;
+                    const uint32_t q = (uint32_t)(j >> 2);
+                    if (q != cq) {
+                        cq = q;
+                        cw = philox(q, 0u, p.filter, TAG_STRAT, p.key0, p.key1);
                     }
+                    n = min(noff, (int)fl + (u23f(word_of(cw, (int)(j & 3))) < y - fl ? 1 : 0));
                 }
-                th.v[i] = __int_as_float(n);
-                last_n = n;
             }
+            th.v[i] = __int_as_float(n);
+            last_n = n;
         }
     }
     // exclusive running maximum of the threads' last counts: where this thread's first run starts
@@ -410,8 +364,8 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
             }
         };
 #pragma unroll
-        for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
-            if ((KK || i < th.K) && ((th.pos >> i) & 1u)) {
+        for (int i = 0; i < KK; ++i) {
+            if ((th.pos >> i) & 1u) {
                 const int b = __float_as_int(th.v[i]);
                 if (b - a >= kLongRun) {
                     put();
@@ -461,22 +415,7 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
         const int32_t tag = (int32_t)(epoch << kLocalBits);
         const int shift = (int)(((uintptr_t)(p.anc + jlo + c0) >> 2) & 3u);  // to a 16-byte boundary
         const int need = c1 - c0 + shift;
-        if constexpr (CAP <= 4 * kThreads) {  // small staging (the multinomial guide): need <= CAP always
-            if (noff <= kChunk)
-                decode_chunk<4, KK, true>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-            else
-                decode_chunk<4, KK>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-        } else if (noff <= kChunk) {  // the tile's only chunk
-            if (need <= 4 * kThreads)
-                decode_chunk<4, KK, true>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-            else if (need <= 8 * kThreads)
-                decode_chunk<8, KK, true>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-            else if (CAP == 16 * kThreads || need <= 16 * kThreads)
-                decode_chunk<16, KK, true>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-            else
-                decode_chunk<(CAP > 16 * kThreads ? CAP : 16 * kThreads + 4) / kThreads, KK, true>(
-                    p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
-        } else if (need <= 4 * kThreads)
+        if (CAP <= 4 * kThreads || need <= 4 * kThreads)  // the multinomial guide's staging: always
             decode_chunk<4, KK>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
         else if (need <= 8 * kThreads)
             decode_chunk<8, KK>(p, sm, out, th, jlo, c0, c1, shift, start0, tile_base, tag);
@@ -1265,13 +1204,13 @@ __device__ __forceinline__ int32_t multinomial_draw_guided(uint32_t x, const Tab
 
 // This thread's samples of its tile: every 16th |v| (and the tile's last)
 // into c2, every 2^c1shift-th (and the last) into c1.
-template <int KK = 0>
+template <int KK>
 __device__ __forceinline__ void write_tile_samples(const TileThread& th, int n, float* c2, float* c1, int c1shift) {
     const int m1 = (1 << c1shift) - 1;
 #pragma unroll
-    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i) {
+    for (int i = 0; i < KK; ++i) {
         const int e = th.e0 + i;
-        if ((KK || i < th.K) && e < n) {
+        if (e < n) {
             const bool lastel = e == n - 1;
             if (((e + 1) & 15) == 0 || lastel) c2[e >> 4] = fabsf(th.v[i]);
             if (((e + 1) & m1) == 0 || lastel) c1[e >> c1shift] = fabsf(th.v[i]);
@@ -1296,65 +1235,51 @@ __device__ __forceinline__ void st_v8(float* p, const float* o) {
 }
 
 // Reloads a tile stored by write_tile_v into th (elements of tile-local
-// indices [0, n)): v from the magnitudes, the positive-weight mask from the
-// sign bits.  Slots at or beyond n are not read: they and, in threads wholly past n, the base
-// hold the last element's v, as after a scan.  SMEM: vg0 is a copy of the
-// tile in shared memory.  Every lane of the warp must call it (the bases come
-// from the lane below).
-template <int KK = 0, bool SMEM = false>  // KK: elements per thread when fixed (the tile was scanned with KK), 0 = from n
+// indices [0, n), KK a thread as scanned): v from the magnitudes, the positive-weight mask from
+// the sign bits.  Slots at or beyond n are not read: they and, in threads wholly past n, the
+// base hold the last element's v, as after a scan.  Every lane of the warp must call it
+// (the bases come from the lane below).
+template <int KK>
 __device__ __forceinline__ void read_tile_v(const float* vg0, int n, TileThread& th) {
-    const int K = KK ? KK : per_thread_count(n);
-    th.K = K;
-    th.e0 = threadIdx.x * K;
+    th.K = KK;
+    th.e0 = threadIdx.x * KK;
     const float* vg = vg0 + th.e0;
-    const bool whole = th.e0 + K <= n;
-    if (!SMEM && KK >= 8 && whole && (((uintptr_t)vg) & 31u) == 0) {
+    if (KK >= 8 && th.e0 + KK <= n && (((uintptr_t)vg) & 31u) == 0) {
 #pragma unroll
         for (int q = 0; q < KK / 8; ++q) ld_cg_v8(vg + 8 * q, th.v + 8 * q);
     } else {
 #pragma unroll
-        for (int q = 0; q < kMaxPerThread / 4; ++q) {
-            if (4 * q < K) {
-                if (th.e0 + 4 * q + 3 < n) {
-                    const float4 t = SMEM ? *reinterpret_cast<const float4*>(vg + 4 * q)
-                                          : __ldcg(reinterpret_cast<const float4*>(vg + 4 * q));
-                    th.v[4 * q] = t.x;
-                    th.v[4 * q + 1] = t.y;
-                    th.v[4 * q + 2] = t.z;
-                    th.v[4 * q + 3] = t.w;
-                } else {
+        for (int q = 0; q < KK / 4; ++q) {
+            if (th.e0 + 4 * q + 3 < n) {
+                const float4 t = __ldcg(reinterpret_cast<const float4*>(vg + 4 * q));
+                th.v[4 * q] = t.x;
+                th.v[4 * q + 1] = t.y;
+                th.v[4 * q + 2] = t.z;
+                th.v[4 * q + 3] = t.w;
+            } else {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        th.v[4 * q + r] = th.e0 + 4 * q + r < n ? (SMEM ? vg[4 * q + r] : __ldcg(vg + 4 * q + r)) : -0.0f;
-                }
+                for (int r = 0; r < 4; ++r) th.v[4 * q + r] = th.e0 + 4 * q + r < n ? __ldcg(vg + 4 * q + r) : -0.0f;
             }
         }
     }
     // the sign bits: none set in the usual thread
-    uint32_t any = 0, pos = K >= 32 ? 0xffffffffu : (1u << K) - 1u;
+    uint32_t any = 0, pos = (1u << KK) - 1u;
 #pragma unroll
-    for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
-        if (KK || i < K) any |= __float_as_uint(th.v[i]);
+    for (int i = 0; i < KK; ++i) any |= __float_as_uint(th.v[i]);
     if (any >> 31) {
         pos = 0;
-        float run = th.e0 >= n ? fabsf(SMEM ? vg0[n - 1] : __ldcg(vg0 + n - 1)) : 0.f;
+        float run = th.e0 >= n ? fabsf(__ldcg(vg0 + n - 1)) : 0.f;
 #pragma unroll
-        for (int i = 0; i < (KK ? KK : kMaxPerThread); ++i)
-            if (KK || i < K) {
-                if (!zero_flag(th.v[i])) pos |= 1u << i;
-                if (th.e0 + i < n) run = fabsf(th.v[i]);
-                th.v[i] = run;  // past the tile's end: the last element's
-            }
+        for (int i = 0; i < KK; ++i) {
+            if (!zero_flag(th.v[i])) pos |= 1u << i;
+            if (th.e0 + i < n) run = fabsf(th.v[i]);
+            th.v[i] = run;  // past the tile's end: the last element's
+        }
     }
     th.pos = pos;
     // the element before this thread's first: the lane below's last, or a load by lane 0
-    float last = th.v[0];
-#pragma unroll
-    for (int i = 1; i < (KK ? KK : kMaxPerThread); ++i)
-        if (KK || i < K) last = th.v[i];
-    th.base = __shfl_up_sync(0xffffffffu, last, 1);
-    if ((threadIdx.x & 31) == 0)
-        th.base = th.e0 == 0 ? 0.f : (th.e0 <= n ? fabsf(SMEM ? vg[-1] : __ldcg(vg - 1)) : th.v[0]);
+    th.base = __shfl_up_sync(0xffffffffu, th.v[KK - 1], 1);
+    if ((threadIdx.x & 31) == 0) th.base = th.e0 == 0 ? 0.f : (th.e0 <= n ? fabsf(__ldcg(vg - 1)) : th.v[0]);
 }
 
 // The tile's cumulative weights to global memory (sign bit: zero weight), for the searches.

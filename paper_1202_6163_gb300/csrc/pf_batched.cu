@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             continue;
         }
         if (KIND != KIND_MULTI) {
-            // ---- systematic / stratified: one tile (a one-tile filter is its own item) ----
-            const int c = c_item == kWhole ? 0 : c_item;
+            // ---- systematic / stratified: one tile of a filter split over CTAs ----
+            const int c = c_item;
             const int64_t t0 = (int64_t)c * kTileMax;
             TileSummary ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, (int)min((int64_t)kTileMax, PA - t0), sm.tile, th);
             uint32_t* rec = reinterpret_cast<uint32_t*>(bp.records + (ticket - c));  // the filter's Tf records
@@ -288,9 +288,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             if (tid == 0) {
                 trace_stamp(bp.trace, bp.trace_cap, ticket, 1);
                 int ok = 1;
-                if (Tf > 1 && c == bp.skip_tile) {
+                if (c == bp.skip_tile) {
                     ok = 0;  // test hook: withhold this tile's record; the filter's other tiles time out
-                } else if (Tf > 1) {
+                } else {
                     st_v4_u32(rec + 4 * c, (uint32_t)ts.k, __float_as_uint(ts.S.hi), __float_as_uint(ts.S.lo),
                               (uint32_t)(ts.i_last + 1) | (ts.bad ? 0x80000000u : 0u));
                     __threadfence();
@@ -304,11 +304,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                         __nanosleep(32);
                     }
                     if (!ok) set_status(bp.ctl + CTL_STATUS, ST_TIMEOUT);
-                } else {
-                    sm.rk[0] = ts.k;
-                    sm.rsh[0] = ts.S.hi;
-                    sm.rsl[0] = ts.S.lo;
-                    sm.ril[0] = ts.i_last;
                 }
                 sm.skip = !ok;
                 trace_stamp(bp.trace, bp.trace_cap, ticket, 2);
@@ -317,12 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             if (!sm.skip) {
                 if (tid < 32) {
                     uint4 r = make_uint4(0, 0, 0, 0);
-                    if (Tf > 1) {
-                        if (lane < Tf) r = ld_cg_v4_u32(rec + 4 * lane);
-                    } else if (lane == 0) {
-                        r = make_uint4((uint32_t)sm.rk[0], __float_as_uint(sm.rsh[0]), __float_as_uint(sm.rsl[0]),
-                                       (uint32_t)(sm.ril[0] + 1) | (ts.bad ? 0x80000000u : 0u));
-                    }
+                    if (lane < Tf) r = ld_cg_v4_u32(rec + 4 * lane);
                     filter_carries<KIND>(sm, bp, Tf, lane, (int)r.x, __uint_as_float(r.y), __uint_as_float(r.z),
                                          (int)(r.w & 0x7fffffffu) - 1, (int)(r.w >> 31), c == 0);
                 }
@@ -346,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 }
             }
             // the last of a split filter's CTAs to leave resets its counters
-            if (Tf > 1 && tid == 0 && atomicAdd(bp.counters + 2 * f + 1, 1u) == (uint32_t)Tf - 1u) {
+            if (tid == 0 && atomicAdd(bp.counters + 2 * f + 1, 1u) == (uint32_t)Tf - 1u) {
                 atomicExch(arrive, 0u);
                 atomicExch(bp.counters + 2 * f + 1, 0u);
             }

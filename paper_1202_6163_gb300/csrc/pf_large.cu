@@ -296,14 +296,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
 }
 
 // ---------------------------------------------------------------------------
-// Launch 3, multinomial: every draw searches the tile table, then its tile's
-// cumulative weights (the plain binary searches of Section 2's description,
-// through L2).
+// Launch 4, multinomial: each draw first reads its guide entry and one 16-element window
+// of v (quad-cooperatively, pf_assign.cuh); a lane whose four draws the guide did not all
+// settle redoes its Philox block by the plain binary searches of Section 2's description
+// over the tile table and the tile's cumulative weights, through L2 (same results).
 // ---------------------------------------------------------------------------
-// GUIDE: each draw first reads its guide entry and one 16-element window of v
-// (quad-cooperatively, pf_assign.cuh); a lane whose four draws the guide did
-// not all settle redoes its Philox block by the plain searches (same results).
-template <bool GUIDE>
 __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, const TableEntry* table,
                                                              const LargeScalars* sc, const int32_t* g, int64_t M) {
     grid_begin();
@@ -320,16 +317,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, con
         const int64_t q = mine ? q0 + threadIdx.x : 0;
         const u32x4 r = philox((uint32_t)q, 0u, p.filter, TAG_MULTI, p.key0, p.key1);
         int32_t a[4];
-        bool settled = false;
-        if (GUIDE) {
-            settled = true;
+        bool settled = true;
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                bool ok;
-                a[s] = multinomial_draw_guided(word_of(r, s), table, p.n_tiles, p.v_out, g, M, kLargeTile, PA,
-                                               p.lead, Wh, Wl, ok);
-                settled = settled && ok;
-            }
+        for (int s = 0; s < 4; ++s) {
+            bool ok;
+            a[s] = multinomial_draw_guided(word_of(r, s), table, p.n_tiles, p.v_out, g, M, kLargeTile, PA, p.lead, Wh, Wl, ok);
+            settled = settled && ok;
         }
         if (!settled)
             multinomial_draws4<false>(r, table, p.n_tiles, p.v_out, kLargeTile, PA, p.lead, Wh, Wl, a);
@@ -405,7 +398,7 @@ cudaError_t launch_large_kind(SortedParams p, unsigned char* scratch, int num_sm
         const int64_t nq = (p.P + 3) >> 2;
         int64_t gd = (nq + kThreads - 1) / kThreads;
         if (gd > (int64_t)num_sms * 16) gd = (int64_t)num_sms * 16;
-        e = launch_overlapped(k_large_draws<true>, (unsigned)gd, kThreads, 0, s, p, table, sc, g, M);
+        e = launch_overlapped(k_large_draws, (unsigned)gd, kThreads, 0, s, p, table, sc, g, M);
     }
     return e;
 }

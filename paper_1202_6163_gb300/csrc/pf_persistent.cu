@@ -747,7 +747,7 @@ static cudaError_t launch_k(const SortedParams& p, int grid, cudaStream_t s) {
         if (q <= 4) return launch_kind<KIND, 4>(p, grid, s);
         if (q <= 8) return launch_kind<KIND, 8>(p, grid, s);
     } else {
-        if (p.tiles_per_cta <= 1 && p.tagged != nullptr && grid == p.n_tiles && grid <= kThreads) {
+        if (p.tiles_per_cta <= 1) {  // one tile per CTA, at most kThreads of them
             if (q <= 4) return launch_one_tile<KIND, 4>(p, grid, s);
             if (q <= 8) return launch_one_tile<KIND, 8>(p, grid, s);
             return launch_one_tile<KIND, 16>(p, grid, s);
