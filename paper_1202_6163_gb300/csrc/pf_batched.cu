@@ -135,14 +135,16 @@ __device__ __forceinline__ void filter_carries(BatchShared& sm, const BatchParam
     }
 }
 
-// One tile's assignment.  No look for long runs: its registers spill in this kernel (612
-// bytes with, 296 without) and a batched filter's are short.  4096 filters, weights exp(N(0,1)),
-// exp(2 N), exp(4 N), systematic: 231, 240, 253 us with it, 228, 235, 276 without;
-// stratified 291, 355, 389 and 286, 339, 387.
-template <int KIND, int KK>
+// One tile's assignment.  LONG (the look for long runs) for the tiles of split filters, where
+// one warp's chunks are what the whole filter waits for: 40 filters of 1000 to 65536 particles,
+// weights exp(4 N(0,1)), systematic 33.2 us without, 18.9 with it; stratified 37.6 and 27.4.
+// Without for one-tile and whole filters: other filters fill the time, and its registers spill
+// (stratified: 320 bytes stored, 384 with it in the split tiles, 588 everywhere; 4096 filters of
+// 256 to 65536 particles, weights exp(N(0,1)): 288 us, 293 with it everywhere).
+template <int KIND, int KK, bool LONG>
 __device__ __forceinline__ void assign_batched(const SortedParams& p, AssignShared& sm, const TileMap map,
                                                int32_t* stage, TileThread& th, const TileSummary& ts, int64_t index0) {
-    assign_tile<KIND, KK, kIoCap, warp_stage_per_lane(KK), false>(p, sm, map, stage, th, ts, index0);
+    assign_tile<KIND, KK, kIoCap, warp_stage_per_lane(KK), LONG>(p, sm, map, stage, th, ts, index0);
 }
 
 // A systematic or stratified filter of one tile: scan, map and assignment with no barrier
@@ -160,7 +162,7 @@ __device__ __forceinline__ void one_tile_filter(const BatchParams& bp, const Sor
     }
     const TileMap map = only_tile_map<KIND>(p, total_pair(ts.total));
     trace_stamp(bp.trace, bp.trace_cap, ticket, 3);
-    assign_batched<KIND, KK>(p, sm.as, map, stage, th, ts, -lead);
+    assign_batched<KIND, KK, false>(p, sm.as, map, stage, th, ts, -lead);
     if (bp.trace) {
         __syncthreads();
         trace_stamp(bp.trace, bp.trace_cap, ticket, 4);
@@ -263,11 +265,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                     ts.i_last = sm.ril[c];
                     const TileMap map = sm.maps[c];
                     if (th.K == 16)
-                        assign_batched<KIND, 16>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 16, false>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else if (th.K == 8)
-                        assign_batched<KIND, 8>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 8, false>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else
-                        assign_batched<KIND, 4>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 4, false>(p, sm.as, map, stage, th, ts, t0 - lead);
                 }
                 if (bp.trace) {
                     __syncthreads();
@@ -324,11 +326,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                     const TileMap map = {sm.as.jlo, sm.as.noff, sm.as.tau0, sm.as.inv_rho};
                     // elements per thread as a constant: 16 for full tiles, fewer for small filters
                     if (th.K == 16)
-                        assign_batched<KIND, 16>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 16, true>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else if (th.K == 8)
-                        assign_batched<KIND, 8>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 8, true>(p, sm.as, map, stage, th, ts, t0 - lead);
                     else
-                        assign_batched<KIND, 4>(p, sm.as, map, stage, th, ts, t0 - lead);
+                        assign_batched<KIND, 4, true>(p, sm.as, map, stage, th, ts, t0 - lead);
                     if (bp.trace) {
                         __syncthreads();
                         trace_stamp(bp.trace, bp.trace_cap, ticket, 4);
