@@ -394,7 +394,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 const u32x4 r = philox((uint32_t)q, 0u, p.filter, TAG_MULTI, p.key0, p.key1);
                 int32_t a[4];
                 if (Tf == 1) {
-                    multinomial_draws4<true>(r, sm.table, Tf, p.v_out, kTileMax, PA, lead, sm.as.W_hi, sm.as.W_lo, a);
+                    multinomial_draws4(r, sm.table, Tf, [&](int, int64_t, int i) { return p.v_out[i]; }, kTileMax, PA, lead,
+                                       sm.as.W_hi, sm.as.W_lo, a);
                 } else {
                     const float* coarse = reinterpret_cast<const float*>(region);
 #pragma unroll

@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, con
             settled = settled && ok;
         }
         if (!settled)
-            multinomial_draws4<false>(r, table, p.n_tiles, p.v_out, kLargeTile, PA, p.lead, Wh, Wl, a);
+            multinomial_draws4(r, table, p.n_tiles,
+                               [&](int t, int64_t, int i) { return __ldcg(p.v_out + (int64_t)t * kLargeTile + i); },
+                               kLargeTile, PA, p.lead, Wh, Wl, a);
         if (!mine) continue;
         const int64_t j = 4 * q;
         if (j + 3 < p.P && (((uintptr_t)(p.anc + j)) & 15u) == 0) {

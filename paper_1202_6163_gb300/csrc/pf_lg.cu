@@ -96,7 +96,7 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* ra, float*
 
 // The initial draw, on the step's tiles of 1024 particles (one filter per CTA, so no
 // division of a particle's index, and as many CTAs as the step), or, where those leave SMs
-// idle, on tiles of 256.  Bound by instruction issue: the noise's arithmetic.  256 filters
+// idle (less than one of them for each), on tiles of 256.  Bound by instruction issue: the noise's arithmetic.  256 filters
 // of 2^16 particles: 141 -> 96 us (as a grid-stride loop over all particles, 37% of the warps
 // resident); its 335 MB take 49 us.  7 filters of 4097 particles of 16 dimensions: 35 CTAs of 1024
 // particles 6.0 us, 119 of 256 2.3.  Rows of many dimensions are drawn in the order of memory: 16 filters
@@ -302,7 +302,7 @@ static cudaError_t lg_init_tiles(LgParams p, cudaStream_t s) {
 
 cudaError_t launch_lg_init(const LgParams& p, int num_sms, cudaStream_t s) {
     const int64_t tiles = (int64_t)p.F * ((p.P + lg_tile() - 1) / lg_tile());
-    return tiles < 2 * num_sms ? lg_init_tiles<1>(p, s) : lg_init_tiles<kLgPerThread>(p, s);
+    return tiles < num_sms ? lg_init_tiles<1>(p, s) : lg_init_tiles<kLgPerThread>(p, s);
 }
 
 cudaError_t launch_lg_step(const LgParams& p, cudaStream_t s) {

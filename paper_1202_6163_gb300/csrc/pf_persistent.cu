@@ -341,7 +341,8 @@ __device__ void multinomial_draws(const SortedParams& p, PersistShared& sm, cons
                 }
             }
         } else {
-            multinomial_draws4<false>(r, table, T, p.v_out, p.tile, p.P + p.lead, p.lead, Wh, Wl, a);
+            multinomial_draws4(r, table, T, [&](int, int64_t b, int i) { return __ldcg(p.v_out + b + i); }, p.tile,
+                               p.P + p.lead, p.lead, Wh, Wl, a);
         }
         const int64_t j = 4 * q;
         if (!mine) continue;

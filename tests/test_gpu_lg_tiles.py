@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("F,P,D", [(303, 1024, 4), (304, 1024, 4), (2, 310001, 4), (5, 70001, 20), (400, 257, 64),
+@pytest.mark.parametrize("F,P,D", [(151, 1024, 4), (152, 1024, 4), (303, 1024, 4), (2, 310001, 4), (5, 70001, 20), (400, 257, 64),
                                    (151, 2047, 8), (310, 1000, 16), (1, 255, 32)])
 def test_init_tiles(F, P, D):
     x = torch.full((F * P * D + 8,), 9.0, device="cuda")
