@@ -173,8 +173,9 @@ pf_status pf_resample_metropolis(const float* logw, int64_t P, int B, uint64_t s
  *   src       [P_src][row_bytes] bytes, row-major   (in)
  *   ancestors [P_dst] int32                         (in)
  *   dst       [P_dst][row_bytes] bytes, row-major   (out; must not overlap src)
- * row_bytes must be a positive multiple of 4.  16-byte alignment of src, dst
- * and row_bytes selects 128-bit accesses; otherwise narrower ones are used.
+ * row_bytes must be a positive multiple of 4.  32-byte alignment of src, dst
+ * and row_bytes selects 256-bit accesses, 16-byte alignment 128-bit ones;
+ * otherwise narrower ones are used.
  * An ancestor outside [0, P_src) leaves that row untouched and sets device
  * status PF_ERR_INVALID.
  */

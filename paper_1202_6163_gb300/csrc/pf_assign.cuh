@@ -438,11 +438,10 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
 // own 32 S staging entries (all -1 between chunks), a warp max-scan fills them,
 // and the entries are set back to -1 as they are read for the last time.
 //
-// The CTA-wide decode below this bound waited at three barriers a tile with 40% of
-// the issue slots used.  Systematic launch at P = 2^25 + 4096 94 us (41 instructions
-// per particle), stratified 156 us (88); whole calls now: stratified at 10^8
-// particles 691 -> 417 us, 4096 filters systematic 293 -> 264 us, the 2^24 heavy-tail
-// step 252 -> 230 us.
+// Bound by instruction issue and latency at two CTAs an SM.  The CTA-wide decode waited at
+// three barriers a tile with 40% of the issue slots used: the assignment launch at P = 2^25 +
+// 4096 took 94 us systematic and 156 stratified, this way 53 and 79 (pf_large.cu); stratified
+// at 10^8 particles 691 and 391 us in all.
 //
 // N by a rounded addition: y + 1.5 2^23 rounded up (down) has ceil(y)
 // (floor(y)) in its low bits, exact for |y| < 2^22; it replaces the conversion,
@@ -451,18 +450,17 @@ __device__ void assign_offspring(const SortedParams& p, AssignShared& sm, const 
 //
 // Skewed weights: a warp whose offsets are several chunks looks for a run that goes on
 // for two chunks or more and stores it as it is, and a warp with more strata than its
-// buffer holds draws them one buffer at a time, passing over those inside a run.  With
+// buffers hold draws them one buffer at a time, passing over those inside a run.  With
 // every chunk decoded and each thread drawing its own strata, systematic, exp(4 N(0,1))
-// weights: 2^20 particles 66 us, now 27; 3 M 127, now 52; 2^24 394, now 150; stratified
-// 2^20 41, now 25; 4096 filters, exp(2 N), which look for no runs: 387, now 339.
+// weights: 2^20 particles 66 us, so 27; 2^24 394 and 150; stratified 2^20 41 and 26.
 // ---------------------------------------------------------------------------
 // A tile with more offsets than this goes to the CTA-wide decode.  One warp may own nearly
 // all of a tile's offsets (one heavy particle, or many): long runs it stores as they are,
 // and where it must decode chunk by chunk, 640 offsets at a time, the CTA's 10236 at a
 // time behind three barriers and two clears of the staging are quicker only for a great
-// many.  One weight in about 1e4 heavy, 2^24 particles, systematic, weights exp(3 N(0,1)): 98 us with the line
-// at 16384, 80 at 65536, 79 at 262144; exp(4 N) at 6e4 particles, stratified: 14.7, 12.4, 11.7;
-// 300 equally heavy particles side by side among 2^20: 56, 50, 89.
+// many.  2^24 particles, systematic, weights exp(3 N(0,1)): 98 us with the line at 16384, 80 at
+// 65536, 79 at 262144; exp(4 N) at 6e4 particles, stratified: 14.7, 12.4, 11.7; 300 equally
+// heavy particles side by side among 2^20: 56, 50, 89.
 // Without the look for long runs (LONG false) the line is at 16384.
 constexpr int kWarpOffsets = 8 * kTileMax, kWarpOffsetsShort = 2 * kTileMax;
 // A run of so many offsets of one particle, two of the warp's chunks, is stored as it is.
@@ -497,7 +495,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
         const bool clamp = nb < 0 || nl > noff;
 #pragma unroll
         for (int i = 0; i < KK; ++i)
-            th.v[i] = __int_as_float(__float_as_int(__fadd_ru(__fmaf_rn(th.v[i], ir, x0), kRoundMagic)) - kRoundMagicBits);
+            th.v[i] =
+                __int_as_float(__float_as_int(__fadd_ru(__fmaf_rn(th.v[i], ir, x0), kRoundMagic)) - kRoundMagicBits);
         if (clamp) {
 #pragma unroll
             for (int i = 0; i < KK; ++i)
@@ -533,7 +532,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
             __syncwarp();  // the last tile's reads of the buffer
             for (int b = lane; b < blocks; b += 32) {
                 const u32x4 r = philox((uint32_t)(g0 + b), 0u, p.filter, TAG_STRAT, p.key0, p.key1);
-                *reinterpret_cast<float4*>(ubuf + from + 4 * b) = make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
+                *reinterpret_cast<float4*>(ubuf + from + 4 * b) =
+                    make_float4(u23f(r.x), u23f(r.y), u23f(r.z), u23f(r.w));
             }
             __syncwarp();
             start0 = min(noff, kb + (ubuf[from + strata_index(at, kb)] < fb ? 1 : 0));
@@ -550,7 +550,8 @@ __device__ __forceinline__ void assign_warp(const SortedParams& p, const TileMap
                     const float y = __fmaf_rn(th.v[i], ir, x0);
                     float frac;
                     const int k = min(max(stratum(y, frac), 0), kmax);
-                    th.v[i] = __int_as_float(min(noff, k + (ubuf[from + strata_index(at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
+                    th.v[i] = __int_as_float(
+                        min(noff, k + (ubuf[from + strata_index(at, k)] < __fsub_rn(y, (float)k) ? 1 : 0)));
                 }
             }
             if (spill) {

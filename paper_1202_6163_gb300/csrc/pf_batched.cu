@@ -20,15 +20,15 @@
 //     CTA waits for has been or will be taken by a running CTA (the launch is
 //     cooperative, so all CTAs are resident);
 //   - unless such filters load the resident CTAs well enough by themselves
-//     (k_batched_plan has the rule): then the plan keeps each one whole, a single item whose CTA scans all its tiles
-//     (cumulative weights to the CTA's scratch), forms the carries and every
-//     tile's offset map, and assigns the tiles, with no wait on another CTA.
+//     (k_batched_plan has the rule): then the plan keeps each one whole, a single
+//     item whose CTA scans all its tiles (cumulative weights to the CTA's scratch),
+//     forms the carries and every tile's offset map, and assigns the tiles, with no
+//     wait on another CTA.
 // What bounds it: the scan's and the decode's instructions and barriers at two
 // CTAs an SM (registers), about 45% of the issue slots.  4096 filters of 256 to
-// 65536 particles, systematic: 254 us with a one-tile filter's records and
-// carries through shared memory and its tile widths found at run time, 229 us
-// now; the next ticket drawn ahead of its item 232, without the prefetch of a
-// filter's next tile into L2 230.
+// 65536 particles of spreads 0.5 to 3, systematic: 236 us (310 with a one-tile
+// filter's records and carries through shared memory, its tile widths found at
+// run time, and the CTA-wide decode).
 // A filter's data may start at any 4-byte boundary: tiles are laid out on the
 // aligned window, with the leading slots taken as zero weights.  The last CTA
 // to finish resets the ticket; the last CTA of a split filter resets its
@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
             // ---- systematic / stratified: one tile of a filter split over CTAs ----
             const int c = c_item;
             const int64_t t0 = (int64_t)c * kTileMax;
-            TileSummary ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, (int)min((int64_t)kTileMax, PA - t0), sm.tile, th);
+            const int n = (int)min((int64_t)kTileMax, PA - t0);
+            TileSummary ts = tile_scan<kReadOnly>(p.lw + t0, c == 0 ? lead : 0, n, sm.tile, th);
             uint32_t* rec = reinterpret_cast<uint32_t*>(bp.records + (ticket - c));  // the filter's Tf records
             uint32_t* arrive = bp.counters + 2 * f;
             if (tid == 0) {
@@ -394,8 +395,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_batched(BatchParams bp) {
                 const u32x4 r = philox((uint32_t)q, 0u, p.filter, TAG_MULTI, p.key0, p.key1);
                 int32_t a[4];
                 if (Tf == 1) {
-                    multinomial_draws4(r, sm.table, Tf, [&](int, int64_t, int i) { return p.v_out[i]; }, kTileMax, PA, lead,
-                                       sm.as.W_hi, sm.as.W_lo, a);
+                    multinomial_draws4(r, sm.table, Tf, [&](int, int64_t, int i) { return p.v_out[i]; }, kTileMax, PA,
+                                       lead, sm.as.W_hi, sm.as.W_lo, a);
                 } else {
                     const float* coarse = reinterpret_cast<const float*>(region);
 #pragma unroll

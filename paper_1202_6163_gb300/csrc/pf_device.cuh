@@ -175,7 +175,8 @@ __device__ __forceinline__ float fmax3_nan(float a, float b, float c) {
 __device__ __forceinline__ long long fixed48_of(float s, float c) {
     const float sc = __fmul_rn(s, 0x1p48f), cc = __fmul_rn(-c, 0x1p48f);
     if (!(s < 64.f)) return __float2ll_rn(sc) + __float2ll_rn(cc);  // weights far above 1, or NaN: c may be large too
-    // s < 64 has an error term below 2^-16, so cc fits 32 bits; sc is an integer from 2^24 on
+    // s < 64: Kahan's term is at most half an ulp of s, |c| <= 2^-19, so cc is below 2^30 and its
+    // conversion to 32 bits exact; sc is an integer from 2^24 on
     const uint32_t b = __float_as_uint(sc);
     const int sh = (int)(b >> 23) - 150;
     const long long whole = (long long)((b & 0x7fffffu) | 0x800000u) << (sh > 0 ? sh : 0);
@@ -201,7 +202,7 @@ __device__ __forceinline__ float fixed48_to_float(long long v) {
 // first lets the next such launch take its place on the GPU; a larger one leaves that
 // to its CTAs' exits, as a grid placed beside another that fills the SMs is spread
 // unevenly over them (Metropolis at P = 65536: 17 us, 36 with the early start).
-constexpr unsigned kEarlyStartCtas = 38;  // a quarter of the SMs
+constexpr unsigned kEarlyStartCtas = 38;  // a quarter of this part's 152 SMs
 __device__ __forceinline__ void grid_begin() {
     if (gridDim.x <= kEarlyStartCtas) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

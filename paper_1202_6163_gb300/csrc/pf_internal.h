@@ -64,7 +64,7 @@ struct SortedParams {
     uint32_t key0, key1, filter;
     uint32_t* ctl;
     uint64_t* slots;   // one 16-byte record per tile
-    uint64_t* tagged;  // kTaggedWords per CTA: epoch-tagged records of the one-tile-per-CTA launches, which alone write them
+    uint64_t* tagged;  // kTaggedWords per CTA: epoch-tagged records, written by the one-tile-per-CTA launches alone
     uint64_t wait_ns;
     int skip_tile;
     float* v_out;     // tile-local cumulative weights (P + lead floats): multinomial, and the tiles
@@ -89,7 +89,7 @@ struct BatchParams {
     const uint64_t* seeds;
     int32_t* anc;
     uint32_t* ctl;
-    float* scratch;           // per CTA: cumulative weights of multi-tile filters; Metropolis: weights beyond the staging
+    float* scratch;           // per CTA: cumulative weights of multi-tile filters; Metropolis: unstaged weights
     int64_t scratch_per_cta;  // floats per CTA
     const int32_t* items;     // work items from the plan pass: f * 32 + tile, or f * 32 + 31 (whole filter)
     uint4* records;           // one 16-byte tile record per item (split filters)

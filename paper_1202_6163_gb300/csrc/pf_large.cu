@@ -7,9 +7,9 @@
 //      scan (pf_tile.cuh), a 16-byte record (k_t, S_t, i_last) and the tile's
 //      cumulative weights v_i (sign bit: zero weight);
 //   2. k_large_carries: one cluster of CTAs: the largest tile exponent K, the exact
-//      prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} (128-bit fixed point), W = B_T, every tile's offset map from B_t and B_{t+1}
-//      (the same function of a boundary for both ends, so neighbouring tiles share their
-//      end exactly), and the multinomial's tile table;
+//      prefix B_t = sum_{t' < t} S_t' 2^{k_t' - K} (128-bit fixed point), W = B_T, every
+//      tile's offset map from B_t and B_{t+1} (the same function of a boundary for both
+//      ends, so neighbouring tiles share their end exactly), and the multinomial's tile table;
 //   3. k_large_assign (systematic, stratified): the tiles' offsets and their run-length
 //      decode (pf_assign.cuh), warp by warp: a warp reads its share of a tile's v_i back
 //      (not rescanned: 6-7% faster at 2^25 - 2^27 for the extra 4 B written and read per
@@ -282,7 +282,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_assign(SortedParams p, in
             read_tile_v<16>(p.v_out + t0, (int)min((int64_t)kLargeTile, PA - t0), th);
             ts.i_last = m.il;
             // without SPILL: stratified, 10^8 particles 391 us, with it 396
-            assign_tile<KIND, 16, kIoCap, S, true, false>(p, sm.as, {m.jlo, m.noff, m.x0, m.ir}, stage, th, ts, t0 - p.lead);
+            assign_tile<KIND, 16, kIoCap, S, true, false>(p, sm.as, {m.jlo, m.noff, m.x0, m.ir}, stage, th, ts,
+                                                          t0 - p.lead);
         };
         bool any = false;
         for (int r = 0; r < n; ++r) {
@@ -321,7 +322,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_large_draws(SortedParams p, con
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             bool ok;
-            a[s] = multinomial_draw_guided(word_of(r, s), table, p.n_tiles, p.v_out, g, M, kLargeTile, PA, p.lead, Wh, Wl, ok);
+            a[s] = multinomial_draw_guided(word_of(r, s), table, p.n_tiles, p.v_out, g, M, kLargeTile, PA, p.lead, Wh,
+                                           Wl, ok);
             settled = settled && ok;
         }
         if (!settled)

@@ -95,11 +95,11 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* ra, float*
 }
 
 // The initial draw, on the step's tiles of 1024 particles (one filter per CTA, so no
-// division of a particle's index, and as many CTAs as the step), or, where those leave SMs
-// idle (less than one of them for each), on tiles of 256.  Bound by instruction issue: the noise's arithmetic.  256 filters
-// of 2^16 particles: 141 -> 96 us (as a grid-stride loop over all particles, 37% of the warps
-// resident); its 335 MB take 49 us.  7 filters of 4097 particles of 16 dimensions: 35 CTAs of 1024
-// particles 6.0 us, 119 of 256 2.3.  Rows of many dimensions are drawn in the order of memory: 16 filters
+// division of a particle's index, and as many CTAs as the step), or, where those are fewer
+// than the SMs, on tiles of 256: 7 filters of 4097 particles of 16 dimensions, 35 CTAs 6.0 us,
+// 119 of them 2.3.  Bound by instruction issue: the noise's arithmetic.  256 filters of 2^16
+// particles: 94 us (141 as a grid-stride loop over all particles, 37% of the warps resident);
+// its 335 MB take 49 us.  Rows of many dimensions are drawn in the order of memory: 16 filters
 // of 70001 particles of 64 dimensions 258 us with a thread to a row, 112 so.
 template <int GS, int PER>
 __global__ void __launch_bounds__(kLgThreads) k_lg_init(LgParams p) {

@@ -74,19 +74,16 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas<VT, Place>())
 
 template <typename VT, int U>
 static cudaError_t gather_vt(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,
-                             void* dst, uint32_t* ctl, int num_sms, cudaStream_t s, int wave, int from = 8, int full = 40) {
+                             void* dst, uint32_t* ctl, int num_sms, cudaStream_t s, int wave, int from = 8,
+                             int full = 40) {
     const int64_t vecs = row_bytes / (int64_t)sizeof(VT);
     const int64_t total = P_dst * vecs;
     const RowSplit split = row_split(vecs, total);
     const unsigned blocks = chunk_grid(total, kGatherThreads * U, num_sms, wave, full, from);
-    if (split.wide())
-        return launch_overlapped(k_gather<VT, U, false, uint64_t>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split,
-                                 anc, total, (VT*)dst, ctl);
-    if (split.pow2)
-        return launch_overlapped(k_gather<VT, U, true>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc,
-                                 total, (VT*)dst, ctl);
-    return launch_overlapped(k_gather<VT, U, false>, blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc, total,
-                             (VT*)dst, ctl);
+    return launch_overlapped(split.wide()   ? k_gather<VT, U, false, uint64_t>
+                             : split.pow2 ? k_gather<VT, U, true>
+                                          : k_gather<VT, U, false>,
+                             blocks, kGatherThreads, 0, s, (const VT*)src, P_src, split, anc, total, (VT*)dst, ctl);
 }
 
 cudaError_t launch_gather(const void* src, int64_t P_src, int64_t row_bytes, const int32_t* anc, int64_t P_dst,

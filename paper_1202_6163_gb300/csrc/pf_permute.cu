@@ -21,9 +21,9 @@
 //
 // Bound by its launches and by L2 latency (five passes of 4 bytes a slot, of which
 // only the first and the last touch the caller's arrays): one memset and four
-// launches where there were three memsets and seven.  Stratified resampling,
-// permutation and in-place move of 3 M rows of 64 bytes: 212 -> 150 us, 136 us
-// with the rows in 256-bit chunks, and 116 us with more of their reads in flight.
+// launches.  Stratified resampling, permutation and in-place move of 3 M rows of 64
+// bytes: 113 us, 35 of them the permutation, 44 the rows (212 us in all with three
+// memsets and seven launches and the rows in 128-bit chunks).
 #include <climits>
 #include <type_traits>
 
@@ -149,7 +149,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_tiles(const int32_t* o, i
         const int xe = t < T ? __ldcg(&pre[t].extra) : 0, xd = t < T ? __ldcg(&pre[t].dead) : 0;
         const int xp = perm_parts(xe);
         int se, sd, sp;
-        const int pe = block_excl_scan(xe, red, se), pd = block_excl_scan(xd, red, sd), pp = block_excl_scan(xp, red, sp);
+        const int pe = block_excl_scan(xe, red, se), pd = block_excl_scan(xd, red, sd);
+        const int pp = block_excl_scan(xp, red, sp);
         if (t < T) pre[t] = {ce + pe, cd + pd, cp + pp};
         ce += se;
         cd += sd;

@@ -614,7 +614,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_one_tile(SortedParams p) {
     const int64_t PA = p.P + p.lead, t0 = (int64_t)t * p.tile;
     TileThread th;
     const TileSummary ts =
-        tile_scan_k<KK, false, kReadOnly>(p.lw + t0, t == 0 ? p.lead : 0, (int)min((int64_t)p.tile, PA - t0), sm.tile, th);
+        tile_scan_k<KK, false, kReadOnly>(p.lw + t0, t == 0 ? p.lead : 0, (int)min((int64_t)p.tile, PA - t0), sm.tile,
+                                          th);
     const uint64_t tag = (uint64_t)epoch << 32;
     if (tid == 0 && t != p.skip_tile) {
         uint64_t* rec = p.tagged + kTaggedWords * t;
@@ -783,8 +784,9 @@ static int blocks_per_sm_kk() {
             n = 0;
         nb = min(nb, n);
     };
-    if constexpr (KIND == KIND_MULTI || KK == 16) take(k_persistent<KIND, KK, false>, persistent_smem_bytes(KIND, kMaxTilesTotal, KK));
-    if constexpr (KIND == KIND_MULTI && KK == 16) take(k_persistent<KIND, KK, true>, persistent_smem_bytes(KIND, kMaxTilesTotal, KK));
+    const size_t smem = persistent_smem_bytes(KIND, kMaxTilesTotal, KK);
+    if constexpr (KIND == KIND_MULTI || KK == 16) take(k_persistent<KIND, KK, false>, smem);
+    if constexpr (KIND == KIND_MULTI && KK == 16) take(k_persistent<KIND, KK, true>, smem);
     if constexpr (KIND != KIND_MULTI) take(k_one_tile<KIND, KK>, one_tile_smem(KK));
     return nb;
 }

@@ -3,8 +3,9 @@
 // the call is an ordinary launch (a cooperative one costs 2.5 us more between calls on
 // a stream), the tiles' records are exchanged through distributed shared memory and the
 // hardware's cluster barrier instead of global memory and an arrival counter, and
-// the multinomial's draws search the cumulative weights in shared memory.  A filter of one tile needs no exchange at all: every thread forms
-// the filter's offset map from the tile's total.
+// the multinomial's draws search the cumulative weights in shared memory.  A filter of one
+// tile needs no exchange at all: every thread forms the filter's offset map from the
+// tile's total.
 //
 // Bound by latency: the load, the scan's shuffles and barriers, the boundaries' 128-bit
 // arithmetic and two divisions follow one another.  Calls back to back in a graph,
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(kThreads) k_small(SortedParams p) {
                 o[r] = ((th.pos >> i) & 1u) ? th.v[i] : -th.v[i];
             }
             if (th.e0 + 4 * q < n)  // a whole piece of four: the slots between n and it belong to this tile
-                *reinterpret_cast<float4*>(vall + t * slot + weight_place(th.e0 + 4 * q)) = make_float4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<float4*>(vall + t * slot + weight_place(th.e0 + 4 * q)) =
+                    make_float4(o[0], o[1], o[2], o[3]);
         }
     } else {
         warp_stage_init<KIND, CAP>(stage);
