@@ -453,7 +453,7 @@ size_t batched_scratch_floats_per_cta() { return (size_t)kMaxOwnB * kTileMax; }
 // counting sort; the order within a class is whatever the shared-memory
 // atomics give, and no filter's result depends on it) and writes the items
 // f * 32 + c (tile c of a split filter) or f * 32 + kWhole.  Masked and empty
-// filters get no item; a negative size or a filter beyond kMaxOwnB tiles sets
+// filters get no item; a negative size or a cumulative filter beyond kMaxOwnB tiles sets
 // PF_ERR_INVALID and gets none.  The item count goes to ctl[CTL_ITEMS].
 constexpr int kPlanThreads = 1024;
 __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* lw, const int64_t* offsets, int F,
@@ -472,11 +472,11 @@ __global__ void __launch_bounds__(kPlanThreads) k_batched_plan(const float* lw, 
         }
         const int lead = (int)(((uintptr_t)(lw + off0) >> 2) & 3u);
         const int64_t T = (n + lead + kTileMax - 1) / kTileMax;
-        if (T > kMaxOwnB) {
+        if (T > kMaxOwnB && !metro) {
             set_status(ctl + CTL_STATUS, ST_INVALID);
             return 0;
         }
-        return (int)T;
+        return (int)min(T, (int64_t)kMaxOwnB);  // a Metropolis filter has no tiles: one item whatever its size
     };
     const int first = tid < F ? tiles(tid) : 0;  // on its way before the barrier, and used twice
     if (tid <= kMaxOwnB) count[tid] = 0;
